@@ -93,6 +93,7 @@ def load(path: str = LIB_PATH):
         "cc_lr_bench_gemm": [I, I, I, I, I, P],
         "cc_lr_bench_hbm": [I, I, I, P, I],
         "cc_lr_selftest_timeout": [I, ctypes.POINTER(ctypes.c_int)],
+        "cc_lr_selftest_f64gemm": [I, I, I, I, D, ctypes.c_uint, P],
         "cc_lr_selftest_precond": [I, D, D, ctypes.c_uint, ctypes.POINTER(ctypes.c_double)],
     }
     for name, args in sig.items():
@@ -417,6 +418,13 @@ def cc_lr_selftest_precond(n=1 << 20, omega=0.0, omega_im=0.0, seed=1):
     err = ctypes.c_double(0.0)
     _check(load().cc_lr_selftest_precond(int(n), float(omega), float(omega_im), int(seed), ctypes.byref(err)))
     return err.value
+
+
+def cc_lr_selftest_f64gemm(M, N, K, layout=0, spread=0.0, seed=1):
+    """(largest error over its bound, misplaced NaNs) of the FP64 tensor-core GEMM (include/cclr_testing.h)."""
+    out = np.zeros(2, dtype=np.float64)
+    _check(load().cc_lr_selftest_f64gemm(M, N, K, layout, float(spread), seed, _ptr(out)))
+    return float(out[0]), float(out[1])
 
 
 def cc_lr_launch_count() -> int:

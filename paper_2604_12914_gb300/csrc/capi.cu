@@ -1196,6 +1196,8 @@ cclr_status cc_lr_init(cclr_ctx **ctx, int o, int v, int naux, const double *eps
     // prepared constant operands of the tensor-core contractions are kept (up to 8 GB) unless the
     // context has a budget
     c->M->E.prep_cache_cap = c->M->lean ? 0 : (size_t)8 << 30;
+    c->M->E.f64_cache_cap = c->M->lean ? 0 : (size_t)6 << 30;
+    c->acct.reclaim = [M = c->M.get()] { return M->E.f64_reclaim(); };
     c->M->upload_inputs(eps, L, mu, t1, t2, device_ptrs);
     c->M->cst_for(prec);      // intermediates in the working precision
     c->M->build_diagonal();
@@ -1860,6 +1862,73 @@ int cc_lr_selftest_precond(int n, double omega, double omega_im, unsigned seed, 
       if (std::abs(ref) > 0) mx = std::max(mx, std::abs(got - ref) / std::abs(ref));
     }
     *max_rel_err = mx;
+  });
+}
+
+int cc_lr_selftest_f64gemm(int M, int N, int K, int layout, double spread, unsigned seed, double *out) {
+  if (M < 1 || N < 1 || K < 1 || layout < 0 || layout > 31 || !(spread >= 0 && spread < 400) || !out)
+    return fail(CCLR_EINVAL, "bad selftest_f64gemm arguments");
+  return guarded([&] {
+    std::mt19937_64 g(seed);
+    std::normal_distribution<double> nd(0.0, 1.0);
+    std::uniform_real_distribution<double> ud(-spread, spread);
+    const bool ak = layout & 1, bk = layout & 2, cm = layout & 4;
+    const zd alpha = layout & 8 ? zd(0.7, -1.3) : zd(-0.5);
+    std::vector<zd> a((size_t)M * K), b((size_t)K * N), c0((size_t)M * N), c((size_t)M * N);
+    std::vector<double> am(M, 0.0), bm(N, 0.0);
+    auto A = [&](int m, int k) -> zd & { return a[ak ? (size_t)m * K + k : (size_t)k * M + m]; };
+    auto B = [&](int k, int n) -> zd & { return b[bk ? (size_t)n * K + k : (size_t)k * N + n]; };
+    auto at = [&](int m, int n) { return cm ? (size_t)n * M + m : (size_t)m * N + n; };
+    for (int m = 0; m < M; ++m) {
+      const double s = std::exp2(std::floor(ud(g)));
+      for (int k = 0; k < K; ++k) {
+        A(m, k) = zd(s * nd(g), s * nd(g));
+        am[m] = std::max({am[m], std::abs(A(m, k).real()), std::abs(A(m, k).imag())});
+      }
+    }
+    for (int n = 0; n < N; ++n) {
+      const double s = std::exp2(std::floor(ud(g)));
+      for (int k = 0; k < K; ++k) {
+        B(k, n) = zd(s * nd(g), s * nd(g));
+        bm[n] = std::max({bm[n], std::abs(B(k, n).real()), std::abs(B(k, n).imag())});
+      }
+    }
+    for (auto &z : c0) z = zd(nd(g), nd(g));
+    if (layout & 16) A(0, K / 2) = zd(std::numeric_limits<double>::quiet_NaN(), 0.0);
+    cudaStream_t st;
+    CCLR_CUDA(cudaStreamCreate(&st));
+    DevBuf Ad(a.size() * 16), Bd(b.size() * 16), Cd(c.size() * 16), As((size_t)f64tc_bytes(M, K, false)),
+        Bs((size_t)f64tc_bytes(N, K, true)), At((size_t)M * 4), Bt((size_t)N * 4), Sc(f64tc_scratch_bytes(M, N));
+    CCLR_CUDA(cudaMemcpyAsync(Ad.p, a.data(), Ad.bytes, cudaMemcpyHostToDevice, st));
+    CCLR_CUDA(cudaMemcpyAsync(Bd.p, b.data(), Bd.bytes, cudaMemcpyHostToDevice, st));
+    CCLR_CUDA(cudaMemcpyAsync(Cd.p, c0.data(), Cd.bytes, cudaMemcpyHostToDevice, st));
+    const F64Op oa = f64tc_prep(Ad.p, view1(ak ? K : 1), view1(ak ? 1 : M), M, K, false, As.p, At.as<uint32_t>(), st);
+    const F64Op ob = f64tc_prep(Bd.p, view1(bk ? K : 1), view1(bk ? 1 : N), N, K, true, Bs.p, Bt.as<uint32_t>(), st);
+    f64tc_gemm(oa, M, ob, N, K, Cd.p, view1(cm ? 1 : N), view1(cm ? M : 1), zc(alpha.real(), alpha.imag()), true, Sc.p, st);
+    CCLR_CUDA(cudaMemcpyAsync(c.data(), Cd.p, Cd.bytes, cudaMemcpyDeviceToHost, st));
+    if (tc_error(st)) throw Error(CCLR_ETIMEOUT, "tensor-core kernel gave up on a bounded wait");
+    CCLR_CUDA(cudaStreamDestroy(st));
+    const double u = std::exp2(-53.0), ext = K * std::exp2(-59.0) + (double)K * K * std::exp2(-67.0);
+    const size_t total = (size_t)M * N, step = std::max<size_t>(1, total / 4000);
+    out[0] = out[1] = 0.0;
+    for (size_t q = 0; q < total; q += step) {
+      const int m = (int)(q / N), n = (int)(q % N);
+      const zd got = c[at(m, n)], old = c0[at(m, n)];
+      const bool nan = (layout & 16) && m == 0;
+      if (nan != std::isnan(got.real()) || nan != std::isnan(got.imag())) out[1] += 1.0;
+      if (nan) continue;
+      long double re = 0.0L, im = 0.0L;
+      for (int k = 0; k < K; ++k) {
+        const zd x = A(m, k), y = B(k, n);
+        re += (long double)x.real() * y.real() - (long double)x.imag() * y.imag();
+        im += (long double)x.real() * y.imag() + (long double)x.imag() * y.real();
+      }
+      const long double wr = old.real() + (alpha.real() * re - alpha.imag() * im);
+      const long double wi = old.imag() + (alpha.real() * im + alpha.imag() * re);
+      const double mag = std::abs(alpha) * std::hypot((double)re, (double)im) + std::abs(old);
+      const double lim = 8 * u * mag + std::abs(alpha) * am[m] * bm[n] * ext;
+      out[0] = std::max({out[0], (double)std::abs(got.real() - wr) / lim, (double)std::abs(got.imag() - wi) / lim});
+    }
   });
 }
 

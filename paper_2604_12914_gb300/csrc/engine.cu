@@ -29,10 +29,16 @@ void DevBuf::alloc(size_t b) {
   release();
   if (b == 0) return;
   MemAcct *a = current_acct();
-  if (a && a->budget && a->used + b > a->budget)
+  auto over = [&] { return a && a->budget && a->used + b > a->budget; };
+  if (over() && a->reclaim) a->reclaim();
+  if (over())
     throw Error(2, "HBM budget of " + std::to_string(a->budget) + " bytes exceeded: " + std::to_string(a->used) +
                        " bytes held, " + std::to_string(b) + " more requested");
   cudaError_t e = cudaMalloc(&p, b);
+  if (e == cudaErrorMemoryAllocation && a && a->reclaim && a->reclaim()) {
+    (void)cudaGetLastError();
+    e = cudaMalloc(&p, b);
+  }
   if (e != cudaSuccess) {
     p = nullptr;
     (void)cudaGetLastError();
@@ -73,6 +79,9 @@ double2 *Engine::dot_scratch() {
   return dots_.as<double2>();
 }
 double2 *Engine::dot_results() { return dot_scratch() + 512; }
+
+// complex128 contractions from this many multiply-adds on run on the tensor cores
+static constexpr double kF64MinWork = 2.0e6;
 
 static int mode_pos(const std::string &m, char c) {
   auto k = m.find(c);
@@ -312,6 +321,14 @@ void Engine::contract(zc alpha, const Tens &A, const std::string &ma, const Tens
     return;
   }
 
+  // complex128 on tensor cores from exact slices, from 2e6 multiply-adds on (below, the slicing costs more than
+  // the CUDA cores): the longer side as rows, the shorter one as the (twice as large) columns
+  if (dt == C128 && nb <= 16 && (double)M * N * K >= kF64MinWork && K < (1ll << 28)) {
+    if (N > M ? contract_f64(alpha, B, mb, A, ma, C, mc, bat, Nm, Mm, Km, nb, N, M, K)
+              : contract_f64(alpha, A, ma, B, mb, C, mc, bat, Mm, Nm, Km, nb, M, N, K))
+      return;
+  }
+
   // An output mode that keeps the M or N group from being one strided index in both of its
   // operands is peeled off as a batch index (stride 0 in the operand that lacks it), so that
   // no operand is permuted; batch modes proper take precedence.
@@ -407,9 +424,187 @@ void Engine::contract(zc alpha, const Tens &A, const std::string &ma, const Tens
   }
 }
 
+bool Engine::f64_reclaim() {
+  if (f64_holds_ || (f64_slots_.empty() && f64_kept_.empty() && !f64_scr_.p)) return false;
+  f64_slots_.clear();
+  f64_scr_.release();
+  f64_kept_.clear();
+  f64_kept_bytes_ = 0;
+  return true;
+}
+
+F64Op Engine::f64_operand(int slot, const void *src, View2 rv, View2 kv, int64_t R, int64_t K, bool embed,
+                          const std::string &key) {
+  const size_t sl = ((size_t)f64tc_bytes(R, K, embed) + 255) / 256 * 256, need = sl + (size_t)R * 4;
+  if (!key.empty()) {
+    PrepEntry *e = nullptr;
+    for (auto &x : f64_kept_)
+      if (x->key == key) e = x.get();
+    if (e && e->filled && e->buf.bytes == need) {
+      F64Op op;
+      op.p = e->buf.p;
+      op.tops = (const uint32_t *)((const char *)e->buf.p + sl);
+      op.stride = R;
+      return op;
+    }
+    if (!e && f64_kept_bytes_ + need <= f64_cache_cap) {
+      auto n = std::make_unique<PrepEntry>();
+      n->key = key;
+      try {
+        n->buf.alloc(need);
+        f64_kept_bytes_ += need;
+        f64_kept_.push_back(std::move(n));
+        e = f64_kept_.back().get();
+      } catch (const Error &x) {  // no room to keep it: the workspace slot serves
+        if (x.status != 2) throw;
+      }
+    }
+    if (e && e->buf.bytes == need) {
+      const F64Op op = f64tc_prep(src, rv, kv, R, K, embed, e->buf.p, (uint32_t *)((char *)e->buf.p + sl), st);
+      e->filled = true;
+      return op;
+    }
+  }
+  f64_reserve(slot, R, K, embed);
+  char *b = (char *)f64_slots_[slot].p;
+  return f64tc_prep(src, rv, kv, R, K, embed, b, (uint32_t *)(b + sl), st);
+}
+
+void Engine::f64_scratch(int64_t M, int64_t N) {
+  const size_t need = f64tc_scratch_bytes(M, N);
+  if (f64_scr_.bytes >= need) return;
+  if (f64_scr_.p) CCLR_CUDA(cudaStreamSynchronize(st));
+  f64_scr_.alloc(need);
+}
+
+void Engine::f64_gemm(const F64Op &A, int64_t M, const F64Op &B, int64_t N, int64_t K, void *C, View2 rv, View2 cv, zc alpha,
+                      bool accumulate) {
+  f64_scratch(M, N);
+  tc_pending = true;
+  f64tc_gemm(A, M, B, N, K, C, rv, cv, alpha, accumulate, f64_scr_.p, st);
+}
+
+void Engine::check_tc() {
+  if (!tc_pending) return;
+  tc_pending = false;
+  if (tc_error(st)) throw Error(5, "a tensor-core kernel gave up on a bounded wait");
+}
+
+void Engine::f64_reserve(int slot, int64_t R, int64_t K, bool embed) {
+  if ((int)f64_slots_.size() <= slot) f64_slots_.resize(slot + 1);
+  DevBuf &b = f64_slots_[slot];
+  const size_t need = ((size_t)f64tc_bytes(R, K, embed) + 255) / 256 * 256 + (size_t)R * 4;
+  if (b.bytes < need) {
+    if (b.p) CCLR_CUDA(cudaStreamSynchronize(st));
+    b.alloc(need);
+  }
+}
+
+// One index of a contraction operand as a strided view that is read in unit-stride runs
+static bool runs_of(const View2 &x, int64_t n) {
+  return x.sin == 1 && (x.din == TC_ONE_LEVEL ? n : x.din) >= std::min<int64_t>(8, n);
+}
+
+bool Engine::contract_f64(zc alpha, const Tens &A, const std::string &ma, const Tens &B, const std::string &mb,
+                          const Tens &C, const std::string &mc, const std::string &bat, const std::string &Mm,
+                          const std::string &Nm, const std::string &Km, int64_t nb, int64_t M, int64_t N, int64_t K) {
+  const size_t es = dt_size(C128);
+  int64_t a0, b0, c0;
+  View2 am, ak, bk, bn, cm, cn;
+  auto view = [&](const Tens &T, const std::string &mt, const std::string &g1, const std::string &g2, int64_t &s0, View2 &v1,
+                  int64_t n1, View2 &v2, int64_t n2) {
+    int64_t z;
+    return group_view(T, mt, bat, z, s0) && group_view2(T, mt, g1, v1) && group_view2(T, mt, g2, v2) &&
+           (runs_of(v1, n1) || runs_of(v2, n2));
+  };
+  // operands and results whose modes need more than two levels, or whose runs are short, go through a
+  // contiguous copy; slices of an operand are bounded (2 GiB), in chunks of whole blocks of a two-level view
+  const bool a_ok = view(A, ma, Mm, Km, a0, am, M, ak, K), b_ok = view(B, mb, Km, Nm, b0, bk, K, bn, N);
+  const bool direct = view(C, mc, Mm, Nm, c0, cm, M, cn, N);
+  if (!a_ok) { a0 = M * K; am = view1(K); ak = view1(1); }
+  if (!b_ok) { b0 = K * N; bk = view1(N); bn = view1(1); }
+  if (!direct) { c0 = M * N; cm = view1(N); cn = view1(1); }
+  auto unit_of = [](const View2 &x, const View2 &y) {
+    int64_t u = 1;
+    if (x.din != TC_ONE_LEVEL) u = std::lcm(u, x.din);
+    if (y.din != TC_ONE_LEVEL) u = std::lcm(u, y.din);
+    return u;
+  };
+  auto chunk = [](int64_t n, int64_t per, int64_t u) {
+    const int64_t cap = (2ll << 30) / per;
+    return n > cap && u < n ? std::max(u, cap / u * u) : n;
+  };
+  const int64_t Mc = chunk(M, f64tc_bytes(1, K, false), unit_of(am, cm)), Nc = chunk(N, f64tc_bytes(1, K, true), unit_of(bn, cn));
+  if ((double)F64_SLICES * std::max(Mc, 2 * Nc) >= 2147483648.0) return false;
+  const void *Ap = A.p, *Bp = B.p;
+  Tens T;
+  std::string akey, bkey;
+  if (f64_cache_cap && cst_hint && (cst_hint == A.p || cst_hint == B.p)) {
+    char hint[40];
+    std::snprintf(hint, sizeof hint, "%p|", cst_hint);
+    if (cst_hint == A.p) akey = std::string("A") + hint + ma + "|" + bat + "|" + Mm + "|" + Km + "|";
+    else bkey = std::string("B") + hint + mb + "|" + bat + "|" + Km + "|" + Nm + "|";
+  }
+  auto at = [](const std::string &key, int64_t b, int64_t r) {
+    return key.empty() ? key : key + std::to_string(b) + "," + std::to_string(r);
+  };
+  // a kept operand whose slices are all there needs no contiguous copy
+  auto have = [&](const std::string &key, int64_t n, int64_t step) {
+    if (key.empty()) return false;
+    for (int64_t b = 0; b < nb; ++b)
+      for (int64_t r = 0; r < n; r += step) {
+        bool f = false;
+        for (auto &x : f64_kept_) f = f || (x->key == at(key, b, r) && x->filled);
+        if (!f) return false;
+      }
+    return true;
+  };
+  F64Hold hold(*this);
+  try {
+    if (!a_ok && !have(akey, M, Mc)) Ap = ws(0, nb * M * K * es);
+    if (!b_ok && !have(bkey, N, Nc)) Bp = ws(1, nb * K * N * es);
+    if (!direct) T = contiguous_like(ws(2, nb * M * N * es), C128, C, mc, bat + Mm + Nm);
+    // the workspace for the slices is claimed before anything is computed
+    f64_scratch(Mc, Nc);
+    if (!have(akey, M, Mc)) f64_reserve(0, Mc, K, false);
+    if (!have(bkey, N, Nc)) f64_reserve(1, Nc, K, true);
+  } catch (const Error &e) {
+    if (e.status != 2) throw;
+    return false;
+  }
+  if (!a_ok && Ap != A.p) {
+    Tens P = contiguous_like((void *)Ap, C128, A, ma, bat + Mm + Km);
+    permute(zc(1.0), A, ma, P, bat + Mm + Km, false);
+  }
+  if (!b_ok && Bp != B.p) {
+    Tens P = contiguous_like((void *)Bp, C128, B, mb, bat + Km + Nm);
+    permute(zc(1.0), B, mb, P, bat + Km + Nm, false);
+  }
+  if (trace_on())
+    std::fprintf(stderr, "cclr contract f64 %s,%s->%s nb=%lld M=%lld N=%lld K=%lld A[%s|%s]%s B[%s|%s]%s C[%s|%s]%s\n", ma.c_str(),
+                 mb.c_str(), mc.c_str(), (long long)nb, (long long)M, (long long)N, (long long)K, vstr(am).c_str(),
+                 vstr(ak).c_str(), Ap == A.p ? "" : "(permuted)", vstr(bk).c_str(), vstr(bn).c_str(),
+                 Bp == B.p ? "" : "(permuted)", vstr(cm).c_str(), vstr(cn).c_str(), direct ? "" : "(temporary)");
+  if (!direct) CCLR_CUDA(cudaMemsetAsync(T.p, 0, (size_t)(nb * M * N) * es, st));
+  for (int64_t b = 0; b < nb; ++b) {
+    char *Cb = (char *)(direct ? C.p : T.p) + b * c0 * es;
+    for (int64_t n0 = 0; n0 < N; n0 += Nc) {
+      const int64_t nn = std::min(Nc, N - n0);
+      const F64Op ob = f64_operand(1, (const char *)Bp + (b * b0 + v2off(bn, n0)) * es, bn, bk, nn, K, true, at(bkey, b, n0));
+      for (int64_t m0 = 0; m0 < M; m0 += Mc) {
+        const int64_t mm = std::min(Mc, M - m0);
+        const F64Op oa = f64_operand(0, (const char *)Ap + (b * a0 + v2off(am, m0)) * es, am, ak, mm, K, false, at(akey, b, m0));
+        f64_gemm(oa, mm, ob, nn, K, Cb + (v2off(cm, m0) + v2off(cn, n0)) * es, cm, cn, alpha, true);
+      }
+    }
+  }
+  if (!direct) permute(zc(1.0), T, bat + Mm + Nm, C, mc, true);
+  return true;
+}
+
 Engine::PrepEntry *Engine::prep_find(const std::string &key) {
   for (auto &e : prep_)
-    if (e->key == key) return e->epoch == state_epoch() ? e.get() : nullptr;
+    if (e->key == key) return e->filled ? e.get() : nullptr;
   return nullptr;
 }
 
@@ -430,6 +625,7 @@ void Engine::contract_tc(zc alpha, const Tens &A, const std::string &ma, const T
                          const std::string &bat, const std::string &Mm, const std::string &Nm,
                          const std::string &Km, int64_t nb, int64_t M, int64_t N, int64_t K) {
   const size_t es = dt_size(C64);
+  tc_pending = true;
   int64_t a0, b0, c0, z;
   View2 am, ak, bk, bn, cm, cn;
   const void *Ap = A.p, *Bp = B.p;
@@ -474,7 +670,7 @@ void Engine::contract_tc(zc alpha, const Tens &A, const std::string &ma, const T
         PrepEntry *fa = cache_a && seg == 1 ? prep_get(akey + "P", (size_t)(nb * M * K * es)) : nullptr;
         Tens T = contiguous_like(fa ? fa->buf.p : ws(0, nb * M * K * es), C64, A, ma, order);
         permute(zc(1.0), A, ma, T, order, false);
-        if (fa) fa->epoch = state_epoch();
+        if (fa) fa->filled = true;
         Ap = T.p;
       }
     }
@@ -558,8 +754,8 @@ void Engine::contract_tc(zc alpha, const Tens &A, const std::string &ma, const T
     }
     ++tc_calls;
   }
-  if (wa && !used_direct) wa->epoch = state_epoch();
-  if (wb) wb->epoch = state_epoch();
+  if (wa && !used_direct) wa->filled = true;
+  if (wb) wb->filled = true;
   if (!direct) permute(zc(1.0), T, bat + Mm + Nm, C, mc, true);
 }
 

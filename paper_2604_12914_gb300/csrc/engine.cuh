@@ -1,10 +1,12 @@
 // Host-side tensor-contraction engine: device buffers, workspace, einsum-style
 // contractions mapped onto the strided complex GEMM, permutes and vector helpers.
 #pragma once
+#include <functional>
 #include <memory>
 #include <string>
 #include <vector>
 
+#include "f64_tc.cuh"
 #include "kernels.cuh"
 
 namespace cclr {
@@ -13,6 +15,9 @@ namespace cclr {
 // an optional limit (0 = none) that every allocation charged to it is checked against.
 struct MemAcct {
   size_t used = 0, peak = 0, budget = 0;
+  // frees what the owner keeps only for speed; true if anything was freed.  An allocation that fails or
+  // would exceed the budget calls it and tries once more.
+  std::function<bool()> reclaim;
 };
 // The account that allocations made on this thread are charged to (nullptr: none).
 MemAcct *&current_acct();
@@ -25,8 +30,8 @@ struct AcctScope {
   AcctScope &operator=(const AcctScope &) = delete;
 };
 
-// Owning device allocation.  An allocation over the current account's budget throws status 2
-// (CCLR_ENOMEM) before cudaMalloc is called; the bytes are returned to the same account when
+// Owning device allocation.  An allocation over the current account's budget (after its reclaim) throws
+// status 2 (CCLR_ENOMEM) before cudaMalloc is called; the bytes are returned to the same account when
 // the buffer is released, whichever thread releases it.
 struct DevBuf {
   void *p = nullptr;
@@ -68,7 +73,11 @@ class Engine {
   // Workspace slot s of at least `bytes` bytes (grown on demand, reused across calls).
   void *ws(int slot, size_t bytes);
   // frees the workspace slots (they grow again on demand)
-  void release_ws() { slots_.clear(); }
+  void release_ws() {
+    slots_.clear();
+    f64_slots_.clear();
+    f64_scr_.release();
+  }
   // C[mc] += alpha * sum A[ma] B[mb] over the modes not in mc (einsum semantics; every
   // mode must appear in exactly two operands or in all three).
   void contract(zc alpha, const Tens &A, const std::string &ma, const Tens &B,
@@ -77,6 +86,34 @@ class Engine {
   void contract_tc(zc alpha, const Tens &A, const std::string &ma, const Tens &B, const std::string &mb,
                    const Tens &C, const std::string &mc, const std::string &bat, const std::string &Mm,
                    const std::string &Nm, const std::string &Km, int64_t nb, int64_t M, int64_t N, int64_t K);
+  // the complex128 tensor-core branch (f64_tc.cuh); false: no memory for the operands' slices, nothing done
+  bool contract_f64(zc alpha, const Tens &A, const std::string &ma, const Tens &B, const std::string &mb, const Tens &C,
+                    const std::string &mc, const std::string &bat, const std::string &Mm, const std::string &Nm,
+                    const std::string &Km, int64_t nb, int64_t M, int64_t N, int64_t K);
+  // Slices of a complex128 operand (f64tc_prep) in workspace slot `slot`, or, with a key, kept until
+  // clear_prep_cache() like the other constant operands (at most f64_cache_cap bytes).  Throws status 2.
+  F64Op f64_operand(int slot, const void *src, View2 rv, View2 kv, int64_t R, int64_t K, bool embed,
+                    const std::string &key);
+  // room for the sums of an M x N f64tc_gemm (throws status 2), and the product itself on this engine's stream
+  void f64_scratch(int64_t M, int64_t N);
+  void f64_gemm(const F64Op &A, int64_t M, const F64Op &B, int64_t N, int64_t K, void *C, View2 rv, View2 cv, zc alpha,
+                bool accumulate);
+  // Throws status 5 if a tensor-core kernel launched since the last check gave up on a bounded wait
+  // (synchronises the stream; nothing is done when none was launched).
+  void check_tc();
+  bool tc_pending = false;
+  // claims workspace slot `slot` for R rows of K entries.  Throws status 2.
+  void f64_reserve(int slot, int64_t R, int64_t K, bool embed);
+  size_t f64_cache_cap = 0;
+  // Holds off f64_reclaim() while prepared slices are in use on the host side.
+  struct F64Hold {
+    Engine &e;
+    explicit F64Hold(Engine &e_) : e(e_) { ++e.f64_holds_; }
+    ~F64Hold() { --e.f64_holds_; }
+    F64Hold(const F64Hold &) = delete;
+  };
+  // frees the FP64 slices (workspace and kept operands); true if there were any
+  bool f64_reclaim();
   // out[mo] (+)= alpha * in[mi]  (same mode set; dtypes may differ -> conversion).
   void permute(zc alpha, const Tens &in, const std::string &mi, const Tens &out,
                const std::string &mo, bool acc);
@@ -84,15 +121,17 @@ class Engine {
   double2 *dot_scratch();  // device: partials [>=304] and results [64]
   double2 *dot_results();
   // Constant operands: while cst_hint points at one operand of a tensor-core contraction, the
-  // prepared form of that operand (its permuted copy, or its TF32 / BF16 embedded rows or columns)
-  // is kept and reused by later contractions of the same operand with the same modes and
-  // precision, as long as state_epoch() has not moved (no device memory freed, no constants
-  // rebuilt); at most prep_cache_cap bytes (0: off).
+  // prepared form of that operand (its permuted copy, its TF32 / BF16 embedded rows or columns, or its
+  // FP64 slices) is kept and reused by later contractions of the same operand with the same modes and
+  // precision; at most prep_cache_cap (f64_cache_cap) bytes (0: off).  Whoever rewrites or frees a
+  // constant calls clear_prep_cache() before and after.
   const void *cst_hint = nullptr;
   size_t prep_cache_cap = 0;
   void clear_prep_cache() {
     prep_.clear();
     prep_bytes_ = 0;
+    f64_kept_.clear();
+    f64_kept_bytes_ = 0;
   }
   size_t prep_cache_bytes() const { return prep_bytes_; }
 
@@ -102,7 +141,7 @@ class Engine {
   struct PrepEntry {
     std::string key;
     DevBuf buf;
-    unsigned long long epoch = 0;  // the entry's content is valid while state_epoch() equals it
+    bool filled = false;
   };
   std::vector<std::unique_ptr<PrepEntry>> prep_;
   size_t prep_bytes_ = 0;
@@ -110,6 +149,11 @@ class Engine {
   PrepEntry *prep_find(const std::string &key);
   // the entry to (re)fill, created if needed; nullptr when it would exceed the cap
   PrepEntry *prep_get(const std::string &key, size_t bytes);
+  std::vector<DevBuf> f64_slots_;  // two per slot: slices, tops
+  std::vector<std::unique_ptr<PrepEntry>> f64_kept_;  // slices, then tops in the same buffer
+  size_t f64_kept_bytes_ = 0;
+  DevBuf f64_scr_;
+  int f64_holds_ = 0;
 };
 
 }  // namespace cclr

@@ -1,0 +1,754 @@
+// FP64-accurate complex GEMM on tcgen05 from exact 8-bit slices; see f64_tc.cuh.
+//
+// This GPU's FP64 pipe does two FMAs per clock and SM, so a complex GEMM on it stops near 1 TFLOP/s.  The
+// 36 BF16 slice products (orders q <= 7) cost 36 times a BF16 GEMM and still leave some 25 times more.
+// Measured (GEMM and output kernel, operands sliced): M = N = K = 1760 complex 1.81 ms (24 TFLOP/s, 870 TFLOP/s of
+// BF16 MMAs) against 42 ms on the FP64 pipe; 12100 x 1760 x 500 3.5 ms against 90; 400^3 51 us against 617.
+// What bounds it: MMAs alone (never waiting for the epilogue) 1.09 ms at 1760^3; handing each order's accumulator to
+// the epilogue and back, 1.5 ms; with the epilogue's integer work, 1.8 ms.
+#include <atomic>
+#include <cmath>
+#include <type_traits>
+
+#include "engine.cuh"
+#include "f64_tc.cuh"
+#include "tc_ptx.cuh"
+
+namespace cclr {
+namespace {
+
+constexpr int S = F64_SLICES;
+constexpr int BM = 128;
+constexpr int KC = 32;                  // real K per chunk: 64-byte slice rows, and S_q <= 8 * 2^14 * 32 = 2^22 exact
+constexpr int A_SLOT = BM * KC * 2;     // bytes of one slice block of A
+constexpr int NSLOT = 12;               // ring of (A_s, B_s) slot pairs: one chunk of 8 and half of the next
+constexpr int NBUF = 4;                 // accumulators in TMEM
+constexpr int MAX_CHUNKS = 2048;        // per launch, 65536 real K: |S_0| 2^32 stays below 2^62
+constexpr int SPLIT_TILES = 76;         // K is split when at most this many tiles (half the SMs) exist
+
+struct F64Params {
+  int sA, sB, rA, rB;   // slice rows per slice of A and B, first slice row
+  int nMt, nNt, band, splits, chunks_per_split;
+  int chunk0, chunk1;   // chunks of KC of this K segment
+  long long *hi;        // integer sums, [split][tile][column][row]: hi + lo 2^-8, in units of 2^(ea + eb - 46)
+  float *lo;
+  int *err;
+};
+
+// C += or = alpha times the sums, through C's views
+struct F64Out {
+  int m0, n0, M, N;     // first row and complex column of the tiles; C's extents
+  int nMt, nNt, splits, cols_fast, accumulate;
+  const long long *hi;
+  const float *lo;
+  const uint32_t *ea, *eb;  // rows' and columns' maxima (scale_of gives the exponents)
+  double *C;
+  View2 rv, cv;
+  double ar, ai;        // alpha (used unless pow2)
+  int pow2, neg, sh;    // alpha = (-1)^neg 2^sh
+};
+
+__device__ __forceinline__ void unit_coords(const F64Params &p, int u, int &mt, int &nt, int &sp) {
+  const int tiles = p.nMt * p.nNt;
+  sp = u / tiles;
+  const int id = u - sp * tiles, per_band = p.band * p.nNt, b = id / per_band, local = id - b * per_band;
+  const int mb = min(p.band, p.nMt - b * p.band);
+  mt = b * p.band + local % mb;
+  nt = local / mb;
+}
+
+// One MMA of K = 16 (32 bytes per row), D (+)= A B^T, both operands K-major with 64-byte swizzled rows (8-row
+// groups 512 bytes apart), given by the low words of their descriptors: address >> 4, leading offset 1.
+__device__ __forceinline__ uint32_t sw64_lo(uint32_t saddr) { return ((saddr & 0x3FFFF) >> 4) | (1u << 16); }
+__device__ __forceinline__ void mma_sw64(uint32_t tmem, uint32_t a, uint32_t b, uint32_t idesc, bool acc) {
+  // high word: stride offset 512 >> 4, version 1, SWIZZLE_64B
+  constexpr uint32_t hi = (512u >> 4) | (1u << 14) | (4u << 29);
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\tmov.b64 da, {%1, %3};\n\tmov.b64 db, {%2, %3};\n\t"
+      "setp.ne.b32 p, %5, 0;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, p;\n\t}"
+      :
+      : "r"(tmem), "r"(a), "r"(b), "r"(hi), "r"(idesc), "r"(acc ? 1 : 0));
+}
+
+// W accumulator columns of the warp's 32 rows into registers (no wait), W = 8, 16 or 32
+template <int W> __device__ __forceinline__ void tmem_ld(uint32_t a, uint32_t (&r)[W]);
+template <> __device__ __forceinline__ void tmem_ld<8>(uint32_t a, uint32_t (&r)[8]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+               : "r"(a));
+}
+template <> __device__ __forceinline__ void tmem_ld<16>(uint32_t a, uint32_t (&r)[16]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+               : "r"(a));
+}
+template <> __device__ __forceinline__ void tmem_ld<32>(uint32_t a, uint32_t (&r)[32]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+               : "r"(a));
+}
+// completes every load issued before it; hold() passes registers through so that no use of them moves above
+__device__ __forceinline__ void tmem_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+template <int W> __device__ __forceinline__ void hold(uint32_t (&r)[W]) {
+#pragma unroll
+  for (int k = 0; k < W; ++k) asm volatile("" : "+r"(r[k])::"memory");
+}
+
+// scale e of a row from the largest high word of its entries' magnitudes: every |x| < 2^e
+__device__ __forceinline__ int scale_of(uint32_t m) {
+  const int ex = (int)(m >> 20);
+  return ex == 0x7ff ? F64_NONFINITE : max(ex, 1) - 1022;
+}
+
+// An integer-valued float of magnitude <= 2^22 as the low bits of x + 1.5 * 2^23 (minus MAGIC)
+constexpr uint32_t MAGIC = 0x4B400000u;
+__device__ __forceinline__ uint32_t fbits(uint32_t r) { return __float_as_uint(__uint_as_float(r) + 12582912.f); }
+
+// lo 2^s rounded to an integer (|result| < 2^62), from the bits of lo
+__device__ __forceinline__ long long scaled_int(float lo, int s) {
+  const uint32_t b = __float_as_uint(lo), ex = (b >> 23) & 0xff;
+  const unsigned long long m = ex ? (b & 0x7fffffu) | 0x800000u : 0u;
+  const int sh = (int)ex - 150 + s;
+  const unsigned long long r = sh >= 0 ? m << sh : sh < -25 ? 0ull : ((m >> (-sh - 1)) + 1) >> 1;
+  return (int)b < 0 ? -(long long)r : (long long)r;
+}
+
+// 2^e (hi 2^-46 + lo 2^-54), negated if neg: hi is shifted up as far as it goes (24 bits at most), lo rounded into
+// the bits below it, and the sum rounded once to FP64 (ties to even), in integer arithmetic: the FP64 pipe would
+// take longer for its conversions and scalings than the MMAs of a short K.
+__device__ __forceinline__ double combine(long long hi, float lo, int e, int neg) {
+  const int s = max(0, min(24, __clzll(hi < 0 ? -hi : hi) - 2));
+  const long long tot = (hi << s) + scaled_int(lo, s - 8);
+  if (tot == 0) return 0.0;
+  unsigned long long m = (unsigned long long)(tot < 0 ? -tot : tot);
+  const unsigned long long sign = ((tot < 0) != (neg != 0)) ? 1ull << 63 : 0ull;
+  const int lz = __clzll(m), ex = 1023 + 63 - lz + e - 46 - s;  // biased exponent of the leading bit
+  m <<= lz;
+  m = (m + 0x3ffull + ((m >> 11) & 1)) < m ? 1ull << 53 : (m + 0x3ffull + ((m >> 11) & 1)) >> 11;
+  if (ex > 0 && ex < 0x7fe) return __longlong_as_double((long long)(sign | (((unsigned long long)(ex - 1) << 52) + m)));
+  // towards the ends of the range: [1, 2] scaled in steps that stay representable
+  const double r = __longlong_as_double((long long)(sign | ((1022ull << 52) + m)));
+  const int d = max(-2200, min(2200, ex - 1023)), d1 = d / 3, d2 = (d - d1) / 2;
+  auto two = [](int k) { return __hiloint2double((1023 + k) << 20, 0); };
+  return r * two(d1) * two(d2) * two(d - d1 - d2);
+}
+
+// The slice products (two MMAs each) of orders 7 - P, 5 - P, 3 - P, 1 - P of the n-th chunk, whose slices 7 .. 0 are
+// in slots G0, G0 + 1, ...
+template <int BN, int G0, int P>
+__device__ __forceinline__ bool issue_chunk(uint8_t *smem, uint32_t tmem, uint32_t idesc, uint64_t *tfull, uint64_t *tempty,
+                                            uint64_t *empty, int *err, volatile int *abort_flag) {
+  constexpr int SLOT = A_SLOT + BN * KC * 2;
+#pragma unroll
+  for (int q = S - 1 - P; q >= 0; q -= 2) {
+    const int buf = (S - 1 - q) % NBUF;
+    // accumulator buf is used twice per chunk; it is free when its previous order has been read
+    if (!mbar_wait_ab(su32(tempty + buf), q < S - NBUF ? 0u : 1u, err, abort_flag)) return false;
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const uint32_t d = tmem + (uint32_t)(buf * BN);
+    uint32_t base = sw64_lo(su32(smem));
+    asm volatile("" : "+r"(base));  // slot addresses are formed here, not kept in registers
+#pragma unroll
+    for (int i = 0; i <= q; ++i) {
+      const uint32_t da = base + (((G0 + S - 1 - i) % NSLOT) * SLOT >> 4);
+      const uint32_t db = base + ((((G0 + S - 1 - (q - i)) % NSLOT) * SLOT + A_SLOT) >> 4);
+      mma_sw64(d, da, db, idesc, i != 0);
+      mma_sw64(d, da + 2, db + 2, idesc, true);
+    }
+    mma_commit(su32(tfull + buf));
+    // slices q and q - 1 (and 7, which the orders of P = 1 never read) are not read by this warp's later orders
+    if (q == S - 2) mma_commit(su32(empty + G0 % NSLOT));
+    mma_commit(su32(empty + (G0 + S - 1 - q) % NSLOT));
+    if (q > 0) mma_commit(su32(empty + (G0 + S - q) % NSLOT));
+  }
+  return true;
+}
+
+// Warp 0 streams slice blocks with TMA into a ring of (A_s, B_s) slots, s = 7 first: the orders of a chunk are
+// issued as q = 7 .. 0, order q is the last to read slice q, so slots free up in the order they were filled.
+// Warp 1 issues the MMAs of order q into TMEM accumulator (7 - q) % 4.  Warps 4-11 add the exact sums of each
+// order to a 64-bit integer (q <= 4, two orders at a time as one 32-bit integer) or a float (q = 5, 6, 7, below
+// 2^-40 of the total) per output, and store both once per unit.  192 accumulator registers per thread:
+// setmaxnreg gives the two epilogue warpgroups 232 and the first one 40 (of 168 at launch).
+template <int BN>
+__global__ void __launch_bounds__(384, 1)
+    f64_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, F64Params p) {
+  constexpr int B_SLOT = BN * KC * 2, SLOT = A_SLOT + B_SLOT, NC = BN / 2;
+  constexpr uint32_t TCOLS = NBUF * BN;
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+  uint64_t *bars = (uint64_t *)(smem + NSLOT * SLOT);
+  uint64_t *full = bars, *empty = full + NSLOT, *tfull = empty + NSLOT, *tempty = tfull + NBUF, *drain = tempty + NBUF;
+  uint32_t *tslot = (uint32_t *)(drain + 2);
+  int *issued = (int *)(tslot + 1), *consumed = issued + 1;
+  volatile int *abort_flag = issued + 2;
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
+  const int units = p.nMt * p.nNt * p.splits;
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < NSLOT; ++s) {
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(su32(full + s)) : "memory");
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 2;" ::"r"(su32(empty + s)) : "memory");
+    }
+    for (int b = 0; b < NBUF; ++b) {
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(su32(tfull + b)) : "memory");
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 8;" ::"r"(su32(tempty + b)) : "memory");
+    }
+    for (int b = 0; b < 2; ++b) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(su32(drain + b)) : "memory");
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    issued[0] = 0;
+    consumed[0] = 0;
+    *abort_flag = 0;
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(su32(tslot)), "r"(TCOLS)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t tmem = __shfl_sync(0xffffffffu, *tslot, 0);
+
+  if (warp < 4) {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 40;");
+    if (warp == 0 && lane == 0) {
+      int g = 0;
+      bool ok = true;
+      for (int u = blockIdx.x; u < units && ok; u += gridDim.x) {
+        int mt, nt, sp;
+        unit_coords(p, u, mt, nt, sp);
+        const int c0 = p.chunk0 + sp * p.chunks_per_split, c1 = min(p.chunk1, c0 + p.chunks_per_split);
+        for (int c = c0; c < c1 && ok; ++c)
+          for (int s = S - 1; s >= 0; --s, ++g) {
+            const int slot = g % NSLOT;
+            if (!mbar_wait_ab(su32(empty + slot), ((uint32_t)(g / NSLOT) & 1u) ^ 1u, p.err, abort_flag)) { ok = false; break; }
+            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(su32(full + slot)),
+                         "r"((uint32_t)SLOT)
+                         : "memory");
+            tma_load_2d(smem + slot * SLOT, &tmA, c * KC, s * p.sA + p.rA + mt * BM, su32(full + slot));
+            tma_load_2d(smem + slot * SLOT + A_SLOT, &tmB, c * KC, s * p.sB + p.rB + nt * BN, su32(full + slot));
+            issued[0] = g + 1;
+          }
+      }
+    } else if ((warp == 1 || warp == 2) && lane == 0) {
+      const uint32_t idesc = idesc_mma(TC_BF16, BM, BN);
+      int g = 0;  // first slot of the chunk
+      bool ok = true;
+      for (int u = blockIdx.x; u < units && ok; u += gridDim.x) {
+        int mt, nt, sp;
+        unit_coords(p, u, mt, nt, sp);
+        const int c0 = p.chunk0 + sp * p.chunks_per_split, c1 = min(p.chunk1, c0 + p.chunks_per_split);
+        for (int c = c0; c < c1 && ok; ++c, g += S) {
+          for (int k = 0; k < S && ok; ++k) {
+            const int slot = (g + k) % NSLOT;
+            ok = mbar_wait_ab(su32(full + slot), (uint32_t)((g + k) / NSLOT) & 1u, p.err, abort_flag);
+            if (ok && warp == 1) consumed[0] = g + k + 1;
+          }
+          if (!ok) break;
+          // the chunk's first slot is 0, 4 or 8: slot offsets are constants in each case, so that the issuing
+          // thread spends a few instructions per MMA
+          const int g0 = g % NSLOT;
+          auto chunk = [&](auto G) {
+            constexpr int G0 = decltype(G)::value;
+            return warp == 1 ? issue_chunk<BN, G0, 0>(smem, tmem, idesc, tfull, tempty, empty, p.err, abort_flag)
+                             : issue_chunk<BN, G0, 1>(smem, tmem, idesc, tfull, tempty, empty, p.err, abort_flag);
+          };
+          ok = g0 == 0 ? chunk(std::integral_constant<int, 0>()) : g0 == 4 ? chunk(std::integral_constant<int, 4>())
+                                                                           : chunk(std::integral_constant<int, 8>());
+        }
+      }
+      mma_commit(su32(drain + warp - 1));
+      mbar_wait(su32(drain + warp - 1), 0, p.err);
+    }
+    __syncwarp();
+  } else {
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 232;");
+    const int quarter = warp & 3, h = (warp - 4) >> 2;
+    const uint32_t tb = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(h * NC);
+    bool ok = true;
+    for (int u = blockIdx.x; u < units && ok; u += gridDim.x) {
+      int mt, nt, sp;
+      unit_coords(p, u, mt, nt, sp);
+      const int c0 = p.chunk0 + sp * p.chunks_per_split, c1 = min(p.chunk1, c0 + p.chunks_per_split);
+      long long hi[NC];
+      float lo[NC];
+#pragma unroll
+      for (int c = 0; c < NC; ++c) { hi[c] = 0; lo[c] = 0.f; }
+      auto wait = [&](int buf, uint32_t use) {
+        const bool w = mbar_wait_ab(su32(tfull + buf), use, p.err, abort_flag);
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        return __all_sync(0xffffffffu, w) != 0;
+      };
+      auto release = [&](int buf) {
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        __syncwarp();
+        if (lane == 0) mbar_arrive(su32(tempty + buf));
+      };
+      for (int ch = c0; ch < c1; ++ch) {
+        constexpr int W1 = NC < 32 ? NC : 32, W2 = 16;  // columns per TMEM load
+        // q = 7, 6, 5 (accumulators 0, 1, 2): a float below the integer
+        auto low = [&](int buf, float w) {
+#pragma unroll
+          for (int c = 0; c < NC; c += W1) {
+            uint32_t x[W1];
+            tmem_ld<W1>(tb + buf * BN + c, x);
+            tmem_wait();
+            hold(x);
+#pragma unroll
+            for (int k = 0; k < W1; ++k) lo[c + k] = fmaf(__uint_as_float(x[k]), w, lo[c + k]);
+          }
+        };
+        // two orders at a time as one 32-bit integer: S_(q-1) 2^8 + S_q
+        auto pair = [&](int bx, int by, int shift) {
+#pragma unroll
+          for (int c = 0; c < NC; c += W2) {
+            uint32_t x[W2], y[W2];
+            tmem_ld<W2>(tb + bx * BN + c, x);
+            tmem_ld<W2>(tb + by * BN + c, y);
+            tmem_wait();
+            hold(x);
+            hold(y);
+#pragma unroll
+            for (int k = 0; k < W2; ++k)
+              hi[c + k] += (long long)(int)((fbits(y[k]) << 8) + fbits(x[k]) - (MAGIC * 257u)) * (1ll << shift);
+          }
+        };
+        if (!(ok = wait(0, 0))) break;
+        low(0, 0x1p-16f);
+        release(0);
+        if (!(ok = wait(1, 0))) break;
+        low(1, 0x1p-8f);
+        release(1);
+        if (!(ok = wait(2, 0))) break;
+        low(2, 1.f);
+        release(2);
+        if (!(ok = wait(3, 0) && wait(0, 1))) break;
+        pair(3, 0, 0);  // q = 4, 3
+        release(3);
+        release(0);
+        if (!(ok = wait(1, 1) && wait(2, 1))) break;
+        pair(1, 2, 16);  // q = 2, 1
+        release(1);
+        release(2);
+        if (!(ok = wait(3, 1))) break;
+#pragma unroll
+        for (int c = 0; c < NC; c += W1) {  // q = 0
+          uint32_t x[W1];
+          tmem_ld<W1>(tb + 3 * BN + c, x);
+          tmem_wait();
+          hold(x);
+#pragma unroll
+          for (int k = 0; k < W1; ++k) hi[c + k] += (long long)((unsigned long long)(fbits(x[k]) - MAGIC) << 32);
+        }
+        release(3);
+      }
+      if (!ok) break;
+      const int64_t at = (((int64_t)sp * p.nMt * p.nNt + (int64_t)nt * p.nMt + mt) * BN + h * NC) * BM + quarter * 32 + lane;
+#pragma unroll
+      for (int c = 0; c < NC; ++c) {
+        p.hi[at + c * BM] = hi[c];
+        p.lo[at + c * BM] = lo[c];
+      }
+    }
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  if (threadIdx.x == 0 && consumed[0] < issued[0])  // error path: drain copies issued but never consumed (bounded)
+    for (int g = consumed[0]; g < issued[0]; ++g) mbar_wait(su32(full + g % NSLOT), (uint32_t)(g / NSLOT) & 1u, p.err);
+  __syncthreads();
+  if (warp == 1)
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TCOLS) : "memory");
+}
+
+// The integer sums to FP64: a block takes 32 rows by 16 complex columns of a tile, reads the sums of every K
+// split along the rows (as the GEMM wrote them), adds them exactly, and writes C along its contiguous direction
+// (through shared memory when that is the columns).  This is a kernel of its own because the conversion is some
+// hundred dependent integer instructions per value: at the GEMM's eight warps per SM, with the accumulators
+// holding all registers, it took 50 us per tile, as long as the MMAs of K = 250.
+template <int BN>
+__global__ void __launch_bounds__(256) f64_out_kernel(F64Out p) {
+  __shared__ double2 T[32][17];
+  const int lane = threadIdx.x, y = threadIdx.y;
+  int b = blockIdx.x;
+  const int cg = b % (BN / 32);
+  b /= BN / 32;
+  const int rg = b % 4, tile = b / 4, mt = tile % p.nMt, nt = tile / p.nMt;
+  const int r0 = p.m0 + mt * BM + rg * 32, c0 = p.n0 + nt * (BN / 2) + cg * 16;
+  if (r0 >= p.M || c0 >= p.N) return;
+  const int row = r0 + lane;
+  const int er = row < p.M ? scale_of(p.ea[row]) : 0;
+  const int64_t plane = (int64_t)p.nMt * p.nNt * BN * BM;
+#pragma unroll
+  for (int q = 0; q < 2; ++q) {
+    const int j = y + 8 * q, n = c0 + j;
+    if (n < p.N) {
+      const int64_t at = ((int64_t)tile * BN + cg * 32 + 2 * j) * BM + rg * 32 + lane;
+      long long hr = 0, hm = 0;
+      double2 v;
+      if (p.splits == 1) {
+        hr = p.hi[at];
+        hm = p.hi[at + BM];
+      }
+      float lr = p.lo[at], lm = p.lo[at + BM];
+      if (p.splits > 1) {  // the low parts as integers of 2^-16
+        long long ir = 0, im = 0;
+#pragma unroll 4
+        for (int s = 0; s < p.splits; ++s) {
+          hr += p.hi[at + s * plane];
+          hm += p.hi[at + s * plane + BM];
+          ir += scaled_int(p.lo[at + s * plane], 16);
+          im += scaled_int(p.lo[at + s * plane + BM], 16);
+        }
+        lr = (float)ir * 0x1p-16f;
+        lm = (float)im * 0x1p-16f;
+      }
+      const int e = er + scale_of(p.eb[n]);
+      v.x = combine(hr, lr, e + p.sh, p.neg);
+      v.y = combine(hm, lm, e + p.sh, p.neg);
+      if (!p.pow2) v = make_double2(p.ar * v.x - p.ai * v.y, p.ar * v.y + p.ai * v.x);
+      if (e >= F64_NONFINITE / 2) v.x = v.y = __longlong_as_double(0x7ff8000000000000ll);
+      if (p.cols_fast) {
+        T[lane][j] = v;
+      } else if (row < p.M) {
+        double2 *dst = (double2 *)p.C + v2off(p.rv, row) + v2off(p.cv, n);
+        if (p.accumulate) { const double2 o = *dst; v.x += o.x; v.y += o.y; }
+        *dst = v;
+      }
+    }
+  }
+  if (!p.cols_fast) return;
+  __syncthreads();
+  const int t = y * 32 + lane, j = t & 15, n = c0 + j;
+  if (n >= p.N) return;
+  const int64_t co = v2off(p.cv, n);
+#pragma unroll
+  for (int q = 0; q < 2; ++q) {
+    const int rl = (t >> 4) + 16 * q;
+    if (r0 + rl >= p.M) break;
+    double2 *dst = (double2 *)p.C + v2off(p.rv, r0 + rl) + co, v = T[rl][j];
+    if (p.accumulate) { const double2 o = *dst; v.x += o.x; v.y += o.y; }
+    *dst = v;
+  }
+}
+
+// The same for many K splits of a small C: a block takes 32 rows of one complex column, its eight warps share the
+// splits.
+template <int BN>
+__global__ void __launch_bounds__(256) f64_out_split_kernel(F64Out p) {
+  __shared__ long long T[4][8][33];
+  const int lane = threadIdx.x, y = threadIdx.y;
+  int b = blockIdx.x;
+  const int j = b % (BN / 2);
+  b /= BN / 2;
+  const int rg = b % 4, tile = b / 4, mt = tile % p.nMt, nt = tile / p.nMt;
+  const int row = p.m0 + mt * BM + rg * 32 + lane, n = p.n0 + nt * (BN / 2) + j;
+  if (n >= p.N || p.m0 + mt * BM + rg * 32 >= p.M) return;
+  const int64_t plane = (int64_t)p.nMt * p.nNt * BN * BM, at = ((int64_t)tile * BN + 2 * j) * BM + rg * 32 + lane;
+  long long t[4] = {0, 0, 0, 0};  // hi and lo 2^16, real and imaginary
+#pragma unroll 4
+  for (int s = y; s < p.splits; s += 8) {
+    t[0] += p.hi[at + s * plane];
+    t[1] += p.hi[at + s * plane + BM];
+    t[2] += scaled_int(p.lo[at + s * plane], 16);
+    t[3] += scaled_int(p.lo[at + s * plane + BM], 16);
+  }
+#pragma unroll
+  for (int k = 0; k < 4; ++k) T[k][y][lane] = t[k];
+  __syncthreads();
+  if (y != 0 || row >= p.M) return;
+#pragma unroll
+  for (int k = 0; k < 4; ++k)
+    for (int q = 1; q < 8; ++q) t[k] += T[k][q][lane];
+  const int e = scale_of(p.ea[row]) + scale_of(p.eb[n]);
+  double2 v;
+  v.x = combine(t[0], (float)t[2] * 0x1p-16f, e + p.sh, p.neg);
+  v.y = combine(t[1], (float)t[3] * 0x1p-16f, e + p.sh, p.neg);
+  if (!p.pow2) v = make_double2(p.ar * v.x - p.ai * v.y, p.ar * v.y + p.ai * v.x);
+  if (e >= F64_NONFINITE / 2) v.x = v.y = __longlong_as_double(0x7ff8000000000000ll);
+  double2 *dst = (double2 *)p.C + v2off(p.rv, row) + v2off(p.cv, n);
+  if (p.accumulate) { const double2 o = *dst; v.x += o.x; v.y += o.y; }
+  *dst = v;
+}
+
+// ---------------- slices ----------------
+__device__ __forceinline__ uint32_t mag(double x) { return (uint32_t)__double2hiint(x) & 0x7fffffffu; }
+__device__ __forceinline__ uint32_t mag2(double2 z) { return max(mag(z.x), mag(z.y)); }
+
+// x 2^(63 - e) rounded to an integer (63 bits and sign), from the bits of x: no FP64 arithmetic
+__device__ __forceinline__ long long fixed63(double x, int e) {
+  const uint32_t h = (uint32_t)__double2hiint(x);
+  const int ex = (int)((h >> 20) & 0x7ff);
+  unsigned long long f = ((unsigned long long)((h & 0xfffffu) | (ex ? 0x100000u : 0u)) << 32) | (uint32_t)__double2loint(x);
+  const int sh = max(ex, 1) - 1012 - e;  // at most 10
+  if (sh >= 0) f <<= sh;
+  else f = sh < -54 ? 0ull : ((f >> (-sh - 1)) + 1) >> 1;
+  return (int)h < 0 ? -(long long)f : (long long)f;
+}
+
+// the next balanced digit (-128 .. 127) from below, as BF16 bits
+__device__ __forceinline__ uint32_t digit(long long &X) {
+  const int d = (int)(signed char)(X & 0xff);
+  X = (X - d) >> 8;
+  return __float_as_uint(__uint_as_float(MAGIC + (uint32_t)d) - 12582912.f) >> 16;
+}
+
+// eight slices of one complex entry at real columns 2k, 2k+1 of slice row r (R rows per slice)
+template <bool EMBED>
+__device__ __forceinline__ void put_slices(uint32_t *dst, int64_t R, int64_t ld2, int64_t r, int64_t k, double2 z, int e) {
+  long long X = fixed63(z.x, e), Y = fixed63(z.y, e);
+  if (e == F64_NONFINITE) X = Y = 0;
+#pragma unroll
+  for (int s = S - 1; s >= 0; --s) {
+    uint32_t a, b;
+    if (s > 0) {
+      a = digit(X);
+      b = digit(Y);
+    } else {  // the top digit, up to +-128
+      a = __float_as_uint(__uint_as_float(MAGIC + (uint32_t)(int)X) - 12582912.f) >> 16;
+      b = __float_as_uint(__uint_as_float(MAGIC + (uint32_t)(int)Y) - 12582912.f) >> 16;
+    }
+    if (EMBED) {
+      uint32_t *row = dst + ((int64_t)s * 2 * R + 2 * r) * ld2 + k;
+      row[0] = a | ((b ^ 0x8000u) << 16);
+      row[ld2] = b | (a << 16);
+    } else {
+      dst[((int64_t)s * R + r) * ld2 + k] = a | (b << 16);
+    }
+  }
+}
+
+// Rows contiguous along k: T threads per row find the row's largest magnitude, then read it again (from
+// L1/L2) and write its slices, coalesced along k.
+template <int T, bool EMBED>
+__global__ void __launch_bounds__(256) f64_slice_rows(const double2 *__restrict__ src, View2 rv, View2 kv, int64_t R, int64_t K,
+                                                      uint32_t *__restrict__ dst, int64_t ld2, uint32_t *__restrict__ tops) {
+  __shared__ uint32_t red[8];
+  const int t = threadIdx.x % T;
+  const int64_t r = (int64_t)blockIdx.x * (256 / T) + threadIdx.x / T;
+  const double2 *row = src + (r < R ? v2off(rv, r) : 0);
+  uint32_t m = 0;
+  if (r < R)
+    for (int64_t k = t; k < K; k += T) m = max(m, mag2(row[v2off(kv, k)]));
+  m = __reduce_max_sync(0xffffffffu, m);
+  if (T > 32) {
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
+    __syncthreads();
+    for (int w = 0; w < T / 32; ++w) m = max(m, red[w]);
+  }
+  if (r >= R) return;
+  if (t == 0) tops[r] = m;
+  const int e = scale_of(m);
+  for (int64_t k = t; k < K; k += T) put_slices<EMBED>(dst, R, ld2, r, k, row[v2off(kv, k)], e);
+}
+
+// The same for a few long rows: blocks over ranges of k, maxima first.
+__global__ void __launch_bounds__(256) f64_rowmax(const double2 *__restrict__ src, View2 rv, View2 kv, int64_t K, int64_t kstep,
+                                                  uint32_t *__restrict__ tops) {
+  const double2 *row = src + v2off(rv, blockIdx.x);
+  const int64_t k1 = min(K, (int64_t)(blockIdx.y + 1) * kstep);
+  uint32_t m = 0;
+  for (int64_t k = (int64_t)blockIdx.y * kstep + threadIdx.x; k < k1; k += 256) m = max(m, mag2(row[v2off(kv, k)]));
+  m = __reduce_max_sync(0xffffffffu, m);
+  if ((threadIdx.x & 31) == 0) atomicMax(tops + blockIdx.x, m);
+}
+template <bool EMBED>
+__global__ void __launch_bounds__(256) f64_slice_range(const double2 *__restrict__ src, View2 rv, View2 kv, int64_t R, int64_t K,
+                                                       int64_t kstep, uint32_t *__restrict__ dst, int64_t ld2,
+                                                       const uint32_t *__restrict__ tops) {
+  const int64_t r = blockIdx.x, k1 = min(K, (int64_t)(blockIdx.y + 1) * kstep);
+  const double2 *row = src + v2off(rv, r);
+  const int e = scale_of(tops[r]);
+  for (int64_t k = (int64_t)blockIdx.y * kstep + threadIdx.x; k < k1; k += 256)
+    put_slices<EMBED>(dst, R, ld2, r, k, row[v2off(kv, k)], e);
+}
+
+// Rows contiguous along r (k strided): maxima by threads along r over a range of k, then 32 x 32 transposing
+// tiles.
+__global__ void __launch_bounds__(256) f64_colmax(const double2 *__restrict__ src, View2 rv, View2 kv, int64_t R, int64_t K,
+                                                  int64_t kstep, uint32_t *__restrict__ tops) {
+  const int64_t r = (int64_t)blockIdx.x * 256 + threadIdx.x;
+  if (r >= R) return;
+  const double2 *row = src + v2off(rv, r);
+  const int64_t k1 = min(K, (int64_t)(blockIdx.y + 1) * kstep);
+  uint32_t m = 0;
+#pragma unroll 4
+  for (int64_t k = (int64_t)blockIdx.y * kstep; k < k1; ++k) m = max(m, mag2(row[v2off(kv, k)]));
+  atomicMax(tops + r, m);
+}
+template <bool EMBED>
+__global__ void __launch_bounds__(256) f64_slice_tiled(const double2 *__restrict__ src, View2 rv, View2 kv, int64_t R, int64_t K,
+                                                       uint32_t *__restrict__ dst, int64_t ld2,
+                                                       const uint32_t *__restrict__ tops) {
+  __shared__ double2 tile[32][33];
+  const int64_t tr = (R + 31) / 32, tk = (K + 31) / 32;
+  for (int64_t t = blockIdx.x; t < tr * tk; t += gridDim.x) {
+    const int64_t r0 = (t % tr) * 32, k0 = (t / tr) * 32;
+    for (int q = threadIdx.y; q < 32; q += 8) {
+      const int64_t r = r0 + threadIdx.x, k = k0 + q;
+      tile[q][threadIdx.x] = (r < R && k < K) ? src[v2off(rv, r) + v2off(kv, k)] : make_double2(0.0, 0.0);
+    }
+    __syncthreads();
+    for (int q = threadIdx.y; q < 32; q += 8) {
+      const int64_t r = r0 + q, k = k0 + threadIdx.x;
+      if (r < R && k < K) put_slices<EMBED>(dst, R, ld2, r, k, tile[threadIdx.x][q], scale_of(tops[r]));
+    }
+    __syncthreads();
+  }
+}
+
+template <bool EMBED>
+void prep_launch(const double2 *src, View2 rv, View2 kv, int64_t R, int64_t K, uint32_t *dst, uint32_t *tops, cudaStream_t st) {
+  const int64_t ld2 = f64tc_ld(K) / 2;
+  const bool kfast = kv.sin == 1 || rv.sin != 1;
+  if (kfast && !(R < 2 * 152 && K >= 2048)) {
+    if (K >= 512) f64_slice_rows<256, EMBED><<<(unsigned)R, 256, 0, st>>>(src, rv, kv, R, K, dst, ld2, tops);
+    else f64_slice_rows<32, EMBED><<<(unsigned)((R + 7) / 8), 256, 0, st>>>(src, rv, kv, R, K, dst, ld2, tops);
+    count_launch();
+    return;
+  }
+  CCLR_CUDA(cudaMemsetAsync(tops, 0, (size_t)R * sizeof(uint32_t), st));
+  if (kfast) {  // about four blocks per SM over ranges of at least 1024
+    const int64_t ky = std::max<int64_t>(1, std::min<int64_t>({(4 * 152 + R - 1) / R, K / 1024, (int64_t)65535}));
+    const int64_t kstep = (K + ky - 1) / ky;
+    const dim3 g((unsigned)R, (unsigned)((K + kstep - 1) / kstep));
+    f64_rowmax<<<g, 256, 0, st>>>(src, rv, kv, K, kstep, tops);
+    f64_slice_range<EMBED><<<g, 256, 0, st>>>(src, rv, kv, R, K, kstep, dst, ld2, tops);
+  } else {
+    const int64_t bx = (R + 255) / 256;
+    const int64_t ky = std::max<int64_t>(1, std::min<int64_t>({(4 * 152 + bx - 1) / bx, (K + 15) / 16, (int64_t)65535}));
+    const int64_t kstep = (K + ky - 1) / ky;
+    f64_colmax<<<dim3((unsigned)bx, (unsigned)((K + kstep - 1) / kstep)), 256, 0, st>>>(src, rv, kv, R, K, kstep, tops);
+    const int64_t nt = ((R + 31) / 32) * ((K + 31) / 32);
+    f64_slice_tiled<EMBED><<<(unsigned)std::min<int64_t>(nt, 152 * 64), dim3(32, 8), 0, st>>>(src, rv, kv, R, K, dst, ld2, tops);
+  }
+  count_launch(2);
+}
+
+template <int BN> size_t smem_bytes() {
+  return 1024 + (size_t)NSLOT * (A_SLOT + BN * KC * 2) + (2 * NSLOT + 2 * NBUF + 2) * 8 + 16;
+}
+
+// one launch of the GEMM over the tiles of p (rows rowsA of A from p.rA, columns of B from p.rB), and its output
+template <int BN>
+void launch(const F64Op &A, const F64Op &B, const F64Params &p, F64Out &o, int64_t K, cudaStream_t st) {
+  static std::atomic<unsigned long long> attr_set{0};  // one bit per device
+  int dev = 0;
+  CCLR_CUDA(cudaGetDevice(&dev));
+  if (dev >= 64 || !(attr_set.load() & (1ull << dev))) {
+    CCLR_CUDA(cudaFuncSetAttribute(f64_gemm_kernel<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes<BN>()));
+    if (dev < 64) attr_set |= 1ull << dev;
+  }
+  const int64_t ld = f64tc_ld(K);
+  const CUtensorMap ma = tc_make_map(A.p, (int64_t)S * p.sA, 2 * K, ld, BM, 64, TC_BF16);
+  const CUtensorMap mb = tc_make_map(B.p, (int64_t)S * p.sB, 2 * K, ld, BN, 64, TC_BF16);
+  const int64_t tiles = (int64_t)p.nMt * p.nNt, units = tiles * p.splits;
+  f64_gemm_kernel<BN><<<(unsigned)std::min<int64_t>(units, tc_num_sms()), 384, smem_bytes<BN>(), st>>>(ma, mb, p);
+  CCLR_CUDA(cudaGetLastError());
+  o.hi = p.hi;
+  o.lo = p.lo;
+  o.nMt = p.nMt;
+  o.nNt = p.nNt;
+  o.splits = p.splits;
+  if (p.splits > 8) f64_out_split_kernel<BN><<<(unsigned)(tiles * 4 * (BN / 2)), dim3(32, 8), 0, st>>>(o);
+  else f64_out_kernel<BN><<<(unsigned)(tiles * 4 * (BN / 32)), dim3(32, 8), 0, st>>>(o);
+  CCLR_CUDA(cudaGetLastError());
+  count_launch(2);
+}
+
+// columns of tiles and rows of tiles of one launch, the K splits and the bytes of their sums
+struct F64Plan {
+  int BN, nMt, nNt, rows, cols;  // tiles in all; tile rows and tile columns per launch
+  int64_t unit;                  // bytes of one tile's sums
+};
+F64Plan plan_of(int64_t M, int64_t N, size_t cap) {
+  F64Plan q;
+  q.BN = 2 * N <= 32 ? 32 : 2 * N <= 64 ? 64 : 128;
+  q.nMt = (int)((M + BM - 1) / BM);
+  q.nNt = (int)((2 * N + q.BN - 1) / q.BN);
+  q.unit = (int64_t)BM * q.BN * 12;
+  const int64_t fit = std::max<int64_t>(1, (int64_t)cap / q.unit);
+  q.rows = (int)std::min<int64_t>(q.nMt, fit);
+  q.cols = (int)std::max<int64_t>(1, std::min<int64_t>(q.nNt, fit / q.rows));
+  return q;
+}
+constexpr size_t SUMS_CAP = 256u << 20;  // the most that the sums of one launch take
+
+}  // namespace
+
+F64Op f64tc_prep(const void *src, View2 rv, View2 kv, int64_t R, int64_t K, bool embed, void *dst, uint32_t *tops,
+                 cudaStream_t st) {
+  CCLR_REQUIRE(R > 0 && K > 0 && (int64_t)S * 2 * R < (1ll << 31) && 2 * K < (1ll << 31), "f64tc_prep: bad dimensions");
+  if (embed) prep_launch<true>((const double2 *)src, rv, kv, R, K, (uint32_t *)dst, tops, st);
+  else prep_launch<false>((const double2 *)src, rv, kv, R, K, (uint32_t *)dst, tops, st);
+  CCLR_CUDA(cudaGetLastError());
+  F64Op op;
+  op.p = dst;
+  op.tops = tops;
+  op.stride = R;
+  return op;
+}
+
+size_t f64tc_scratch_bytes(int64_t M, int64_t N) {
+  const F64Plan q = plan_of(M, N, SUMS_CAP);
+  // split K: at most one unit per SM
+  return (size_t)std::max<int64_t>((int64_t)q.rows * q.cols, (int64_t)q.nMt * q.nNt <= SPLIT_TILES ? tc_num_sms() : 0) * q.unit;
+}
+
+void f64tc_gemm(const F64Op &A, int64_t M, const F64Op &B, int64_t N, int64_t K, void *C, View2 rv, View2 cv, zc alpha,
+                bool accumulate, void *scratch, cudaStream_t st) {
+  if (M <= 0 || N <= 0 || K <= 0) return;
+  CCLR_REQUIRE(A.r0 + M <= A.stride && B.r0 + N <= B.stride, "f64tc_gemm: rows outside the prepared operand");
+  CCLR_REQUIRE((uintptr_t)A.p % 16 == 0 && (uintptr_t)B.p % 16 == 0, "f64tc_gemm: operands must be 16-byte aligned");
+  const F64Plan pl = plan_of(M, N, SUMS_CAP);
+  F64Params p;
+  p.sA = (int)A.stride;
+  p.sB = (int)(2 * B.stride);
+  p.err = tc_device_err();
+  F64Out o;
+  o.M = (int)M;
+  o.N = (int)N;
+  o.C = (double *)C;
+  o.rv = rv;
+  o.cv = cv;
+  o.cols_fast = cv.sin == 1 && (cv.din == TC_ONE_LEVEL || cv.din >= 4) ? 1 : 0;
+  o.ea = A.tops + A.r0;
+  o.eb = B.tops + B.r0;
+  o.ar = alpha.re;
+  o.ai = alpha.im;
+  int ex = 0;
+  o.pow2 = alpha.im == 0.0 && std::abs(std::frexp(alpha.re, &ex)) == 0.5;
+  o.sh = o.pow2 ? ex - 1 : 0;
+  o.neg = o.pow2 && alpha.re < 0.0;
+  const int nk = (int)((2 * K + KC - 1) / KC);
+  for (int t0 = 0; t0 < pl.nNt; t0 += pl.cols)
+    for (int r0 = 0; r0 < pl.nMt; r0 += pl.rows) {
+      p.nMt = std::min(pl.rows, pl.nMt - r0);
+      p.nNt = std::min(pl.cols, pl.nNt - t0);
+      p.band = std::min(p.nMt, 12);
+      o.m0 = r0 * BM;
+      o.n0 = t0 * (pl.BN / 2);
+      p.rA = (int)A.r0 + r0 * BM;
+      p.rB = (int)(2 * B.r0) + t0 * pl.BN;
+      const int64_t tiles = (int64_t)p.nMt * p.nNt;
+      // segments of K that the integer sums can hold, one launch each; within one, K is split when the tiles of
+      // the whole product leave half the SMs idle, four chunks at least per split
+      for (p.chunk0 = 0; p.chunk0 < nk; p.chunk0 += MAX_CHUNKS) {
+        p.chunk1 = std::min(nk, p.chunk0 + MAX_CHUNKS);
+        const int n = p.chunk1 - p.chunk0;
+        const int64_t splits = (int64_t)pl.nMt * pl.nNt > SPLIT_TILES
+                                   ? 1 : std::max<int64_t>(1, std::min<int64_t>(tc_num_sms() / tiles, n / 4));
+        p.chunks_per_split = (int)((n + splits - 1) / splits);
+        p.splits = (n + p.chunks_per_split - 1) / p.chunks_per_split;
+        p.hi = (long long *)scratch;
+        p.lo = (float *)(p.hi + tiles * p.splits * BM * pl.BN);
+        o.accumulate = accumulate || p.chunk0 > 0;
+        if (pl.BN == 32) launch<32>(A, B, p, o, K, st);
+        else if (pl.BN == 64) launch<64>(A, B, p, o, K, st);
+        else launch<128>(A, B, p, o, K, st);
+      }
+    }
+}
+
+}  // namespace cclr

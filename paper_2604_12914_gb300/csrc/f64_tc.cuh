@@ -1,0 +1,54 @@
+// FP64-accurate complex GEMM on the tcgen05 tensor cores: every FP64 operand row is written as eight
+// 8-bit integer slices with one power-of-two scale (the error-free splitting of Ozaki, Ogita, Oishi and
+// Rump, Numer. Algorithms 59 (2012), on matrix engines as in Mukunoki, Ozaki, Ogita and Imamura, ISC 2020),
+// the slice products are BF16 MMAs whose FP32 sums are exact integers, and the sums are combined in 64-bit
+// integers.
+//
+//   x = 2^e sum_{s=0..7} d_s 2^-(8 s + 7),   |d_s| <= 128 (63 bits under the largest entry of the row),
+//   sum_k a_k b_k = 2^(ea + eb) sum_{q=0..7} S_q 2^-(8 q + 14),   S_q = sum_k sum_{i+j=q} d_i(a_k) d_j(b_k);
+// the orders q >= 8 (below 2^-64 of the largest product per term) are dropped, so the error is a few 2^-64
+// of (largest entry of the row) x (largest entry of the column) per term, below the rounding of an FP64
+// accumulation (2^-53 of the partial sums).
+#pragma once
+#include <cstdint>
+
+#include "kernels.cuh"
+#include "tc_gemm.cuh"
+
+namespace cclr {
+
+constexpr int F64_SLICES = 8;
+// Scale of a row that holds a NaN or an infinity: its products are written as NaN.
+constexpr int F64_NONFINITE = 1 << 20;
+
+// Real elements per slice row of K complex entries (whole 16-byte units) and the bytes of a prepared
+// operand of R rows (embed: two slice rows per complex column, as the GEMM's column operand needs).
+inline int64_t f64tc_ld(int64_t K) { return (2 * K + 7) / 8 * 8; }
+inline int64_t f64tc_bytes(int64_t R, int64_t K, bool embed) { return F64_SLICES * R * (embed ? 2 : 1) * f64tc_ld(K) * 2; }
+
+// A prepared operand, or the rows [r0, r0 + rows) of one: slice s of row r is row s * stride + r0 + r of p
+// (embedded operands have two slice rows per complex column; stride, r0 and rows count columns then).
+struct F64Op {
+  const void *p = nullptr;
+  const uint32_t *tops = nullptr;  // high word of the largest magnitude of each row: its scale
+  int64_t stride = 0, r0 = 0;
+  F64Op rows(int64_t first) const {
+    F64Op o = *this;
+    o.r0 += first;
+    return o;
+  }
+};
+
+// Slices of the complex128 operand X(r, k) = src[v2off(rv, r) + v2off(kv, k)], r < R, k < K, into dst, and the
+// rows' largest magnitudes into tops[R].  embed: the column operand, (re, -im) and (im, re).
+F64Op f64tc_prep(const void *src, View2 rv, View2 kv, int64_t R, int64_t K, bool embed, void *dst, uint32_t *tops,
+                 cudaStream_t st);
+
+// C(m, n) (+)= alpha sum_k A(m, k) B(k, n), complex128, from prepared operands (A: M rows, B: N embedded
+// columns).  C(m, n) at C + v2off(rv, m) + v2off(cv, n) complex entries; accumulate: added to C, else C is
+// overwritten.  scratch: f64tc_scratch_bytes(M, N) of device memory for the integer sums (at most 256 MB).
+void f64tc_gemm(const F64Op &A, int64_t M, const F64Op &B, int64_t N, int64_t K, void *C, View2 rv, View2 cv, zc alpha,
+                bool accumulate, void *scratch, cudaStream_t st);
+size_t f64tc_scratch_bytes(int64_t M, int64_t N);
+
+}  // namespace cclr

@@ -1,4 +1,6 @@
 // Packed particle-particle ladder on the CUDA cores; see ladder_cc.cuh.
+#include <cstdio>
+#include <string>
 #include <vector>
 
 #include "ladder_cc.cuh"
@@ -131,6 +133,29 @@ void LadderCC::apply(Engine &E, int dt, const Tens &Lvv, int o, int v, int naux,
   if (sig.bytes < sg) sig.alloc(sg);
   const int2 *op = opairs.as<int2>(), *vp = vpairs.as<int2>();
   const bool f64 = dt == C128;
+  // complex128: formation and contraction on the tensor cores from exact slices (f64_tc.cuh), when the
+  // formation has 2e7 multiply-adds (o = 10, v = 40 has 2.5e8) and the slices find room; CUDA cores otherwise
+  Engine::F64Hold hold(E);
+  bool tc = f64 && (double)naux * Pv * vv >= 2.0e7 && Pv < (1ll << 26) && NR * Po < (1ll << 26) && vv < (1ll << 26);
+  F64Op La, Lb, Xo;
+  if (tc) {
+    try {
+      char hint[64];
+      std::snprintf(hint, sizeof hint, "ladder|%p|%d|%d|", Lvv.p, v, naux);
+      // L~ rows (b,f) and embedded columns (a,e), K = naux; kept while L~_vv stands, in unbudgeted contexts
+      La = E.f64_operand(2, Lvv.p, view1(1), view1(vv), vv, naux, false, std::string(hint) + "A");
+      Lb = E.f64_operand(3, Lvv.p, view1(1), view1(vv), vv, naux, true, std::string(hint) + "B");
+      E.f64_scratch((int64_t)v * v, (int64_t)ga * v);
+      if (dir > 0) E.f64_scratch(maxpairs, NR * Po);
+      else E.f64_scratch(NR * Po, Pv);
+      // the packed block's and the packed vectors' slices for the largest group
+      E.f64_reserve(4, dir > 0 ? maxpairs : Pv, dir > 0 ? Pv : maxpairs, dir < 0);
+      E.f64_reserve(5, NR * Po, dir > 0 ? Pv : maxpairs, dir > 0);
+    } catch (const Error &e) {
+      if (e.status != 2) throw;
+      tc = false;
+    }
+  }
   if (dir > 0) {
     for (int64_t r = 0; r < NR; ++r) {
       if (f64)
@@ -141,6 +166,8 @@ void LadderCC::apply(Engine &E, int dt, const Tens &Lvv, int o, int v, int naux,
                                                         Xp.as<float2>() + r * Po);
       count_launch();
     }
+    // every group's products read all of X: its slices are made once
+    if (tc) Xo = E.f64_operand(5, Xp.p, view1(1), view1(NR * Po), NR * Po, Pv, true, "");
   } else {
     CCLR_CUDA(cudaMemsetAsync(sig.p, 0, sg, st));
   }
@@ -150,16 +177,21 @@ void LadderCC::apply(Engine &E, int dt, const Tens &Lvv, int o, int v, int naux,
     if (np == 0) continue;
     // formation: W[(b - a0, f)][(a - a0, e)] = sum_P L[P,b,f] L[P,a,e], b >= a0
     const int64_t rows = (int64_t)(v - a0) * v, cols = (int64_t)(a1 - a0) * v;
-    GemmArgs g;
-    g.A = (const char *)Lvv.p + (size_t)a0 * v * es;
-    g.sAm = 1; g.sAk = vv;
-    g.B = (const char *)Lvv.p + (size_t)a0 * v * es;
-    g.sBk = vv; g.sBn = 1;
-    g.C = W.p;
-    g.sCm = cols; g.sCn = 1;
-    g.M = rows; g.N = cols; g.K = naux;
-    g.overwrite = 1;
-    launch_gemm(g, dt, st);
+    if (tc) {
+      E.f64_gemm(La.rows((int64_t)a0 * v), rows, Lb.rows((int64_t)a0 * v), cols, naux, W.p, view1(cols), view1(1), zc(1.0),
+                 false);
+    } else {
+      GemmArgs g;
+      g.A = (const char *)Lvv.p + (size_t)a0 * v * es;
+      g.sAm = 1; g.sAk = vv;
+      g.B = (const char *)Lvv.p + (size_t)a0 * v * es;
+      g.sBk = vv; g.sBn = 1;
+      g.C = W.p;
+      g.sCm = cols; g.sCn = 1;
+      g.M = rows; g.N = cols; g.K = naux;
+      g.overwrite = 1;
+      launch_gemm(g, dt, st);
+    }
     if (f64)
       cc_pack_w<double><<<grid1d(np * Pv), 256, 0, st>>>(W.as<double2>(), cols, v, a0, vp, p0, np, Pv, Wp.as<double2>());
     else
@@ -167,6 +199,11 @@ void LadderCC::apply(Engine &E, int dt, const Tens &Lvv, int o, int v, int naux,
     count_launch();
     if (dir > 0) {
       // sig[(ab)][(r, ij)] = sum_{e<f} <ab||ef>~ X_r[i,j,e,f] for the group's pairs
+      if (tc) {
+        const F64Op wo = E.f64_operand(4, Wp.p, view1(Pv), view1(1), np, Pv, false, "");
+        E.f64_gemm(wo, np, Xo, NR * Po, Pv, (char *)sig.p + (size_t)p0 * NR * Po * es, view1(NR * Po), view1(1), zc(1.0), false);
+        continue;
+      }
       GemmArgs c;
       c.A = Wp.p; c.sAm = Pv; c.sAk = 1;
       c.B = Xp.p; c.sBk = NR * Po; c.sBn = 1;
@@ -186,6 +223,12 @@ void LadderCC::apply(Engine &E, int dt, const Tens &Lvv, int o, int v, int naux,
         count_launch();
       }
       // Z[(r, ij)][(ef)] += sum_{(ab) in group} Y'_r[(ij)][(ab)] <ab||ef>~
+      if (tc) {
+        const F64Op yo = E.f64_operand(5, Xp.p, view1(np), view1(1), NR * Po, np, false, "");
+        const F64Op wo = E.f64_operand(4, Wp.p, view1(1), view1(Pv), Pv, np, true, "");
+        E.f64_gemm(yo, NR * Po, wo, Pv, np, sig.p, view1(Pv), view1(1), zc(1.0), true);
+        continue;
+      }
       GemmArgs c;
       c.A = Xp.p; c.sAm = np; c.sAk = 1;
       c.B = Wp.p; c.sBk = Pv; c.sBn = 1;

@@ -289,6 +289,7 @@ void LadderTC::apply(Engine &E, int dir, zc alpha, int nrhs, const void *const *
   const int o = o_, v = v_, seg = seg_, kind = kind_;
   const int64_t Po = Po_, Pv = Pv_;
   if (Po == 0 || Pv == 0 || nrhs < 1) return;
+  E.tc_pending = true;
   const int64_t vv = (int64_t)v * v, es = tc_esize(kind);
   const int64_t ldL = 2 * tc_kpad(naux_) * seg;
   const int ga = std::min(ga_, v);

@@ -92,6 +92,7 @@ void Model::upload_inputs(const double *eps_h, const double *L, const double *mu
     apply_denominator(o, v, eps.as<double>(), t2.p, st);
   }
   CCLR_CUDA(cudaStreamSynchronize(st));
+  E.check_tc();
 }
 
 // Complex64 copies of the undressed inputs (made once, for complex64 rebuilds).
@@ -112,6 +113,8 @@ void Model::build_set(const void *t1d, const void *t2d, CstSet &out, int dt, int
   // CCLR_OPTIME=1 also prints the wall time of every build (diagnostics)
   static const bool optime = std::getenv("CCLR_OPTIME") && std::getenv("CCLR_OPTIME")[0] == '1';
   const auto wall0 = std::chrono::steady_clock::now();
+  E.clear_prep_cache();  // the set's buffers are rewritten
+  out.valid = false;
   out.dt = dt;
   const size_t es = dt_size(dt);
   const int P = naux;
@@ -244,6 +247,7 @@ void Model::build_set(const void *t1d, const void *t2d, CstSet &out, int dt, int
     }
     CCLR_CUDA(cudaStreamSynchronize(st));
   }
+  E.check_tc();
   E.tc_mode = tc_saved;
   if (lean) E.release_ws();  // the builds' permuted operands are not needed by the products
   for (int k = 0; k < 3; ++k)  // a ladder prepared from this buffer is stale
@@ -262,6 +266,8 @@ void Model::build_set(const void *t1d, const void *t2d, CstSet &out, int dt, int
 // B~ = (1 - t) B (1 + t): Fov = B~_ov, Foo = B~_oo, Fvv = B~_vv, Wovoo = -Fov_me t_ij^be; every
 // element with a two-body integral (Woooo, Wovvo, Wooov, <mn||ef>, L~) vanishes.
 void Model::build_set_onebody(const void *Bd, const void *t1d, const void *t2d, CstSet &out) {
+  E.clear_prep_cache();
+  out.valid = false;
   out.dt = C128;
   const int tc_saved = E.tc_mode;
   E.tc_mode = 0;
@@ -292,6 +298,7 @@ void Model::build_set_onebody(const void *Bd, const void *t1d, const void *t2d, 
   for (int k : {K_FOO, K_FOV, K_FVV, K_T2, K_WOVOO}) out.zero[k] = false;
   for (int k = 0; k < K_NCST; ++k)
     if (out.zero[k]) out.buf[k].release();
+  E.check_tc();
   E.tc_mode = tc_saved;
   CCLR_CUDA(cudaStreamSynchronize(st));
   bump_state_epoch();
@@ -314,6 +321,8 @@ void Model::build_diagonal() {
 // complex64 rounding of a complex128 set (same shapes, contiguous)
 void Model::round_set(const CstSet &src, CstSet &dst) {
   CCLR_REQUIRE(src.valid && src.dt == C128, "round_set: source must be a valid complex128 set");
+  E.clear_prep_cache();
+  dst.valid = false;
   dst.dt = C64;
   dst.zero = src.zero;
   for (int k = 0; k < K_NCST; ++k) {
@@ -411,6 +420,7 @@ const void *Model::oovv_packed() {
       E.contract(zc(-1), Lov, "Pmf", Lov, "Pne", F, "mnef");
       pack_doubles(C128, C128, o, v, full.p, oovvp.p, st);
       CCLR_CUDA(cudaStreamSynchronize(st));
+      E.check_tc();
     }
     CCLR_CUDA(cudaStreamSynchronize(st));
   }
@@ -495,6 +505,15 @@ void Model::apply_body(int dir, const CstSet &C, int nr, const void *const *x1, 
     for (int k = 4; k < nv; ++k) ptr[r][k] = tv[k].p;
   auto V = [&](int r, int id) { return var_tens(id, dt, ptr[r][id]); };
   auto Cst = [&](int id) { return C.t[id]; };
+  // a contraction whose constant operand is marked as one (also when it throws: the mark is taken back)
+  auto hinted = [&](const Op &op, auto &&f) {
+    struct Mark {
+      const void *&h;
+      ~Mark() { h = nullptr; }
+    } mark{E.cst_hint};
+    E.cst_hint = Cst(op.cst).p;
+    f();
+  };
   auto run_ladder = [&](int d, zc a, int in_id, int out_id) {
     if (C.zero[K_LVV]) return;
     std::vector<Tens> in(nr), out(nr);
@@ -536,9 +555,7 @@ void Model::apply_body(int dir, const CstSet &C, int nr, const void *const *x1, 
         if (oe0 && r == 0) CCLR_CUDA(cudaEventRecord(oe0, st));
         switch (op.kind) {
           case OP_CONTRACT:
-            E.cst_hint = Cst(op.cst).p;
-            E.contract(op.alpha, Cst(op.cst), op.mc, V(r, op.in), op.mi, V(r, op.out), op.mo);
-            E.cst_hint = nullptr;
+            hinted(op, [&] { E.contract(op.alpha, Cst(op.cst), op.mc, V(r, op.in), op.mi, V(r, op.out), op.mo); });
             break;
           case OP_PERM: E.permute(op.alpha, V(r, op.in), op.mi, V(r, op.out), op.mo, true); break;
           case OP_ZERO: E.zero(V(r, op.out)); break;
@@ -584,9 +601,7 @@ void Model::apply_body(int dir, const CstSet &C, int nr, const void *const *x1, 
         if (op.kind == OP_LADDER || (op.kind == OP_CONTRACT && C.zero[op.cst])) continue;
         switch (op.kind) {
           case OP_CONTRACT:
-            E.cst_hint = Cst(op.cst).p;
-            E.contract(op.alpha, Cst(op.cst), op.mc, V(r, op.out), op.mo, V(r, op.in), op.mi);
-            E.cst_hint = nullptr;
+            hinted(op, [&] { E.contract(op.alpha, Cst(op.cst), op.mc, V(r, op.out), op.mo, V(r, op.in), op.mi); });
             break;
           case OP_PERM: E.permute(op.alpha, V(r, op.out), op.mo, V(r, op.in), op.mi, true); break;
           case OP_ZERO: E.zero(V(r, op.out)); break;
@@ -697,7 +712,8 @@ void Model::apply_batch(int dir, const CstSet &C, int nr, const void *const *x1,
       ms_last[2] = tot;
       ms_last[3] = -1.f;
       ++graph_launches;
-      if (E.tc_mode && tc_error(st)) throw Error(5, "a tensor-core kernel gave up on a bounded wait");
+      E.tc_pending = true;
+      E.check_tc();
       return;
     }
   }
@@ -720,7 +736,7 @@ void Model::apply_batch(int dir, const CstSet &C, int nr, const void *const *x1,
   ms_last[1] = tot - lad_ms;
   ms_last[2] = tot;
   ms_last[3] = form_ms;
-  if (E.tc_mode && tc_error(st)) throw Error(5, "a tensor-core kernel gave up on a bounded wait");
+  E.check_tc();
   if (graphs) {
     for (size_t w = 0; w < warm.size(); ++w)
       if (warm[w].key == key) {
@@ -767,6 +783,7 @@ void Model::xi(const void *mub, const void *t1d, const void *t2d, void *xi1, voi
   antisym_project(C128, o, v, X2.p, st);
   vec_scal(C128, X2.numel(), zc(2.0), X2.p, st);
   CCLR_CUDA(cudaStreamSynchronize(st));
+  E.check_tc();
 }
 
 // ---------------------------------------------------------------------------------------

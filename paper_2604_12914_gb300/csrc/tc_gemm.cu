@@ -19,6 +19,7 @@
 
 #include "engine.cuh"
 #include "tc_gemm.cuh"
+#include "tc_ptx.cuh"
 
 namespace cclr {
 namespace {
@@ -26,7 +27,6 @@ namespace {
 constexpr int BM = 128;      // UMMA M
 constexpr int BKB = 128;     // bytes per K block = one 128-byte swizzle row (32 TF32 or 64 BF16)
 constexpr int STAGES = 4;
-constexpr unsigned long long TIMEOUT_NS = 2000000000ull;  // 2 s per wait
 
 struct TcParams {
   int M, N, K, BN;
@@ -41,121 +41,6 @@ struct TcParams {
   int atomic;           // split-K: combine partial tiles with atomicAdd
   int *err;
 };
-
-__device__ __forceinline__ uint32_t su32(const void *p) {
-  return static_cast<uint32_t>(__cvta_generic_to_shared(p));
-}
-
-__device__ __forceinline__ unsigned long long gtime() {
-  unsigned long long t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
-}
-
-__device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok)
-      : "r"(bar), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-
-__device__ bool mbar_wait(uint32_t bar, uint32_t parity, int *err) {
-  if (mbar_try(bar, parity)) return true;
-  const unsigned long long t0 = gtime();
-  while (true) {
-    if (mbar_try(bar, parity)) return true;
-    if (gtime() - t0 > TIMEOUT_NS) {
-      atomicExch(err, 1);
-      return false;
-    }
-  }
-}
-
-__device__ __forceinline__ void tma_load_2d(void *dst, const CUtensorMap *map, int x, int y,
-                                            uint32_t bar) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
-      :
-      : "r"(su32(dst)), "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(bar)
-      : "memory");
-}
-
-// Shared-memory matrix descriptor: K-major operand, 128-byte swizzle, rows of 128 bytes,
-// 8-row groups 1024 bytes apart (stride byte offset), descriptor version 1.
-__device__ __forceinline__ uint64_t sw128_desc(uint32_t saddr) {
-  uint64_t d = 0;
-  d |= (uint64_t)((saddr & 0x3FFFF) >> 4);
-  d |= (uint64_t)1 << 16;            // leading byte offset (unused with 128B swizzle)
-  d |= (uint64_t)(1024 >> 4) << 32;  // stride byte offset
-  d |= (uint64_t)1 << 46;            // version
-  d |= (uint64_t)2 << 61;            // SWIZZLE_128B
-  return d;
-}
-
-// Instruction descriptor of kind::tf32 / kind::f16: D FP32 (bits 4-5), A and B type (bits 7-9
-// and 10-12: TF32 = 2, BF16 = 1), both K-major, N >> 3 (bits 17-22), M >> 4 (bits 24-28).
-__host__ __device__ constexpr uint32_t idesc_mma(int kind, int M, int N) {
-  return (1u << 4) | ((kind == TC_BF16 ? 1u : 2u) << 7) | ((kind == TC_BF16 ? 1u : 2u) << 10) |
-         ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
-}
-
-// one MMA of K = 32 bytes per row (8 TF32 or 16 BF16), D (+)= A B^T in TMEM
-template <int KIND>
-__device__ __forceinline__ void mma_issue(uint32_t tmem, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
-  if constexpr (KIND == TC_BF16) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-        :
-        : "r"(tmem), "l"(a), "l"(b), "r"(idesc), "r"(acc));
-  } else {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}"
-        :
-        : "r"(tmem), "l"(a), "l"(b), "r"(idesc), "r"(acc));
-  }
-}
-
-__device__ __forceinline__ void mma_commit(uint32_t bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
-               : "memory");
-}
-
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-        "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
-        "=r"(r[14]), "=r"(r[15])
-      : "r"(taddr));
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-}
-
-// Bounded wait that also gives up when another role of the CTA has aborted.
-__device__ bool mbar_wait_ab(uint32_t bar, uint32_t parity, int *err, volatile int *abort_flag) {
-  if (mbar_try(bar, parity)) return true;
-  const unsigned long long t0 = gtime();
-  while (true) {
-    if (mbar_try(bar, parity)) return true;
-    if (*abort_flag) return false;
-    if (gtime() - t0 > TIMEOUT_NS) {
-      atomicExch(err, 1);
-      *abort_flag = 1;
-      return false;
-    }
-  }
-}
-
-__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
-}
 
 // work unit -> (m tile, n tile, split); banded rasterisation: consecutive units share one B
 // tile column across a band of M tiles, so the band's A tiles and the current B tiles stay in L2
@@ -508,17 +393,18 @@ int *device_err() {
 }
 
 // 2-D tensor map over a row-major operand (rows x cols elements, ld elements apart), boxes of
-// one 128-byte K block by box_rows rows, 128-byte swizzle
-CUtensorMap make_map(const void *base, int64_t rows, int64_t cols, int64_t ld, int box_rows, int kind) {
+// box_bytes of K (one 128- or 64-byte swizzle row) by box_rows rows
+CUtensorMap make_map(const void *base, int64_t rows, int64_t cols, int64_t ld, int box_rows, int box_bytes, int kind) {
   CUtensorMap m;
   const int64_t es = tc_esize(kind);
   cuuint64_t gdim[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
   cuuint64_t gstride[1] = {(cuuint64_t)(ld * es)};
-  cuuint32_t box[2] = {(cuuint32_t)(BKB / es), (cuuint32_t)box_rows};
+  cuuint32_t box[2] = {(cuuint32_t)(box_bytes / es), (cuuint32_t)box_rows};
   cuuint32_t estr[2] = {1, 1};
   CUresult r = g_encode(&m, kind == TC_BF16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2,
                         (void *)base, gdim, gstride, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                        CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+                        box_bytes == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B,
+                        CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS) throw Error(4, "cuTensorMapEncodeTiled failed: " + std::to_string((int)r));
   return m;
 }
@@ -628,8 +514,8 @@ static void tc_launch(const void *A, int64_t lda, const void *B, int64_t ldb, in
                       int *err, cudaStream_t st, int64_t a_cols, TcCfg cfg, TcCfg *used) {
   const int64_t es = tc_esize(kind), BK = BKB / es;
   const int BN = cfg.BN > 0 ? cfg.BN : pick_bn(Nreal);
-  const CUtensorMap ma = make_map(A, M, a_cols < 0 ? Kreal : a_cols, lda, BM, kind);
-  const CUtensorMap mb = make_map(B, Nreal, Kreal, ldb, BN, kind);
+  const CUtensorMap ma = make_map(A, M, a_cols < 0 ? Kreal : a_cols, lda, BM, BKB, kind);
+  const CUtensorMap mb = make_map(B, Nreal, Kreal, ldb, BN, BKB, kind);
   TcParams p;
   p.M = (int)M;
   p.N = (int)Nreal;
@@ -864,6 +750,12 @@ int tc_selftest_timeout(int timeout_us, cudaStream_t st) {
   count_launch();
   CCLR_CUDA(cudaGetLastError());
   return tc_error(st);
+}
+
+int *tc_device_err() { return device_err(); }
+int tc_num_sms() { return num_sms(); }
+CUtensorMap tc_make_map(const void *base, int64_t rows, int64_t cols, int64_t ld, int box_rows, int box_bytes, int kind) {
+  return make_map(base, rows, cols, ld, box_rows, box_bytes, kind);
 }
 
 void tc_set_autotune(bool on) { g_tune_on = on; }

@@ -13,6 +13,7 @@
 // operands (bf16x3, the three-product split of Henry, Tang and Heinecke, ARITH 2019) about
 // 2^-16 relative, at the BF16 rate (twice the TF32 rate).
 #pragma once
+#include <cuda.h>
 #include <cuda_bf16.h>
 
 #include "kernels.cuh"
@@ -157,6 +158,14 @@ void tc_set_autotune(bool on);
 // Rows of 10 doubles per tuned shape of the current device (kind, M, N, K, BN, splits, band,
 // best ms, the rule's ms, candidates timed), up to cap rows; returns the number of shapes.
 int tc_tuning_table(int cap, double *rec);
+
+// For kernels of other translation units: the current device's bounded-wait flag (the first use on a device
+// sets it up and fetches the tensor-map encoder), its SM count, and the 2-D tensor map of a row-major operand
+// (rows x cols elements of the operand type, ld apart; boxes of box_bytes = 128 or 64 bytes, the swizzle, by
+// box_rows rows).
+int *tc_device_err();
+int tc_num_sms();
+CUtensorMap tc_make_map(const void *base, int64_t rows, int64_t cols, int64_t ld, int box_rows, int box_bytes, int kind);
 
 // Reads (and clears) the device-side error flag of the tensor-core kernels: 0 = fine,
 // 1 = a bounded wait gave up.
