@@ -116,25 +116,116 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN))
   }
 }
 
+// The same with one output per thread in a TM x TN tile (TM TN = 256): little padding and many blocks.  In FP64,
+// whose pipe does two FMAs per clock and SM, this is the kernel for every size: the pipe is busy 512 clocks per k
+// of a 16 x 16 tile, far longer than its loads take, and what counts is that no padded entry is computed and that
+// every SM has a block (o=10 v=40: M=40 N=10 K=40 98 us as one 128 x 16 tile, 28 so; M=N=10 K=16000 520 us as
+// 64 x 64 tiles, 34 so).  In FP32 it serves the products whose 64 x 64 tiles would leave most SMs idle.
+template <typename T, int TM, int TN>
+__global__ void __launch_bounds__(256) zgemm_small(GemmArgs g, int64_t b0) {
+  using C = typename cpx<T>::t;
+  constexpr int BK = TM > 64 || TN > 64 ? 8 : 16, NA = (TM * BK + 255) / 256, NB = (TN * BK + 255) / 256;
+  __shared__ C As[BK][TM + 1], Bs[BK][TN + 1];
+  const int64_t nMt = (g.M + TM - 1) / TM;
+  const int64_t m0 = ((int64_t)blockIdx.x % nMt) * TM, n0 = ((int64_t)blockIdx.x / nMt) * TN, b = b0 + blockIdx.z;
+  const C *A = (const C *)g.A + b * g.sAb, *B = (const C *)g.B + b * g.sBb;
+  const int tid = threadIdx.x, tn = tid % TN, tm = tid / TN;
+  const bool a_kfast = g.sAk == 1, b_nfast = g.sBn == 1;
+  const int64_t kbeg = g.kchunk > 0 ? (int64_t)blockIdx.y * g.kchunk : 0;
+  const int64_t kend = g.kchunk > 0 ? min(g.K, kbeg + g.kchunk) : g.K;
+  C ra[NA], rb[NB];
+  auto fetch = [&](int64_t k0) {
+#pragma unroll
+    for (int q = 0; q < NA; ++q) {
+      const int e = tid + q * 256, kk = a_kfast ? e % BK : e / TM, mm = a_kfast ? e / BK : e % TM;
+      const int64_t m = m0 + mm, k = k0 + kk;
+      ra[q] = (e < TM * BK && m < g.M && k < kend) ? A[m * g.sAm + k * g.sAk] : C{T(0), T(0)};
+    }
+#pragma unroll
+    for (int q = 0; q < NB; ++q) {
+      const int e = tid + q * 256, kk = b_nfast ? e / TN : e % BK, nn = b_nfast ? e % TN : e / BK;
+      const int64_t n = n0 + nn, k = k0 + kk;
+      rb[q] = (e < TN * BK && n < g.N && k < kend) ? B[k * g.sBk + n * g.sBn] : C{T(0), T(0)};
+    }
+  };
+  C acc{T(0), T(0)};
+  fetch(kbeg);
+  for (int64_t k0 = kbeg; k0 < kend; k0 += BK) {
+#pragma unroll
+    for (int q = 0; q < NA; ++q) {
+      const int e = tid + q * 256;
+      if (e < TM * BK) As[a_kfast ? e % BK : e / TM][a_kfast ? e / BK : e % TM] = ra[q];
+    }
+#pragma unroll
+    for (int q = 0; q < NB; ++q) {
+      const int e = tid + q * 256;
+      if (e < TN * BK) Bs[b_nfast ? e / TN : e % BK][b_nfast ? e % TN : e / BK] = rb[q];
+    }
+    __syncthreads();
+    if (k0 + BK < kend) fetch(k0 + BK);  // the next block's loads overlap this block's sums
+    if (m0 + tm < g.M && n0 + tn < g.N) {
+      const int nk = (int)min((int64_t)BK, kend - k0);
+#pragma unroll 4
+      for (int kk = 0; kk < nk; ++kk) {
+        const C x = As[kk][tm], y = Bs[kk][tn];
+        acc.x = fma(x.x, y.x, acc.x);
+        acc.x = fma(-x.y, y.y, acc.x);
+        acc.y = fma(x.x, y.y, acc.y);
+        acc.y = fma(x.y, y.x, acc.y);
+      }
+    }
+    __syncthreads();
+  }
+  const int64_t m = m0 + tm, n = n0 + tn;
+  if (m >= g.M || n >= g.N) return;
+  C *dst = (C *)g.C + b * g.sCb + m * g.sCm + n * g.sCn;
+  const T ar = (T)g.alr, ai = (T)g.ali;
+  C r;
+  r.x = ar * acc.x - ai * acc.y;
+  r.y = ar * acc.y + ai * acc.x;
+  if (g.kchunk > 0) {
+    atomicAdd(&dst->x, r.x);
+    atomicAdd(&dst->y, r.y);
+    return;
+  }
+  if (!g.overwrite) {
+    const C o = *dst;
+    r.x += o.x;
+    r.y += o.y;
+  }
+  *dst = r;
+}
+
 void launch_gemm(const GemmArgs &g, int dt, cudaStream_t st) {
   if (g.M <= 0 || g.N <= 0) return;
   if (g.K <= 0) {
     CCLR_REQUIRE(!g.overwrite, "gemm with K=0 and overwrite is not supported");
     return;
   }
-  // Tile shape by output shape: the CUDA cores compute every element of a tile, so a skinny
-  // output gets a flat tile (128 x 16 or 16 x 128) instead of 64 x 64 -- FP64 work is dear on
-  // this GPU (about 8 GFLOP/s per SM).
+  auto tiles_of = [&](int64_t tm, int64_t tn) { return ((g.M + tm - 1) / tm) * ((g.N + tn - 1) / tn); };
+  // complex64: 64 x 64 tiles (flat ones for skinny outputs) when they fill two thirds of the SMs
   const int shape = (g.N <= 16 && g.M > 16) ? 1 : (g.M <= 16 && g.N > 16) ? 2 : 0;
-  const int64_t BMs = shape == 1 ? 128 : shape == 2 ? 16 : 64, BNs = shape == 1 ? 16 : shape == 2 ? 128 : 64;
-  const int64_t tiles = ((g.M + BMs - 1) / BMs) * ((g.N + BNs - 1) / BNs);
-  // split K over blocks (partial sums added atomically) when the tile grid cannot fill the
-  // GPU: the skinny and matrix-vector shapes; at least 64 of K per split
+  const int64_t big = shape == 1 ? tiles_of(128, 16) : shape == 2 ? tiles_of(16, 128) : tiles_of(64, 64);
+  const bool small = dt == C128 || big * g.batch < 100;
+  // one output per thread: the tile shape with the least padding (complex64, which its loads bound, keeps the square
+  // one down to four columns: 64 x 4 tiles read A three times for N = 11, 37 us against 21)
+  int tm = 16, tn = 16;
+  if (small && (dt == C128 || std::min(g.M, g.N) <= 4))
+    for (int t : {64, 256})
+      for (int side = 0; side < 2; ++side) {
+        const int m = side == 0 ? t : 256 / t, n = 256 / m;
+        if (tiles_of(m, n) < tiles_of(tm, tn)) { tm = m; tn = n; }
+      }
+  const int64_t tiles = small ? tiles_of(tm, tn) : big;
+  // split K over blocks (partial sums added atomically) when the tile grid cannot fill the GPU: at least 32 of K
+  // per split in complex128; in complex64 as many splits as the large tiles would take, of at least 64 (twice as
+  // many atomic FP32 additions made the error of an o=11 v=67 sigma half as large again)
   int64_t splits = 1;
-  const int64_t bk = dt == C128 ? 8 : 16;
+  const int64_t bk = dt == C128 ? 8 : 16, fill = dt == C128 ? 4 * 152 : 2 * 152, least = dt == C128 ? 32 : 64;
+  const int64_t units = (dt == C128 ? tiles : big) * g.batch;
   const bool plain_c = g.sCn == 1 && g.sCm == g.N && (g.batch == 1 || g.sCb == g.M * g.N);
-  if (tiles * g.batch < 2 * 152 && g.K >= 128 && (!g.overwrite || plain_c) && g.batch <= 65535)
-    splits = std::min<int64_t>((2 * 152 + tiles * g.batch - 1) / (tiles * g.batch), g.K / 64);
+  if (units < fill && g.K >= 2 * least && (!g.overwrite || plain_c) && g.batch <= 65535)
+    splits = std::min<int64_t>((fill + units - 1) / units, g.K / least);
   GemmArgs ga = g;
   if (splits > 1) {
     ga.kchunk = ((g.K + splits - 1) / splits + bk - 1) / bk * bk;
@@ -147,15 +238,19 @@ void launch_gemm(const GemmArgs &g, int dt, cudaStream_t st) {
   for (int64_t b0 = 0; b0 < g.batch; b0 += 65535) {
     int64_t nb = std::min<int64_t>(65535, g.batch - b0);
     dim3 grid((unsigned)tiles, (unsigned)splits, (unsigned)nb);
-    if (dt == C128) {
-      if (shape == 1) zgemm_simt<double, 128, 16, 8, 8, 1><<<grid, 256, 0, st>>>(ga, b0);
-      else if (shape == 2) zgemm_simt<double, 16, 128, 8, 1, 8><<<grid, 256, 0, st>>>(ga, b0);
-      else zgemm_simt<double, 64, 64, 8, 4, 4><<<grid, 256, 0, st>>>(ga, b0);
-    } else {
-      if (shape == 1) zgemm_simt<float, 128, 16, 16, 8, 1><<<grid, 256, 0, st>>>(ga, b0);
-      else if (shape == 2) zgemm_simt<float, 16, 128, 16, 1, 8><<<grid, 256, 0, st>>>(ga, b0);
-      else zgemm_simt<float, 64, 64, 16, 4, 4><<<grid, 256, 0, st>>>(ga, b0);
-    }
+    auto run_small = [&](auto zero) {
+      using T = decltype(zero);
+      if (tm == 16) zgemm_small<T, 16, 16><<<grid, 256, 0, st>>>(ga, b0);
+      else if (tm == 64) zgemm_small<T, 64, 4><<<grid, 256, 0, st>>>(ga, b0);
+      else if (tm == 4) zgemm_small<T, 4, 64><<<grid, 256, 0, st>>>(ga, b0);
+      else if (tm == 256) zgemm_small<T, 256, 1><<<grid, 256, 0, st>>>(ga, b0);
+      else zgemm_small<T, 1, 256><<<grid, 256, 0, st>>>(ga, b0);
+    };
+    if (dt == C128) run_small(0.0);
+    else if (small) run_small(0.0f);
+    else if (shape == 1) zgemm_simt<float, 128, 16, 16, 8, 1><<<grid, 256, 0, st>>>(ga, b0);
+    else if (shape == 2) zgemm_simt<float, 16, 128, 16, 1, 8><<<grid, 256, 0, st>>>(ga, b0);
+    else zgemm_simt<float, 64, 64, 16, 4, 4><<<grid, 256, 0, st>>>(ga, b0);
     count_launch();
     CCLR_CUDA(cudaGetLastError());
   }
