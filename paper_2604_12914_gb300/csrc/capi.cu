@@ -1950,7 +1950,7 @@ int cc_lr_bench_gemm(int M, int N, int K, int mode, int reps, double *ms) {
     cudaStream_t st;
     CCLR_CUDA(cudaStreamCreate(&st));
     const int seg = mode == 1 ? 1 : 3, kind = mode == 3 ? TC_BF16 : TC_TF32;
-    const int64_t ld = 2 * tc_kpad(K) * seg, es = tc_esize(kind);
+    const int64_t ld = 2 * tc_kpad(K, kind) * seg, es = tc_esize(kind);
     DevBuf A((size_t)M * ld * es), B((size_t)2 * N * ld * es), C((size_t)M * N * 8);
     // deterministic small values (exact content is irrelevant for timing)
     CCLR_CUDA(cudaMemsetAsync(A.p, 0, A.bytes, st));
@@ -1959,10 +1959,10 @@ int cc_lr_bench_gemm(int M, int N, int K, int mode, int reps, double *ms) {
     cudaEvent_t e0, e1;
     CCLR_CUDA(cudaEventCreate(&e0));
     CCLR_CUDA(cudaEventCreate(&e1));
-    tc_gemm_seg(A.p, ld, B.p, ld, M, 2 * N, 2 * tc_kpad(K), seg, kind, C.as<float>(), 2 * N, zc(1), false, st);
+    tc_gemm_seg(A.p, ld, B.p, ld, M, 2 * N, ld / seg, seg, kind, C.as<float>(), 2 * N, zc(1), false, st);
     CCLR_CUDA(cudaEventRecord(e0, st));
     for (int r = 0; r < reps; ++r)
-      tc_gemm_seg(A.p, ld, B.p, ld, M, 2 * N, 2 * tc_kpad(K), seg, kind, C.as<float>(), 2 * N, zc(1), false, st);
+      tc_gemm_seg(A.p, ld, B.p, ld, M, 2 * N, ld / seg, seg, kind, C.as<float>(), 2 * N, zc(1), false, st);
     CCLR_CUDA(cudaEventRecord(e1, st));
     CCLR_CUDA(cudaEventSynchronize(e1));
     float t = 0;

@@ -480,10 +480,10 @@ void Engine::f64_scratch(int64_t M, int64_t N) {
 }
 
 void Engine::f64_gemm(const F64Op &A, int64_t M, const F64Op &B, int64_t N, int64_t K, void *C, View2 rv, View2 cv, zc alpha,
-                      bool accumulate) {
+                      bool accumulate, UpperTiles *upper) {
   f64_scratch(M, N);
   tc_pending = true;
-  f64tc_gemm(A, M, B, N, K, C, rv, cv, alpha, accumulate, f64_scr_.p, st);
+  f64tc_gemm(A, M, B, N, K, C, rv, cv, alpha, accumulate, f64_scr_.p, st, upper);
 }
 
 void Engine::check_tc() {
@@ -644,7 +644,7 @@ void Engine::contract_tc(zc alpha, const Tens &A, const std::string &ma, const T
   };
   const int seg = tc_mode == 1 ? 1 : 3;
   const int kind = tc_mode == 3 ? TC_BF16 : TC_TF32;
-  const int64_t ld = 2 * tc_kpad(K) * seg, tes = tc_esize(kind);
+  const int64_t ld = 2 * tc_kpad(K, kind) * seg, tes = tc_esize(kind);
   const int64_t per_col = 2 * ld * tes, per_row = ld * tes, capb = 2ll << 30;
   // A constant operand (cst_hint) keeps its prepared form: "P" entries hold its permuted
   // contiguous copy, "R" entries its prepared rows (A) or columns (B) for every batch and chunk.
@@ -750,7 +750,7 @@ void Engine::contract_tc(zc alpha, const Tens &A, const std::string &ma, const T
         void *Am = Arows ? (void *)(Arows + (b * M + m0) * per_row) : Ao;
         if (Arows ? (!ra && n0 == 0) : (n0 == 0 || Mc < M))
           tc_prep_a2((const char *)Ab + v2off(am, m0) * es, am, ak, mm, K, seg, kind, Am, ld, st);
-        tc_gemm_seg_v(Am, ld, Bn, ld, mm, 2 * nn, 2 * tc_kpad(K), seg, kind, Cn + 2 * v2off(cm, m0), cm, cn, alpha,
+        tc_gemm_seg_v(Am, ld, Bn, ld, mm, 2 * nn, ld / seg, seg, kind, Cn + 2 * v2off(cm, m0), cm, cn, alpha,
                       direct, st);
       }
     }

@@ -56,6 +56,32 @@ struct DevBuf {
   template <typename T> T *as() const { return (T *)p; }
 };
 
+// The tiles of a ladder group's formation W[(b, f)][(a, e)] (b and a counted from the group's first a, v rows and
+// columns each) that hold an entry with b > a, which are all that is read of it: a group of g values of a computes
+// g (g + 1) / 2 of the v g blocks less (a fifth of the work at v = 160, g = 32).  Lists are made once per tiling and
+// kept; get() returns nullptr (compute every tile) where it cannot make one (no memory, inside a capture).
+class UpperTiles {
+ public:
+  explicit UpperTiles(int v = 1) : v_(v) {}
+  // nMt x nNt tiles of rows x cols entries from row m0 and column n0 on, of M rows in all, in bands of `band` tile
+  // rows; *n: tiles in the list
+  const uint32_t *get(int nMt, int nNt, int band, int rows, int cols, int64_t m0, int64_t n0, int64_t M, cudaStream_t st,
+                      int *n);
+  void reset(int v) {
+    lists_.clear();
+    v_ = v;
+  }
+
+ private:
+  struct List {
+    int nMt, nNt, band, rows, cols, n;
+    int64_t m0, n0, M;
+    DevBuf buf;
+  };
+  std::vector<std::unique_ptr<List>> lists_;
+  int v_;
+};
+
 size_t device_bytes_in_use();
 // Counter bumped whenever device memory is freed (and by callers that rewrite state a captured
 // CUDA graph depends on): a graph captured at one value is valid while the counter keeps it.
@@ -97,7 +123,7 @@ class Engine {
   // room for the sums of an M x N f64tc_gemm (throws status 2), and the product itself on this engine's stream
   void f64_scratch(int64_t M, int64_t N);
   void f64_gemm(const F64Op &A, int64_t M, const F64Op &B, int64_t N, int64_t K, void *C, View2 rv, View2 cv, zc alpha,
-                bool accumulate);
+                bool accumulate, UpperTiles *upper = nullptr);
   // Throws status 5 if a tensor-core kernel launched since the last check gave up on a bounded wait
   // (synchronises the stream; nothing is done when none was launched).
   void check_tc();

@@ -29,6 +29,8 @@ constexpr int SPLIT_TILES = 76;         // K is split when at most this many til
 struct F64Params {
   int sA, sB, rA, rB;   // slice rows per slice of A and B, first slice row
   int nMt, nNt, band, splits, chunks_per_split;
+  const uint32_t *list; // the tiles to compute, (m << 16) | n, ntiles of them (nullptr: all, in raster order)
+  int ntiles;
   int chunk0, chunk1;   // chunks of KC of this K segment
   long long *hi;        // integer sums, [split][tile][column][row]: hi + lo 2^-8, in units of 2^(ea + eb - 46)
   float *lo;
@@ -39,6 +41,8 @@ struct F64Params {
 struct F64Out {
   int m0, n0, M, N;     // first row and complex column of the tiles; C's extents
   int nMt, nNt, splits, cols_fast, accumulate;
+  const uint32_t *list; // as the GEMM's (K is not split then)
+  int ntiles;
   const long long *hi;
   const float *lo;
   const uint32_t *ea, *eb;  // rows' and columns' maxima (scale_of gives the exponents)
@@ -49,9 +53,15 @@ struct F64Out {
 };
 
 __device__ __forceinline__ void unit_coords(const F64Params &p, int u, int &mt, int &nt, int &sp) {
-  const int tiles = p.nMt * p.nNt;
-  sp = u / tiles;
-  const int id = u - sp * tiles, per_band = p.band * p.nNt, b = id / per_band, local = id - b * per_band;
+  sp = u / p.ntiles;
+  const int id = u - sp * p.ntiles;
+  if (p.list) {
+    const uint32_t mn = __ldg(p.list + id);
+    mt = (int)(mn >> 16);
+    nt = (int)(mn & 0xffff);
+    return;
+  }
+  const int per_band = p.band * p.nNt, b = id / per_band, local = id - b * per_band;
   const int mb = min(p.band, p.nMt - b * p.band);
   mt = b * p.band + local % mb;
   nt = local / mb;
@@ -184,7 +194,7 @@ __global__ void __launch_bounds__(384, 1)
   int *issued = (int *)(tslot + 1), *consumed = issued + 1;
   volatile int *abort_flag = issued + 2;
   const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
-  const int units = p.nMt * p.nNt * p.splits;
+  const int units = p.ntiles * p.splits;
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < NSLOT; ++s) {
@@ -374,7 +384,14 @@ __global__ void __launch_bounds__(256) f64_out_kernel(F64Out p) {
   int b = blockIdx.x;
   const int cg = b % (BN / 32);
   b /= BN / 32;
-  const int rg = b % 4, tile = b / 4, mt = tile % p.nMt, nt = tile / p.nMt;
+  const int rg = b % 4;
+  int tile = b / 4, mt = tile % p.nMt, nt = tile / p.nMt;
+  if (p.list) {
+    const uint32_t mn = __ldg(p.list + tile);
+    mt = (int)(mn >> 16);
+    nt = (int)(mn & 0xffff);
+    tile = nt * p.nMt + mt;
+  }
   const int r0 = p.m0 + mt * BM + rg * 32, c0 = p.n0 + nt * (BN / 2) + cg * 16;
   if (r0 >= p.M || c0 >= p.N) return;
   const int row = r0 + lane;
@@ -643,7 +660,7 @@ void launch(const F64Op &A, const F64Op &B, const F64Params &p, F64Out &o, int64
   const int64_t ld = f64tc_ld(K);
   const CUtensorMap ma = tc_make_map(A.p, (int64_t)S * p.sA, 2 * K, ld, BM, 64, TC_BF16);
   const CUtensorMap mb = tc_make_map(B.p, (int64_t)S * p.sB, 2 * K, ld, BN, 64, TC_BF16);
-  const int64_t tiles = (int64_t)p.nMt * p.nNt, units = tiles * p.splits;
+  const int64_t units = (int64_t)p.ntiles * p.splits;
   f64_gemm_kernel<BN><<<(unsigned)std::min<int64_t>(units, tc_num_sms()), 384, smem_bytes<BN>(), st>>>(ma, mb, p);
   CCLR_CUDA(cudaGetLastError());
   o.hi = p.hi;
@@ -651,8 +668,10 @@ void launch(const F64Op &A, const F64Op &B, const F64Params &p, F64Out &o, int64
   o.nMt = p.nMt;
   o.nNt = p.nNt;
   o.splits = p.splits;
-  if (p.splits > 8) f64_out_split_kernel<BN><<<(unsigned)(tiles * 4 * (BN / 2)), dim3(32, 8), 0, st>>>(o);
-  else f64_out_kernel<BN><<<(unsigned)(tiles * 4 * (BN / 32)), dim3(32, 8), 0, st>>>(o);
+  o.list = p.list;
+  o.ntiles = p.ntiles;
+  if (p.splits > 8) f64_out_split_kernel<BN><<<(unsigned)(p.ntiles * 4 * (BN / 2)), dim3(32, 8), 0, st>>>(o);
+  else f64_out_kernel<BN><<<(unsigned)(p.ntiles * 4 * (BN / 32)), dim3(32, 8), 0, st>>>(o);
   CCLR_CUDA(cudaGetLastError());
   count_launch(2);
 }
@@ -697,7 +716,7 @@ size_t f64tc_scratch_bytes(int64_t M, int64_t N) {
 }
 
 void f64tc_gemm(const F64Op &A, int64_t M, const F64Op &B, int64_t N, int64_t K, void *C, View2 rv, View2 cv, zc alpha,
-                bool accumulate, void *scratch, cudaStream_t st) {
+                bool accumulate, void *scratch, cudaStream_t st, UpperTiles *upper) {
   if (M <= 0 || N <= 0 || K <= 0) return;
   CCLR_REQUIRE(A.r0 + M <= A.stride && B.r0 + N <= B.stride, "f64tc_gemm: rows outside the prepared operand");
   CCLR_REQUIRE((uintptr_t)A.p % 16 == 0 && (uintptr_t)B.p % 16 == 0, "f64tc_gemm: operands must be 16-byte aligned");
@@ -732,6 +751,10 @@ void f64tc_gemm(const F64Op &A, int64_t M, const F64Op &B, int64_t N, int64_t K,
       p.rA = (int)A.r0 + r0 * BM;
       p.rB = (int)(2 * B.r0) + t0 * pl.BN;
       const int64_t tiles = (int64_t)p.nMt * p.nNt;
+      p.ntiles = (int)tiles;
+      // (a product with few tiles splits K instead)
+      p.list = upper && (int64_t)pl.nMt * pl.nNt > SPLIT_TILES
+                   ? upper->get(p.nMt, p.nNt, p.band, BM, pl.BN / 2, o.m0, o.n0, M, st, &p.ntiles) : nullptr;
       // segments of K that the integer sums can hold, one launch each; within one, K is split when the tiles of
       // the whole product leave half the SMs idle, four chunks at least per split
       for (p.chunk0 = 0; p.chunk0 < nk; p.chunk0 += MAX_CHUNKS) {

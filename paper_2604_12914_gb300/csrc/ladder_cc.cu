@@ -118,6 +118,7 @@ void LadderCC::apply(Engine &E, int dt, const Tens &Lvv, int o, int v, int naux,
     CCLR_CUDA(cudaMemcpyAsync(opairs.p, op.data(), op.size() * sizeof(int2), cudaMemcpyHostToDevice, st));
     CCLR_CUDA(cudaMemcpyAsync(vpairs.p, vp.data(), vp.size() * sizeof(int2), cudaMemcpyHostToDevice, st));
     CCLR_CUDA(cudaStreamSynchronize(st));
+    if (v_ != v) upper_.reset(v);
     o_ = o;
     v_ = v;
   }
@@ -179,7 +180,7 @@ void LadderCC::apply(Engine &E, int dt, const Tens &Lvv, int o, int v, int naux,
     const int64_t rows = (int64_t)(v - a0) * v, cols = (int64_t)(a1 - a0) * v;
     if (tc) {
       E.f64_gemm(La.rows((int64_t)a0 * v), rows, Lb.rows((int64_t)a0 * v), cols, naux, W.p, view1(cols), view1(1), zc(1.0),
-                 false);
+                 false, &upper_);
     } else {
       GemmArgs g;
       g.A = (const char *)Lvv.p + (size_t)a0 * v * es;

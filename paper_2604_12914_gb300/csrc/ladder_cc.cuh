@@ -23,6 +23,7 @@ class LadderCC {
  private:
   int o_ = -1, v_ = -1;
   DevBuf opairs, vpairs;       // pair tables (p, q), p < q
+  UpperTiles upper_;           // the formation's tiles with b > a
   DevBuf W, Wp, Xp, sig;       // group formation block, packed group block, packed X / Y', packed result
 };
 

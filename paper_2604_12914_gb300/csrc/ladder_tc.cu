@@ -205,10 +205,11 @@ void ladder_unpack_sig_bench(int o, int v, const void *S, void *out, cudaStream_
 void LadderTC::prepare(Engine &E, const Tens &Lvv, int o, int v, int naux, int seg, int kind, bool lean) {
   cudaStream_t st = E.st;
   wall_ready_ = false;  // a stored block belongs to the previous L~_vv
+  if (v_ != v) upper_.reset(v);
   o_ = o; v_ = v; naux_ = naux; seg_ = seg; kind_ = kind;
   Po_ = (int64_t)o * (o - 1) / 2;
   Pv_ = (int64_t)v * (v - 1) / 2;
-  const int64_t ld = 2 * tc_kpad(naux) * seg, es = tc_esize(kind);
+  const int64_t ld = 2 * tc_kpad(naux, kind) * seg, es = tc_esize(kind);
   const int64_t vv = (int64_t)v * v;
   Lvv_ = Lvv.p;
   LA.alloc((size_t)vv * ld * es);
@@ -291,19 +292,19 @@ void LadderTC::apply(Engine &E, int dir, zc alpha, int nrhs, const void *const *
   if (Po == 0 || Pv == 0 || nrhs < 1) return;
   E.tc_pending = true;
   const int64_t vv = (int64_t)v * v, es = tc_esize(kind);
-  const int64_t ldL = 2 * tc_kpad(naux_) * seg;
+  const int64_t ldL = 2 * tc_kpad(naux_, kind) * seg;
   const int ga = std::min(ga_, v);
   const int64_t NR = (int64_t)nrhs;
   const bool use_wall = store_ && dir > 0;
   // buffers sized for the first (largest) group
   const int64_t maxpairs = pair_start(v, ga);
-  const int64_t kpg = tc_kpad(maxpairs);
+  const int64_t kpg = tc_kpad(maxpairs, kind);
   // the (e<f) pairs in chunks of QC, so that a packed block (rows of the group's pairs, or
   // rows of the chunk's pairs in the transpose) stays within 2 GiB; the stored ablation keeps one
   const int64_t cap = 2ll << 30;
   int64_t QC = use_wall ? Pv : std::max<int64_t>(64, cap / (4 * std::max<int64_t>(kpg, 1) * seg * es) / 8 * 8);
   QC = std::min(QC, Pv);
-  const int64_t nch = (Pv + QC - 1) / QC, Kc = tc_kpad(QC), ldc = 2 * Kc * seg;
+  const int64_t nch = (Pv + QC - 1) / QC, Kc = tc_kpad(QC, kind), ldc = 2 * Kc * seg;
   if (W.bytes < (size_t)vv * ga * v * 8) W.alloc((size_t)vv * ga * v * 8);
   if (!lb_all_ && LB.bytes < (size_t)2 * ga * v * ldL * es) LB.alloc((size_t)2 * ga * v * ldL * es);
   const size_t wp_bytes = dir > 0 ? (size_t)maxpairs * ldc * es : (size_t)2 * QC * (2 * kpg * seg) * es;
@@ -365,7 +366,7 @@ void LadderTC::apply(Engine &E, int dir, zc alpha, int nrhs, const void *const *
     if (!lb_all_) tc_prep_b((const char *)Lvv_ + (size_t)a0 * v * 8, vv, 1, naux_, cols, seg, kind, LBb, ldL, st);
     CCLR_CUDA(cudaEventRecord(fev[2 * nform_], st));
     tc_gemm_seg(LAb + (int64_t)a0 * v * ldL * es, ldL, LBg, ldL, rows, 2 * cols, ldL / seg, seg, kind, W.as<float>(),
-                2 * cols, zc(1.0), false, st);
+                2 * cols, zc(1.0), false, st, &upper_);
     CCLR_CUDA(cudaEventRecord(fev[2 * nform_ + 1], st));
     ++nform_;
     if (use_wall) {  // pack the group's rows into the stored block; contract once afterwards
@@ -380,7 +381,7 @@ void LadderTC::apply(Engine &E, int dir, zc alpha, int nrhs, const void *const *
                     sig.as<float>() + 2 * p0 * Po * NR, 2 * Po * NR, zc(1.0), c > 0, st);
       }
     } else {
-      const int64_t kg = tc_kpad(np), ldg = 2 * kg * seg;
+      const int64_t kg = tc_kpad(np, kind), ldg = 2 * kg * seg;
       for (int64_t r = 0; r < NR; ++r) {
         void *dst = Xpb + Po * r * ldg * es;
         if (kind == TC_BF16)

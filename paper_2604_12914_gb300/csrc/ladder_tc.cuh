@@ -66,6 +66,7 @@ class LadderTC {
   bool lb_all_ = false;     // LB holds the embedded rows (a,e) of every a (prepared once per L~_vv)
   const void *Lvv_ = nullptr;  // the complex64 L~_vv the operands are prepared from
   DevBuf opairs, vpairs;    // pair tables (p, q), p < q, row-major pair order
+  UpperTiles upper_;        // the formation's tiles with b > a
   DevBuf W, Wp, Xp, sig;    // group formation block, packed group block, packed X, packed result
   int ga_ = 32;             // a values per group (set by tune())
   bool tuned_ = false;

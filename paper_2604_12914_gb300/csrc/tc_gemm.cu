@@ -33,6 +33,8 @@ struct TcParams {
   int nMt, nNt, band;   // tile counts; M tiles per raster band (N varies fastest inside a band)
   int kb_per_split;     // K blocks per split (splits of K are atomically summed)
   int splits;           // work units = tiles x splits, walked with stride gridDim.x
+  const uint32_t *list; // the tiles to compute, (m << 16) | n, ntiles of them (nullptr: all, in raster order)
+  int ntiles;
   int transposed;       // epilogue: 1 = lanes along columns (C columns contiguous), 0 = lane per row
   float *C;
   View2 rv, cv;         // C rows and complex columns
@@ -45,9 +47,14 @@ struct TcParams {
 // work unit -> (m tile, n tile, split); banded rasterisation: consecutive units share one B
 // tile column across a band of M tiles, so the band's A tiles and the current B tiles stay in L2
 __device__ __forceinline__ void unit_coords(const TcParams &p, int u, int &m_tile, int &n_tile, int &split) {
-  const int tiles = p.nMt * p.nNt;
-  split = u / tiles;
-  const int id = u - split * tiles;
+  split = u / p.ntiles;
+  const int id = u - split * p.ntiles;
+  if (p.list) {
+    const uint32_t mn = __ldg(p.list + id);
+    m_tile = (int)(mn >> 16);
+    n_tile = (int)(mn & 0xffff);
+    return;
+  }
   const int per_band = p.band * p.nNt;
   const int b = id / per_band;
   const int local = id - b * per_band;
@@ -78,7 +85,7 @@ __global__ void __launch_bounds__(320, 1)
   int *consumed = issued + 1;        // K blocks whose full barrier the MMA warp passed
   volatile int *abort_flag = issued + 2;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int units = p.nMt * p.nNt * p.splits;
+  const int units = p.ntiles * p.splits;
   const int nk_all = (p.K + BK - 1) / BK;
   // accumulator columns: one buffer per power of two >= BN, two buffers
   const uint32_t half = BN <= 32 ? 32u : BN <= 64 ? 64u : BN <= 128 ? 128u : 256u;
@@ -409,21 +416,6 @@ CUtensorMap make_map(const void *base, int64_t rows, int64_t cols, int64_t ld, i
   return m;
 }
 
-int pick_bn(int64_t N) {
-  if (N <= 256) return (int)((N + 15) / 16 * 16);
-  int best = 256;
-  int64_t best_waste = -1;
-  for (int bn = 256; bn >= 128; bn -= 16) {
-    int64_t tiles = (N + bn - 1) / bn;
-    int64_t waste = tiles * bn - N;
-    if (best_waste < 0 || waste < best_waste) {
-      best = bn;
-      best_waste = waste;
-    }
-  }
-  return best;
-}
-
 int num_sms() {
   int dev = 0, n = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
@@ -442,7 +434,7 @@ template <int KIND>
 void prep_launch(const void *src, View2 mv, View2 kv, int64_t MN, int64_t K, int seg, int isB, void *dst, int64_t ldd,
                  cudaStream_t st) {
   using T = typename TcElem<KIND>::T;
-  const int64_t Kp = tc_kpad(K);
+  const int64_t Kp = ldd / (2 * seg);
   const bool tiled = kv.sin != 1 && mv.sin == 1 && MN >= 8;
   if (tiled) {
     const int64_t nt = ((MN + 31) / 32) * ((Kp + 31) / 32);
@@ -459,7 +451,7 @@ void prep_launch(const void *src, View2 mv, View2 kv, int64_t MN, int64_t K, int
 
 void tc_prep_a2(const void *A, View2 mv, View2 kv, int64_t M, int64_t K, int seg, int kind, void *dst, int64_t ldd,
                 cudaStream_t st) {
-  CCLR_REQUIRE(ldd >= 2 * tc_kpad(K) * seg, "tc_prep_a: row too short");
+  CCLR_REQUIRE(ldd >= 2 * K * seg && ldd % (2 * seg) == 0, "tc_prep_a: row too short");
   if (kind == TC_BF16) prep_launch<TC_BF16>(A, mv, kv, M, K, seg, 0, dst, ldd, st);
   else prep_launch<TC_TF32>(A, mv, kv, M, K, seg, 0, dst, ldd, st);
   count_launch();
@@ -468,7 +460,7 @@ void tc_prep_a2(const void *A, View2 mv, View2 kv, int64_t M, int64_t K, int seg
 
 void tc_prep_b2(const void *B, View2 kv, View2 nv, int64_t K, int64_t N, int seg, int kind, void *dst, int64_t ldd,
                 cudaStream_t st) {
-  CCLR_REQUIRE(ldd >= 2 * tc_kpad(K) * seg, "tc_prep_b: row too short");
+  CCLR_REQUIRE(ldd >= 2 * K * seg && ldd % (2 * seg) == 0, "tc_prep_b: row too short");
   if (kind == TC_BF16) prep_launch<TC_BF16>(B, nv, kv, N, K, seg, 1, dst, ldd, st);
   else prep_launch<TC_TF32>(B, nv, kv, N, K, seg, 1, dst, ldd, st);
   count_launch();
@@ -489,6 +481,50 @@ void tc_prep_b(const void *B, int64_t sbk, int64_t sbn, int64_t K, int64_t N, in
 struct TcCfg {
   int BN = 0, splits = 0, band = 0;
 };
+
+// Clocks of a 128-byte K block of a BN-wide tile (four MMAs of BN / 2, but an MMA never takes less than 93, which
+// makes narrow tiles dear: M = N = K = 5056 complex 497 TFLOP/s in 128-wide tiles, 800 in 256-wide ones), and of a
+// tile's epilogue.
+constexpr int64_t block_clocks(int BN) { return 4 * std::max(BN / 2, 93); }
+constexpr int64_t epilogue_clocks(int BN) { return 32 * BN; }
+
+// Time in clocks of M x N tiles of width BN with K in `splits`, each SM taking every num_sms-th unit: whole waves
+// of the longer of main loop and epilogue, and the last epilogue.
+static int64_t cfg_clocks(int64_t M, int64_t Nreal, int nk, int BN, int splits, int nsm) {
+  const int64_t units = ((M + BM - 1) / BM) * ((Nreal + BN - 1) / BN) * splits, waves = (units + nsm - 1) / nsm;
+  const int64_t main = (nk + splits - 1) / splits * block_clocks(BN), epi = epilogue_clocks(BN) * (splits > 1 ? 2 : 1);
+  return waves * std::max(main, epi) + epi;
+}
+
+// the cheapest number of K splits of at least eight blocks, from min_splits on (1 unless it gains a twentieth)
+static int best_splits(int64_t M, int64_t Nreal, int nk, int BN, int min_splits, bool allow, int nsm) {
+  int best = min_splits;
+  if (!allow) return best;
+  int64_t t = cfg_clocks(M, Nreal, nk, BN, best, nsm);
+  const int64_t tiles = ((M + BM - 1) / BM) * ((Nreal + BN - 1) / BN);
+  const int most = (int)std::min<int64_t>(nk / 8, std::max<int64_t>(min_splits + 32, 2 * nsm / std::max<int64_t>(tiles, 1)));
+  for (int s = min_splits + 1; s <= most; ++s) {
+    const int64_t c = cfg_clocks(M, Nreal, nk, BN, s, nsm);
+    if (c * 20 < t * 19) { t = c; best = s; }
+  }
+  return best;
+}
+
+// the rule's tile width and splits: the cheapest by cfg_clocks, a narrower tile where it gains a tenth (per column it
+// loads more of A: 25600 x 2560 x 800 complex 838 TFLOP/s at 256, 732 at 208, which would save half a wave)
+static void rule_cfg(int64_t M, int64_t Nreal, int nk, int min_splits, bool allow, int nsm, int &BN, int &splits) {
+  if (Nreal <= 256) {
+    BN = (int)((Nreal + 15) / 16 * 16);
+    splits = best_splits(M, Nreal, nk, BN, min_splits, allow, nsm);
+    return;
+  }
+  int64_t t = -1;
+  for (int bn = 256; bn >= 128; bn -= 16) {
+    const int s = best_splits(M, Nreal, nk, bn, min_splits, allow, nsm);
+    const int64_t c = cfg_clocks(M, Nreal, nk, bn, s, nsm);
+    if (t < 0 || c * 10 < t * 9) { t = c; BN = bn; splits = s; }
+  }
+}
 
 struct TuneKey {
   int dev, kind, transposed;
@@ -511,9 +547,17 @@ thread_local bool g_tune_on = false;
 // configuration launched.
 static void tc_launch(const void *A, int64_t lda, const void *B, int64_t ldb, int64_t M, int64_t Nreal, int64_t Kreal,
                       int kind, float *C, View2 rv, View2 cv, zc alpha, bool accumulate, int max_kb_per_split,
-                      int *err, cudaStream_t st, int64_t a_cols, TcCfg cfg, TcCfg *used) {
+                      int *err, cudaStream_t st, int64_t a_cols, TcCfg cfg, TcCfg *used, UpperTiles *upper) {
   const int64_t es = tc_esize(kind), BK = BKB / es;
-  const int BN = cfg.BN > 0 ? cfg.BN : pick_bn(Nreal);
+  const int nk = (int)((Kreal + BK - 1) / BK), nsm = num_sms();
+  // the length of each accumulation chain is bounded (accuracy of the split-precision passes)
+  const int min_splits = max_kb_per_split > 0 ? (nk + max_kb_per_split - 1) / max_kb_per_split : 1;
+  // K splits need an accumulating or plain output (split partial tiles are added atomically)
+  const bool plain = rv.din == TC_ONE_LEVEL && cv.din == TC_ONE_LEVEL && cv.sin == 1;
+  int BN = cfg.BN, splits = std::max(cfg.splits, min_splits);
+  if (BN <= 0) rule_cfg(M, Nreal, nk, min_splits, accumulate || plain, nsm, BN, splits);
+  else if (cfg.splits <= 0) splits = best_splits(M, Nreal, nk, BN, min_splits, accumulate || plain, nsm);
+  splits = std::min({splits, nk, 65535});
   const CUtensorMap ma = make_map(A, M, a_cols < 0 ? Kreal : a_cols, lda, BM, BKB, kind);
   const CUtensorMap mb = make_map(B, Nreal, Kreal, ldb, BN, BKB, kind);
   TcParams p;
@@ -523,21 +567,11 @@ static void tc_launch(const void *A, int64_t lda, const void *B, int64_t ldb, in
   p.BN = BN;
   p.nMt = (int)((M + BM - 1) / BM);
   p.nNt = (int)((Nreal + BN - 1) / BN);
-  // band of M tiles whose A rows (about 32 MB) stay in L2 while N sweeps
+  // band of M tiles swept by N: as many A rows as take 32 MB (they stay in L2), and at least 20 tiles, which makes
+  // the running tiles' block of C about square (M = N = K = 7680 complex: 4 tiles 839 TFLOP/s, 20 tiles 894)
   p.band = cfg.band > 0 ? std::min(cfg.band, p.nMt)
-                        : (int)std::max<int64_t>(1, std::min<int64_t>(p.nMt, (32ll << 20) / (BM * Kreal * es + 1)));
-  const int nk = (int)((Kreal + BK - 1) / BK);
+                        : (int)std::min<int64_t>(p.nMt, std::max<int64_t>(20, (32ll << 20) / (BM * Kreal * es + 1)));
   const int64_t tiles = (int64_t)p.nMt * p.nNt;
-  const int nsm = num_sms();
-  // split K when the tile list cannot fill the GPU (two units per SM), at least 16 K blocks
-  // per split
-  int splits = 1;
-  if (cfg.splits > 0) splits = std::min(cfg.splits, nk);
-  else if (tiles < 2 * nsm && nk >= 32)
-    splits = (int)std::max<int64_t>(1, std::min<int64_t>((2 * nsm + tiles - 1) / tiles, nk / 16));
-  // bound the length of each accumulation chain (accuracy of the split-precision passes)
-  if (max_kb_per_split > 0) splits = std::max(splits, (nk + max_kb_per_split - 1) / max_kb_per_split);
-  splits = std::min(splits, 65535);
   p.kb_per_split = (nk + splits - 1) / splits;
   splits = (nk + p.kb_per_split - 1) / p.kb_per_split;  // every split has at least one K block
   p.splits = splits;
@@ -556,7 +590,9 @@ static void tc_launch(const void *A, int64_t lda, const void *B, int64_t ldb, in
                  "tc_gemm: split K without accumulation needs a plain C layout");
     CCLR_CUDA(cudaMemset2DAsync(C, (size_t)rv.sin * 8, 0, (size_t)Nreal * 4, (size_t)M, st));
   }
-  const int64_t units = tiles * splits;
+  p.ntiles = (int)tiles;
+  p.list = upper ? upper->get(p.nMt, p.nNt, p.band, BM, BN / 2, 0, 0, M, st, &p.ntiles) : nullptr;
+  const int64_t units = (int64_t)p.ntiles * splits;
   CCLR_REQUIRE(units < (1ll << 31), "tc_gemm: too many work units");
   static const bool trace = std::getenv("CCLR_TRACE") && std::getenv("CCLR_TRACE")[0] == '1';
   if (trace)
@@ -577,25 +613,29 @@ static void tc_launch(const void *A, int64_t lda, const void *B, int64_t ldb, in
   }
 }
 
-// Candidate configurations around the rule's choice: other tile widths for wide outputs, more or
-// fewer K splits where the tile list is short, and the two extreme raster bands.
-static std::vector<TcCfg> candidates(const TcCfg &rule, int64_t M, int64_t Nreal, int64_t Kreal, int kind,
-                                     bool allow_split) {
+// Candidate configurations around the rule's choice: other tile widths for wide outputs (each with its own best
+// number of splits), more or fewer K splits, and the two extreme raster bands.
+static std::vector<TcCfg> candidates(const TcCfg &rule, int64_t M, int64_t Nreal, int64_t Kreal, int kind, bool allow_split,
+                                     int max_kb_per_split) {
   std::vector<TcCfg> c{rule};
   auto add = [&](TcCfg x) {
     for (const auto &y : c)
       if (y.BN == x.BN && y.splits == x.splits && y.band == x.band) return;
     c.push_back(x);
   };
+  const int nk = (int)((Kreal + BKB / tc_esize(kind) - 1) / (BKB / tc_esize(kind)));
+  const int least = max_kb_per_split > 0 ? (nk + max_kb_per_split - 1) / max_kb_per_split : 1;
   if (Nreal > 256)
-    for (int bn : {128, 192, 256}) { TcCfg x = rule; x.BN = bn; add(x); }
-  const int64_t nk = (Kreal + BKB / tc_esize(kind) - 1) / (BKB / tc_esize(kind));
-  if (!allow_split) {
-  } else if (rule.splits > 1) {
-    TcCfg x = rule; x.splits = std::max(1, rule.splits / 2); add(x);
-    x.splits = (int)std::min<int64_t>(nk, 2 * rule.splits); add(x);
-  } else if (nk >= 16) {
-    TcCfg x = rule; x.splits = 2; add(x);
+    for (int bn : {192, 256}) {
+      TcCfg x = rule;
+      x.BN = bn;
+      x.splits = best_splits(M, Nreal, nk, bn, least, allow_split, num_sms());
+      add(x);
+    }
+  if (allow_split) {
+    TcCfg x = rule;
+    x.splits = std::max(least, rule.splits / 2); add(x);
+    if (nk >= 16) { x.splits = std::min(nk / 4, 2 * rule.splits); add(x); }
   }
   const int nMt = (int)((M + BM - 1) / BM);
   if (nMt > 1) {
@@ -607,7 +647,7 @@ static std::vector<TcCfg> candidates(const TcCfg &rule, int64_t M, int64_t Nreal
 
 static void tc_gemm_core(const void *A, int64_t lda, const void *B, int64_t ldb, int64_t M, int64_t Nreal,
                          int64_t Kreal, int kind, float *C, View2 rv, View2 cv, zc alpha, bool accumulate,
-                         int max_kb_per_split, int *err, cudaStream_t st, int64_t a_cols = -1) {
+                         int max_kb_per_split, int *err, cudaStream_t st, int64_t a_cols = -1, UpperTiles *upper = nullptr) {
   if (M <= 0 || Nreal <= 0) return;
   const int64_t es = tc_esize(kind);
   CCLR_REQUIRE(Nreal % 2 == 0, "tc_gemm: real N must be even (complex pairs)");
@@ -615,7 +655,7 @@ static void tc_gemm_core(const void *A, int64_t lda, const void *B, int64_t ldb,
   CCLR_REQUIRE(((uintptr_t)A % 16) == 0 && ((uintptr_t)B % 16) == 0, "tc_gemm: operands must be 16-byte aligned");
   CCLR_REQUIRE(M < (1ll << 31) && Nreal < (1ll << 31) && Kreal < (1ll << 31), "tc_gemm: dimension too large");
   const int transposed = (cv.sin == 1 && (cv.din == TC_ONE_LEVEL || cv.din >= 8)) ? 1 : 0;
-  const TuneKey key{current_device(), kind, transposed, M, Nreal, Kreal};
+  const TuneKey key{current_device(), kind, transposed + (upper ? 2 : 0), M, Nreal, Kreal};
   TcCfg cfg;
   bool have = false;
   {
@@ -652,7 +692,7 @@ static void tc_gemm_core(const void *A, int64_t lda, const void *B, int64_t ldb,
     if (ok) {
       TcCfg rule;
       tc_launch(A, lda, B, ldb, M, Nreal, Kreal, kind, Ct, trv, tcv, alpha, false, max_kb_per_split, err, st, a_cols,
-                TcCfg(), &rule);
+                TcCfg(), &rule, upper);
       rec.rule = rule;
       cudaEvent_t e0, e1;
       CCLR_CUDA(cudaEventCreate(&e0));
@@ -660,11 +700,11 @@ static void tc_gemm_core(const void *A, int64_t lda, const void *B, int64_t ldb,
       float best = 1e30f;
       // K splits need an accumulating or plain output (split partial tiles are added atomically)
       const bool plain = trv.din == TC_ONE_LEVEL && tcv.din == TC_ONE_LEVEL && tcv.sin == 1;
-      for (const TcCfg &cand : candidates(rule, M, Nreal, Kreal, kind, accumulate || plain)) {
+      for (const TcCfg &cand : candidates(rule, M, Nreal, Kreal, kind, accumulate || plain, max_kb_per_split)) {
         TcCfg used;
         CCLR_CUDA(cudaEventRecord(e0, st));
         tc_launch(A, lda, B, ldb, M, Nreal, Kreal, kind, Ct, trv, tcv, alpha, false, max_kb_per_split, err, st, a_cols,
-                  cand, &used);
+                  cand, &used, upper);
         CCLR_CUDA(cudaEventRecord(e1, st));
         CCLR_CUDA(cudaEventSynchronize(e1));
         float ms = 0.f;
@@ -687,7 +727,7 @@ static void tc_gemm_core(const void *A, int64_t lda, const void *B, int64_t ldb,
     cfg = rec.cfg;
   }
   tc_launch(A, lda, B, ldb, M, Nreal, Kreal, kind, C, rv, cv, alpha, accumulate, max_kb_per_split, err, st, a_cols, cfg,
-            nullptr);
+            nullptr, upper);
 }
 
 void tc_gemm(const float *A, int64_t lda, const float *B, int64_t ldb, int64_t M, int64_t Nreal,
@@ -700,21 +740,22 @@ void tc_gemm(const float *A, int64_t lda, const float *B, int64_t ldb, int64_t M
 // so the split passes keep every accumulator to at most 64 K blocks (2048 real K in TF32, 4096
 // in BF16) and sum the partial tiles in FP32.
 void tc_gemm_seg_v(const void *A, int64_t lda, const void *B, int64_t ldb, int64_t M, int64_t Nreal, int64_t Kseg,
-                   int seg, int kind, float *C, View2 rv, View2 cv, zc alpha, bool accumulate, cudaStream_t st) {
+                   int seg, int kind, float *C, View2 rv, View2 cv, zc alpha, bool accumulate, cudaStream_t st,
+                   UpperTiles *upper) {
   int *err = device_err();
   if (seg == 1) {
-    tc_gemm_core(A, lda, B, ldb, M, Nreal, Kseg, kind, C, rv, cv, alpha, accumulate, 0, err, st);
+    tc_gemm_core(A, lda, B, ldb, M, Nreal, Kseg, kind, C, rv, cv, alpha, accumulate, 0, err, st, -1, upper);
     return;
   }
   const int64_t es = tc_esize(kind);
   tc_gemm_core((const char *)A + Kseg * es, lda, (const char *)B + Kseg * es, ldb, M, Nreal, 2 * Kseg, kind, C, rv,
-               cv, alpha, accumulate, 64, err, st);
-  tc_gemm_core(A, lda, B, ldb, M, Nreal, Kseg, kind, C, rv, cv, alpha, true, 64, err, st);
+               cv, alpha, accumulate, 64, err, st, -1, upper);
+  tc_gemm_core(A, lda, B, ldb, M, Nreal, Kseg, kind, C, rv, cv, alpha, true, 64, err, st, -1, upper);
 }
 
 void tc_gemm_a_inplace(const void *A, int64_t lda_cpx, int64_t K, const float *B, int64_t ldb, int64_t M,
                        int64_t Nreal, float *C, View2 rv, View2 cv, zc alpha, bool accumulate, cudaStream_t st) {
-  tc_gemm_core(A, 2 * lda_cpx, B, ldb, M, Nreal, 2 * tc_kpad(K), TC_TF32, C, rv, cv, alpha, accumulate, 0,
+  tc_gemm_core(A, 2 * lda_cpx, B, ldb, M, Nreal, ldb, TC_TF32, C, rv, cv, alpha, accumulate, 0,
                device_err(), st, 2 * K);
 }
 
@@ -723,8 +764,47 @@ bool tc_a_inplace_ok(const void *A, int64_t lda_cpx, int64_t K) {
 }
 
 void tc_gemm_seg(const void *A, int64_t lda, const void *B, int64_t ldb, int64_t M, int64_t Nreal, int64_t Kseg,
-                 int seg, int kind, float *C, int64_t ldc_floats, zc alpha, bool accumulate, cudaStream_t st) {
-  tc_gemm_seg_v(A, lda, B, ldb, M, Nreal, Kseg, seg, kind, C, view1(ldc_floats / 2), view1(1), alpha, accumulate, st);
+                 int seg, int kind, float *C, int64_t ldc_floats, zc alpha, bool accumulate, cudaStream_t st,
+                 UpperTiles *upper) {
+  tc_gemm_seg_v(A, lda, B, ldb, M, Nreal, Kseg, seg, kind, C, view1(ldc_floats / 2), view1(1), alpha, accumulate, st, upper);
+}
+
+const uint32_t *UpperTiles::get(int nMt, int nNt, int band, int rows, int cols, int64_t m0, int64_t n0, int64_t M,
+                                cudaStream_t st, int *n) {
+  if (nMt > 0xffff || nNt > 0xffff) return nullptr;
+  for (const auto &e : lists_)
+    if (e->nMt == nMt && e->nNt == nNt && e->band == band && e->rows == rows && e->cols == cols && e->m0 == m0 &&
+        e->n0 == n0 && e->M == M) {
+      *n = e->n;
+      return (const uint32_t *)e->buf.p;
+    }
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  CCLR_CUDA(cudaStreamIsCapturing(st, &cap));
+  if (cap != cudaStreamCaptureStatusNone) return nullptr;
+  std::vector<uint32_t> t;
+  for (int b0 = 0; b0 < nMt; b0 += band)
+    for (int nt = 0; nt < nNt; ++nt)
+      for (int mt = b0; mt < std::min(nMt, b0 + band); ++mt) {
+        const int64_t last_b = (std::min<int64_t>(M, m0 + (int64_t)(mt + 1) * rows) - 1) / v_;
+        const int64_t first_a = (n0 + (int64_t)nt * cols) / v_;
+        if (last_b > first_a) t.push_back((uint32_t)mt << 16 | (uint32_t)nt);
+      }
+  if (t.empty()) return nullptr;
+  auto e = std::make_unique<List>();
+  e->nMt = nMt; e->nNt = nNt; e->band = band; e->rows = rows; e->cols = cols;
+  e->m0 = m0; e->n0 = n0; e->M = M;
+  e->n = (int)t.size();
+  try {
+    e->buf.alloc(t.size() * sizeof(uint32_t));
+  } catch (const Error &x) {
+    if (x.status != 2) throw;
+    return nullptr;  // no room: every tile is computed
+  }
+  CCLR_CUDA(cudaMemcpyAsync(e->buf.p, t.data(), e->buf.bytes, cudaMemcpyHostToDevice, st));
+  CCLR_CUDA(cudaStreamSynchronize(st));  // t is pageable and goes out of scope
+  lists_.push_back(std::move(e));
+  *n = lists_.back()->n;
+  return (const uint32_t *)lists_.back()->buf.p;
 }
 
 void tc_setup_device_flagged() {

@@ -106,9 +106,16 @@ inline View2 view1(int64_t stride) {
 // Complex K padded so that every operand row is a whole number of 16-byte units for every
 // operand type and split (2 K seg elements of 2 or 4 bytes: K a multiple of 4).
 inline int64_t tc_kpad(int64_t K) { return (K + 3) / 4 * 4; }
+// The same for rows that the tensor-core kernel streams: from K = 64 on whole 128-byte K blocks, so that every row
+// of every segment starts on a 128-byte line and a block's load touches one line per row, not two (K = 3600
+// against 3604 complex, M = N = 3600: TF32 752 against 685 TFLOP/s, BF16 x 3 1271 against 922).
+inline int64_t tc_kpad(int64_t K, int kind) {
+  const int64_t q = kind == TC_BF16 ? 32 : 16;
+  return K < 64 ? tc_kpad(K) : (K + q - 1) / q * q;
+}
 
 // seg = 1 (one pass) or 3 (split); kind = TC_TF32 or TC_BF16.  dst rows have ldd elements of
-// the operand type (>= 2*tc_kpad(K)*seg).
+// the operand type, seg segments of ldd / (2 seg) >= K complex entries each, zero beyond K.
 void tc_prep_a(const void *A, int64_t sam, int64_t sak, int64_t M, int64_t K, int seg, int kind, void *dst,
                int64_t ldd, cudaStream_t st);
 void tc_prep_b(const void *B, int64_t sbk, int64_t sbn, int64_t K, int64_t N, int seg, int kind, void *dst,
@@ -124,12 +131,15 @@ void tc_prep_b2(const void *B, View2 kv, View2 nv, int64_t K, int64_t N, int seg
 void tc_gemm(const float *A, int64_t lda, const float *B, int64_t ldb, int64_t M, int64_t Nreal,
              int64_t Kreal, float *C, int64_t ldc_floats, zc alpha, bool accumulate, cudaStream_t st);
 
+class UpperTiles;
+
 // Complex GEMM on prepared operands (elements of the operand type kind) with seg segments of
 // Kseg elements each (Kseg = 2*Kp).  seg = 1: one pass.  seg = 3: the correction terms
 // hi.lo + lo.hi (segments 1-2) and the main term hi.hi (segment 0) run as two passes with
 // separate TMEM accumulators, summed into C in FP32 by the epilogues.
 void tc_gemm_seg(const void *A, int64_t lda, const void *B, int64_t ldb, int64_t M, int64_t Nreal, int64_t Kseg,
-                 int seg, int kind, float *C, int64_t ldc_floats, zc alpha, bool accumulate, cudaStream_t st);
+                 int seg, int kind, float *C, int64_t ldc_floats, zc alpha, bool accumulate, cudaStream_t st,
+                 UpperTiles *upper = nullptr);
 // TF32 GEMM whose A is read in place: complex64 rows of K contiguous elements, lda_cpx complex
 // elements apart (no prepared copy; TF32 needs no split of A).  tc_a_inplace_ok tells whether
 // the TMA rules allow it (16-byte aligned base, row pitch a multiple of 16 bytes).
@@ -148,7 +158,8 @@ void tc_gemm_seg_flagged(const float *A, int64_t lda, const float *B, int64_t ld
 // the same with C addressed through views of its rows and its complex columns
 // (complex element (m, n) at C + 2 * (v2off(rv, m) + v2off(cv, n)) floats)
 void tc_gemm_seg_v(const void *A, int64_t lda, const void *B, int64_t ldb, int64_t M, int64_t Nreal, int64_t Kseg,
-                   int seg, int kind, float *C, View2 rv, View2 cv, zc alpha, bool accumulate, cudaStream_t st);
+                   int seg, int kind, float *C, View2 rv, View2 cv, zc alpha, bool accumulate, cudaStream_t st,
+                   UpperTiles *upper = nullptr);
 
 // Tile autotuner: while on (per host thread), the first use of a GEMM shape (operand kind, M,
 // real N, real K, epilogue layout) on a device times a handful of launch configurations (tile
