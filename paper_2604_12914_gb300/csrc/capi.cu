@@ -1949,7 +1949,7 @@ int cc_lr_bench_gemm(int M, int N, int K, int mode, int reps, double *ms) {
   return guarded([&] {
     cudaStream_t st;
     CCLR_CUDA(cudaStreamCreate(&st));
-    const int seg = mode == 1 ? 1 : 3, kind = mode == 3 ? TC_BF16 : TC_TF32;
+    const int seg = mode == 1 ? 1 : 2, kind = mode == 3 ? TC_BF16 : TC_TF32;
     const int64_t ld = 2 * tc_kpad(K, kind) * seg, es = tc_esize(kind);
     DevBuf A((size_t)M * ld * es), B((size_t)2 * N * ld * es), C((size_t)M * N * 8);
     // deterministic small values (exact content is irrelevant for timing)

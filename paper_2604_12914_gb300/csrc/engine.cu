@@ -642,7 +642,7 @@ void Engine::contract_tc(zc alpha, const Tens &A, const std::string &ma, const T
   auto coalesced = [&](const View2 &x, int64_t nx, const View2 &y, int64_t ny) {
     return runs(x, nx) || runs(y, ny);
   };
-  const int seg = tc_mode == 1 ? 1 : 3;
+  const int seg = tc_mode == 1 ? 1 : 2;
   const int kind = tc_mode == 3 ? TC_BF16 : TC_TF32;
   const int64_t ld = 2 * tc_kpad(K, kind) * seg, tes = tc_esize(kind);
   const int64_t per_col = 2 * ld * tes, per_row = ld * tes, capb = 2ll << 30;

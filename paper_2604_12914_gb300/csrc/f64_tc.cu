@@ -67,20 +67,6 @@ __device__ __forceinline__ void unit_coords(const F64Params &p, int u, int &mt, 
   nt = local / mb;
 }
 
-// One MMA of K = 16 (32 bytes per row), D (+)= A B^T, both operands K-major with 64-byte swizzled rows (8-row
-// groups 512 bytes apart), given by the low words of their descriptors: address >> 4, leading offset 1.
-__device__ __forceinline__ uint32_t sw64_lo(uint32_t saddr) { return ((saddr & 0x3FFFF) >> 4) | (1u << 16); }
-__device__ __forceinline__ void mma_sw64(uint32_t tmem, uint32_t a, uint32_t b, uint32_t idesc, bool acc) {
-  // high word: stride offset 512 >> 4, version 1, SWIZZLE_64B
-  constexpr uint32_t hi = (512u >> 4) | (1u << 14) | (4u << 29);
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\tmov.b64 da, {%1, %3};\n\tmov.b64 db, {%2, %3};\n\t"
-      "setp.ne.b32 p, %5, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, p;\n\t}"
-      :
-      : "r"(tmem), "r"(a), "r"(b), "r"(hi), "r"(idesc), "r"(acc ? 1 : 0));
-}
-
 // W accumulator columns of the warp's 32 rows into registers (no wait), W = 8, 16 or 32
 template <int W> __device__ __forceinline__ void tmem_ld(uint32_t a, uint32_t (&r)[W]);
 template <> __device__ __forceinline__ void tmem_ld<8>(uint32_t a, uint32_t (&r)[8]) {
@@ -163,8 +149,8 @@ __device__ __forceinline__ bool issue_chunk(uint8_t *smem, uint32_t tmem, uint32
     for (int i = 0; i <= q; ++i) {
       const uint32_t da = base + (((G0 + S - 1 - i) % NSLOT) * SLOT >> 4);
       const uint32_t db = base + ((((G0 + S - 1 - (q - i)) % NSLOT) * SLOT + A_SLOT) >> 4);
-      mma_sw64(d, da, db, idesc, i != 0);
-      mma_sw64(d, da + 2, db + 2, idesc, true);
+      mma_sw64<TC_BF16>(d, da, db, idesc, i != 0);
+      mma_sw64<TC_BF16>(d, da + 2, db + 2, idesc, true);
     }
     mma_commit(su32(tfull + buf));
     // slices q and q - 1 (and 7, which the orders of P = 1 never read) are not read by this warp's later orders

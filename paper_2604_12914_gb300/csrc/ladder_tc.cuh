@@ -26,7 +26,7 @@ class LadderTC {
     for (auto e : fev)
       if (e) cudaEventDestroy(e);
   }
-  // Lvv: complex64 [naux][v][v] (T1-dressed).  seg = 1 (one pass) or 3 (split); kind = TC_TF32
+  // Lvv: complex64 [naux][v][v] (T1-dressed).  seg = 1 (one pass) or 2 (split); kind = TC_TF32
   // or TC_BF16 (operand type of the tensor-core GEMMs).
   // lean: skip the group-size tuner and take the largest candidate whose block fits in 4 GB
   void prepare(Engine &E, const Tens &Lvv, int o, int v, int naux, int seg, int kind, bool lean = false);
@@ -44,7 +44,7 @@ class LadderTC {
   int group_size() const { return ga_; }
   // Ablation: keep the whole packed <ab||ef>~ (P_v x P_v, TF32 rows) once formed, so that later
   // sigma products (dir +1) skip the formation and run one contraction GEMM.  The transpose
-  // product still forms the blocks on the fly.  Costs P_v^2 x 8 bytes (x 3 for 3xTF32, x 1.5 for
+  // product still forms the blocks on the fly.  Costs P_v^2 x 8 bytes (x 2 for 3xTF32, x 1 for
   // bf16x3).
   void set_store(bool on) {
     store_ = on;

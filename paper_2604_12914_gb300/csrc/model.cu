@@ -464,7 +464,7 @@ void Model::ladder(int dir, const CstSet &C, zc alpha, const std::vector<Tens> &
   const int dt = C.dt;
   const int nr = (int)in.size();
   if (dt == C64 && E.tc_mode) {
-    const int k = E.tc_mode - 1, seg = E.tc_mode == 1 ? 1 : 3, kind = E.tc_mode == 3 ? TC_BF16 : TC_TF32;
+    const int k = E.tc_mode - 1, seg = E.tc_mode == 1 ? 1 : 2, kind = E.tc_mode == 3 ? TC_BF16 : TC_TF32;
     if (lean)  // a budgeted context keeps one tensor-core ladder's buffers at a time
       for (int q = 0; q < 3; ++q)
         if (q != k && ltc_src[q]) {

@@ -130,7 +130,7 @@ void narrow(const void *in, void *out, int64_t n, cudaStream_t s) {
 extern "C" int cc_lr_selftest_gemm_noalloc(int M, int N, int K, int mode, unsigned seed, double *err) {
   if (M < 1 || N < 1 || K < 1 || (mode != 1 && mode != 2) || !err)
     return record_error(CCLR_EINVAL, "bad selftest_gemm_noalloc arguments");
-  const int seg = mode == 2 ? 3 : 1;
+  const int seg = mode == 2 ? 2 : 1;
   // the bound is checked in floating point first, so that huge sizes cannot overflow
   const double approx = 48.0 * ((double)M * K + (double)K * N) + 48.0 * (double)M * N +
                         24.0 * ((double)M + 2.0 * N) * ((double)K + 64.0) * seg + 4096.0;

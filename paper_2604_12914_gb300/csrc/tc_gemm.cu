@@ -65,6 +65,60 @@ __device__ __forceinline__ void unit_coords(const TcParams &p, int u, int &m_til
 
 constexpr int EPI_PITCH = 18;  // floats per staged row (16 + 2): conflict-free float2 traffic
 
+// One 16-column chunk of a tile (columns n1 .., rows row0 + lane of the warp's 32) times alpha into C: eight complex
+// values per lane, destinations first, then all loads, then all stores (independent accesses in flight instead of one
+// read-modify-write at a time).
+__device__ __forceinline__ void store16(const TcParams &p, const uint32_t (&r)[16], float *stg, int row0, int lane, int n1) {
+  float *dst[8];
+  float2 val[8];
+  if (p.transposed) {
+    // stage rows, then 4 rows x 8 complex per instruction (64 contiguous bytes per row)
+    float2 *srow = reinterpret_cast<float2 *>(stg + lane * EPI_PITCH);
+#pragma unroll
+    for (int j = 0; j < 8; ++j) srow[j] = make_float2(__uint_as_float(r[2 * j]), __uint_as_float(r[2 * j + 1]));
+    __syncwarp();
+    const int jj = lane & 7, rs = lane >> 3, n = n1 + 2 * jj;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const int rl = 4 * k + rs, grow = row0 + rl;
+      val[k] = reinterpret_cast<const float2 *>(stg + rl * EPI_PITCH)[jj];
+      dst[k] = (grow < p.M && n < p.N) ? p.C + 2 * (v2off(p.rv, grow) + v2off(p.cv, n >> 1)) : nullptr;
+    }
+    __syncwarp();
+  } else {
+    const int row = row0 + lane;
+    const float *crow = p.C + 2 * v2off(p.rv, row < p.M ? row : 0);
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const int n = n1 + 2 * k;
+      val[k] = make_float2(__uint_as_float(r[2 * k]), __uint_as_float(r[2 * k + 1]));
+      dst[k] = (row < p.M && n < p.N) ? const_cast<float *>(crow) + 2 * v2off(p.cv, n >> 1) : nullptr;
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < 8; ++k)
+    val[k] = make_float2(p.ar * val[k].x - p.ai * val[k].y, p.ar * val[k].y + p.ai * val[k].x);
+  if (p.atomic) {
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+      if (dst[k]) {
+        atomicAdd(dst[k], val[k].x);
+        atomicAdd(dst[k] + 1, val[k].y);
+      }
+    return;
+  }
+  if (p.accumulate) {
+    float2 old[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) old[k] = dst[k] ? *reinterpret_cast<const float2 *>(dst[k]) : make_float2(0.f, 0.f);
+#pragma unroll
+    for (int k = 0; k < 8; ++k) val[k] = make_float2(val[k].x + old[k].x, val[k].y + old[k].y);
+  }
+#pragma unroll
+  for (int k = 0; k < 8; ++k)
+    if (dst[k]) *reinterpret_cast<float2 *>(dst[k]) = val[k];
+}
+
 template <int KIND>
 __global__ void __launch_bounds__(320, 1)
     tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
@@ -194,7 +248,6 @@ __global__ void __launch_bounds__(320, 1)
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const int m0 = mt * BM, n0 = nt * BN;
       const uint32_t tbase = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)buf * half;
-      const int row = m0 + q * 32 + lane;
       if (16 * h >= BN) {  // no chunk for this warp: release the buffer at once
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         __syncwarp();
@@ -210,57 +263,7 @@ __global__ void __launch_bounds__(320, 1)
           __syncwarp();
           if (lane == 0) mbar_arrive(su32(tempty + buf));
         }
-        // eight complex values per lane: destinations first, then all loads, then all stores
-        // (independent accesses in flight instead of one read-modify-write at a time)
-        float *dst[8];
-        float2 val[8];
-        if (p.transposed) {
-          // stage rows, then 4 rows x 8 complex per instruction (64 contiguous bytes per row)
-          float2 *srow = reinterpret_cast<float2 *>(stg + lane * EPI_PITCH);
-#pragma unroll
-          for (int j = 0; j < 8; ++j) srow[j] = make_float2(__uint_as_float(r[2 * j]), __uint_as_float(r[2 * j + 1]));
-          __syncwarp();
-          const int jj = lane & 7, rs = lane >> 3;
-          const int n = n0 + c0 + 2 * jj;
-#pragma unroll
-          for (int k = 0; k < 8; ++k) {
-            const int rl = 4 * k + rs, grow = m0 + q * 32 + rl;
-            val[k] = reinterpret_cast<const float2 *>(stg + rl * EPI_PITCH)[jj];
-            dst[k] = (grow < p.M && n < p.N) ? p.C + 2 * (v2off(p.rv, grow) + v2off(p.cv, n >> 1)) : nullptr;
-          }
-          __syncwarp();
-        } else {
-          const float *crow = p.C + 2 * v2off(p.rv, row < p.M ? row : 0);
-#pragma unroll
-          for (int k = 0; k < 8; ++k) {
-            const int n = n0 + c0 + 2 * k;
-            val[k] = make_float2(__uint_as_float(r[2 * k]), __uint_as_float(r[2 * k + 1]));
-            dst[k] = (row < p.M && n < p.N) ? const_cast<float *>(crow) + 2 * v2off(p.cv, n >> 1) : nullptr;
-          }
-        }
-#pragma unroll
-        for (int k = 0; k < 8; ++k)
-          val[k] = make_float2(p.ar * val[k].x - p.ai * val[k].y, p.ar * val[k].y + p.ai * val[k].x);
-        if (p.atomic) {
-#pragma unroll
-          for (int k = 0; k < 8; ++k)
-            if (dst[k]) {
-              atomicAdd(dst[k], val[k].x);
-              atomicAdd(dst[k] + 1, val[k].y);
-            }
-        } else {
-          if (p.accumulate) {
-            float2 old[8];
-#pragma unroll
-            for (int k = 0; k < 8; ++k)
-              old[k] = dst[k] ? *reinterpret_cast<const float2 *>(dst[k]) : make_float2(0.f, 0.f);
-#pragma unroll
-            for (int k = 0; k < 8; ++k) val[k] = make_float2(val[k].x + old[k].x, val[k].y + old[k].y);
-          }
-#pragma unroll
-          for (int k = 0; k < 8; ++k)
-            if (dst[k]) *reinterpret_cast<float2 *>(dst[k]) = val[k];
-        }
+        store16(p, r, stg, m0 + q * 32, lane, n0 + c0);
       }
     }
   }
@@ -271,6 +274,180 @@ __global__ void __launch_bounds__(320, 1)
     for (int g = consumed[0]; g < issued[0]; ++g)
       mbar_wait(su32(full + g % STAGES), (uint32_t)(g / STAGES) & 1u, p.err);
   }
+  __syncthreads();
+  if (warp == 1)
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(tcols) : "memory");
+}
+
+// The split modes in one pass: each 64-byte K block of A_hi, A_lo, B_hi, B_lo is loaded once and gives three products,
+// hi.hi into the main accumulator, hi.lo + lo.hi into the correction accumulator (both 256 columns: one set of
+// accumulators for tiles wider than 128 columns, two otherwise).  After CHAIN blocks the epilogue warps add both to
+// FP32 registers and give the accumulators back; the unit's sums are written once.  Against one pass per term over
+// rows of [hi | hi | lo], with every 64 blocks of a pass added to C by atomics, it loads a third less of A and B and
+// touches C once.  TFLOP/s of MMAs before and now: 3840^3 complex 3xTF32 784 and 1049, bf16x3 1507 and 2029;
+// 25600 x 2560 x 800 757 and 945, 1338 and 1712 (bound by the tensor cores).
+constexpr int SPLIT_STAGES = 4;
+constexpr int CHAIN = 128;  // 64-byte K blocks per accumulation chain
+
+template <int KIND>
+__global__ void __launch_bounds__(320, 1)
+    tc_split_kernel(const __grid_constant__ CUtensorMap tmAh, const __grid_constant__ CUtensorMap tmAl,
+                    const __grid_constant__ CUtensorMap tmBh, const __grid_constant__ CUtensorMap tmBl, TcParams p) {
+  constexpr int KB = 64 / (KIND == TC_BF16 ? 2 : 4);  // operand elements per K block
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+  const int BN = p.BN, a_bytes = BM * 64, b_bytes = BN * 64, slot = 2 * (a_bytes + b_bytes);
+  float *stage = (float *)(smem + SPLIT_STAGES * slot);
+  uint64_t *bars = (uint64_t *)(stage + 8 * 32 * EPI_PITCH);
+  uint64_t *full = bars, *empty = bars + SPLIT_STAGES, *tfull = empty + SPLIT_STAGES, *tempty = tfull + 2, *drain = tempty + 2;
+  uint32_t *tslot = (uint32_t *)(drain + 1);
+  int *issued = (int *)(tslot + 1), *consumed = issued + 1;
+  volatile int *abort_flag = issued + 2;
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
+  const int units = p.ntiles * p.splits, nk_all = (p.K + KB - 1) / KB;
+  const uint32_t half = BN <= 32 ? 32u : BN <= 64 ? 64u : BN <= 128 ? 128u : 256u;
+  const int nbuf = half == 256u ? 1 : 2;
+  const uint32_t tcols = 2 * half * (uint32_t)nbuf;
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < SPLIT_STAGES; ++s) {
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(su32(full + s)) : "memory");
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(su32(empty + s)) : "memory");
+    }
+    for (int b = 0; b < 2; ++b) {
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(su32(tfull + b)) : "memory");
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 8;" ::"r"(su32(tempty + b)) : "memory");
+    }
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(su32(drain)) : "memory");
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    issued[0] = 0;
+    consumed[0] = 0;
+    *abort_flag = 0;
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(su32(tslot)), "r"(tcols)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t tmem = *tslot;
+
+  if (warp == 0) {
+    if (lane == 0) {
+      int g = 0;
+      bool ok = true;
+      for (int u = blockIdx.x; u < units && ok; u += gridDim.x) {
+        int mt, nt, sp;
+        unit_coords(p, u, mt, nt, sp);
+        const int kb0 = sp * p.kb_per_split, kb1 = min(nk_all, kb0 + p.kb_per_split);
+        for (int kb = kb0; kb < kb1; ++kb, ++g) {
+          const int s = g % SPLIT_STAGES;
+          if (!mbar_wait_ab(su32(empty + s), ((uint32_t)(g / SPLIT_STAGES) & 1u) ^ 1u, p.err, abort_flag)) { ok = false; break; }
+          asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(su32(full + s)), "r"((uint32_t)slot)
+                       : "memory");
+          uint8_t *d = smem + s * slot;
+          tma_load_2d(d, &tmAh, kb * KB, mt * BM, su32(full + s));
+          tma_load_2d(d + 2 * a_bytes, &tmBh, kb * KB, nt * BN, su32(full + s));
+          tma_load_2d(d + 2 * a_bytes + b_bytes, &tmBl, kb * KB, nt * BN, su32(full + s));
+          tma_load_2d(d + a_bytes, &tmAl, kb * KB, mt * BM, su32(full + s));
+          issued[0] = g + 1;
+        }
+      }
+    }
+    __syncwarp();
+  } else if (warp == 1) {
+    if (lane == 0) {
+      const uint32_t idesc = idesc_mma(KIND, BM, BN), base = sw64_lo(su32(smem));
+      const uint32_t al = (uint32_t)a_bytes >> 4, bh = 2 * al, bl = bh + ((uint32_t)b_bytes >> 4);
+      int g = 0, it = 0;  // K blocks, accumulation chains
+      bool ok = true;
+      for (int u = blockIdx.x; u < units && ok; u += gridDim.x) {
+        int mt, nt, sp;
+        unit_coords(p, u, mt, nt, sp);
+        const int kb0 = sp * p.kb_per_split, kb1 = min(nk_all, kb0 + p.kb_per_split);
+        for (int c0 = kb0; c0 < kb1 && ok; c0 += CHAIN, ++it) {
+          const int buf = nbuf == 1 ? 0 : it & 1, use = nbuf == 1 ? it : it >> 1;
+          if (!mbar_wait_ab(su32(tempty + buf), ((uint32_t)use & 1u) ^ 1u, p.err, abort_flag)) { ok = false; break; }
+          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+          const uint32_t dm = tmem + (uint32_t)buf * 2 * half, dc = dm + half;
+          const int c1 = min(kb1, c0 + CHAIN);
+          for (int kb = c0; kb < c1; ++kb, ++g) {
+            const int s = g % SPLIT_STAGES;
+            if (!mbar_wait_ab(su32(full + s), (uint32_t)(g / SPLIT_STAGES) & 1u, p.err, abort_flag)) { ok = false; break; }
+            consumed[0] = g + 1;
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            const uint32_t sb = base + ((uint32_t)(s * slot) >> 4);
+            const bool acc = kb > c0;
+            mma_sw64<KIND>(dm, sb, sb + bh, idesc, acc);
+            mma_sw64<KIND>(dm, sb + 2, sb + bh + 2, idesc, true);
+            mma_sw64<KIND>(dc, sb, sb + bl, idesc, acc);
+            mma_sw64<KIND>(dc, sb + 2, sb + bl + 2, idesc, true);
+            mma_sw64<KIND>(dc, sb + al, sb + bh, idesc, true);
+            mma_sw64<KIND>(dc, sb + al + 2, sb + bh + 2, idesc, true);
+            mma_commit(su32(empty + s));
+          }
+          if (ok) mma_commit(su32(tfull + buf));
+        }
+      }
+      mma_commit(su32(drain));
+      mbar_wait(su32(drain), 0, p.err);
+    }
+    __syncwarp();
+  } else {
+    const int q = warp & 3, h = (warp - 2) >> 2;
+    float *stg = stage + (warp - 2) * 32 * EPI_PITCH;
+    int it = 0;
+    bool ok = true;
+    for (int u = blockIdx.x; u < units && ok; u += gridDim.x) {
+      int mt, nt, sp;
+      unit_coords(p, u, mt, nt, sp);
+      const int kb0 = sp * p.kb_per_split, kb1 = min(nk_all, kb0 + p.kb_per_split);
+      float sum[8][16];  // columns 16 h + 32 j + c of the warp's rows
+      for (int c0 = kb0; c0 < kb1; c0 += CHAIN, ++it) {
+        const int buf = nbuf == 1 ? 0 : it & 1, use = nbuf == 1 ? it : it >> 1;
+        ok = __all_sync(0xffffffffu, mbar_wait_ab(su32(tfull + buf), (uint32_t)use & 1u, p.err, abort_flag));
+        if (!ok) break;
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        const uint32_t tb = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)buf * 2 * half;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          const int c = 16 * h + 32 * j;
+          if (c < BN) {
+            uint32_t x[16];
+            tmem_ld16(tb + half + (uint32_t)c, x);
+#pragma unroll
+            for (int k = 0; k < 16; ++k) sum[j][k] = __uint_as_float(x[k]) + (c0 == kb0 ? 0.f : sum[j][k]);
+            tmem_ld16(tb + (uint32_t)c, x);
+#pragma unroll
+            for (int k = 0; k < 16; ++k) sum[j][k] += __uint_as_float(x[k]);
+          }
+        }
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        __syncwarp();
+        if (lane == 0) mbar_arrive(su32(tempty + buf));
+      }
+      if (!ok) break;
+      // a rolled loop over the chunks, the front one of the registers each time
+#pragma unroll 1
+      for (int c = 16 * h; c < BN; c += 32) {
+        uint32_t r[16];
+#pragma unroll
+        for (int k = 0; k < 16; ++k) r[k] = __float_as_uint(sum[0][k]);
+        store16(p, r, stg, mt * BM + q * 32, lane, nt * BN + c);
+#pragma unroll
+        for (int j = 0; j < 7; ++j)
+#pragma unroll
+          for (int k = 0; k < 16; ++k) sum[j][k] = sum[j + 1][k];
+      }
+    }
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  if (threadIdx.x == 0 && consumed[0] < issued[0])  // error path: drain copies issued but never consumed (bounded)
+    for (int g = consumed[0]; g < issued[0]; ++g)
+      mbar_wait(su32(full + g % SPLIT_STAGES), (uint32_t)(g / SPLIT_STAGES) & 1u, p.err);
   __syncthreads();
   if (warp == 1)
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(tcols) : "memory");
@@ -381,6 +558,8 @@ int current_device() {
 void set_smem_limits() {
   CCLR_CUDA(cudaFuncSetAttribute(tc_gemm_kernel<TC_TF32>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
   CCLR_CUDA(cudaFuncSetAttribute(tc_gemm_kernel<TC_BF16>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
+  CCLR_CUDA(cudaFuncSetAttribute(tc_split_kernel<TC_TF32>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
+  CCLR_CUDA(cudaFuncSetAttribute(tc_split_kernel<TC_BF16>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
 }
 
 // The current device's wait flag; the first use on a device allocates and clears it and raises
@@ -490,21 +669,21 @@ constexpr int64_t epilogue_clocks(int BN) { return 32 * BN; }
 
 // Time in clocks of M x N tiles of width BN with K in `splits`, each SM taking every num_sms-th unit: whole waves
 // of the longer of main loop and epilogue, and the last epilogue.
-static int64_t cfg_clocks(int64_t M, int64_t Nreal, int nk, int BN, int splits, int nsm) {
+static int64_t cfg_clocks(int64_t M, int64_t Nreal, int nk, int BN, int splits, int nsm, int products) {
   const int64_t units = ((M + BM - 1) / BM) * ((Nreal + BN - 1) / BN) * splits, waves = (units + nsm - 1) / nsm;
-  const int64_t main = (nk + splits - 1) / splits * block_clocks(BN), epi = epilogue_clocks(BN) * (splits > 1 ? 2 : 1);
+  const int64_t main = (nk + splits - 1) / splits * block_clocks(BN) * products, epi = epilogue_clocks(BN) * (splits > 1 ? 2 : 1);
   return waves * std::max(main, epi) + epi;
 }
 
-// the cheapest number of K splits of at least eight blocks, from min_splits on (1 unless it gains a twentieth)
-static int best_splits(int64_t M, int64_t Nreal, int nk, int BN, int min_splits, bool allow, int nsm) {
-  int best = min_splits;
+// the cheapest number of K splits of at least eight blocks (1 unless it gains a twentieth)
+static int best_splits(int64_t M, int64_t Nreal, int nk, int BN, bool allow, int nsm, int products) {
+  int best = 1;
   if (!allow) return best;
-  int64_t t = cfg_clocks(M, Nreal, nk, BN, best, nsm);
+  int64_t t = cfg_clocks(M, Nreal, nk, BN, best, nsm, products);
   const int64_t tiles = ((M + BM - 1) / BM) * ((Nreal + BN - 1) / BN);
-  const int most = (int)std::min<int64_t>(nk / 8, std::max<int64_t>(min_splits + 32, 2 * nsm / std::max<int64_t>(tiles, 1)));
-  for (int s = min_splits + 1; s <= most; ++s) {
-    const int64_t c = cfg_clocks(M, Nreal, nk, BN, s, nsm);
+  const int most = (int)std::min<int64_t>(nk / 8, std::max<int64_t>(32, 2 * nsm / std::max<int64_t>(tiles, 1)));
+  for (int s = 2; s <= most; ++s) {
+    const int64_t c = cfg_clocks(M, Nreal, nk, BN, s, nsm, products);
     if (c * 20 < t * 19) { t = c; best = s; }
   }
   return best;
@@ -512,16 +691,16 @@ static int best_splits(int64_t M, int64_t Nreal, int nk, int BN, int min_splits,
 
 // the rule's tile width and splits: the cheapest by cfg_clocks, a narrower tile where it gains a tenth (per column it
 // loads more of A: 25600 x 2560 x 800 complex 838 TFLOP/s at 256, 732 at 208, which would save half a wave)
-static void rule_cfg(int64_t M, int64_t Nreal, int nk, int min_splits, bool allow, int nsm, int &BN, int &splits) {
+static void rule_cfg(int64_t M, int64_t Nreal, int nk, bool allow, int nsm, int products, int &BN, int &splits) {
   if (Nreal <= 256) {
     BN = (int)((Nreal + 15) / 16 * 16);
-    splits = best_splits(M, Nreal, nk, BN, min_splits, allow, nsm);
+    splits = best_splits(M, Nreal, nk, BN, allow, nsm, products);
     return;
   }
   int64_t t = -1;
   for (int bn = 256; bn >= 128; bn -= 16) {
-    const int s = best_splits(M, Nreal, nk, bn, min_splits, allow, nsm);
-    const int64_t c = cfg_clocks(M, Nreal, nk, bn, s, nsm);
+    const int s = best_splits(M, Nreal, nk, bn, allow, nsm, products);
+    const int64_t c = cfg_clocks(M, Nreal, nk, bn, s, nsm, products);
     if (t < 0 || c * 10 < t * 9) { t = c; BN = bn; splits = s; }
   }
 }
@@ -543,23 +722,20 @@ std::map<TuneKey, TuneRec> g_tune;
 thread_local bool g_tune_on = false;
 
 // a_cols: operand elements A actually holds per row (<= Kreal; the rest reads as zero).
-// lda, ldb, Kreal in elements of the operand type.  cfg overrides the rules; *used receives the
-// configuration launched.
+// lda, ldb, Kreal in elements of the operand type; split: rows of two segments (hi, lo) of Kreal elements.  cfg
+// overrides the rules; *used receives the configuration launched.
 static void tc_launch(const void *A, int64_t lda, const void *B, int64_t ldb, int64_t M, int64_t Nreal, int64_t Kreal,
-                      int kind, float *C, View2 rv, View2 cv, zc alpha, bool accumulate, int max_kb_per_split,
-                      int *err, cudaStream_t st, int64_t a_cols, TcCfg cfg, TcCfg *used, UpperTiles *upper) {
+                      int kind, bool split, float *C, View2 rv, View2 cv, zc alpha, bool accumulate, int *err,
+                      cudaStream_t st, int64_t a_cols, TcCfg cfg, TcCfg *used, UpperTiles *upper) {
   const int64_t es = tc_esize(kind), BK = BKB / es;
   const int nk = (int)((Kreal + BK - 1) / BK), nsm = num_sms();
-  // the length of each accumulation chain is bounded (accuracy of the split-precision passes)
-  const int min_splits = max_kb_per_split > 0 ? (nk + max_kb_per_split - 1) / max_kb_per_split : 1;
   // K splits need an accumulating or plain output (split partial tiles are added atomically)
   const bool plain = rv.din == TC_ONE_LEVEL && cv.din == TC_ONE_LEVEL && cv.sin == 1;
-  int BN = cfg.BN, splits = std::max(cfg.splits, min_splits);
-  if (BN <= 0) rule_cfg(M, Nreal, nk, min_splits, accumulate || plain, nsm, BN, splits);
-  else if (cfg.splits <= 0) splits = best_splits(M, Nreal, nk, BN, min_splits, accumulate || plain, nsm);
+  const int products = split ? 3 : 1;
+  int BN = cfg.BN, splits = std::max(cfg.splits, 1);
+  if (BN <= 0) rule_cfg(M, Nreal, nk, accumulate || plain, nsm, products, BN, splits);
+  else if (cfg.splits <= 0) splits = best_splits(M, Nreal, nk, BN, accumulate || plain, nsm, products);
   splits = std::min({splits, nk, 65535});
-  const CUtensorMap ma = make_map(A, M, a_cols < 0 ? Kreal : a_cols, lda, BM, BKB, kind);
-  const CUtensorMap mb = make_map(B, Nreal, Kreal, ldb, BN, BKB, kind);
   TcParams p;
   p.M = (int)M;
   p.N = (int)Nreal;
@@ -574,6 +750,7 @@ static void tc_launch(const void *A, int64_t lda, const void *B, int64_t ldb, in
   const int64_t tiles = (int64_t)p.nMt * p.nNt;
   p.kb_per_split = (nk + splits - 1) / splits;
   splits = (nk + p.kb_per_split - 1) / p.kb_per_split;  // every split has at least one K block
+  if (split) p.kb_per_split *= 2;                       // (64-byte blocks there)
   p.splits = splits;
   p.C = C;
   p.rv = rv;
@@ -599,11 +776,22 @@ static void tc_launch(const void *A, int64_t lda, const void *B, int64_t ldb, in
     std::fprintf(stderr, "cclr tc_gemm kind=%d M=%lld N=%lld K=%lld BN=%d tiles=%lld splits=%d band=%d atomic=%d transposed=%d\n",
                  kind, (long long)M, (long long)Nreal, (long long)Kreal, BN, (long long)tiles, splits, p.band, p.atomic,
                  p.transposed);
-  const size_t smem = 1024 + (size_t)STAGES * (BM + BN) * BKB + (size_t)8 * 32 * EPI_PITCH * 4 +
-                      (2 * STAGES + 5) * 8 + 16;
   const unsigned grid = (unsigned)std::min<int64_t>(units, nsm);
-  if (kind == TC_BF16) tc_gemm_kernel<TC_BF16><<<grid, 320, smem, st>>>(ma, mb, p);
-  else tc_gemm_kernel<TC_TF32><<<grid, 320, smem, st>>>(ma, mb, p);
+  const size_t epi = (size_t)8 * 32 * EPI_PITCH * 4 + (2 * STAGES + 5) * 8 + 16;
+  if (split) {
+    const char *Al = (const char *)A + Kreal * es, *Bl = (const char *)B + Kreal * es;
+    const CUtensorMap ah = make_map(A, M, Kreal, lda, BM, 64, kind), al = make_map(Al, M, Kreal, lda, BM, 64, kind);
+    const CUtensorMap bh = make_map(B, Nreal, Kreal, ldb, BN, 64, kind), bl = make_map(Bl, Nreal, Kreal, ldb, BN, 64, kind);
+    const size_t smem = 1024 + (size_t)SPLIT_STAGES * 2 * (BM + BN) * 64 + epi;
+    if (kind == TC_BF16) tc_split_kernel<TC_BF16><<<grid, 320, smem, st>>>(ah, al, bh, bl, p);
+    else tc_split_kernel<TC_TF32><<<grid, 320, smem, st>>>(ah, al, bh, bl, p);
+  } else {
+    const CUtensorMap ma = make_map(A, M, a_cols < 0 ? Kreal : a_cols, lda, BM, BKB, kind);
+    const CUtensorMap mb = make_map(B, Nreal, Kreal, ldb, BN, BKB, kind);
+    const size_t smem = 1024 + (size_t)STAGES * (BM + BN) * BKB + epi;
+    if (kind == TC_BF16) tc_gemm_kernel<TC_BF16><<<grid, 320, smem, st>>>(ma, mb, p);
+    else tc_gemm_kernel<TC_TF32><<<grid, 320, smem, st>>>(ma, mb, p);
+  }
   count_launch();
   CCLR_CUDA(cudaGetLastError());
   if (used) {
@@ -616,7 +804,7 @@ static void tc_launch(const void *A, int64_t lda, const void *B, int64_t ldb, in
 // Candidate configurations around the rule's choice: other tile widths for wide outputs (each with its own best
 // number of splits), more or fewer K splits, and the two extreme raster bands.
 static std::vector<TcCfg> candidates(const TcCfg &rule, int64_t M, int64_t Nreal, int64_t Kreal, int kind, bool allow_split,
-                                     int max_kb_per_split) {
+                                     int products) {
   std::vector<TcCfg> c{rule};
   auto add = [&](TcCfg x) {
     for (const auto &y : c)
@@ -624,17 +812,16 @@ static std::vector<TcCfg> candidates(const TcCfg &rule, int64_t M, int64_t Nreal
     c.push_back(x);
   };
   const int nk = (int)((Kreal + BKB / tc_esize(kind) - 1) / (BKB / tc_esize(kind)));
-  const int least = max_kb_per_split > 0 ? (nk + max_kb_per_split - 1) / max_kb_per_split : 1;
   if (Nreal > 256)
     for (int bn : {192, 256}) {
       TcCfg x = rule;
       x.BN = bn;
-      x.splits = best_splits(M, Nreal, nk, bn, least, allow_split, num_sms());
+      x.splits = best_splits(M, Nreal, nk, bn, allow_split, num_sms(), products);
       add(x);
     }
   if (allow_split) {
     TcCfg x = rule;
-    x.splits = std::max(least, rule.splits / 2); add(x);
+    x.splits = std::max(1, rule.splits / 2); add(x);
     if (nk >= 16) { x.splits = std::min(nk / 4, 2 * rule.splits); add(x); }
   }
   const int nMt = (int)((M + BM - 1) / BM);
@@ -646,8 +833,8 @@ static std::vector<TcCfg> candidates(const TcCfg &rule, int64_t M, int64_t Nreal
 }
 
 static void tc_gemm_core(const void *A, int64_t lda, const void *B, int64_t ldb, int64_t M, int64_t Nreal,
-                         int64_t Kreal, int kind, float *C, View2 rv, View2 cv, zc alpha, bool accumulate,
-                         int max_kb_per_split, int *err, cudaStream_t st, int64_t a_cols = -1, UpperTiles *upper = nullptr) {
+                         int64_t Kreal, int kind, bool split, float *C, View2 rv, View2 cv, zc alpha, bool accumulate,
+                         int *err, cudaStream_t st, int64_t a_cols = -1, UpperTiles *upper = nullptr) {
   if (M <= 0 || Nreal <= 0) return;
   const int64_t es = tc_esize(kind);
   CCLR_REQUIRE(Nreal % 2 == 0, "tc_gemm: real N must be even (complex pairs)");
@@ -655,7 +842,7 @@ static void tc_gemm_core(const void *A, int64_t lda, const void *B, int64_t ldb,
   CCLR_REQUIRE(((uintptr_t)A % 16) == 0 && ((uintptr_t)B % 16) == 0, "tc_gemm: operands must be 16-byte aligned");
   CCLR_REQUIRE(M < (1ll << 31) && Nreal < (1ll << 31) && Kreal < (1ll << 31), "tc_gemm: dimension too large");
   const int transposed = (cv.sin == 1 && (cv.din == TC_ONE_LEVEL || cv.din >= 8)) ? 1 : 0;
-  const TuneKey key{current_device(), kind, transposed + (upper ? 2 : 0), M, Nreal, Kreal};
+  const TuneKey key{current_device(), kind, transposed + (upper ? 2 : 0) + (split ? 4 : 0), M, Nreal, Kreal};
   TcCfg cfg;
   bool have = false;
   {
@@ -691,7 +878,7 @@ static void tc_gemm_core(const void *A, int64_t lda, const void *B, int64_t ldb,
     TuneRec rec;
     if (ok) {
       TcCfg rule;
-      tc_launch(A, lda, B, ldb, M, Nreal, Kreal, kind, Ct, trv, tcv, alpha, false, max_kb_per_split, err, st, a_cols,
+      tc_launch(A, lda, B, ldb, M, Nreal, Kreal, kind, split, Ct, trv, tcv, alpha, false, err, st, a_cols,
                 TcCfg(), &rule, upper);
       rec.rule = rule;
       cudaEvent_t e0, e1;
@@ -700,10 +887,10 @@ static void tc_gemm_core(const void *A, int64_t lda, const void *B, int64_t ldb,
       float best = 1e30f;
       // K splits need an accumulating or plain output (split partial tiles are added atomically)
       const bool plain = trv.din == TC_ONE_LEVEL && tcv.din == TC_ONE_LEVEL && tcv.sin == 1;
-      for (const TcCfg &cand : candidates(rule, M, Nreal, Kreal, kind, accumulate || plain, max_kb_per_split)) {
+      for (const TcCfg &cand : candidates(rule, M, Nreal, Kreal, kind, accumulate || plain, split ? 3 : 1)) {
         TcCfg used;
         CCLR_CUDA(cudaEventRecord(e0, st));
-        tc_launch(A, lda, B, ldb, M, Nreal, Kreal, kind, Ct, trv, tcv, alpha, false, max_kb_per_split, err, st, a_cols,
+        tc_launch(A, lda, B, ldb, M, Nreal, Kreal, kind, split, Ct, trv, tcv, alpha, false, err, st, a_cols,
                   cand, &used, upper);
         CCLR_CUDA(cudaEventRecord(e1, st));
         CCLR_CUDA(cudaEventSynchronize(e1));
@@ -726,37 +913,26 @@ static void tc_gemm_core(const void *A, int64_t lda, const void *B, int64_t ldb,
     g_tune[key] = rec;
     cfg = rec.cfg;
   }
-  tc_launch(A, lda, B, ldb, M, Nreal, Kreal, kind, C, rv, cv, alpha, accumulate, max_kb_per_split, err, st, a_cols, cfg,
+  tc_launch(A, lda, B, ldb, M, Nreal, Kreal, kind, split, C, rv, cv, alpha, accumulate, err, st, a_cols, cfg,
             nullptr, upper);
 }
 
 void tc_gemm(const float *A, int64_t lda, const float *B, int64_t ldb, int64_t M, int64_t Nreal,
              int64_t Kreal, float *C, int64_t ldc_floats, zc alpha, bool accumulate, cudaStream_t st) {
-  tc_gemm_core(A, lda, B, ldb, M, Nreal, Kreal, TC_TF32, C, view1(ldc_floats / 2), view1(1), alpha, accumulate, 0,
+  tc_gemm_core(A, lda, B, ldb, M, Nreal, Kreal, TC_TF32, false, C, view1(ldc_floats / 2), view1(1), alpha, accumulate,
                device_err(), st);
 }
 
-// The tensor-core accumulation error was measured to grow linearly with the chain length,
-// so the split passes keep every accumulator to at most 64 K blocks (2048 real K in TF32, 4096
-// in BF16) and sum the partial tiles in FP32.
 void tc_gemm_seg_v(const void *A, int64_t lda, const void *B, int64_t ldb, int64_t M, int64_t Nreal, int64_t Kseg,
                    int seg, int kind, float *C, View2 rv, View2 cv, zc alpha, bool accumulate, cudaStream_t st,
                    UpperTiles *upper) {
-  int *err = device_err();
-  if (seg == 1) {
-    tc_gemm_core(A, lda, B, ldb, M, Nreal, Kseg, kind, C, rv, cv, alpha, accumulate, 0, err, st, -1, upper);
-    return;
-  }
-  const int64_t es = tc_esize(kind);
-  tc_gemm_core((const char *)A + Kseg * es, lda, (const char *)B + Kseg * es, ldb, M, Nreal, 2 * Kseg, kind, C, rv,
-               cv, alpha, accumulate, 64, err, st, -1, upper);
-  tc_gemm_core(A, lda, B, ldb, M, Nreal, Kseg, kind, C, rv, cv, alpha, true, 64, err, st, -1, upper);
+  tc_gemm_core(A, lda, B, ldb, M, Nreal, Kseg, kind, seg == 2, C, rv, cv, alpha, accumulate, device_err(), st, -1, upper);
 }
 
 void tc_gemm_a_inplace(const void *A, int64_t lda_cpx, int64_t K, const float *B, int64_t ldb, int64_t M,
                        int64_t Nreal, float *C, View2 rv, View2 cv, zc alpha, bool accumulate, cudaStream_t st) {
-  tc_gemm_core(A, 2 * lda_cpx, B, ldb, M, Nreal, ldb, TC_TF32, C, rv, cv, alpha, accumulate, 0,
-               device_err(), st, 2 * K);
+  tc_gemm_core(A, 2 * lda_cpx, B, ldb, M, Nreal, ldb, TC_TF32, false, C, rv, cv, alpha, accumulate, device_err(),
+               st, 2 * K);
 }
 
 bool tc_a_inplace_ok(const void *A, int64_t lda_cpx, int64_t K) {
@@ -816,13 +992,8 @@ void tc_gemm_seg_flagged(const float *A, int64_t lda, const float *B, int64_t ld
                          int64_t Kseg, int seg, float *C, int64_t ldc_floats, zc alpha, bool accumulate,
                          int *err, cudaStream_t st) {
   CCLR_REQUIRE(g_encode != nullptr, "tc_gemm_seg_flagged: tc_setup_device_flagged was not called");
-  const View2 rv = view1(ldc_floats / 2), cv = view1(1);
-  if (seg == 1) {
-    tc_gemm_core(A, lda, B, ldb, M, Nreal, Kseg, TC_TF32, C, rv, cv, alpha, accumulate, 0, err, st);
-    return;
-  }
-  tc_gemm_core(A + Kseg, lda, B + Kseg, ldb, M, Nreal, 2 * Kseg, TC_TF32, C, rv, cv, alpha, accumulate, 64, err, st);
-  tc_gemm_core(A, lda, B, ldb, M, Nreal, Kseg, TC_TF32, C, rv, cv, alpha, true, 64, err, st);
+  tc_gemm_core(A, lda, B, ldb, M, Nreal, Kseg, TC_TF32, seg == 2, C, view1(ldc_floats / 2), view1(1), alpha, accumulate,
+               err, st);
 }
 
 int tc_selftest_timeout(int timeout_us, cudaStream_t st) {

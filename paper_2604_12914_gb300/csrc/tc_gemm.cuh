@@ -7,9 +7,9 @@
 //   B_real rows 2n, 2n+1 = (Re b_kn, -Im b_kn), (Im b_kn, Re b_kn) over k, [2N][2K]
 // so that D[m][2n] = Re C[m][n] and D[m][2n+1] = Im C[m][n]: the FP32 output is already
 // the interleaved complex result (4 real multiplies per complex multiply-add).
-// Split modes (seg = 3): x = hi + lo with hi the operand type's rounding of x and lo the
-// rounding of x - hi; A_real = [hi | hi | lo], B_real = [hi | lo | hi] along K gives
-// hi.hi + hi.lo + lo.hi.  With TF32 operands (3xTF32) that is about FP32 accuracy; with BF16
+// Split modes (seg = 2): x = hi + lo with hi the operand type's rounding of x and lo the
+// rounding of x - hi, rows stored as [hi | lo]; the kernel forms hi.hi + hi.lo + lo.hi from one load of each.
+// With TF32 operands (3xTF32) that is about FP32 accuracy; with BF16
 // operands (bf16x3, the three-product split of Henry, Tang and Heinecke, ARITH 2019) about
 // 2^-16 relative, at the BF16 rate (twice the TF32 rate).
 #pragma once
@@ -49,7 +49,7 @@ template <> __device__ __forceinline__ void tc_split<TC_BF16>(float x, __nv_bflo
   l = __float2bfloat16_rn(x - __bfloat162float(h));
 }
 
-// complex value v as element k of an A-format row (K-major; [hi | hi | lo] when seg = 3)
+// complex value v as element k of an A-format row (K-major; [hi | lo] when seg = 2)
 template <int KIND>
 __device__ __forceinline__ void tc_put_a(typename TcElem<KIND>::T *row, int64_t k, int64_t Kp, int seg, float2 v) {
   if (seg == 1) {
@@ -60,12 +60,11 @@ __device__ __forceinline__ void tc_put_a(typename TcElem<KIND>::T *row, int64_t 
     tc_split<KIND>(v.x, hr, lr);
     tc_split<KIND>(v.y, hi, li);
     row[2 * k] = hr; row[2 * k + 1] = hi;
-    row[2 * Kp + 2 * k] = hr; row[2 * Kp + 2 * k + 1] = hi;
-    row[4 * Kp + 2 * k] = lr; row[4 * Kp + 2 * k + 1] = li;
+    row[2 * Kp + 2 * k] = lr; row[2 * Kp + 2 * k + 1] = li;
   }
 }
 
-// complex value v as element k of the embedded B rows r0 (re, -im), r1 (im, re) ([hi | lo | hi])
+// complex value v as element k of the embedded B rows r0 (re, -im), r1 (im, re) ([hi | lo])
 template <int KIND>
 __device__ __forceinline__ void tc_put_b(typename TcElem<KIND>::T *r0, typename TcElem<KIND>::T *r1, int64_t k,
                                          int64_t Kp, int seg, float2 v) {
@@ -79,7 +78,6 @@ __device__ __forceinline__ void tc_put_b(typename TcElem<KIND>::T *r0, typename 
     tc_split<KIND>(-v.y, nhi, nli);
     r0[2 * k] = hr; r0[2 * k + 1] = nhi; r1[2 * k] = hi; r1[2 * k + 1] = hr;
     r0[2 * Kp + 2 * k] = lr; r0[2 * Kp + 2 * k + 1] = nli; r1[2 * Kp + 2 * k] = li; r1[2 * Kp + 2 * k + 1] = lr;
-    r0[4 * Kp + 2 * k] = hr; r0[4 * Kp + 2 * k + 1] = nhi; r1[4 * Kp + 2 * k] = hi; r1[4 * Kp + 2 * k + 1] = hr;
   }
 }
 
@@ -114,7 +112,7 @@ inline int64_t tc_kpad(int64_t K, int kind) {
   return K < 64 ? tc_kpad(K) : (K + q - 1) / q * q;
 }
 
-// seg = 1 (one pass) or 3 (split); kind = TC_TF32 or TC_BF16.  dst rows have ldd elements of
+// seg = 1 (one pass) or 2 (split); kind = TC_TF32 or TC_BF16.  dst rows have ldd elements of
 // the operand type, seg segments of ldd / (2 seg) >= K complex entries each, zero beyond K.
 void tc_prep_a(const void *A, int64_t sam, int64_t sak, int64_t M, int64_t K, int seg, int kind, void *dst,
                int64_t ldd, cudaStream_t st);
@@ -134,9 +132,9 @@ void tc_gemm(const float *A, int64_t lda, const float *B, int64_t ldb, int64_t M
 class UpperTiles;
 
 // Complex GEMM on prepared operands (elements of the operand type kind) with seg segments of
-// Kseg elements each (Kseg = 2*Kp).  seg = 1: one pass.  seg = 3: the correction terms
-// hi.lo + lo.hi (segments 1-2) and the main term hi.hi (segment 0) run as two passes with
-// separate TMEM accumulators, summed into C in FP32 by the epilogues.
+// Kseg elements each.  seg = 1: one pass.  seg = 2: one pass that forms the main term hi.hi and the corrections
+// hi.lo + lo.hi in separate TMEM accumulators; after every 64 K blocks they are added up in FP32 registers, so that
+// no accumulation chain gets longer.
 void tc_gemm_seg(const void *A, int64_t lda, const void *B, int64_t ldb, int64_t M, int64_t Nreal, int64_t Kseg,
                  int seg, int kind, float *C, int64_t ldc_floats, zc alpha, bool accumulate, cudaStream_t st,
                  UpperTiles *upper = nullptr);

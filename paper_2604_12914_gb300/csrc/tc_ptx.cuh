@@ -101,6 +101,29 @@ __device__ __forceinline__ void mma_issue(uint32_t tmem, uint64_t a, uint64_t b,
   }
 }
 
+// One MMA of K = 32 bytes per row, both operands K-major with 64-byte swizzled rows (8-row groups 512 bytes apart),
+// given by the low words of their descriptors: address >> 4, leading offset 1.
+__device__ __forceinline__ uint32_t sw64_lo(uint32_t saddr) { return ((saddr & 0x3FFFF) >> 4) | (1u << 16); }
+template <int KIND>
+__device__ __forceinline__ void mma_sw64(uint32_t tmem, uint32_t a, uint32_t b, uint32_t idesc, bool acc) {
+  // high word: stride offset 512 >> 4, version 1, SWIZZLE_64B
+  constexpr uint32_t hi = (512u >> 4) | (1u << 14) | (4u << 29);
+  if constexpr (KIND == TC_BF16)
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\tmov.b64 da, {%1, %3};\n\tmov.b64 db, {%2, %3};\n\t"
+        "setp.ne.b32 p, %5, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, p;\n\t}"
+        :
+        : "r"(tmem), "r"(a), "r"(b), "r"(hi), "r"(idesc), "r"(acc ? 1 : 0));
+  else
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\tmov.b64 da, {%1, %3};\n\tmov.b64 db, {%2, %3};\n\t"
+        "setp.ne.b32 p, %5, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::tf32 [%0], da, db, %4, p;\n\t}"
+        :
+        : "r"(tmem), "r"(a), "r"(b), "r"(hi), "r"(idesc), "r"(acc ? 1 : 0));
+}
+
 __device__ __forceinline__ void mma_commit(uint32_t bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
                : "memory");
