@@ -1,4 +1,5 @@
 // Packed particle-particle ladder on tcgen05 tensor cores; see ladder_tc.cuh.
+#include <type_traits>
 #include <vector>
 
 #include "ladder_tc.cuh"
@@ -51,26 +52,64 @@ __global__ void pack_y_a(const float2 *Y, int o, int v, const int2 *op, const in
 // for the (e<f) pairs q0 .. q0 + nq - 1 (q below is the pair's offset from q0).
 // mode 0: A operand rows r = (a,b) pair - p0, K = q          (forward contraction)
 // mode 1: B operand rows 2q, 2q+1, K = r                      (transpose contraction)
-template <int KIND>
-__global__ void pack_w(const float2 *W, int64_t ldw, int v, int a0, const int2 *vp, int64_t p0,
-                       int64_t np, int64_t q0, int64_t nq, int64_t Kp, int seg, int mode, typename TcElem<KIND>::T *dst,
-                       int64_t ldd) {
-  const int64_t total = mode == 0 ? np * Kp : nq * Kp;
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total;
-       e += (int64_t)gridDim.x * blockDim.x) {
-    int64_t r, q;  // r: (a,b) pair within the group; q: (e<f) pair offset
-    if (mode == 0) { r = e / Kp; q = e % Kp; } else { q = e / Kp; r = e % Kp; }
-    const bool inside = mode == 0 ? (q < nq) : (r < np);
-    float2 val = make_float2(0.f, 0.f);
-    if (inside) {
-      const int2 ab = vp[p0 + r], ef = vp[q0 + q];
-      const int64_t rb = (int64_t)(ab.y - a0) * v, ca = (int64_t)(ab.x - a0) * v;
-      const float2 w1 = W[(rb + ef.y) * ldw + ca + ef.x];
-      const float2 w2 = W[(rb + ef.x) * ldw + ca + ef.y];
-      val = make_float2(w1.x - w2.x, w1.y - w2.y);
-    }
-    if (mode == 0) tc_put_a<KIND>(dst + r * ldd, q, Kp, seg, val);
-    else tc_put_b<KIND>(dst + (2 * q) * ldd, dst + (2 * q + 1) * ldd, r, Kp, seg, val);
+// A block takes one a, PW values of b and a PW x PW tile of (e, f), e-tile <= f-tile: both images are read along
+// their rows (whole 128-byte lines, 32 of them in flight per thread), one is turned around through shared memory,
+// and the result is written along q (mode 0) or, turned again, along r (mode 1), in 128-byte runs.  HBM-bound: W is
+// read once and the block written once.
+constexpr int PW = 16;
+template <int KIND, int MODE>
+__global__ void __launch_bounds__(PW *PW) pack_w(const float2 *__restrict__ W, int64_t ldw, int v, int a0, int64_t p0,
+                                                 int64_t q0, int64_t nq, int64_t Kp, int seg,
+                                                 typename TcElem<KIND>::T *__restrict__ dst, int64_t ldd) {
+  __shared__ float2 T[PW][PW][PW + 1];  // [b][e][f]
+  const int a = a0 + blockIdx.z, b0 = a + 1 + blockIdx.y * PW;
+  if (b0 >= v) return;
+  int te = 0, t = blockIdx.x;  // the upper triangle of tiles, row by row
+  const int nt = (v + PW - 1) / PW;
+  while (t >= nt - te) { t -= nt - te; ++te; }
+  const int e0 = te * PW, f0 = (te + t) * PW, x = threadIdx.x & (PW - 1), y = threadIdx.x / PW;
+  auto pair = [&](int p, int q) { return (int64_t)p * v - (int64_t)p * (p + 1) / 2 + (q - p - 1); };
+  const int nb = min(PW, v - b0);
+  const float2 *Wa = W + (int64_t)(a - a0) * v;
+  float2 w[PW];
+#pragma unroll
+  for (int k = 0; k < PW; ++k) {  // <ab|ef> at (f = f0 + y, e = e0 + x)
+    const bool in = k < nb && f0 + y < v && e0 + x < v;
+    w[k] = in ? Wa[((int64_t)(b0 + k - a0) * v + f0 + y) * ldw + e0 + x] : make_float2(0.f, 0.f);
+  }
+#pragma unroll
+  for (int k = 0; k < PW; ++k) T[k][x][y] = w[k];
+#pragma unroll
+  for (int k = 0; k < PW; ++k) {  // <ab|fe> at (e = e0 + y, f = f0 + x)
+    const bool in = k < nb && e0 + y < v && f0 + x < v;
+    w[k] = in ? Wa[((int64_t)(b0 + k - a0) * v + e0 + y) * ldw + f0 + x] : make_float2(0.f, 0.f);
+  }
+  __syncthreads();
+  if (MODE == 0) {
+    const int e = e0 + y, f = f0 + x;
+    const int64_t q = pair(e, f) - q0, r0 = pair(a, b0) - p0;
+    if (!(e < f && f < v && q >= 0 && q < nq)) return;
+#pragma unroll
+    for (int k = 0; k < PW; ++k)
+      if (k < nb) {
+        const float2 z = T[k][y][x];
+        tc_put_a<KIND>(dst + (r0 + k) * ldd, q, Kp, seg, make_float2(z.x - w[k].x, z.y - w[k].y));
+      }
+    return;
+  }
+#pragma unroll
+  for (int k = 0; k < PW; ++k) {
+    const float2 z = T[k][y][x];
+    T[k][y][x] = make_float2(z.x - w[k].x, z.y - w[k].y);
+  }
+  __syncthreads();
+  const int64_t r = pair(a, b0) - p0 + x;
+  if (x >= nb) return;
+  for (int j = 0; j < PW; ++j) {  // (e = e0 + j, f = f0 + y), r along the threads
+    const int e = e0 + j, f = f0 + y;
+    const int64_t q = pair(e, f) - q0;
+    if (e < f && f < v && q >= 0 && q < nq)
+      tc_put_b<KIND>(dst + (2 * q) * ldd, dst + (2 * q + 1) * ldd, r, Kp, seg, T[x][j][y]);
   }
 }
 
@@ -337,16 +376,27 @@ void LadderTC::apply(Engine &E, int dir, zc alpha, int nrhs, const void *const *
     const size_t wall_bytes = (size_t)Pv * ldc * es;
     if (Wall.bytes != wall_bytes) Wall.alloc(wall_bytes);
   }
-  // pack_w launch into dst (rows of ldd elements of the mode's operand type)
-  auto packw = [&](int a0, int64_t p0, int64_t np, int64_t q0, int64_t nq, int64_t cols, int64_t Kp, int mode,
+  // pack_w of the group a0 .. a1 - 1 into dst (rows of ldd elements of the mode's operand type); the columns beyond
+  // the pairs, up to Kp, are cleared
+  auto packw = [&](int a0, int a1, int64_t p0, int64_t np, int64_t q0, int64_t nq, int64_t cols, int64_t Kp, int mode,
                    void *dst, int64_t ldd) {
-    const int64_t total = mode == 0 ? np * Kp : nq * Kp;
-    if (kind == TC_BF16)
-      pack_w<TC_BF16><<<grid1d(total), 256, 0, st>>>(W.as<float2>(), cols, v, a0, vp, p0, np, q0, nq, Kp, seg, mode,
-                                                     (__nv_bfloat16 *)dst, ldd);
-    else
-      pack_w<TC_TF32><<<grid1d(total), 256, 0, st>>>(W.as<float2>(), cols, v, a0, vp, p0, np, q0, nq, Kp, seg, mode,
-                                                     (float *)dst, ldd);
+    const int64_t nt = (v + PW - 1) / PW, used = mode == 0 ? nq : np, rows = mode == 0 ? np : 2 * nq;
+    if (Kp > used)
+      for (int s = 0; s < seg; ++s)
+        CCLR_CUDA(cudaMemset2DAsync((char *)dst + (2 * Kp * s + 2 * used) * es, (size_t)(ldd * es), 0,
+                                    (size_t)(2 * (Kp - used) * es), (size_t)rows, st));
+    const dim3 g((unsigned)(nt * (nt + 1) / 2), (unsigned)((v - 1 - a0 + PW - 1) / PW), (unsigned)(a1 - a0));
+    auto go = [&](auto K, auto M) {
+      constexpr int KIND = decltype(K)::value, MODE = decltype(M)::value;
+      pack_w<KIND, MODE><<<g, PW * PW, 0, st>>>(W.as<float2>(), cols, v, a0, p0, q0, nq, Kp, seg,
+                                                (typename TcElem<KIND>::T *)dst, ldd);
+    };
+    using Bf = std::integral_constant<int, TC_BF16>;
+    using Tf = std::integral_constant<int, TC_TF32>;
+    using M0 = std::integral_constant<int, 0>;
+    using M1 = std::integral_constant<int, 1>;
+    if (kind == TC_BF16) mode == 0 ? go(Bf(), M0()) : go(Bf(), M1());
+    else mode == 0 ? go(Tf(), M0()) : go(Tf(), M1());
     count_launch();
   };
   for (int a0 = 0; a0 < v - 1 && !(use_wall && wall_ready_); a0 += ga) {
@@ -370,13 +420,13 @@ void LadderTC::apply(Engine &E, int dir, zc alpha, int nrhs, const void *const *
     CCLR_CUDA(cudaEventRecord(fev[2 * nform_ + 1], st));
     ++nform_;
     if (use_wall) {  // pack the group's rows into the stored block; contract once afterwards
-      packw(a0, p0, np, 0, Pv, cols, Kc, 0, (char *)Wall.p + p0 * ldc * es, ldc);
+      packw(a0, a1, p0, np, 0, Pv, cols, Kc, 0, (char *)Wall.p + p0 * ldc * es, ldc);
     } else if (dir > 0) {
       // sigT[(ab)][(r, ij)] = sum_{e<f} <ab||ef>~ X_r[i,j,e,f] for the group's pairs, all RHS, summed
       // over the chunks of (e<f)
       for (int64_t c = 0; c < nch; ++c) {
         const int64_t q0 = c * QC, nq = std::min(QC, Pv - q0);
-        packw(a0, p0, np, q0, nq, cols, Kc, 0, Wpb, ldc);
+        packw(a0, a1, p0, np, q0, nq, cols, Kc, 0, Wpb, ldc);
         tc_gemm_seg(Wpb, ldc, Xpb + c * xchunk, ldc, np, 2 * Po * NR, ldc / seg, seg, kind,
                     sig.as<float>() + 2 * p0 * Po * NR, 2 * Po * NR, zc(1.0), c > 0, st);
       }
@@ -395,7 +445,7 @@ void LadderTC::apply(Engine &E, int dir, zc alpha, int nrhs, const void *const *
       // Z[(r, ij)][(ef)] += sum_{(ab) in group} Y'_r[(ij)][(ab)] <ab||ef>~, a chunk of (e<f) at a time
       for (int64_t c = 0; c < nch; ++c) {
         const int64_t q0 = c * QC, nq = std::min(QC, Pv - q0);
-        packw(a0, p0, np, q0, nq, cols, kg, 1, Wpb, ldg);
+        packw(a0, a1, p0, np, q0, nq, cols, kg, 1, Wpb, ldg);
         tc_gemm_seg(Xpb, ldg, Wpb, ldg, Po * NR, 2 * nq, ldg / seg, seg, kind, sig.as<float>() + 2 * q0, 2 * Pv,
                     zc(1.0), true, st);
       }
