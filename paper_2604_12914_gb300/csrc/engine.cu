@@ -296,6 +296,23 @@ void Engine::contract(zc alpha, const Tens &A, const std::string &ma, const Tens
           ss[off + q] = Sv.str[mode_pos(msm, mch)];
         }
       }
+      // the leading mode contracted, all others of the result in the same contiguous order
+      {
+        const std::string rest = mbig.substr(1);
+        bool lead = Bt.rank >= 2 && rest == mc && mode_pos(mc, mbig[0]) < 0;
+        int64_t e2 = 1;
+        for (int q = C.rank - 1; q >= 0 && lead; --q) {
+          lead = C.str[q] == e2 || C.dim[q] == 1;
+          e2 *= C.dim[q];
+        }
+        if (lead && e2 < ((int64_t)1 << 38)) {
+          if (trace_on())
+            std::fprintf(stderr, "cclr contract colsum %s,%s->%s P=%lld R=%lld dt=%d\n", ma.c_str(), mb.c_str(), mc.c_str(),
+                         (long long)Bt.dim[0], (long long)e2, dt);
+          contract_colsum_gemv(dt, Bt.dim[0], e2, Bt.p, Sv.p, Sv.str[mode_pos(msm, mbig[0])], C.p, alpha, st);
+          return;
+        }
+      }
       if (!((rmask & 4) && (rmask & 8))) {
         if (trace_on())
           std::fprintf(stderr, "cclr contract gemv %s,%s->%s dims %lld %lld %lld %lld rmask %d dt=%d\n", ma.c_str(),

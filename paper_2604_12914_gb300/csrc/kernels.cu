@@ -992,8 +992,10 @@ __global__ void __launch_bounds__(128) smallk_kernel(int64_t P, int K, int J, in
   }
 }
 
-// The complex64 case with k <= 32: each thread keeps its column X[p][.][q] in registers (all K loads
-// issued at once), prefetches eight outputs at a time, and reads S from shared memory.
+// The complex64 case with k <= 32: each thread keeps two columns X[p][.][q], X[p][.][q + 128] in registers (all loads
+// issued at once; KT is k rounded up to 8, S zero beyond), prefetches four outputs of each, and reads S two entries per
+// load from shared memory, eight loads' issue time for 32 FMAs' (with one column and one entry per load the loads
+// took as long as the FMAs: 32 x 32 on 32 x 32 x 240 x 240, 0.80 ms; the FMAs alone are 0.20, the memory 0.21).
 template <int KT>
 __global__ void __launch_bounds__(128) smallk_reg_kernel(int64_t P, int K, int J, int64_t Q,
                                                          const float2 *__restrict__ S, int64_t sSk, int64_t sSj,
@@ -1001,52 +1003,59 @@ __global__ void __launch_bounds__(128) smallk_reg_kernel(int64_t P, int K, int J
                                                          float2 *__restrict__ Y, int64_t sYp, int64_t sYj, float ar,
                                                          float ai) {
   extern __shared__ __align__(16) unsigned char smr_raw[];
-  float2 *Ss = (float2 *)smr_raw;  // [K][J]
-  for (int e = threadIdx.x; e < K * J; e += blockDim.x) {
-    const int k = e / J, j = e % J;
-    Ss[e] = S[(int64_t)k * sSk + (int64_t)j * sSj];
+  float2 *Ss = (float2 *)smr_raw;  // [KT][JP], JP = J rounded up to 4
+  const int JP = (J + 3) & ~3;
+  for (int e = threadIdx.x; e < KT * JP; e += blockDim.x) {
+    const int k = e / JP, j = e % JP;
+    Ss[e] = k < K && j < J ? S[(int64_t)k * sSk + (int64_t)j * sSj] : make_float2(0.f, 0.f);
   }
   __syncthreads();
-  const int64_t nqt = (Q + 127) / 128;
+  const int64_t nqt = (Q + 255) / 256;
   for (int64_t t = blockIdx.x; t < P * nqt; t += gridDim.x) {
-    const int64_t p = t / nqt, q = (t % nqt) * 128 + threadIdx.x;
-    if (q >= Q) continue;
+    const int64_t p = t / nqt, q = (t % nqt) * 256 + threadIdx.x;
+    const bool in[2] = {q < Q, q + 128 < Q};
+    if (!in[0]) continue;
     const float2 *xp = X + p * sXp + q;
-    float2 x[KT];
+    float2 x[2][KT];
 #pragma unroll
-    for (int k = 0; k < KT; ++k) x[k] = k < K ? xp[(int64_t)k * sXk] : make_float2(0.f, 0.f);
+    for (int k = 0; k < KT; ++k)
+#pragma unroll
+      for (int c = 0; c < 2; ++c)
+        x[c][k] = k < K && in[c] ? xp[(int64_t)k * sXk + c * 128] : make_float2(0.f, 0.f);
     float2 *yp = Y + p * sYp + q;
-    for (int j0 = 0; j0 < J; j0 += 8) {
-      float2 yv[8];
+    for (int j0 = 0; j0 < J; j0 += 4) {
+      float2 yv[2][4], acc[2][4];
 #pragma unroll
-      for (int u = 0; u < 8; ++u)
-        if (j0 + u < J) yv[u] = yp[(int64_t)(j0 + u) * sYj];
-      float re[8], im[8];
+      for (int c = 0; c < 2; ++c)
 #pragma unroll
-      for (int u = 0; u < 8; ++u) { re[u] = 0.f; im[u] = 0.f; }
+        for (int u = 0; u < 4; ++u) {
+          yv[c][u] = j0 + u < J && in[c] ? yp[(int64_t)(j0 + u) * sYj + c * 128] : make_float2(0.f, 0.f);
+          acc[c][u] = make_float2(0.f, 0.f);
+        }
 #pragma unroll
       for (int k = 0; k < KT; ++k) {
-        if (k < K) {
-          const float2 *sr = Ss + k * J + j0;
+        const float4 s01 = *reinterpret_cast<const float4 *>(Ss + k * JP + j0);
+        const float4 s23 = *reinterpret_cast<const float4 *>(Ss + k * JP + j0 + 2);
+        const float2 sv[4] = {make_float2(s01.x, s01.y), make_float2(s01.z, s01.w), make_float2(s23.x, s23.y),
+                              make_float2(s23.z, s23.w)};
 #pragma unroll
-          for (int u = 0; u < 8; ++u) {
-            if (j0 + u < J) {
-              const float2 sv = sr[u];
-              re[u] += sv.x * x[k].x - sv.y * x[k].y;
-              im[u] += sv.x * x[k].y + sv.y * x[k].x;
-            }
+        for (int c = 0; c < 2; ++c)
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            acc[c][u].x += sv[u].x * x[c][k].x - sv[u].y * x[c][k].y;
+            acc[c][u].y += sv[u].x * x[c][k].y + sv[u].y * x[c][k].x;
           }
-        }
       }
 #pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        if (j0 + u < J) {
-          float2 y = yv[u];
-          y.x += ar * re[u] - ai * im[u];
-          y.y += ar * im[u] + ai * re[u];
-          yp[(int64_t)(j0 + u) * sYj] = y;
-        }
-      }
+      for (int c = 0; c < 2; ++c)
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (j0 + u < J && in[c]) {
+            float2 y = yv[c][u];
+            y.x += ar * acc[c][u].x - ai * acc[c][u].y;
+            y.y += ar * acc[c][u].y + ai * acc[c][u].x;
+            yp[(int64_t)(j0 + u) * sYj + c * 128] = y;
+          }
     }
   }
 }
@@ -1071,9 +1080,18 @@ void contract_smallk(int dt, int64_t P, int K, int J, int64_t Q, const void *S, 
   const int64_t tiles = P * ((Q + 127) / 128);
   const unsigned grid = (unsigned)std::min<int64_t>(tiles, (int64_t)152 * 16);
   if (dt == C64 && K <= 32) {
-    smallk_reg_kernel<32><<<grid, 128, (size_t)K * J * 8, st>>>(P, K, J, Q, (const float2 *)S, sSk, sSj,
-                                                                (const float2 *)X, sXp, sXk, (float2 *)Y, sYp, sYj,
-                                                                (float)alpha.re, (float)alpha.im);
+    const int64_t t2 = P * ((Q + 255) / 256);
+    const unsigned g2 = (unsigned)std::min<int64_t>(t2, (int64_t)152 * 16);
+    auto go = [&](auto kt) {
+      constexpr int KT = decltype(kt)::value;
+      smallk_reg_kernel<KT><<<g2, 128, (size_t)KT * ((J + 3) & ~3) * 8, st>>>(
+          P, K, J, Q, (const float2 *)S, sSk, sSj, (const float2 *)X, sXp, sXk, (float2 *)Y, sYp, sYj, (float)alpha.re,
+          (float)alpha.im);
+    };
+    if (K <= 8) go(std::integral_constant<int, 8>());
+    else if (K <= 16) go(std::integral_constant<int, 16>());
+    else if (K <= 24) go(std::integral_constant<int, 24>());
+    else go(std::integral_constant<int, 32>());
     count_launch();
     CCLR_CUDA(cudaGetLastError());
     return;
@@ -1122,6 +1140,7 @@ __global__ void __launch_bounds__(256) slab_gemv_kernel(int64_t d0, int64_t d1, 
     if (r2) {  // one warp per row x2, lanes along the contiguous contracted x3
       for (int64_t x2 = warp; x2 < d2; x2 += nwarps) {
         T re = 0, im = 0;
+#pragma unroll 4
         for (int64_t x3 = lane; x3 < d3; x3 += 32) {
           const C2 b = slab[x2 * d3 + x3], sv = sb[x3 * s3];
           re += b.x * sv.x - b.y * sv.y;
@@ -1137,6 +1156,7 @@ __global__ void __launch_bounds__(256) slab_gemv_kernel(int64_t d0, int64_t d1, 
       if (g < G) {
         for (int64_t x3 = c; x3 < d3; x3 += w3) {
           T re = 0, im = 0;
+#pragma unroll 8
           for (int64_t x2 = g; x2 < d2; x2 += G) {
             const C2 b = slab[x2 * d3 + x3], sv = sb[(r3 ? 0 : x3 * s3) + x2 * s2];
             re += b.x * sv.x - b.y * sv.y;
@@ -1176,6 +1196,44 @@ void contract_slab_gemv(int dt, const int64_t *d, int rmask, const void *B, cons
     slab_gemv_kernel<float><<<grid, 256, smem, st>>>(d[0], d[1], d[2], d[3], rmask, (const float2 *)B,
                                                      (const float2 *)S, ss[0], ss[1], ss[2], ss[3], (float2 *)Y, ys[0],
                                                      ys[1], ys[2], ys[3], (float)alpha.re, (float)alpha.im);
+  count_launch();
+  CCLR_CUDA(cudaGetLastError());
+}
+
+// y[r] += alpha sum_p B[p][r] w[p] for a contiguous [P][R] array: threads along r, blocks over ranges of p whose
+// partial sums are added with atomics; one coalesced pass over B (memory-bound: 800 x 25600 complex64 113 us as a
+// GEMM with one column).
+template <typename T>
+__global__ void __launch_bounds__(256) colsum_gemv_kernel(int64_t P, int64_t R, int64_t step, const typename cpx<T>::t *__restrict__ B,
+                                                          const typename cpx<T>::t *__restrict__ w, int64_t sw,
+                                                          typename cpx<T>::t *__restrict__ y, T ar, T ai) {
+  const int64_t r = (int64_t)blockIdx.x * 256 + threadIdx.x;
+  if (r >= R) return;
+  const int64_t p1 = min(P, (int64_t)(blockIdx.y + 1) * step);
+  T re = 0, im = 0;
+#pragma unroll 8
+  for (int64_t p = (int64_t)blockIdx.y * step; p < p1; ++p) {
+    const auto b = B[p * R + r], s = w[p * sw];
+    re += b.x * s.x - b.y * s.y;
+    im += b.x * s.y + b.y * s.x;
+  }
+  atomicAdd(&y[r].x, ar * re - ai * im);
+  atomicAdd(&y[r].y, ar * im + ai * re);
+}
+
+void contract_colsum_gemv(int dt, int64_t P, int64_t R, const void *B, const void *w, int64_t sw, void *y, zc alpha,
+                          cudaStream_t st) {
+  const int64_t bx = (R + 255) / 256;
+  // about eight blocks per SM, of at least 32 rows
+  const int64_t ny = std::max<int64_t>(1, std::min<int64_t>({(8 * 152 + bx - 1) / bx, P / 32, (int64_t)65535}));
+  const int64_t step = (P + ny - 1) / ny;
+  const dim3 g((unsigned)bx, (unsigned)((P + step - 1) / step));
+  if (dt == C128)
+    colsum_gemv_kernel<double><<<g, 256, 0, st>>>(P, R, step, (const double2 *)B, (const double2 *)w, sw, (double2 *)y,
+                                                  alpha.re, alpha.im);
+  else
+    colsum_gemv_kernel<float><<<g, 256, 0, st>>>(P, R, step, (const float2 *)B, (const float2 *)w, sw, (float2 *)y,
+                                                 (float)alpha.re, (float)alpha.im);
   count_launch();
   CCLR_CUDA(cudaGetLastError());
 }

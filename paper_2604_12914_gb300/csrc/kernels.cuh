@@ -54,6 +54,10 @@ void vec_precond(int dt, int64_t n, const double *D, double omega, double omega_
 void build_diag(int o, int v, const void *Foo, const void *Fvv, double *D1, double *D2p,
                 cudaStream_t st);
 
+// y[r] += alpha sum_p B[p][r] w[p * sw], B [P][R] contiguous, y contiguous
+void contract_colsum_gemv(int dt, int64_t P, int64_t R, const void *B, const void *w, int64_t sw, void *y, zc alpha,
+                          cudaStream_t st);
+
 // Packed (unique-amplitude) doubles: P[(i<j) * P_v + (a<b)], pairs (p<q) of n indices numbered
 // row by row, pair(p, q) = p n - p (p + 1) / 2 + q - p - 1.  The full tensor F[o][o][v][v] is
 // antisymmetric in (i,j) and (a,b).

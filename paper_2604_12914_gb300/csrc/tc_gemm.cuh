@@ -81,6 +81,35 @@ __device__ __forceinline__ void tc_put_b(typename TcElem<KIND>::T *r0, typename 
   }
 }
 
+// The same for two neighbouring entries k (even), k + 1: four operand elements per store.
+__device__ __forceinline__ void tc_store4(float *p, float a, float b, float c, float d) {
+  *reinterpret_cast<float4 *>(p) = make_float4(a, b, c, d);
+}
+__device__ __forceinline__ void tc_store4(__nv_bfloat16 *p, __nv_bfloat16 a, __nv_bfloat16 b, __nv_bfloat16 c, __nv_bfloat16 d) {
+  __nv_bfloat162 v[2] = {__halves2bfloat162(a, b), __halves2bfloat162(c, d)};
+  *reinterpret_cast<uint2 *>(p) = *reinterpret_cast<uint2 *>(v);
+}
+template <int KIND>
+__device__ __forceinline__ void tc_put_a_pair(typename TcElem<KIND>::T *row, int64_t k, int64_t Kp, int seg, float2 v, float2 w) {
+  if (seg == 1) {
+    tc_store4(row + 2 * k, tc_one<KIND>(v.x), tc_one<KIND>(v.y), tc_one<KIND>(w.x), tc_one<KIND>(w.y));
+    return;
+  }
+  typename TcElem<KIND>::T h[4], l[4];
+  tc_split<KIND>(v.x, h[0], l[0]);
+  tc_split<KIND>(v.y, h[1], l[1]);
+  tc_split<KIND>(w.x, h[2], l[2]);
+  tc_split<KIND>(w.y, h[3], l[3]);
+  tc_store4(row + 2 * k, h[0], h[1], h[2], h[3]);
+  tc_store4(row + 2 * Kp + 2 * k, l[0], l[1], l[2], l[3]);
+}
+template <int KIND>
+__device__ __forceinline__ void tc_put_b_pair(typename TcElem<KIND>::T *r0, typename TcElem<KIND>::T *r1, int64_t k, int64_t Kp,
+                                              int seg, float2 v, float2 w) {
+  tc_put_a_pair<KIND>(r0, k, Kp, seg, make_float2(v.x, -v.y), make_float2(w.x, -w.y));
+  tc_put_a_pair<KIND>(r1, k, Kp, seg, make_float2(v.y, v.x), make_float2(w.y, w.x));
+}
+
 // Two-level strided index view: offset(i) = (i / din) * sout + (i % din) * sin (elements).
 // One level: din = TC_ONE_LEVEL, sout = 0.
 constexpr int64_t TC_ONE_LEVEL = (int64_t)1 << 62;
