@@ -279,6 +279,172 @@ __global__ void __launch_bounds__(320, 1)
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(tcols) : "memory");
 }
 
+// The same GEMM by pairs of CTAs: a pair computes 256 x BN tiles (BN a multiple of 32), each CTA loading its 128 rows
+// of A and half the rows of B, and the first CTA issuing the MMAs for both.  A 128-row CTA of its own loads 94 bytes
+// per clock and SM at BN = 256, which L2 does not keep up with; here it is 62, and the ring holds six blocks instead
+// of four.  TFLOP/s before and now: 28800 x 7680 x 1200 complex 924 and 1144, 3840^3 860 and 1131, 7680^3 894 and 1187,
+// 25600 x 2560 x 800 849 and 1063.
+constexpr int PAIR_STAGES = 6;
+
+template <int KIND>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(320, 1)
+    tc_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, TcParams p) {
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+  constexpr int BK = BKB / (KIND == TC_BF16 ? 2 : 4);  // operand elements per K block
+  const int BN = p.BN, HN = BN / 2;
+  uint8_t *sA = smem;
+  uint8_t *sB = smem + PAIR_STAGES * BM * BKB;
+  float *stage = (float *)(smem + PAIR_STAGES * (BM + HN) * BKB);  // 8 warps x 32 rows x EPI_PITCH
+  // full and tempty are waited for in CTA 0 only; empty and tfull arrive in both
+  uint64_t *bars = (uint64_t *)(stage + 8 * 32 * EPI_PITCH);
+  uint64_t *full = bars, *empty = bars + PAIR_STAGES, *tfull = empty + PAIR_STAGES, *tempty = tfull + 2, *drain = tempty + 2;
+  uint32_t *tslot = (uint32_t *)(drain + 1);
+  int *issued = (int *)(tslot + 1), *consumed = issued + 1;
+  volatile int *abort_flag = issued + 2;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint32_t rank = cta_rank();
+  const int pair = blockIdx.x >> 1, npairs = gridDim.x >> 1;
+  const int units = p.ntiles * p.splits, nk_all = (p.K + BK - 1) / BK;
+  const uint32_t half = BN <= 32 ? 32u : BN <= 64 ? 64u : BN <= 128 ? 128u : 256u;
+  const uint32_t tcols = 2 * half;
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < PAIR_STAGES; ++s) {
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(su32(full + s)) : "memory");
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(su32(empty + s)) : "memory");
+    }
+    for (int b = 0; b < 2; ++b) {
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(su32(tfull + b)) : "memory");
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 16;" ::"r"(su32(tempty + b)) : "memory");  // 8 warps of both CTAs
+    }
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(su32(drain)) : "memory");
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmA)) : "memory");
+    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmB)) : "memory");
+    issued[0] = 0;
+    consumed[0] = 0;
+    *abort_flag = 0;
+  }
+  __syncthreads();
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(su32(tslot)), "r"(tcols)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  pair_sync();  // both CTAs' barriers are initialised
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t tmem = *tslot;
+
+  if (warp == 0) {
+    if (lane == 0) {
+      // TMA producer of this CTA's half of the operands; both halves count on CTA 0's full barrier
+      const uint32_t bytes = (uint32_t)(2 * BM + BN) * BKB;
+      int g = 0, s = 0;
+      uint32_t ph = 0;
+      bool ok = true;
+      for (int u = pair; u < units && ok; u += npairs) {
+        int mt, nt, sp;
+        unit_coords(p, u, mt, nt, sp);
+        const int kb0 = sp * p.kb_per_split;
+        const int nk = max(0, min(nk_all - kb0, p.kb_per_split));
+        const int y_a = (2 * mt + (int)rank) * BM, y_b = nt * BN + (int)rank * HN;
+        for (int kb = 0; kb < nk; ++kb, ++g) {
+          if (!mbar_wait_ab(su32(empty + s), ph ^ 1u, p.err, abort_flag)) { ok = false; break; }
+          const uint32_t fb = pair_addr(su32(full + s), 0);
+          if (rank == 0)
+            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(su32(full + s)), "r"(bytes)
+                         : "memory");
+          tma_load_2d_pair(sA + s * BM * BKB, &tmA, (kb0 + kb) * BK, y_a, fb);
+          tma_load_2d_pair(sB + s * HN * BKB, &tmB, (kb0 + kb) * BK, y_b, fb);
+          issued[0] = g + 1;
+          if (++s == PAIR_STAGES) { s = 0; ph ^= 1u; }
+        }
+      }
+    }
+    __syncwarp();
+  } else if (warp == 1) {
+    if (rank == 0 && elect_one()) {
+      // MMA issuer of the pair: accumulator buffer it & 1 for the it-th unit
+      const uint32_t idesc = idesc_mma(KIND, 2 * BM, BN);
+      int g = 0, it = 0, s = 0;
+      uint32_t ph = 0;
+      bool ok = true;
+      for (int u = pair; u < units && ok; u += npairs, ++it) {
+        int mt, nt, sp;
+        unit_coords(p, u, mt, nt, sp);
+        const int kb0 = sp * p.kb_per_split;
+        const int nk = max(0, min(nk_all - kb0, p.kb_per_split));
+        const int buf = it & 1;
+        if (!mbar_wait_ab(su32(tempty + buf), ((uint32_t)(it >> 1) & 1u) ^ 1u, p.err, abort_flag)) break;
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        const uint32_t dacc = tmem + (uint32_t)buf * half;
+        for (int kb = 0; kb < nk; ++kb, ++g) {
+          if (!mbar_wait_ab(su32(full + s), ph, p.err, abort_flag)) { ok = false; break; }
+          consumed[0] = g + 1;
+          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+          const uint64_t da = sw128_desc(su32(sA + s * BM * BKB));
+          const uint64_t db = sw128_desc(su32(sB + s * HN * BKB));
+#pragma unroll
+          for (int kk = 0; kk < BKB / 32; ++kk)  // 32 bytes of K per instruction (+2 in 16-byte units)
+            mma_issue_pair<KIND>(dacc, da + 2 * kk, db + 2 * kk, idesc, (kb | kk) != 0 ? 1u : 0u);
+          mma_commit_pair(su32(empty + s));
+          if (++s == PAIR_STAGES) { s = 0; ph ^= 1u; }
+        }
+        if (ok) mma_commit_pair(su32(tfull + buf));  // arrives once this unit's MMAs have completed
+      }
+      // every MMA issued above has completed once this arrives
+      mma_commit_pair(su32(drain));
+      mbar_wait(su32(drain), 0, p.err);
+    }
+    __syncwarp();
+  } else {
+    // epilogue warps 2..9, as above, for this CTA's 128 rows
+    const int q = warp & 3, h = (warp - 2) >> 2;
+    float *stg = stage + (warp - 2) * 32 * EPI_PITCH;
+    int it = 0;
+    for (int u = pair; u < units; u += npairs, ++it) {
+      int mt, nt, sp;
+      unit_coords(p, u, mt, nt, sp);
+      const int buf = it & 1;
+      bool ok = mbar_wait_ab(su32(tfull + buf), (uint32_t)(it >> 1) & 1u, p.err, abort_flag);
+      ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
+      if (!ok) break;
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      const int m0 = (2 * mt + (int)rank) * BM, n0 = nt * BN;
+      const uint32_t tbase = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)buf * half;
+      for (int c0 = 16 * h; c0 < BN; c0 += 32) {
+        uint32_t r[16];
+        tmem_ld16(tbase + (uint32_t)c0, r);
+        if (c0 + 32 >= BN) {
+          // the accumulator buffer is free for the next unit once every warp of both CTAs has read its part
+          asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+          __syncwarp();
+          if (lane == 0) mbar_arrive_cluster(pair_addr(su32(tempty + buf), 0));
+        }
+        store16(p, r, stg, m0 + q * 32, lane, n0 + c0);
+      }
+    }
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  if (threadIdx.x == 0 && *abort_flag) {
+    // error path: drain the copies of both CTAs that CTA 0 expected but never consumed (bounded); copies of CTA 1 that
+    // CTA 0 never expected have no barrier to wait for, so both CTAs stay for 10 ms, which no copy takes
+    if (rank == 0)
+      for (int g = consumed[0]; g < issued[0]; ++g)
+        mbar_wait(su32(full + g % PAIR_STAGES), (uint32_t)(g / PAIR_STAGES) & 1u, p.err);
+    const unsigned long long t0 = gtime();
+    while (gtime() - t0 < 10000000ull) {}
+  }
+  __syncthreads();
+  pair_sync();  // neither CTA leaves (or frees its TMEM) while the other's MMAs, copies or arrivals may touch it
+  if (warp == 1)
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(tcols) : "memory");
+}
+
 // The split modes in one pass: each 64-byte K block of A_hi, A_lo, B_hi, B_lo is loaded once and gives three products,
 // hi.hi into the main accumulator, hi.lo + lo.hi into the correction accumulator (both 256 columns: one set of
 // accumulators for tiles wider than 128 columns, two otherwise).  After CHAIN blocks the epilogue warps add both to
@@ -550,6 +716,8 @@ int current_device() {
 void set_smem_limits() {
   CCLR_CUDA(cudaFuncSetAttribute(tc_gemm_kernel<TC_TF32>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
   CCLR_CUDA(cudaFuncSetAttribute(tc_gemm_kernel<TC_BF16>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
+  CCLR_CUDA(cudaFuncSetAttribute(tc_pair_kernel<TC_TF32>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
+  CCLR_CUDA(cudaFuncSetAttribute(tc_pair_kernel<TC_BF16>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
   CCLR_CUDA(cudaFuncSetAttribute(tc_split_kernel<TC_TF32>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
   CCLR_CUDA(cudaFuncSetAttribute(tc_split_kernel<TC_BF16>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
 }
@@ -653,53 +821,72 @@ void tc_prep_b(const void *B, int64_t sbk, int64_t sbn, int64_t K, int64_t N, in
   tc_prep_b2(B, view1(sbk), view1(sbn), K, N, seg, kind, dst, ldd, st);
 }
 
-// Launch configuration: tile width BN, K splits and raster band (0 = the rule's choice).
+// Launch configuration: tile width BN, K splits and raster band (0 = the rule's choice), and whether pairs of CTAs take
+// 256-row tiles (read with BN > 0 only).
 struct TcCfg {
   int BN = 0, splits = 0, band = 0;
+  bool pair = false;
 };
 
-// Clocks of a 128-byte K block of a BN-wide tile (four MMAs of BN / 2, but an MMA never takes less than 93, which
-// makes narrow tiles dear: M = N = K = 5056 complex 497 TFLOP/s in 128-wide tiles, 800 in 256-wide ones), and of a
-// tile's epilogue.
-constexpr int64_t block_clocks(int BN) { return 4 * std::max(BN / 2, 93); }
+// Clocks of a 128-byte K block of a BN-wide tile: four MMAs of BN / 2, but an MMA never takes less than 93, which
+// makes narrow tiles dear (M = N = K = 5056 complex 497 TFLOP/s in 128-wide tiles, 800 in 256-wide ones), and in the
+// one-pass kernels not less than L2 takes to feed an SM, about 84 bytes per clock.
+constexpr int64_t block_clocks(int BN, bool pair, bool split) {
+  const int64_t mma = 4 * std::max(BN / 2, 93), feed = (BM + (pair ? BN / 2 : BN)) * BKB / 84;
+  return split ? 3 * mma : std::max(mma, feed);
+}
 constexpr int64_t epilogue_clocks(int BN) { return 32 * BN; }
 
-// Time in clocks of M x N tiles of width BN with K in `splits`, each SM taking every num_sms-th unit: whole waves
-// of the longer of main loop and epilogue, and the last epilogue.
-static int64_t cfg_clocks(int64_t M, int64_t Nreal, int nk, int BN, int splits, int nsm, int products) {
-  const int64_t units = ((M + BM - 1) / BM) * ((Nreal + BN - 1) / BN) * splits, waves = (units + nsm - 1) / nsm;
-  const int64_t main = (nk + splits - 1) / splits * block_clocks(BN) * products, epi = epilogue_clocks(BN) * (splits > 1 ? 2 : 1);
+// Time in clocks of M x N tiles of width BN with K in `splits`, each SM (or pair of SMs) taking every num_sms-th (or
+// num_sms / 2-th) unit: whole waves of the longer of main loop and epilogue, and the last epilogue.
+static int64_t cfg_clocks(int64_t M, int64_t Nreal, int nk, int BN, bool pair, int splits, int nsm, bool split) {
+  const int64_t rows = pair ? 2 * BM : BM, slots = pair ? std::max(nsm / 2, 1) : nsm;
+  const int64_t units = ((M + rows - 1) / rows) * ((Nreal + BN - 1) / BN) * splits, waves = (units + slots - 1) / slots;
+  const int64_t main = (nk + splits - 1) / splits * block_clocks(BN, pair, split), epi = epilogue_clocks(BN) * (splits > 1 ? 2 : 1);
   return waves * std::max(main, epi) + epi;
 }
 
 // the cheapest number of K splits of at least eight blocks (1 unless it gains a twentieth)
-static int best_splits(int64_t M, int64_t Nreal, int nk, int BN, bool allow, int nsm, int products) {
+static int best_splits(int64_t M, int64_t Nreal, int nk, int BN, bool pair, bool allow, int nsm, bool split) {
   int best = 1;
   if (!allow) return best;
-  int64_t t = cfg_clocks(M, Nreal, nk, BN, best, nsm, products);
-  const int64_t tiles = ((M + BM - 1) / BM) * ((Nreal + BN - 1) / BN);
-  const int most = (int)std::min<int64_t>(nk / 8, std::max<int64_t>(32, 2 * nsm / std::max<int64_t>(tiles, 1)));
+  int64_t t = cfg_clocks(M, Nreal, nk, BN, pair, best, nsm, split);
+  const int64_t rows = pair ? 2 * BM : BM, tiles = ((M + rows - 1) / rows) * ((Nreal + BN - 1) / BN);
+  const int most = (int)std::min<int64_t>(nk / 8, std::max<int64_t>(32, (pair ? nsm : 2 * nsm) / std::max<int64_t>(tiles, 1)));
   for (int s = 2; s <= most; ++s) {
-    const int64_t c = cfg_clocks(M, Nreal, nk, BN, s, nsm, products);
+    const int64_t c = cfg_clocks(M, Nreal, nk, BN, pair, s, nsm, split);
     if (c * 20 < t * 19) { t = c; best = s; }
   }
   return best;
 }
 
 // the rule's tile width and splits: the cheapest by cfg_clocks, a narrower tile where it gains a tenth (per column it
-// loads more of A: 25600 x 2560 x 800 complex 838 TFLOP/s at 256, 732 at 208, which would save half a wave)
-static void rule_cfg(int64_t M, int64_t Nreal, int nk, bool allow, int nsm, int products, int &BN, int &splits) {
+// loads more of A: 25600 x 2560 x 800 complex 838 TFLOP/s at 256, 732 at 208, which would save half a wave); then
+// pairs of CTAs for one pass if their best tile gains a twentieth (92160 x 160 x 160, bound by its output: 66 us by
+// single CTAs, 80 by pairs)
+static TcCfg rule_cfg(int64_t M, int64_t Nreal, int nk, bool allow, int nsm, bool split) {
+  TcCfg r, q;
+  int64_t t = -1, tq = -1;
   if (Nreal <= 256) {
-    BN = (int)((Nreal + 15) / 16 * 16);
-    splits = best_splits(M, Nreal, nk, BN, allow, nsm, products);
-    return;
+    r.BN = (int)((Nreal + 15) / 16 * 16);
+    r.splits = best_splits(M, Nreal, nk, r.BN, false, allow, nsm, split);
+    t = cfg_clocks(M, Nreal, nk, r.BN, false, r.splits, nsm, split);
+  } else {
+    for (int bn = 256; bn >= 128; bn -= 16) {
+      const int s = best_splits(M, Nreal, nk, bn, false, allow, nsm, split);
+      const int64_t c = cfg_clocks(M, Nreal, nk, bn, false, s, nsm, split);
+      if (t < 0 || c * 10 < t * 9) { t = c; r.BN = bn; r.splits = s; }
+    }
   }
-  int64_t t = -1;
-  for (int bn = 256; bn >= 128; bn -= 16) {
-    const int s = best_splits(M, Nreal, nk, bn, allow, nsm, products);
-    const int64_t c = cfg_clocks(M, Nreal, nk, bn, s, nsm, products);
-    if (t < 0 || c * 10 < t * 9) { t = c; BN = bn; splits = s; }
+  if (split || Nreal < 128 || M <= BM) return r;
+  q.pair = true;
+  for (int bn = 256; bn >= 128; bn -= 32) {
+    if (bn > 128 && bn - 32 >= Nreal) continue;
+    const int s = best_splits(M, Nreal, nk, bn, true, allow, nsm, split);
+    const int64_t c = cfg_clocks(M, Nreal, nk, bn, true, s, nsm, split);
+    if (tq < 0 || c * 10 < tq * 9) { tq = c; q.BN = bn; q.splits = s; }
   }
+  return tq * 20 < t * 19 ? q : r;
 }
 
 struct TuneKey {
@@ -728,22 +915,26 @@ static void tc_launch(const void *A, int64_t lda, const void *B, int64_t ldb, in
   const int nk = (int)((Kreal + BK - 1) / BK), nsm = num_sms();
   // K splits need an accumulating or plain output (split partial tiles are added atomically)
   const bool plain = rv.din == TC_ONE_LEVEL && cv.din == TC_ONE_LEVEL && cv.sin == 1;
-  const int products = split ? 3 : 1;
-  int BN = cfg.BN, splits = std::max(cfg.splits, 1);
-  if (BN <= 0) rule_cfg(M, Nreal, nk, accumulate || plain, nsm, products, BN, splits);
-  else if (cfg.splits <= 0) splits = best_splits(M, Nreal, nk, BN, accumulate || plain, nsm, products);
-  splits = std::min({splits, nk, 65535});
+  if (cfg.BN <= 0) {
+    const int band = cfg.band;
+    cfg = rule_cfg(M, Nreal, nk, accumulate || plain, nsm, split);
+    cfg.band = band;
+  } else if (cfg.splits <= 0) {
+    cfg.splits = best_splits(M, Nreal, nk, cfg.BN, cfg.pair, accumulate || plain, nsm, split);
+  }
+  const int BN = cfg.BN, rows = cfg.pair ? 2 * BM : BM;
+  int splits = std::min({cfg.splits, nk, 65535});
   TcParams p;
   p.M = (int)M;
   p.N = (int)Nreal;
   p.K = (int)Kreal;
   p.BN = BN;
-  p.nMt = (int)((M + BM - 1) / BM);
+  p.nMt = (int)((M + rows - 1) / rows);
   p.nNt = (int)((Nreal + BN - 1) / BN);
   // band of M tiles swept by N: as many A rows as take 32 MB (they stay in L2), and at least 20 tiles, which makes
   // the running tiles' block of C about square (M = N = K = 7680 complex: 4 tiles 839 TFLOP/s, 20 tiles 894)
   p.band = cfg.band > 0 ? std::min(cfg.band, p.nMt)
-                        : (int)std::min<int64_t>(p.nMt, std::max<int64_t>(20, (32ll << 20) / (BM * Kreal * es + 1)));
+                        : (int)std::min<int64_t>(p.nMt, std::max<int64_t>(20 * BM / rows, (32ll << 20) / (rows * Kreal * es + 1)));
   const int64_t tiles = (int64_t)p.nMt * p.nNt;
   p.kb_per_split = (nk + splits - 1) / splits;
   splits = (nk + p.kb_per_split - 1) / p.kb_per_split;  // every split has at least one K block
@@ -765,16 +956,16 @@ static void tc_launch(const void *A, int64_t lda, const void *B, int64_t ldb, in
     CCLR_CUDA(cudaMemset2DAsync(C, (size_t)rv.sin * 8, 0, (size_t)Nreal * 4, (size_t)M, st));
   }
   p.ntiles = (int)tiles;
-  p.list = upper ? upper->get(p.nMt, p.nNt, p.band, BM, BN / 2, 0, 0, M, st, &p.ntiles) : nullptr;
+  p.list = upper ? upper->get(p.nMt, p.nNt, p.band, rows, BN / 2, 0, 0, M, st, &p.ntiles) : nullptr;
   const int64_t units = (int64_t)p.ntiles * splits;
   CCLR_REQUIRE(units < (1ll << 31), "tc_gemm: too many work units");
   static const bool trace = std::getenv("CCLR_TRACE") && std::getenv("CCLR_TRACE")[0] == '1';
   if (trace)
-    std::fprintf(stderr, "cclr tc_gemm kind=%d M=%lld N=%lld K=%lld BN=%d tiles=%lld splits=%d band=%d atomic=%d transposed=%d\n",
-                 kind, (long long)M, (long long)Nreal, (long long)Kreal, BN, (long long)tiles, splits, p.band, p.atomic,
+    std::fprintf(stderr, "cclr tc_gemm kind=%d M=%lld N=%lld K=%lld BN=%d pair=%d tiles=%lld splits=%d band=%d atomic=%d transposed=%d\n",
+                 kind, (long long)M, (long long)Nreal, (long long)Kreal, BN, (int)cfg.pair, (long long)tiles, splits, p.band, p.atomic,
                  p.transposed);
   const unsigned grid = (unsigned)std::min<int64_t>(units, nsm);
-  const size_t epi = (size_t)8 * 32 * EPI_PITCH * 4 + (2 * STAGES + 5) * 8 + 16;
+  const size_t epi = (size_t)8 * 32 * EPI_PITCH * 4 + (2 * PAIR_STAGES + 5) * 8 + 16;
   if (split) {
     const char *Al = (const char *)A + Kreal * es, *Bl = (const char *)B + Kreal * es;
     const CUtensorMap ah = make_map(A, M, Kreal, lda, BM, 64, kind), al = make_map(Al, M, Kreal, lda, BM, 64, kind);
@@ -784,9 +975,13 @@ static void tc_launch(const void *A, int64_t lda, const void *B, int64_t ldb, in
     else tc_split_kernel<TC_TF32><<<grid, 320, smem, st>>>(ah, al, bh, bl, p);
   } else {
     const CUtensorMap ma = make_map(A, M, a_cols < 0 ? Kreal : a_cols, lda, BM, BKB, kind);
-    const CUtensorMap mb = make_map(B, Nreal, Kreal, ldb, BN, BKB, kind);
-    const size_t smem = 1024 + (size_t)STAGES * (BM + BN) * BKB + epi;
-    if (kind == TC_BF16) tc_gemm_kernel<TC_BF16><<<grid, 320, smem, st>>>(ma, mb, p);
+    const CUtensorMap mb = make_map(B, Nreal, Kreal, ldb, cfg.pair ? BN / 2 : BN, BKB, kind);
+    const size_t smem = 1024 + (cfg.pair ? (size_t)PAIR_STAGES * (BM + BN / 2) : (size_t)STAGES * (BM + BN)) * BKB + epi;
+    if (cfg.pair) {
+      const unsigned pairs = (unsigned)std::min<int64_t>(units, std::max(nsm / 2, 1));
+      if (kind == TC_BF16) tc_pair_kernel<TC_BF16><<<2 * pairs, 320, smem, st>>>(ma, mb, p);
+      else tc_pair_kernel<TC_TF32><<<2 * pairs, 320, smem, st>>>(ma, mb, p);
+    } else if (kind == TC_BF16) tc_gemm_kernel<TC_BF16><<<grid, 320, smem, st>>>(ma, mb, p);
     else tc_gemm_kernel<TC_TF32><<<grid, 320, smem, st>>>(ma, mb, p);
   }
   count_launch();
@@ -795,17 +990,18 @@ static void tc_launch(const void *A, int64_t lda, const void *B, int64_t ldb, in
     used->BN = BN;
     used->splits = splits;
     used->band = p.band;
+    used->pair = cfg.pair;
   }
 }
 
 // Candidate configurations around the rule's choice: other tile widths for wide outputs (each with its own best
 // number of splits), more or fewer K splits, and the two extreme raster bands.
 static std::vector<TcCfg> candidates(const TcCfg &rule, int64_t M, int64_t Nreal, int64_t Kreal, int kind, bool allow_split,
-                                     int products) {
+                                     bool split) {
   std::vector<TcCfg> c{rule};
   auto add = [&](TcCfg x) {
     for (const auto &y : c)
-      if (y.BN == x.BN && y.splits == x.splits && y.band == x.band) return;
+      if (y.BN == x.BN && y.splits == x.splits && y.band == x.band && y.pair == x.pair) return;
     c.push_back(x);
   };
   const int nk = (int)((Kreal + BKB / tc_esize(kind) - 1) / (BKB / tc_esize(kind)));
@@ -813,15 +1009,22 @@ static std::vector<TcCfg> candidates(const TcCfg &rule, int64_t M, int64_t Nreal
     for (int bn : {192, 256}) {
       TcCfg x = rule;
       x.BN = bn;
-      x.splits = best_splits(M, Nreal, nk, bn, allow_split, num_sms(), products);
+      x.splits = best_splits(M, Nreal, nk, bn, x.pair, allow_split, num_sms(), split);
       add(x);
     }
+  if (rule.pair) {  // the same width by single CTAs
+    TcCfg x = rule;
+    x.pair = false;
+    x.splits = best_splits(M, Nreal, nk, x.BN, false, allow_split, num_sms(), split);
+    x.band = 0;
+    add(x);
+  }
   if (allow_split) {
     TcCfg x = rule;
     x.splits = std::max(1, rule.splits / 2); add(x);
     if (nk >= 16) { x.splits = std::min(nk / 4, 2 * rule.splits); add(x); }
   }
-  const int nMt = (int)((M + BM - 1) / BM);
+  const int rows = rule.pair ? 2 * BM : BM, nMt = (int)((M + rows - 1) / rows);
   if (nMt > 1) {
     TcCfg x = rule; x.band = 1; add(x);
     x.band = nMt; add(x);
@@ -884,7 +1087,7 @@ static void tc_gemm_core(const void *A, int64_t lda, const void *B, int64_t ldb,
       float best = 1e30f;
       // K splits need an accumulating or plain output (split partial tiles are added atomically)
       const bool plain = trv.din == TC_ONE_LEVEL && tcv.din == TC_ONE_LEVEL && tcv.sin == 1;
-      for (const TcCfg &cand : candidates(rule, M, Nreal, Kreal, kind, accumulate || plain, split ? 3 : 1)) {
+      for (const TcCfg &cand : candidates(rule, M, Nreal, Kreal, kind, accumulate || plain, split)) {
         TcCfg used;
         CCLR_CUDA(cudaEventRecord(e0, st));
         tc_launch(A, lda, B, ldb, M, Nreal, Kreal, kind, split, Ct, trv, tcv, alpha, false, err, st, a_cols,
