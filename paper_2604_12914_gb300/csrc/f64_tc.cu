@@ -2,10 +2,12 @@
 //
 // This GPU's FP64 pipe does two FMAs per clock and SM, so a complex GEMM on it stops near 1 TFLOP/s.  The
 // 36 BF16 slice products (orders q <= 7) cost 36 times a BF16 GEMM and still leave some 25 times more.
-// Measured (GEMM and output kernel, operands sliced): M = N = K = 1760 complex 1.81 ms (24 TFLOP/s, 870 TFLOP/s of
-// BF16 MMAs) against 42 ms on the FP64 pipe; 12100 x 1760 x 500 3.5 ms against 90; 400^3 51 us against 617.
-// What bounds it: MMAs alone (never waiting for the epilogue) 1.09 ms at 1760^3; handing each order's accumulator to
-// the epilogue and back, 1.5 ms; with the epilogue's integer work, 1.8 ms.
+// Measured (GEMM and output kernel, operands sliced): M = N = K = 1760 complex 1.24 ms (35 TFLOP/s, 1270 TFLOP/s of
+// BF16 MMAs) against 42 ms on the FP64 pipe; 12100 x 1760 x 500 2.6 ms against 90; 400^3 44 us against 617.
+// What bounds it: MMAs alone (never waiting for the epilogue) 0.89 ms at 1760^3; handing each sum to the epilogue and
+// its accumulator back, 0.99 ms; with the epilogue's integer work, 1.24 ms.  With chunks of 32 real K (eight sums per
+// chunk, each of its own order) and 128-row tiles by single CTAs it was 1.09, 1.5 and 1.81 ms: twice as many sums to
+// hand over per MMA, and MMAs of 93 clocks instead of 64.
 #include <atomic>
 #include <cmath>
 #include <type_traits>
@@ -19,19 +21,24 @@ namespace {
 
 constexpr int S = F64_SLICES;
 constexpr int BM = 128;
-constexpr int KC = 32;                  // real K per chunk: 64-byte slice rows, and S_q <= 8 * 2^14 * 32 = 2^22 exact
+constexpr int KC = 64;                  // real K per chunk: 128-byte slice rows, and |S_q| <= 6 2^14 64 < 2^24 exact (q <= 5)
 constexpr int A_SLOT = BM * KC * 2;     // bytes of one slice block of A
-constexpr int NSLOT = 12;               // ring of (A_s, B_s) slot pairs: one chunk of 8 and half of the next
-constexpr int NBUF = 4;                 // accumulators in TMEM
-constexpr int MAX_CHUNKS = 2048;        // per launch, 65536 real K: |S_0| 2^32 stays below 2^62
+constexpr int NSLOT = S + 1;            // slots of (A_s, B_s): one chunk, and slice 0 of the next
+__host__ __device__ constexpr int b_slot(int BN, bool pair) { return (pair ? BN / 2 : BN) * KC * 2; }
+// slot of slice s in a chunk of parity par
+__host__ __device__ constexpr int slot_of(int s, int par) { return s == 0 && par ? S : s; }
+constexpr int NBUF = 4;                 // accumulators in TMEM, taken in turn
+constexpr int MAX_CHUNKS = 1024;        // per launch, 65536 real K: |S_0| 2^32 stays below 2^62
 constexpr int SPLIT_TILES = 76;         // K is split when at most this many tiles (half the SMs) exist
 
 struct F64Params {
   int sA, sB, rA, rB;   // slice rows per slice of A and B, first slice row
-  int nMt, nNt, band, splits, chunks_per_split;
-  const uint32_t *list; // the tiles to compute, (m << 16) | n, ntiles of them (nullptr: all, in raster order)
+  int nMt, nNt, splits, chunks_per_split;
+  int uMt, band;        // work units: rows of tiles (of two tiles for pairs of CTAs), and those per raster band
+  const uint32_t *list; // the units to compute, (m << 16) | n, ntiles of them (nullptr: all, in raster order)
   int ntiles;
   int chunk0, chunk1;   // chunks of KC of this K segment
+  int K;                // real K
   long long *hi;        // integer sums, [split][tile][column][row]: hi + lo 2^-8, in units of 2^(ea + eb - 46)
   float *lo;
   int *err;
@@ -62,7 +69,7 @@ __device__ __forceinline__ void unit_coords(const F64Params &p, int u, int &mt, 
     return;
   }
   const int per_band = p.band * p.nNt, b = id / per_band, local = id - b * per_band;
-  const int mb = min(p.band, p.nMt - b * p.band);
+  const int mb = min(p.band, p.uMt - b * p.band);
   mt = b * p.band + local % mb;
   nt = local / mb;
 }
@@ -97,9 +104,14 @@ __device__ __forceinline__ int scale_of(uint32_t m) {
   return ex == 0x7ff ? F64_NONFINITE : max(ex, 1) - 1022;
 }
 
-// An integer-valued float of magnitude <= 2^22 as the low bits of x + 1.5 * 2^23 (minus MAGIC)
-constexpr uint32_t MAGIC = 0x4B400000u;
-__device__ __forceinline__ uint32_t fbits(uint32_t r) { return __float_as_uint(__uint_as_float(r) + 12582912.f); }
+// H 2^8 + L for integers H = h wh and L = l wl (floats; |H| <= 3 2^20, |L| <= 2^22), from the bits of 2^23 + 0x34C000 + H
+// and -(2^23 + 2^22 + L): H and L are their low bits, and the constants cancel modulo 2^32.
+__device__ __forceinline__ int two_orders(uint32_t h, uint32_t l, float wh, float wl) {
+  const uint32_t x = __float_as_uint(fmaf(__uint_as_float(h), wh, 11845632.f));
+  const uint32_t y = __float_as_uint(fmaf(__uint_as_float(l), -wl, -12582912.f));
+  return (int)((x << 8) + y);
+}
+constexpr uint32_t MAGIC = 0x4B400000u;  // 2^23 + 2^22: an integer of up to 22 bits is its low bits when added to it
 
 // lo 2^s rounded to an integer (|result| < 2^62), from the bits of lo
 __device__ __forceinline__ long long scaled_int(float lo, int s) {
@@ -130,133 +142,235 @@ __device__ __forceinline__ double combine(long long hi, float lo, int e, int neg
   return r * two(d1) * two(d2) * two(d - d1 - d2);
 }
 
-// The slice products (two MMAs each) of orders 7 - P, 5 - P, 3 - P, 1 - P of the n-th chunk, whose slices 7 .. 0 are
-// in slots G0, G0 + 1, ...
-template <int BN, int G0, int P>
-__device__ __forceinline__ bool issue_chunk(uint8_t *smem, uint32_t tmem, uint32_t idesc, uint64_t *tfull, uint64_t *tempty,
-                                            uint64_t *empty, int *err, volatile int *abort_flag) {
-  constexpr int SLOT = A_SLOT + BN * KC * 2;
-#pragma unroll
-  for (int q = S - 1 - P; q >= 0; q -= 2) {
-    const int buf = (S - 1 - q) % NBUF;
-    // accumulator buf is used twice per chunk; it is free when its previous order has been read
-    if (!mbar_wait_ab(su32(tempty + buf), q < S - NBUF ? 0u : 1u, err, abort_flag)) return false;
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    const uint32_t d = tmem + (uint32_t)(buf * BN);
-    uint32_t base = sw64_lo(su32(smem));
-    asm volatile("" : "+r"(base));  // slot addresses are formed here, not kept in registers
-#pragma unroll
-    for (int i = 0; i <= q; ++i) {
-      const uint32_t da = base + (((G0 + S - 1 - i) % NSLOT) * SLOT >> 4);
-      const uint32_t db = base + ((((G0 + S - 1 - (q - i)) % NSLOT) * SLOT + A_SLOT) >> 4);
-      mma_sw64<TC_BF16>(d, da, db, idesc, i != 0);
-      mma_sw64<TC_BF16>(d, da + 2, db + 2, idesc, true);
-    }
-    mma_commit(su32(tfull + buf));
-    // slices q and q - 1 (and 7, which the orders of P = 1 never read) are not read by this warp's later orders
-    if (q == S - 2) mma_commit(su32(empty + G0 % NSLOT));
-    mma_commit(su32(empty + (G0 + S - 1 - q) % NSLOT));
-    if (q > 0) mma_commit(su32(empty + (G0 + S - q) % NSLOT));
+// product of slices i of A and j of B of a chunk of parity par, MMAs of 16 real K each (two if half, else four), into
+// the accumulator at d (added to it if acc)
+template <int BN, bool PAIR>
+__device__ __forceinline__ void issue_product(uint32_t base, int par, bool half, int i, int j, uint32_t d, uint32_t idesc,
+                                              bool acc) {
+  constexpr uint32_t SLOT = (A_SLOT + b_slot(BN, PAIR)) >> 4;
+  const uint32_t da = base + slot_of(i, par) * SLOT, db = base + slot_of(j, par) * SLOT + (A_SLOT >> 4);
+  mma_sw128<PAIR>(d, da, db, idesc, acc);
+  mma_sw128<PAIR>(d, da + 2, db + 2, idesc, true);
+  if (half) return;
+  mma_sw128<PAIR>(d, da + 4, db + 4, idesc, true);
+  mma_sw128<PAIR>(d, da + 6, db + 6, idesc, true);
+}
+// `count` products of order q, slices of A from the digits of `list`, lowest first (a loop: unrolled, its addresses
+// spill from the forty registers)
+template <int BN, bool PAIR>
+__device__ __forceinline__ void issue_list(uint32_t base, int par, bool half, int q, uint32_t list, int count, uint32_t d,
+                                           uint32_t idesc, bool acc) {
+#pragma unroll 1
+  for (int k = 0; k < count; ++k, list >>= 4)
+    issue_product<BN, PAIR>(base, par, half, (int)(list & 7), q - (int)(list & 7), d, idesc, acc || k > 0);
+}
+template <bool PAIR> __device__ __forceinline__ void commit(uint32_t bar) {
+  if constexpr (PAIR) mma_commit_pair(bar);
+  else mma_commit(bar);
+}
+
+// The accumulators are taken in turn: the next one and the parity of its use.
+struct Turn {
+  int buf = 0;
+  uint32_t parity = 0;
+  __device__ __forceinline__ Turn next() const {
+    Turn t;
+    t.buf = (buf + 1) % NBUF;
+    t.parity = t.buf == 0 ? parity ^ 1u : parity;
+    return t;
   }
+};
+
+struct Bars {
+  uint32_t base;  // of the barriers: full, empty, tfull, tempty
+  int *err;
+  volatile int *abort_flag;
+  __device__ __forceinline__ uint32_t at(int i) const {
+    uint32_t a = base;
+    asm volatile("" : "+r"(a));  // formed here, not kept in a register of its own
+    return a + 8 * (uint32_t)i;
+  }
+};
+
+// full barriers: slice 0 of even and odd chunks, slice 1, slices 6 and 7, 2 and 5, 3 and 4; empty barriers: slices 7,
+// 6, 1, (3 and 5), 2, 4 (and 0, which is free when the next chunk's 4 is)
+enum { F_0 = 0, F_1 = 2, F_67, F_25, F_34, NFULL };
+enum { E_7 = 0, E_6, E_1, E_35, E_2, E_4, NEMPTY };
+enum { B_EMPTY = NFULL, B_TFULL = B_EMPTY + NEMPTY, B_TEMPTY = B_TFULL + NBUF };
+constexpr int GROUPS = 5;  // full barriers per chunk, in the order they are expected: 0, 67, 1, 25, 34
+
+// All MMAs of the n-th chunk: order 0, order 1, orders 7 and 6 (one sum), then 2, 3, 5 and 4.  The sum of an order is
+// handed over, and its accumulator handed back, about a microsecond after its MMAs have run; in this sequence each finds
+// its accumulator, that of the fourth sum before it, free.  A slice block arrives as long after its slot was freed: the
+// last orders read first what the next chunk begins with (slice 0 has two slots, slice 1 is read by their first four
+// products, and order 7 begins with the slices that come first).
+template <int BN, bool PAIR>
+__device__ __forceinline__ bool issue_chunk(uint32_t base, uint32_t tmem, uint32_t idesc, const Bars &b, Turn &t, uint32_t n,
+                                            bool half, int *consumed) {
+  const int par = (int)(n & 1u);
+  auto wait = [&](int bar, uint32_t parity) {
+    const bool ok = mbar_wait_ab(b.at(bar), parity, b.err, b.abort_flag);
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    return ok;
+  };
+  auto list = [&](int q, uint32_t l, int count, int buf, bool acc) {
+    issue_list<BN, PAIR>(base, par, half, q, l, count, tmem + (uint32_t)(buf * BN), idesc, acc);
+  };
+#pragma unroll 1
+  for (int q = 0; q < 4; ++q) {
+    if (q == 0 && !wait(F_0 + par, (n >> 1) & 1u)) return false;
+    if (q == 1 && !wait(F_1, n & 1u)) return false;
+    if (!wait(B_TEMPTY + t.buf, t.parity ^ 1u)) return false;
+    list(q, 0x3210u, q + 1, t.buf, false);
+    commit<PAIR>(b.at(B_TFULL + t.buf));
+    t = t.next();
+    if (q == 1) {
+      if (!wait(F_67, n & 1u)) return false;
+      consumed[0] = GROUPS * (int)n + 3;
+      if (!wait(B_TEMPTY + t.buf, t.parity ^ 1u)) return false;
+      list(7, 0x6170u, 4, t.buf, false);
+      if (!wait(F_25, n & 1u)) return false;
+      list(7, 0x52u, 2, t.buf, true);
+      if (!wait(F_34, n & 1u)) return false;
+      consumed[0] = GROUPS * (int)n + GROUPS;
+      list(7, 0x43u, 2, t.buf, true);
+      commit<PAIR>(b.at(B_EMPTY + E_7));
+      list(6, 0x6543210u, 7, t.buf, true);
+      commit<PAIR>(b.at(B_EMPTY + E_6));
+      commit<PAIR>(b.at(B_TFULL + t.buf));
+      t = t.next();
+    }
+  }
+  const Turn t4 = t.next();
+  if (!wait(B_TEMPTY + t.buf, t.parity ^ 1u)) return false;
+  list(5, 0x41u, 2, t.buf, false);
+  if (!wait(B_TEMPTY + t4.buf, t4.parity ^ 1u)) return false;
+  list(4, 0x31u, 2, t4.buf, false);
+  commit<PAIR>(b.at(B_EMPTY + E_1));
+  list(5, 0x3250u, 4, t.buf, true);
+  commit<PAIR>(b.at(B_TFULL + t.buf));
+  commit<PAIR>(b.at(B_EMPTY + E_35));
+  list(4, 0x2u, 1, t4.buf, true);
+  commit<PAIR>(b.at(B_EMPTY + E_2));
+  list(4, 0x40u, 2, t4.buf, true);
+  commit<PAIR>(b.at(B_TFULL + t4.buf));
+  commit<PAIR>(b.at(B_EMPTY + E_4));
+  t = t4.next();
   return true;
 }
 
-// Warp 0 streams slice blocks with TMA into a ring of (A_s, B_s) slots, s = 7 first: the orders of a chunk are
-// issued as q = 7 .. 0, order q is the last to read slice q, so slots free up in the order they were filled.
-// Warp 1 issues the MMAs of order q into TMEM accumulator (7 - q) % 4.  Warps 4-11 add the exact sums of each
-// order to a 64-bit integer (q <= 4, two orders at a time as one 32-bit integer) or a float (q = 5, 6, 7, below
-// 2^-40 of the total) per output, and store both once per unit.  192 accumulator registers per thread:
-// setmaxnreg gives the two epilogue warpgroups 232 and the first one 40 (of 168 at launch).
-template <int BN>
+// Warp 0 streams slice blocks with TMA, each as its slot is freed.  Warp 1 issues the MMAs.  Warps 4-11 add the sums of
+// the orders 0 .. 4 to a 64-bit integer (two orders at a time as one 32-bit integer) and those of 5 and of 6 and 7 to a
+// float per output, and store both once per unit.  The orders 6 and 7 share an accumulator: slice s is stored times
+// 2^(-8 s), so they add up with their weights, and below 2^-48 of the total its 24 bits are plenty.  192 accumulator
+// registers per thread: setmaxnreg gives the two epilogue warpgroups 232 and the first one 40 (of 168 at launch).
+// PAIR: two CTAs share a unit of 256 rows; each loads its rows of A and half the rows of B, the first one issues the
+// MMAs of both.  An MMA of 128 x 128 reads 8 KB of shared memory and takes 93 clocks instead of 64 for that; as half
+// of a pair's it reads 6.
+template <int BN, bool PAIR>
 __global__ void __launch_bounds__(384, 1)
     f64_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, F64Params p) {
-  constexpr int B_SLOT = BN * KC * 2, SLOT = A_SLOT + B_SLOT, NC = BN / 2;
+  constexpr int SLOT = A_SLOT + b_slot(BN, PAIR), NC = BN / 2;
   constexpr uint32_t TCOLS = NBUF * BN;
   extern __shared__ uint8_t smem_raw[];
   uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+  // (pairs: full and tempty are waited for in CTA 0 only; empty and tfull arrive in both)
   uint64_t *bars = (uint64_t *)(smem + NSLOT * SLOT);
-  uint64_t *full = bars, *empty = full + NSLOT, *tfull = empty + NSLOT, *tempty = tfull + NBUF, *drain = tempty + NBUF;
-  uint32_t *tslot = (uint32_t *)(drain + 2);
+  uint64_t *full = bars, *empty = full + NFULL, *tfull = empty + NEMPTY, *tempty = tfull + NBUF, *drain = tempty + NBUF;
+  uint32_t *tslot = (uint32_t *)(drain + 1);
   int *issued = (int *)(tslot + 1), *consumed = issued + 1;
   volatile int *abort_flag = issued + 2;
   const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
   const int units = p.ntiles * p.splits;
+  const int rank = PAIR ? (int)cta_rank() : 0, first = PAIR ? blockIdx.x >> 1 : blockIdx.x,
+            step = PAIR ? gridDim.x >> 1 : gridDim.x;
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < NSLOT; ++s) {
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(su32(full + s)) : "memory");
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], 2;" ::"r"(su32(empty + s)) : "memory");
-    }
+    for (int s = 0; s < NFULL; ++s) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(su32(full + s)) : "memory");
+    for (int s = 0; s < NEMPTY; ++s) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(su32(empty + s)) : "memory");
     for (int b = 0; b < NBUF; ++b) {
       asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(su32(tfull + b)) : "memory");
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], 8;" ::"r"(su32(tempty + b)) : "memory");
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(su32(tempty + b)), "r"(PAIR ? 16 : 8) : "memory");
     }
-    for (int b = 0; b < 2; ++b) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(su32(drain + b)) : "memory");
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(su32(drain)) : "memory");
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     issued[0] = 0;
     consumed[0] = 0;
     *abort_flag = 0;
   }
+  __syncthreads();
   if (warp == 1) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(su32(tslot)), "r"(TCOLS)
-                 : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    if constexpr (PAIR) {
+      asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(su32(tslot)), "r"(TCOLS)
+                   : "memory");
+      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+    } else {
+      asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(su32(tslot)), "r"(TCOLS)
+                   : "memory");
+      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
+  if constexpr (PAIR) pair_sync();  // both CTAs' barriers are initialised
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = __shfl_sync(0xffffffffu, *tslot, 0);
 
   if (warp < 4) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 40;");
     if (warp == 0 && lane == 0) {
-      int g = 0;
+      uint32_t n = 0;  // chunks so far
       bool ok = true;
-      for (int u = blockIdx.x; u < units && ok; u += gridDim.x) {
+      for (int u = first; u < units && ok; u += step) {
         int mt, nt, sp;
         unit_coords(p, u, mt, nt, sp);
+        if (PAIR) mt = 2 * mt + rank;
         const int c0 = p.chunk0 + sp * p.chunks_per_split, c1 = min(p.chunk1, c0 + p.chunks_per_split);
-        for (int c = c0; c < c1 && ok; ++c)
-          for (int s = S - 1; s >= 0; --s, ++g) {
-            const int slot = g % NSLOT;
-            if (!mbar_wait_ab(su32(empty + slot), ((uint32_t)(g / NSLOT) & 1u) ^ 1u, p.err, abort_flag)) { ok = false; break; }
-            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(su32(full + slot)),
-                         "r"((uint32_t)SLOT)
-                         : "memory");
-            tma_load_2d(smem + slot * SLOT, &tmA, c * KC, s * p.sA + p.rA + mt * BM, su32(full + slot));
-            tma_load_2d(smem + slot * SLOT + A_SLOT, &tmB, c * KC, s * p.sB + p.rB + nt * BN, su32(full + slot));
-            issued[0] = g + 1;
+        const int yA = p.rA + mt * BM, yB = p.rB + nt * BN + (PAIR ? rank * (BN / 2) : 0);
+        for (int c = c0; c < c1 && ok; ++c, ++n) {
+          const int par = (int)(n & 1u);
+          // slices 0, 7, 6, 1, 5, 3, 2, 4, as they are freed (slice 0's slot was last read two chunks ago, before
+          // slice 4 of the last one could be loaded); a loop, as forty registers do not hold eight slices' addresses
+#pragma unroll 1
+          for (int j = 0; j < S; ++j) {
+            const int s = (0x42351670u >> (4 * j)) & 7, f = s == 0 ? F_0 + par : (0x33455420u >> (4 * s)) & 7;
+            if (j > 0 && !(ok = mbar_wait_ab(su32(empty + (j <= 4 ? j - 1 : j - 2)), (n & 1u) ^ 1u, p.err, abort_flag))) break;
+            if (j < 6 && j != 2) {  // the first slice of its group: one slice (0 and 1) or two
+              if (!PAIR || rank == 0)
+                asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(su32(full + f)),
+                             "r"((uint32_t)(SLOT * (PAIR ? 2 : 1) * (s < 2 ? 1 : 2)))
+                             : "memory");
+              issued[0] = issued[0] + 1;
+            }
+            uint8_t *dst = smem + slot_of(s, par) * SLOT;
+            if constexpr (PAIR) {
+              const uint32_t fb = pair_addr(su32(full + f), 0);
+              tma_load_2d_pair(dst, &tmA, c * KC, s * p.sA + yA, fb);
+              tma_load_2d_pair(dst + A_SLOT, &tmB, c * KC, s * p.sB + yB, fb);
+            } else {
+              tma_load_2d(dst, &tmA, c * KC, s * p.sA + yA, su32(full + f));
+              tma_load_2d(dst + A_SLOT, &tmB, c * KC, s * p.sB + yB, su32(full + f));
+            }
           }
-      }
-    } else if ((warp == 1 || warp == 2) && lane == 0) {
-      const uint32_t idesc = idesc_mma(TC_BF16, BM, BN);
-      int g = 0;  // first slot of the chunk
-      bool ok = true;
-      for (int u = blockIdx.x; u < units && ok; u += gridDim.x) {
-        int mt, nt, sp;
-        unit_coords(p, u, mt, nt, sp);
-        const int c0 = p.chunk0 + sp * p.chunks_per_split, c1 = min(p.chunk1, c0 + p.chunks_per_split);
-        for (int c = c0; c < c1 && ok; ++c, g += S) {
-          for (int k = 0; k < S && ok; ++k) {
-            const int slot = (g + k) % NSLOT;
-            ok = mbar_wait_ab(su32(full + slot), (uint32_t)((g + k) / NSLOT) & 1u, p.err, abort_flag);
-            if (ok && warp == 1) consumed[0] = g + k + 1;
-          }
-          if (!ok) break;
-          // the chunk's first slot is 0, 4 or 8: slot offsets are constants in each case, so that the issuing
-          // thread spends a few instructions per MMA
-          const int g0 = g % NSLOT;
-          auto chunk = [&](auto G) {
-            constexpr int G0 = decltype(G)::value;
-            return warp == 1 ? issue_chunk<BN, G0, 0>(smem, tmem, idesc, tfull, tempty, empty, p.err, abort_flag)
-                             : issue_chunk<BN, G0, 1>(smem, tmem, idesc, tfull, tempty, empty, p.err, abort_flag);
-          };
-          ok = g0 == 0 ? chunk(std::integral_constant<int, 0>()) : g0 == 4 ? chunk(std::integral_constant<int, 4>())
-                                                                           : chunk(std::integral_constant<int, 8>());
         }
       }
-      mma_commit(su32(drain + warp - 1));
-      mbar_wait(su32(drain + warp - 1), 0, p.err);
+    } else if (warp == 1 && rank == 0 && elect_one()) {
+      const uint32_t idesc = idesc_mma(TC_BF16, PAIR ? 2 * BM : BM, BN), base = sw64_lo(su32(smem));
+      const Bars b{su32(bars), p.err, abort_flag};
+      Turn t;
+      uint32_t n = 0;  // chunks so far
+      bool ok = true;
+      for (int u = first; u < units && ok; u += step) {
+        int mt, nt, sp;
+        unit_coords(p, u, mt, nt, sp);
+        const int c0 = p.chunk0 + sp * p.chunks_per_split, c1 = min(p.chunk1, c0 + p.chunks_per_split);
+        for (int c = c0; c < c1 && ok; ++c, ++n) {
+          // half: the rest of the chunk is zeros
+          ok = issue_chunk<BN, PAIR>(base, tmem, idesc, b, t, n, p.K - c * KC <= KC / 2, consumed);
+        }
+      }
+      commit<PAIR>(su32(drain));
+      mbar_wait(su32(drain), 0, p.err);
     }
     __syncwarp();
   } else {
@@ -264,83 +378,88 @@ __global__ void __launch_bounds__(384, 1)
     const int quarter = warp & 3, h = (warp - 4) >> 2;
     const uint32_t tb = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(h * NC);
     bool ok = true;
-    for (int u = blockIdx.x; u < units && ok; u += gridDim.x) {
+    uint32_t n = 0;  // chunks so far
+    Turn t;
+    for (int u = first; u < units && ok; u += step) {
       int mt, nt, sp;
       unit_coords(p, u, mt, nt, sp);
+      if (PAIR) mt = 2 * mt + rank;
       const int c0 = p.chunk0 + sp * p.chunks_per_split, c1 = min(p.chunk1, c0 + p.chunks_per_split);
       long long hi[NC];
       float lo[NC];
 #pragma unroll
       for (int c = 0; c < NC; ++c) { hi[c] = 0; lo[c] = 0.f; }
-      auto wait = [&](int buf, uint32_t use) {
-        const bool w = mbar_wait_ab(su32(tfull + buf), use, p.err, abort_flag);
+      auto wait = [&](int buf, uint32_t parity) {
+        const bool w = mbar_wait_ab(su32(tfull + buf), parity, p.err, abort_flag);
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         return __all_sync(0xffffffffu, w) != 0;
       };
       auto release = [&](int buf) {
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         __syncwarp();
-        if (lane == 0) mbar_arrive(su32(tempty + buf));
+        if (lane == 0) {
+          if constexpr (PAIR) mbar_arrive_cluster(pair_addr(su32(tempty + buf), 0));
+          else mbar_arrive(su32(tempty + buf));
+        }
       };
-      for (int ch = c0; ch < c1; ++ch) {
-        constexpr int W1 = NC < 32 ? NC : 32, W2 = 16;  // columns per TMEM load
-        // q = 7, 6, 5 (accumulators 0, 1, 2): a float below the integer
-        auto low = [&](int buf, float w) {
+      for (int ch = c0; ch < c1; ++ch, ++n) {
+        constexpr int W1 = NC < 32 ? NC : 32, W2 = 8;  // columns per TMEM load (16 in pairs of accumulators spill)
+        // two orders as one 32-bit integer, S_q 2^8 + S_(q+1), from the next two accumulators
+        auto pair = [&](float wh, float wl, int shift) {
+          const Turn x = t, y = t.next();
+          t = y.next();
+          if (!wait(x.buf, x.parity) || !wait(y.buf, y.parity)) return false;
+#pragma unroll
+          for (int c = 0; c < NC; c += W2) {
+            uint32_t a[W2], b[W2];
+            tmem_ld<W2>(tb + x.buf * BN + c, a);
+            tmem_ld<W2>(tb + y.buf * BN + c, b);
+            tmem_wait();
+            hold(a);
+            hold(b);
+#pragma unroll
+            for (int k = 0; k < W2; ++k) hi[c + k] += (long long)two_orders(a[k], b[k], wh, wl) * (1ll << shift);
+          }
+          release(x.buf);
+          release(y.buf);
+          return true;
+        };
+        auto low = [&]() {
+          const Turn z = t;
+          t = t.next();
+          if (!wait(z.buf, z.parity)) return false;
 #pragma unroll
           for (int c = 0; c < NC; c += W1) {
             uint32_t x[W1];
-            tmem_ld<W1>(tb + buf * BN + c, x);
+            tmem_ld<W1>(tb + z.buf * BN + c, x);
             tmem_wait();
             hold(x);
 #pragma unroll
-            for (int k = 0; k < W1; ++k) lo[c + k] = fmaf(__uint_as_float(x[k]), w, lo[c + k]);
+            for (int k = 0; k < W1; ++k) lo[c + k] = fmaf(__uint_as_float(x[k]), 0x1p40f, lo[c + k]);
           }
+          release(z.buf);
+          return true;
         };
-        // two orders at a time as one 32-bit integer: S_(q-1) 2^8 + S_q
-        auto pair = [&](int bx, int by, int shift) {
+        if (!(ok = pair(1.f, 0x1p8f, 24))) break;      // q = 0, 1
+        if (!(ok = low())) break;                      // q = 7, 6
+        if (!(ok = pair(0x1p16f, 0x1p24f, 8))) break;  // q = 2, 3
+        if (!(ok = low())) break;                      // q = 5
+        const Turn z = t;  // q = 4 (too large for the bits of a float near 2^23)
+        t = t.next();
+        if (!(ok = wait(z.buf, z.parity))) break;
 #pragma unroll
-          for (int c = 0; c < NC; c += W2) {
-            uint32_t x[W2], y[W2];
-            tmem_ld<W2>(tb + bx * BN + c, x);
-            tmem_ld<W2>(tb + by * BN + c, y);
-            tmem_wait();
-            hold(x);
-            hold(y);
-#pragma unroll
-            for (int k = 0; k < W2; ++k)
-              hi[c + k] += (long long)(int)((fbits(y[k]) << 8) + fbits(x[k]) - (MAGIC * 257u)) * (1ll << shift);
-          }
-        };
-        if (!(ok = wait(0, 0))) break;
-        low(0, 0x1p-16f);
-        release(0);
-        if (!(ok = wait(1, 0))) break;
-        low(1, 0x1p-8f);
-        release(1);
-        if (!(ok = wait(2, 0))) break;
-        low(2, 1.f);
-        release(2);
-        if (!(ok = wait(3, 0) && wait(0, 1))) break;
-        pair(3, 0, 0);  // q = 4, 3
-        release(3);
-        release(0);
-        if (!(ok = wait(1, 1) && wait(2, 1))) break;
-        pair(1, 2, 16);  // q = 2, 1
-        release(1);
-        release(2);
-        if (!(ok = wait(3, 1))) break;
-#pragma unroll
-        for (int c = 0; c < NC; c += W1) {  // q = 0
-          uint32_t x[W1];
-          tmem_ld<W1>(tb + 3 * BN + c, x);
+        for (int c = 0; c < NC; c += W2) {
+          uint32_t x[W2];
+          tmem_ld<W2>(tb + z.buf * BN + c, x);
           tmem_wait();
           hold(x);
 #pragma unroll
-          for (int k = 0; k < W1; ++k) hi[c + k] += (long long)((unsigned long long)(fbits(x[k]) - MAGIC) << 32);
+          for (int k = 0; k < W2; ++k) hi[c + k] += (long long)__float2int_rn(__uint_as_float(x[k]) * 0x1p32f);
         }
-        release(3);
+        release(z.buf);
       }
       if (!ok) break;
+      if (PAIR && mt >= p.nMt) continue;
       const int64_t at = (((int64_t)sp * p.nMt * p.nNt + (int64_t)nt * p.nMt + mt) * BN + h * NC) * BM + quarter * 32 + lane;
 #pragma unroll
       for (int c = 0; c < NC; ++c) {
@@ -351,11 +470,26 @@ __global__ void __launch_bounds__(384, 1)
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
-  if (threadIdx.x == 0 && consumed[0] < issued[0])  // error path: drain copies issued but never consumed (bounded)
-    for (int g = consumed[0]; g < issued[0]; ++g) mbar_wait(su32(full + g % NSLOT), (uint32_t)(g / NSLOT) & 1u, p.err);
+  // error path: drain copies issued but never consumed (bounded)
+  if (threadIdx.x == 0 && (PAIR ? *abort_flag != 0 : consumed[0] < issued[0])) {
+    if (rank == 0)
+      for (int g = consumed[0]; g < issued[0]; ++g) {
+        const int n = g / GROUPS, k = g % GROUPS, f = k == 0 ? F_0 + (n & 1) : k == 1 ? F_67 : k == 2 ? F_1 : k == 3 ? F_25 : F_34;
+        mbar_wait(su32(full + f), (uint32_t)(k == 0 ? n >> 1 : n) & 1u, p.err);
+      }
+    if (PAIR) {  // copies of CTA 1 that CTA 0 never expected have no barrier to wait for: 10 ms, which no copy takes
+      const unsigned long long t0 = gtime();
+      while (gtime() - t0 < 10000000ull) {}
+    }
+  }
   __syncthreads();
-  if (warp == 1)
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TCOLS) : "memory");
+  if constexpr (PAIR) pair_sync();  // neither CTA leaves while the other's MMAs, copies or arrivals may touch it
+  if (warp == 1) {
+    if constexpr (PAIR)
+      asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TCOLS) : "memory");
+    else
+      asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TCOLS) : "memory");
+  }
 }
 
 // The integer sums to FP64: a block takes 32 rows by 16 complex columns of a tile, reads the sums of every K
@@ -490,11 +624,15 @@ __device__ __forceinline__ long long fixed63(double x, int e) {
   return (int)h < 0 ? -(long long)f : (long long)f;
 }
 
-// the next balanced digit (-128 .. 127) from below, as BF16 bits
-__device__ __forceinline__ uint32_t digit(long long &X) {
+// digit d (-128 .. 128) times 2^(-8 s) as BF16 bits
+__device__ __forceinline__ uint32_t digit_bits(int d, int s) {
+  return __float_as_uint((__uint_as_float(MAGIC + (uint32_t)d) - 12582912.f) * __uint_as_float((uint32_t)(127 - 8 * s) << 23)) >> 16;
+}
+// slice s > 0 from below: the next balanced digit (-128 .. 127)
+__device__ __forceinline__ uint32_t digit(long long &X, int s) {
   const int d = (int)(signed char)(X & 0xff);
   X = (X - d) >> 8;
-  return __float_as_uint(__uint_as_float(MAGIC + (uint32_t)d) - 12582912.f) >> 16;
+  return digit_bits(d, s);
 }
 
 // eight slices of one complex entry at real columns 2k, 2k+1 of slice row r (R rows per slice)
@@ -506,11 +644,11 @@ __device__ __forceinline__ void put_slices(uint32_t *dst, int64_t R, int64_t ld2
   for (int s = S - 1; s >= 0; --s) {
     uint32_t a, b;
     if (s > 0) {
-      a = digit(X);
-      b = digit(Y);
+      a = digit(X, s);
+      b = digit(Y, s);
     } else {  // the top digit, up to +-128
-      a = __float_as_uint(__uint_as_float(MAGIC + (uint32_t)(int)X) - 12582912.f) >> 16;
-      b = __float_as_uint(__uint_as_float(MAGIC + (uint32_t)(int)Y) - 12582912.f) >> 16;
+      a = digit_bits((int)X, 0);
+      b = digit_bits((int)Y, 0);
     }
     if (EMBED) {
       uint32_t *row = dst + ((int64_t)s * 2 * R + 2 * r) * ld2 + k;
@@ -629,35 +767,49 @@ void prep_launch(const double2 *src, View2 rv, View2 kv, int64_t R, int64_t K, u
   count_launch(2);
 }
 
-template <int BN> size_t smem_bytes() {
-  return 1024 + (size_t)NSLOT * (A_SLOT + BN * KC * 2) + (2 * NSLOT + 2 * NBUF + 2) * 8 + 16;
+template <int BN, bool PAIR> constexpr size_t smem_bytes() {
+  return 1024 + (size_t)NSLOT * (A_SLOT + b_slot(BN, PAIR)) + (NFULL + NEMPTY + 2 * NBUF + 1) * 8 + 16;
 }
 
-// one launch of the GEMM over the tiles of p (rows rowsA of A from p.rA, columns of B from p.rB), and its output
-template <int BN>
+// one launch of the GEMM over the units of p (rows of A from p.rA, columns of B from p.rB), and its output
+template <int BN, bool PAIR>
 void launch(const F64Op &A, const F64Op &B, const F64Params &p, F64Out &o, int64_t K, cudaStream_t st) {
   static std::atomic<unsigned long long> attr_set{0};  // one bit per device
+  constexpr int smem = (int)smem_bytes<BN, PAIR>();
   int dev = 0;
   CCLR_CUDA(cudaGetDevice(&dev));
   if (dev >= 64 || !(attr_set.load() & (1ull << dev))) {
-    CCLR_CUDA(cudaFuncSetAttribute(f64_gemm_kernel<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes<BN>()));
+    CCLR_CUDA(cudaFuncSetAttribute(f64_gemm_kernel<BN, PAIR>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
     if (dev < 64) attr_set |= 1ull << dev;
   }
   const int64_t ld = f64tc_ld(K);
-  const CUtensorMap ma = tc_make_map(A.p, (int64_t)S * p.sA, 2 * K, ld, BM, 64, TC_BF16);
-  const CUtensorMap mb = tc_make_map(B.p, (int64_t)S * p.sB, 2 * K, ld, BN, 64, TC_BF16);
+  const CUtensorMap ma = tc_make_map(A.p, (int64_t)S * p.sA, 2 * K, ld, BM, 128, TC_BF16);
+  const CUtensorMap mb = tc_make_map(B.p, (int64_t)S * p.sB, 2 * K, ld, PAIR ? BN / 2 : BN, 128, TC_BF16);
   const int64_t units = (int64_t)p.ntiles * p.splits;
-  f64_gemm_kernel<BN><<<(unsigned)std::min<int64_t>(units, tc_num_sms()), 384, smem_bytes<BN>(), st>>>(ma, mb, p);
+  if constexpr (PAIR) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(2 * (unsigned)std::min<int64_t>(units, std::max(tc_num_sms() / 2, 1)));
+    cfg.blockDim = dim3(384);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = 2;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    CCLR_CUDA(cudaLaunchKernelEx(&cfg, f64_gemm_kernel<BN, PAIR>, ma, mb, p));
+  } else {
+    f64_gemm_kernel<BN, PAIR><<<(unsigned)std::min<int64_t>(units, tc_num_sms()), 384, smem, st>>>(ma, mb, p);
+  }
   CCLR_CUDA(cudaGetLastError());
   o.hi = p.hi;
   o.lo = p.lo;
   o.nMt = p.nMt;
   o.nNt = p.nNt;
   o.splits = p.splits;
-  o.list = p.list;
-  o.ntiles = p.ntiles;
-  if (p.splits > 8) f64_out_split_kernel<BN><<<(unsigned)(p.ntiles * 4 * (BN / 2)), dim3(32, 8), 0, st>>>(o);
-  else f64_out_kernel<BN><<<(unsigned)(p.ntiles * 4 * (BN / 32)), dim3(32, 8), 0, st>>>(o);
+  if (p.splits > 8) f64_out_split_kernel<BN><<<(unsigned)(o.ntiles * 4 * (BN / 2)), dim3(32, 8), 0, st>>>(o);
+  else f64_out_kernel<BN><<<(unsigned)(o.ntiles * 4 * (BN / 32)), dim3(32, 8), 0, st>>>(o);
   CCLR_CUDA(cudaGetLastError());
   count_launch(2);
 }
@@ -677,6 +829,10 @@ F64Plan plan_of(int64_t M, int64_t N, size_t cap) {
   q.rows = (int)std::min<int64_t>(q.nMt, fit);
   q.cols = (int)std::max<int64_t>(1, std::min<int64_t>(q.nNt, fit / q.rows));
   return q;
+}
+// K splits of one launch: only when the tiles of the whole product leave half the SMs idle, two chunks at least each
+int64_t splits_of(int64_t all_tiles, int64_t units, int slots, int n) {
+  return all_tiles > SPLIT_TILES ? 1 : std::max<int64_t>(1, std::min<int64_t>(slots / units, n / 2));
 }
 constexpr size_t SUMS_CAP = 256u << 20;  // the most that the sums of one launch take
 
@@ -727,35 +883,48 @@ void f64tc_gemm(const F64Op &A, int64_t M, const F64Op &B, int64_t N, int64_t K,
   o.sh = o.pow2 ? ex - 1 : 0;
   o.neg = o.pow2 && alpha.re < 0.0;
   const int nk = (int)((2 * K + KC - 1) / KC);
+  p.K = (int)(2 * K);
   for (int t0 = 0; t0 < pl.nNt; t0 += pl.cols)
     for (int r0 = 0; r0 < pl.nMt; r0 += pl.rows) {
       p.nMt = std::min(pl.rows, pl.nMt - r0);
       p.nNt = std::min(pl.cols, pl.nNt - t0);
-      p.band = std::min(p.nMt, 12);
       o.m0 = r0 * BM;
       o.n0 = t0 * (pl.BN / 2);
       p.rA = (int)A.r0 + r0 * BM;
       p.rB = (int)(2 * B.r0) + t0 * pl.BN;
-      const int64_t tiles = (int64_t)p.nMt * p.nNt;
-      p.ntiles = (int)tiles;
-      // (a product with few tiles splits K instead)
-      p.list = upper && (int64_t)pl.nMt * pl.nNt > SPLIT_TILES
-                   ? upper->get(p.nMt, p.nNt, p.band, BM, pl.BN / 2, o.m0, o.n0, M, st, &p.ntiles) : nullptr;
-      // segments of K that the integer sums can hold, one launch each; within one, K is split when the tiles of
-      // the whole product leave half the SMs idle, four chunks at least per split
+      const int64_t tiles = (int64_t)p.nMt * p.nNt, all = (int64_t)pl.nMt * pl.nNt;
+      // tiles of 128 columns by pairs of CTAs, also where the second one has no rows (M <= 128): a single CTA's MMAs
+      // take 93 clocks for 64 columns
+      const bool pair = pl.BN == 128;
+      const int slots = pair ? std::max(tc_num_sms() / 2, 1) : tc_num_sms();
+      p.uMt = pair ? (p.nMt + 1) / 2 : p.nMt;
+      p.band = std::min(p.uMt, pair ? 6 : 12);
+      p.ntiles = p.uMt * p.nNt;
+      o.ntiles = (int)tiles;
+      p.list = o.list = nullptr;
+      if (upper && all > SPLIT_TILES) {  // (a product with few tiles splits K instead)
+        o.list = upper->get(p.nMt, p.nNt, 12, BM, pl.BN / 2, o.m0, o.n0, M, st, &o.ntiles);
+        p.list = pair ? upper->get(p.uMt, p.nNt, p.band, 2 * BM, pl.BN / 2, o.m0, o.n0, M, st, &p.ntiles) : o.list;
+        if (!pair && o.list) p.ntiles = o.ntiles;
+        if (!p.list || !o.list) {
+          p.list = o.list = nullptr;
+          p.ntiles = p.uMt * p.nNt;
+          o.ntiles = (int)tiles;
+        }
+      }
+      // segments of K that the integer sums can hold, one launch each
       for (p.chunk0 = 0; p.chunk0 < nk; p.chunk0 += MAX_CHUNKS) {
         p.chunk1 = std::min(nk, p.chunk0 + MAX_CHUNKS);
         const int n = p.chunk1 - p.chunk0;
-        const int64_t splits = (int64_t)pl.nMt * pl.nNt > SPLIT_TILES
-                                   ? 1 : std::max<int64_t>(1, std::min<int64_t>(tc_num_sms() / tiles, n / 4));
+        const int64_t splits = splits_of(all, (int64_t)p.uMt * p.nNt, slots, n);
         p.chunks_per_split = (int)((n + splits - 1) / splits);
         p.splits = (n + p.chunks_per_split - 1) / p.chunks_per_split;
         p.hi = (long long *)scratch;
         p.lo = (float *)(p.hi + tiles * p.splits * BM * pl.BN);
         o.accumulate = accumulate || p.chunk0 > 0;
-        if (pl.BN == 32) launch<32>(A, B, p, o, K, st);
-        else if (pl.BN == 64) launch<64>(A, B, p, o, K, st);
-        else launch<128>(A, B, p, o, K, st);
+        if (pl.BN == 32) launch<32, false>(A, B, p, o, K, st);
+        else if (pl.BN == 64) launch<64, false>(A, B, p, o, K, st);
+        else launch<128, true>(A, B, p, o, K, st);
       }
     }
 }

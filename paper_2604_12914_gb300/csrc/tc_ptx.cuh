@@ -202,6 +202,26 @@ __device__ __forceinline__ void mma_issue_pair(uint32_t tmem, uint64_t a, uint64
         : "r"(tmem), "l"(a), "l"(b), "r"(idesc), "r"(acc));
   }
 }
+// one BF16 MMA (of the pair's 256 rows if PAIR) on 128-byte swizzled rows, operands as sw64_lo gives them
+template <bool PAIR>
+__device__ __forceinline__ void mma_sw128(uint32_t tmem, uint32_t a, uint32_t b, uint32_t idesc, bool acc) {
+  // high word: stride offset 1024 >> 4, version 1, SWIZZLE_128B
+  constexpr uint32_t hi = (1024u >> 4) | (1u << 14) | (2u << 29);
+  if constexpr (PAIR)
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\tmov.b64 da, {%1, %3};\n\tmov.b64 db, {%2, %3};\n\t"
+        "setp.ne.b32 p, %5, 0;\n\t"
+        "tcgen05.mma.cta_group::2.kind::f16 [%0], da, db, %4, p;\n\t}"
+        :
+        : "r"(tmem), "r"(a), "r"(b), "r"(hi), "r"(idesc), "r"(acc ? 1 : 0));
+  else
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\tmov.b64 da, {%1, %3};\n\tmov.b64 db, {%2, %3};\n\t"
+        "setp.ne.b32 p, %5, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, p;\n\t}"
+        :
+        : "r"(tmem), "r"(a), "r"(b), "r"(hi), "r"(idesc), "r"(acc ? 1 : 0));
+}
 // arrives on the barrier at this offset in both CTAs once the MMAs issued before have completed
 __device__ __forceinline__ void mma_commit_pair(uint32_t bar) {
   asm volatile(
