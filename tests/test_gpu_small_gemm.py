@@ -15,3 +15,12 @@ from paper_2604_12914_gb300 import binding
 def test_small_products(M, N, K):
     tc, fp32 = binding.cc_lr_selftest_gemm(M, N, K, 2, seed=M + N + K)
     assert 0 <= fp32 < 2e-5
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("M,N", [(700, 650), (13000, 16), (16, 13000)])
+@pytest.mark.parametrize("K", [1, 7, 8, 9, 100])
+def test_large_tiles(M, N, K):
+    """64 x 64, 128 x 16 and 16 x 128 tiles at the edges of their K blocks of 8 and 16."""
+    tc, fp32 = binding.cc_lr_selftest_gemm(M, N, K, 2, seed=M + N + K)
+    assert 0 <= fp32 < 2e-5
