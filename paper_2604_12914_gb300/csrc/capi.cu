@@ -429,6 +429,7 @@ struct cclr_ctx {
     blk.clear();
     fullA.b.release();
     fullB.b.release();
+    release_gs_vectors();
   }
 
   // Block solve: nr independent systems (Op - omega_r) x_r = b_r advanced in lockstep, so that
@@ -814,6 +815,14 @@ struct cclr_ctx {
 
   // ---- ground-state CCSD: the amplitude equations Omega(T) = 0 and the energy (Sec. 2.2) ----
   CstSet gs;  // intermediates at s T, s a quadrature node of the residual (scratch)
+  // amplitudes, residual and product of a residual call, and the energy's effective doubles: kept for the next call up to
+  // 64 MB each, outside budgeted contexts
+  AVec gv[3];
+  DevBuf gtau;
+  void release_gs_vectors() {
+    for (auto &b : gv) b.b.release();
+    gtau.release();
+  }
 
   // the arithmetic of a ground-state product: a cclr_prec, or -1 for the context's own
   int gs_prec(int p) const {
@@ -834,7 +843,7 @@ struct cclr_ctx {
   void ccsd_residual(int p, const void *tp, void *r) {
     alloc_full(fullA);
     alloc_full(fullB);
-    AVec sv;
+    AVec &sv = gv[2];
     alloc_vec(sv);
     unpack_to(tp, fullA.b.p, C128);
     CCLR_CUDA(cudaMemsetAsync(r, 0, (size_t)n1 * 16, st));
@@ -863,11 +872,11 @@ struct cclr_ctx {
   // E(T) = sum_ia f_ia t_ia + 1/4 sum <ij||ab> t_ijab + 1/2 sum <ij||ab> t_ia t_jb
   //      = sum over i<j, a<b of <ij||ab> tau_ijab (f_ia = 0), packed amplitudes tp
   zd ccsd_energy(const void *tp) {
-    DevBuf tau((size_t)std::max<int64_t>(1, n2p) * 16);
-    tau_packed(o, v, tp, (const char *)tp + n1 * 16, tau.p, st);
+    if (!gtau.p) gtau.alloc((size_t)std::max<int64_t>(1, n2p) * 16);
+    tau_packed(o, v, tp, (const char *)tp + n1 * 16, gtau.p, st);
     double2 *part = M->E.dot_scratch();
     double2 *res = M->E.dot_results();
-    vec_dot(C128, n2p, M->oovv_packed(), tau.p, 0, part, res, 0, st);
+    vec_dot(C128, n2p, M->oovv_packed(), gtau.p, 0, part, res, 0, st);
     double2 e;
     CCLR_CUDA(cudaMemcpyAsync(&e, res, sizeof(e), cudaMemcpyDeviceToHost, st));
     CCLR_CUDA(cudaStreamSynchronize(st));
@@ -1650,7 +1659,7 @@ cclr_status cc_lr_ccsd_residual(cclr_ctx *c, int prec, const double *t1, const d
   return (cclr_status)guarded_ctx(c, [&] {
     const int p = c->gs_prec(prec);
     c->alloc_full(c->fullB);
-    AVec tv, rv;
+    AVec &tv = c->gv[0], &rv = c->gv[1];
     c->alloc_vec(tv);
     c->alloc_vec(rv);
     to_dev(c, t1, c->fullB.p1(), (size_t)c->n1 * 16);
@@ -1666,8 +1675,9 @@ cclr_status cc_lr_ccsd_residual(cclr_ctx *c, int prec, const double *t1, const d
     from_dev(c, c->fullA.p1(), r1, (size_t)c->n1 * 16);
     from_dev(c, c->fullA.p2(c->n1), r2, (size_t)c->n2 * 16);
     CCLR_CUDA(cudaStreamSynchronize(c->st));
-    c->M->release_set(c->gs);
+    c->M->retire_set(c->gs);
     if (c->M->lean) c->release_scratch();
+    else if ((size_t)c->ntot() * 16 > (64u << 20)) c->release_gs_vectors();
   });
 }
 

@@ -109,6 +109,25 @@ void Model::ensure_src64() {
   conv(h, h64, (int64_t)n * n);
 }
 
+namespace {
+// A buffer that one build needs: a workspace of the engine (kept for the next build) up to 64 MB, an allocation of its
+// own above that and in a budgeted context.  cudaMalloc and cudaFree cost a few hundred microseconds per buffer, and
+// drain the stream; the ground-state residual builds two sets.
+struct BuildTmp {
+  DevBuf own;
+  void *p;
+  BuildTmp(Engine &E, bool lean, int slot, size_t bytes) {
+    if (!lean && bytes <= (64u << 20)) {
+      p = E.ws(slot, bytes);
+    } else {
+      own.alloc(bytes);
+      p = own.p;
+    }
+  }
+};
+enum { WS_T1 = 8, WS_T2, WS_LTOO, WS_EYE, WS_EYE_T, WS_TRACE, WS_ONES, WS_OVOO, WS_MBEF };  // (contractions use 0-4)
+}  // namespace
+
 void Model::build_set(const void *t1d, const void *t2d, CstSet &out, int dt, int tc) {
   // CCLR_OPTIME=1 also prints the wall time of every build (diagnostics)
   static const bool optime = std::getenv("CCLR_OPTIME") && std::getenv("CCLR_OPTIME")[0] == '1';
@@ -138,13 +157,13 @@ void Model::build_set(const void *t1d, const void *t2d, CstSet &out, int dt, int
        Lvo = src(Lvo0, Lvo64, {P, v, o}), Lvv = src(Lvv0, Lvv64, {P, v, v});
   Tens Hf = src(h, h64, {n, n});
   // amplitudes in the build precision
-  DevBuf t1b, t2b;
   Tens t1t = make_tens((void *)t1d, C128, {o, v});
   Tens t2t = make_tens((void *)t2d, C128, {o, o, v, v});
+  std::unique_ptr<BuildTmp> t1b, t2b;
   if (dt == C64) {
-    t1b.alloc((size_t)o * v * 8);
-    t2b.alloc((size_t)o * o * v * v * 8);
-    Tens a = make_tens(t1b.p, C64, {o, v}), b = make_tens(t2b.p, C64, {o, o, v, v});
+    t1b = std::make_unique<BuildTmp>(E, lean, WS_T1, (size_t)o * v * 8);
+    t2b = std::make_unique<BuildTmp>(E, lean, WS_T2, (size_t)o * o * v * v * 8);
+    Tens a = make_tens(t1b->p, C64, {o, v}), b = make_tens(t2b->p, C64, {o, o, v, v});
     E.permute(zc(1), t1t, "ia", a, "ia", false);
     E.permute(zc(1), t2t, "ijab", b, "ijab", false);
     t1t = a;
@@ -152,7 +171,7 @@ void Model::build_set(const void *t1d, const void *t2d, CstSet &out, int dt, int
   }
 
   // ---- T1 dressing of the Cholesky blocks: L~ = (1 - t) L (1 + t)
-  DevBuf Ltoo_b((size_t)P * o * o * es);
+  BuildTmp Ltoo_b(E, lean, WS_LTOO, (size_t)P * o * o * es);
   Tens Ltoo = make_tens(Ltoo_b.p, dt, {P, o, o});
   E.permute(zc(1), Loo, "Pij", Ltoo, "Pij", false);
   E.contract(zc(1), Lov, "Pib", t1t, "jb", Ltoo, "Pij");
@@ -176,12 +195,13 @@ void Model::build_set(const void *t1d, const void *t2d, CstSet &out, int dt, int
   E.permute(zc(1), hvv, "ab", Fvv, "ab", false);
   E.contract(zc(-1), t1t, "ma", hov, "mb", Fvv, "ab");
   {
-    DevBuf Ib((size_t)o * o * 16), Id((size_t)o * o * es), trb((size_t)P * es), ones(sizeof(double) * o);
-    Tens I128 = T(Ib, {o, o}), I = make_tens(Id.p, dt, {o, o}), tr = make_tens(trb.p, dt, {P});
+    BuildTmp Ib(E, lean, WS_EYE, (size_t)o * o * 16), Id(E, lean, WS_EYE_T, (size_t)o * o * es),
+        trb(E, lean, WS_TRACE, (size_t)P * es), ones(E, lean, WS_ONES, sizeof(double) * o);
+    Tens I128 = make_tens(Ib.p, C128, {o, o}), I = make_tens(Id.p, dt, {o, o}), tr = make_tens(trb.p, dt, {P});
     E.zero(I128);
     std::vector<double> one(o, 1.0);
     CCLR_CUDA(cudaMemcpyAsync(ones.p, one.data(), sizeof(double) * o, cudaMemcpyHostToDevice, st));
-    set_diag(o, ones.as<double>(), Ib.p, st);
+    set_diag(o, (const double *)ones.p, Ib.p, st);
     E.permute(zc(1), I128, "kl", I, "kl", false);
     E.zero(tr);
     E.contract(zc(1), Ltoo, "Pkl", I, "kl", tr, "P");
@@ -228,7 +248,7 @@ void Model::build_set(const void *t1d, const void *t2d, CstSet &out, int dt, int
   E.contract(zc(-1), Ltoo, "Pmj", Ltvo, "Pbi", Wovoo, "mbij");
   E.contract(zc(-1), Fov, "me", T2, "ijbe", Wovoo, "mbij");
   {
-    DevBuf tb((size_t)o * v * o * o * es);
+    BuildTmp tb(E, lean, WS_OVOO, (size_t)o * v * o * o * es);
     Tens tmp = make_tens(tb.p, dt, {o, v, o, o});
     E.zero(tmp);
     E.contract(zc(1), Wooov, "mnie", T2, "jnbe", tmp, "mbij");
@@ -237,7 +257,7 @@ void Model::build_set(const void *t1d, const void *t2d, CstSet &out, int dt, int
     // 1/2 sum_ef <mb||ef>~ t_ij^ef = sum_ef <mb|ef>~ t_ij^ef, formed in chunks of b
     int64_t per_b = (int64_t)o * v * v * es;
     int64_t bc = std::max<int64_t>(1, std::min<int64_t>(v, (int64_t)(1ll << 30) / per_b));
-    DevBuf Gb((size_t)(bc * per_b));
+    BuildTmp Gb(E, lean, WS_MBEF, (size_t)(bc * per_b));
     for (int64_t b0 = 0; b0 < v; b0 += bc) {
       int64_t b1 = std::min<int64_t>(v, b0 + bc);
       Tens G = make_tens(Gb.p, dt, {o, b1 - b0, v, v});
@@ -351,6 +371,17 @@ void Model::release_set(CstSet &s) {
   for (int k = 0; k < 3; ++k)
     if (s.t[K_LVV].p && ltc_src[k] == s.t[K_LVV].p) ltc_src[k] = nullptr;
   for (auto &b : s.buf) b.release();
+  s.valid = false;
+}
+
+void Model::retire_set(CstSet &s) {
+  size_t held = 0;
+  for (const auto &b : s.buf) held += b.bytes;
+  if (lean || held > (256u << 20)) return release_set(s);
+  E.clear_prep_cache();
+  for (int k = 0; k < 3; ++k)
+    if (s.t[K_LVV].p && ltc_src[k] == s.t[K_LVV].p) ltc_src[k] = nullptr;
+  bump_state_epoch();
   s.valid = false;
 }
 

@@ -128,6 +128,8 @@ class Model {
   void round_set(const CstSet &src, CstSet &dst);
   // frees a set's buffers (it is rebuilt on its next use)
   void release_set(CstSet &s);
+  // ends the use of a scratch set: its buffers stay for the next one up to 256 MB, outside budgeted contexts
+  void retire_set(CstSet &s);
   // frees everything the FP64 products hold (the complex128 set, temporaries and the CUDA-core
   // ladder's blocks); an FP64 product afterwards rebuilds them
   void release_fp64();
