@@ -35,7 +35,7 @@ struct TcParams {
   int splits;           // work units = tiles x splits, walked with stride gridDim.x
   const uint32_t *list; // the tiles to compute, (m << 16) | n, ntiles of them (nullptr: all, in raster order)
   int ntiles;
-  int transposed;       // epilogue: 1 = lanes along columns (C columns contiguous), 0 = lane per row
+  int store;            // epilogue: a StoreMode
   float *C;
   View2 rv, cv;         // C rows and complex columns
   float ar, ai;
@@ -65,34 +65,99 @@ __device__ __forceinline__ void unit_coords(const TcParams &p, int u, int &m_til
 
 constexpr int EPI_PITCH = 18;  // floats per staged row (16 + 2): conflict-free float2 traffic
 
-// One 16-column chunk of a tile (columns n1 .., rows row0 + lane of the warp's 32) times alpha into C: eight complex
-// values per lane, destinations first, then all loads, then all stores (independent accesses in flight instead of one
-// read-modify-write at a time).
-__device__ __forceinline__ void store16(const TcParams &p, const uint32_t (&r)[16], float *stg, int row0, int lane, int n1) {
+// How a warp writes its part of C: a lane per row; lanes along contiguous columns; the same two complex columns at a time
+// (C 16-byte aligned, everything that its views add up to even)
+enum StoreMode { STORE_ROWS = 0, STORE_COLS = 1, STORE_PAIRS = 2 };
+
+// The rows of C (nullptr: beyond M) that a lane writes in every chunk of a unit, rows row0 + .. of the warp's 32
+struct RowPtrs {
+  float *p[8];
+  __device__ __forceinline__ RowPtrs(const TcParams &q, int row0, int lane) {
+    const int step = q.store == STORE_PAIRS ? 8 : 4;
+    const int first = row0 + (q.store == STORE_PAIRS ? lane >> 2 : q.store == STORE_COLS ? lane >> 3 : lane);
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const int row = first + k * step;
+      p[k] = row < q.M && k < (q.store == STORE_PAIRS ? 4 : q.store == STORE_COLS ? 8 : 1) ? q.C + 2 * v2off(q.rv, row) : nullptr;
+    }
+  }
+};
+
+// One 16-column chunk of a tile (columns n1 .., 32 rows) times alpha into C: sixteen values per lane, all loads before
+// the stores (independent accesses in flight instead of one read-modify-write at a time).  The epilogue's two warps per
+// scheduler are bound by their instructions: with the rows' addresses formed once per unit and 16 bytes per access a
+// chunk takes a fraction of the 416 that it took (245760 x 240 x 240 complex 277 us before, 180 now; 92160 x 160 x 160
+// 74 and 55).
+__device__ __forceinline__ void store16(const TcParams &p, const uint32_t (&r)[16], float *stg, const RowPtrs &rows, int lane,
+                                        int n1) {
+  if (p.store == STORE_PAIRS) {
+    // rows of 16 floats, their 16-byte units permuted so that neither side conflicts; 8 rows x 64 bytes per instruction
+    float4 *st4 = reinterpret_cast<float4 *>(stg);
+    const int u = lane & 3, rs = lane >> 2, n = n1 + 4 * u;
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      st4[4 * lane + (j ^ ((lane >> 1) & 3))] = make_float4(__uint_as_float(r[4 * j]), __uint_as_float(r[4 * j + 1]),
+                                                            __uint_as_float(r[4 * j + 2]), __uint_as_float(r[4 * j + 3]));
+    __syncwarp();
+    const int64_t co = 2 * v2off(p.cv, n >> 1);
+    float4 v[4];
+    float *dst[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int rl = 8 * k + rs;
+      v[k] = st4[4 * rl + (u ^ ((rl >> 1) & 3))];
+      dst[k] = rows.p[k] && n < p.N ? rows.p[k] + co : nullptr;
+    }
+    __syncwarp();
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      v[k] = make_float4(p.ar * v[k].x - p.ai * v[k].y, p.ar * v[k].y + p.ai * v[k].x, p.ar * v[k].z - p.ai * v[k].w,
+                         p.ar * v[k].w + p.ai * v[k].z);
+    if (p.atomic) {
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        if (dst[k]) atomicAdd(reinterpret_cast<float4 *>(dst[k]), v[k]);
+      return;
+    }
+    if (p.accumulate) {
+      float4 old[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) old[k] = dst[k] ? *reinterpret_cast<const float4 *>(dst[k]) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        v[k].x += old[k].x;
+        v[k].y += old[k].y;
+        v[k].z += old[k].z;
+        v[k].w += old[k].w;
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      if (dst[k]) *reinterpret_cast<float4 *>(dst[k]) = v[k];
+    return;
+  }
   float *dst[8];
   float2 val[8];
-  if (p.transposed) {
+  if (p.store == STORE_COLS) {
     // stage rows, then 4 rows x 8 complex per instruction (64 contiguous bytes per row)
     float2 *srow = reinterpret_cast<float2 *>(stg + lane * EPI_PITCH);
 #pragma unroll
     for (int j = 0; j < 8; ++j) srow[j] = make_float2(__uint_as_float(r[2 * j]), __uint_as_float(r[2 * j + 1]));
     __syncwarp();
     const int jj = lane & 7, rs = lane >> 3, n = n1 + 2 * jj;
+    const int64_t co = 2 * v2off(p.cv, n >> 1);
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
-      const int rl = 4 * k + rs, grow = row0 + rl;
-      val[k] = reinterpret_cast<const float2 *>(stg + rl * EPI_PITCH)[jj];
-      dst[k] = (grow < p.M && n < p.N) ? p.C + 2 * (v2off(p.rv, grow) + v2off(p.cv, n >> 1)) : nullptr;
+      val[k] = reinterpret_cast<const float2 *>(stg + (4 * k + rs) * EPI_PITCH)[jj];
+      dst[k] = rows.p[k] && n < p.N ? rows.p[k] + co : nullptr;
     }
     __syncwarp();
   } else {
-    const int row = row0 + lane;
-    const float *crow = p.C + 2 * v2off(p.rv, row < p.M ? row : 0);
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
       const int n = n1 + 2 * k;
       val[k] = make_float2(__uint_as_float(r[2 * k]), __uint_as_float(r[2 * k + 1]));
-      dst[k] = (row < p.M && n < p.N) ? const_cast<float *>(crow) + 2 * v2off(p.cv, n >> 1) : nullptr;
+      dst[k] = rows.p[0] && n < p.N ? rows.p[0] + 2 * v2off(p.cv, n >> 1) : nullptr;
     }
   }
 #pragma unroll
@@ -242,11 +307,12 @@ __global__ void __launch_bounds__(320, 1)
       int mt, nt, sp;
       unit_coords(p, u, mt, nt, sp);
       const int buf = it & 1;
+      const RowPtrs rows(p, mt * BM + q * 32, lane);
       bool ok = mbar_wait_ab(su32(tfull + buf), (uint32_t)(it >> 1) & 1u, p.err, abort_flag);
       ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
       if (!ok) break;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const int m0 = mt * BM, n0 = nt * BN;
+      const int n0 = nt * BN;
       const uint32_t tbase = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)buf * half;
       if (16 * h >= BN) {  // no chunk for this warp: release the buffer at once
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -263,7 +329,7 @@ __global__ void __launch_bounds__(320, 1)
           __syncwarp();
           if (lane == 0) mbar_arrive(su32(tempty + buf));
         }
-        store16(p, r, stg, m0 + q * 32, lane, n0 + c0);
+        store16(p, r, stg, rows, lane, n0 + c0);
       }
     }
   }
@@ -409,11 +475,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(320, 1)
       int mt, nt, sp;
       unit_coords(p, u, mt, nt, sp);
       const int buf = it & 1;
+      const RowPtrs rows(p, (2 * mt + (int)rank) * BM + q * 32, lane);
       bool ok = mbar_wait_ab(su32(tfull + buf), (uint32_t)(it >> 1) & 1u, p.err, abort_flag);
       ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
       if (!ok) break;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const int m0 = (2 * mt + (int)rank) * BM, n0 = nt * BN;
+      const int n0 = nt * BN;
       const uint32_t tbase = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)buf * half;
       for (int c0 = 16 * h; c0 < BN; c0 += 32) {
         uint32_t r[16];
@@ -424,7 +491,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(320, 1)
           __syncwarp();
           if (lane == 0) mbar_arrive_cluster(pair_addr(su32(tempty + buf), 0));
         }
-        store16(p, r, stg, m0 + q * 32, lane, n0 + c0);
+        store16(p, r, stg, rows, lane, n0 + c0);
       }
     }
   }
@@ -601,7 +668,8 @@ __global__ void __launch_bounds__(320, 1)
         uint32_t r[16];
 #pragma unroll
         for (int k = 0; k < 16; ++k) r[k] = __float_as_uint(sum[0][k]);
-        store16(p, r, stg, mt * BM + q * 32, lane, nt * BN + c);
+        const RowPtrs rows(p, mt * BM + q * 32, lane);  // (kept over the loop they would spill)
+        store16(p, r, stg, rows, lane, nt * BN + c);
 #pragma unroll
         for (int j = 0; j < 7; ++j)
 #pragma unroll
@@ -862,7 +930,7 @@ static int best_splits(int64_t M, int64_t Nreal, int nk, int BN, bool pair, bool
 
 // the rule's tile width and splits: the cheapest by cfg_clocks, a narrower tile where it gains a tenth (per column it
 // loads more of A: 25600 x 2560 x 800 complex 838 TFLOP/s at 256, 732 at 208, which would save half a wave); then
-// pairs of CTAs for one pass if their best tile gains a twentieth (92160 x 160 x 160, bound by its output: 66 us by
+// pairs of CTAs for one pass if their best tile gains a twentieth (92160 x 160 x 160, bound by its output: 76 us by
 // single CTAs, 80 by pairs)
 static TcCfg rule_cfg(int64_t M, int64_t Nreal, int nk, bool allow, int nsm, bool split) {
   TcCfg r, q;
@@ -943,8 +1011,12 @@ static void tc_launch(const void *A, int64_t lda, const void *B, int64_t ldb, in
   p.C = C;
   p.rv = rv;
   p.cv = cv;
-  // lanes along columns when C's columns run contiguously, one lane per row otherwise
-  p.transposed = (cv.sin == 1 && (cv.din == TC_ONE_LEVEL || cv.din >= 8)) ? 1 : 0;
+  // lanes along columns when C's columns run contiguously (two at a time where they make whole 16-byte units), one lane
+  // per row otherwise
+  const bool two_r = rv.din != TC_ONE_LEVEL, two_c = cv.din != TC_ONE_LEVEL;
+  const bool even = Nreal % 4 == 0 && (uintptr_t)C % 16 == 0 && rv.sin % 2 == 0 && (!two_r || rv.sout % 2 == 0) &&
+                    (!two_c || (cv.din % 2 == 0 && cv.sout % 2 == 0));
+  p.store = cv.sin != 1 || (two_c && cv.din < 8) ? STORE_ROWS : even ? STORE_PAIRS : STORE_COLS;
   p.ar = (float)alpha.re;
   p.ai = (float)alpha.im;
   p.atomic = splits > 1 ? 1 : 0;
@@ -961,9 +1033,9 @@ static void tc_launch(const void *A, int64_t lda, const void *B, int64_t ldb, in
   CCLR_REQUIRE(units < (1ll << 31), "tc_gemm: too many work units");
   static const bool trace = std::getenv("CCLR_TRACE") && std::getenv("CCLR_TRACE")[0] == '1';
   if (trace)
-    std::fprintf(stderr, "cclr tc_gemm kind=%d M=%lld N=%lld K=%lld BN=%d pair=%d tiles=%lld splits=%d band=%d atomic=%d transposed=%d\n",
+    std::fprintf(stderr, "cclr tc_gemm kind=%d M=%lld N=%lld K=%lld BN=%d pair=%d tiles=%lld splits=%d band=%d atomic=%d store=%d\n",
                  kind, (long long)M, (long long)Nreal, (long long)Kreal, BN, (int)cfg.pair, (long long)tiles, splits, p.band, p.atomic,
-                 p.transposed);
+                 p.store);
   const unsigned grid = (unsigned)std::min<int64_t>(units, nsm);
   const size_t epi = (size_t)8 * 32 * EPI_PITCH * 4 + (2 * PAIR_STAGES + 5) * 8 + 16;
   if (split) {
