@@ -89,12 +89,13 @@ def algorithmic(o, v, naux):
 # K = 1200: 1.793388 GB read + 1.740861 GB written for 8 M N K = 2.1234e12 FLOP).  With K =
 # naux fixed, both the output writes and the per-band operand reads scale with M N, so the
 # ratio carries over to every group of the same workload.
-FORMATION_BYTES_PER_FLOP = (1.793388e9 + 1.740861e9) / (8 * 28800 * 7680 * 1200)
+FORMATION_BYTES_PER_FLOP = (2.618338e9 + 1.743082e9) / (8 * 28800 * 7680 * 1200)
 
 
 def formation_flops_executed(v, naux, ga):
     """Real FLOP the formation GEMMs execute per sigma with group size ga (rows (b,f) with
-    b >= a0 for each group of ga a values)."""
+    b >= a0 for each group of ga a values; an upper bound, as tiles without an entry b > a are
+    left out)."""
     tot = 0
     for a0 in range(0, v - 1, ga):
         a1 = min(v, a0 + ga)
@@ -121,8 +122,8 @@ def ladder_peak(prec):
     if prec == "fp32":
         # 152 SMs x 128 FP32 lanes x 2 flops x 2.07 GHz
         return "alu", 152 * 128 * 2 * 2.07e9 / 1e12, "derived: SM count x FP32 lanes x max clock"
-    # FP64: nominal per-GPU rate (no measured figure on this machine)
-    return "alu", 1.25, "nominal FP64 rate"
+    # FP64: 36 BF16 slice products per contraction
+    return "tensor", d["bf16_tflops"] / 36, f"{how} bf16 / 36 slice products"
 
 
 def reduce_max(x: float) -> float:
@@ -359,7 +360,7 @@ def time_to_alpha_large(cfg, scale, comps=(2,), omegas=(0.0,), tol=1e-6):
     Krylov subspace and alpha contractions), then alpha again by the left-hand route
     (cc_lr_solve_left): the two routes agree to the solves' accuracy, so |alpha_left -
     alpha_right| is an a-posteriori estimate of the error.  (One FP64 sigma at this size takes
-    tens of seconds on this GPU; the FP64 path's solve is not run here.)"""
+    about a second on this GPU; the FP64 path's solve is not run here.)"""
     import numpy as np
     from paper_2604_12914_gb300 import binding
     from paper_2604_12914_gb300.inputs import make_config
@@ -708,7 +709,7 @@ def run_cclr(args):
     # the dominant kernel: the tensor-core GEMMs that form <ab|ef>~ (CUDA events around each)
     traffic = None
     if form_ms > 0:
-        kernel = "tc_gemm_kernel: pp-ladder formation <ab|ef>~ = sum_P L~_ae L~_bf (all groups of one sigma)"
+        kernel = "tc_pair_kernel: pp-ladder formation <ab|ef>~ = sum_P L~_ae L~_bf (all groups of one sigma)"
         achieved = alg["form_cmac"] * 8 / (form_ms * 1e-3) / 1e12
         if args.prec == "tf32" and tga:
             traffic = FORMATION_BYTES_PER_FLOP * formation_flops_executed(v, naux, tga)

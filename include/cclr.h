@@ -241,10 +241,11 @@ cclr_status cc_lr_graph_stats(cclr_ctx *ctx, int *captures, int *launches);
 
 /* Arithmetic of the mixed modes' accurate sigma products: the residual of every refinement
  * step, the polish that finishes a refinement which stalls, and the sigma^T products of the
- * F X stencil.  CCLR_FP64 (default): FP64 on CUDA cores; CCLR_C64_3XTF32: complex64 with
+ * F X stencil.  CCLR_FP64 (default): FP64; CCLR_C64_3XTF32: complex64 with
  * 3xTF32 on the tensor cores (about FP32 accuracy; the residual norms, vector updates, Krylov
- * subspace and alpha contractions stay FP64 either way).  The FP64 sigma is slow on GPUs with
- * a reduced FP64 rate, so large systems use CCLR_C64_3XTF32 with CCLR_C64_TF32 corrections. */
+ * subspace and alpha contractions stay FP64 either way).  The FP64 sigma executes 36 slice
+ * products per contraction and holds a complex128 set, so large systems use CCLR_C64_3XTF32
+ * with CCLR_C64_TF32 corrections. */
 cclr_status cc_lr_set_refinement(cclr_ctx *ctx, int prec);
 
 /* Linear solver of cc_lr_solve / cc_lr_solve_x / cc_lr_lambda: method 1 = restarted

@@ -1,4 +1,4 @@
-// Packed particle-particle ladder on the CUDA cores; see ladder_cc.cuh.
+// Packed particle-particle ladder outside the complex64 tensor-core modes; see ladder_cc.cuh.
 #include <cstdio>
 #include <string>
 #include <vector>

@@ -1,6 +1,6 @@
-// Packed particle-particle ladder on the CUDA cores (FP64 DFMA for complex128, FP32 FFMA for
-// complex64): the same packed algorithm as the tensor-core ladder (LadderTC), for the
-// precision modes that do not use tensor cores.
+// Packed particle-particle ladder of the FP64 and FP32 modes (complex128: from exact slices on the
+// tensor cores where the formation is large and the slices find room, else FP64 CUDA cores;
+// complex64: FP32 CUDA cores): the same packed algorithm as LadderTC.
 //   out[i,j,a,b] += alpha * sum_{e<f} <ab||ef>~ X[i,j,e,f],   <ab|ef>~ = sum_P L~[P,a,e] L~[P,b,f]
 // over packed pairs i<j, a<b, e<f, <ab|ef>~ formed on the fly for one group of a at a time
 // (formation GEMM, K = naux), antisymmetrised and packed, then contracted with packed X; the

@@ -415,8 +415,7 @@ void Model::release_fp64_inputs() {
 }
 
 // The FP64 mode reads intermediates built in FP64.  The complex64 modes read the rounding of
-// those when they exist, else a set built in FP32 on the CUDA cores (this GPU's FP64 rate makes
-// the FP64 build of the o^3 v^3 and o v^3 naux terms take minutes at o=56, v=480).
+// those when they exist, else a set built in FP32 on the CUDA cores (half the memory of an FP64 set).
 const CstSet &Model::cst_for(int p) {
   if (p == 0) {
     if (!c128.valid) {
@@ -489,7 +488,7 @@ Tens Model::var_tens(int id, int dt, void *p) const {
 // pp-ladder: out[i,j,a,b] += alpha sum_ef <ab|ef>~ in[i,j,e,f] (dir +1), or the transpose
 // in'[i,j,e,f] += alpha sum_ab <ab|ef>~ in[i,j,a,b] (dir -1), over packed pairs with <ab|ef>~
 // formed per group of a from L~_vv and never stored whole: tcgen05 tensor cores in the TF32 /
-// 3xTF32 modes, CUDA cores otherwise.
+// 3xTF32 modes and (from exact slices) in FP64, CUDA cores otherwise.
 void Model::ladder(int dir, const CstSet &C, zc alpha, const std::vector<Tens> &in,
                    const std::vector<Tens> &out) {
   const int dt = C.dt;
@@ -512,7 +511,7 @@ void Model::ladder(int dir, const CstSet &C, zc alpha, const std::vector<Tens> &
     ltc[k].apply(E, dir, alpha, nr, ip.data(), outp.data());
     return;
   }
-  // CUDA cores (FP64 DFMA or FP32 FFMA): the same packed algorithm
+  // FP64 slices or CUDA cores: the same packed algorithm
   std::vector<const void *> ip(nr);
   std::vector<void *> outp(nr);
   for (int r = 0; r < nr; ++r) { ip[r] = in[r].p; outp[r] = out[r].p; }

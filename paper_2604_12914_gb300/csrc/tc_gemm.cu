@@ -4,7 +4,8 @@
 // swizzle) into a 4-stage shared-memory ring, warp 1 issues tcgen05.mma into one of two TMEM
 // accumulators, and warps 2-9 drain the other accumulator (tcgen05.ld -> registers ->
 // shared-memory staging -> coalesced global stores), so the epilogue of one tile overlaps
-// the main loop of the next.  Every mbarrier wait is bounded (globaltimer); on timeout the
+// the main loop of the next.  Large products run as pairs of CTAs on 256-row tiles
+// (tc_pair_kernel), the split modes as tc_split_kernel.  Every mbarrier wait is bounded (globaltimer); on timeout the
 // kernel raises a device flag, stops every role, drains its own copies and MMAs with bounded
 // waits, frees its TMEM and returns.
 #include <cstdio>
