@@ -76,6 +76,9 @@ int cc_lr_selftest_gemm_noalloc(int M, int N, int K, int mode, unsigned seed, do
  * should not be, or not NaN where they should.  Returns 0 on success, else a cclr_status code. */
 int cc_lr_selftest_f64gemm(int M, int N, int K, int layout, double spread, unsigned seed, double *out);
 
+/* Device bytes that the FP64 tensor-core GEMM's callers claim for its sums before M x N products (no device call). */
+int cc_lr_selftest_f64_scratch(long long M, long long N, unsigned long long *bytes);
+
 /* The diagonal preconditioner out = r / (D - (omega + i omega_im)) on n seeded complex128 entries
  * (D uniform in [0.1, 20], r normal), whose kernel forms the FP64 reciprocal by Newton-Raphson
  * iteration from the FP32 reciprocal: writes max |out - r/(D - z)| / |r/(D - z)| over the entries,

@@ -1942,6 +1942,12 @@ int cc_lr_selftest_f64gemm(int M, int N, int K, int layout, double spread, unsig
   });
 }
 
+int cc_lr_selftest_f64_scratch(long long M, long long N, unsigned long long *bytes) {
+  if (M < 1 || N < 1 || !bytes) return fail(CCLR_EINVAL, "bad selftest_f64_scratch arguments");
+  *bytes = f64tc_scratch_bytes(M, N);
+  return CCLR_OK;
+}
+
 int cc_lr_selftest_timeout(int timeout_us, int *flag) {
   if (timeout_us < 1 || timeout_us > 10000000 || !flag) return fail(CCLR_EINVAL, "bad selftest_timeout arguments");
   int st = guarded([&] {

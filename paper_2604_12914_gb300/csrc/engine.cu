@@ -498,7 +498,7 @@ void Engine::f64_scratch(int64_t M, int64_t N) {
 
 void Engine::f64_gemm(const F64Op &A, int64_t M, const F64Op &B, int64_t N, int64_t K, void *C, View2 rv, View2 cv, zc alpha,
                       bool accumulate, UpperTiles *upper) {
-  f64_scratch(M, N);
+  CCLR_REQUIRE(f64_scr_.bytes >= f64tc_scratch_bytes(M, N), "f64_gemm: no room claimed for the sums");
   tc_pending = true;
   f64tc_gemm(A, M, B, N, K, C, rv, cv, alpha, accumulate, f64_scr_.p, st, upper);
 }

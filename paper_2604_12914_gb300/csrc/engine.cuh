@@ -120,7 +120,8 @@ class Engine {
   // clear_prep_cache() like the other constant operands (at most f64_cache_cap bytes).  Throws status 2.
   F64Op f64_operand(int slot, const void *src, View2 rv, View2 kv, int64_t R, int64_t K, bool embed,
                     const std::string &key);
-  // room for the sums of an M x N f64tc_gemm (throws status 2), and the product itself on this engine's stream
+  // room for the sums of f64tc_gemms of up to M x N (throws status 2), and a product itself on this engine's stream; the
+  // room has to be claimed before: nothing is allocated, and so nothing can fail, between the products of a call
   void f64_scratch(int64_t M, int64_t N);
   void f64_gemm(const F64Op &A, int64_t M, const F64Op &B, int64_t N, int64_t K, void *C, View2 rv, View2 cv, zc alpha,
                 bool accumulate, UpperTiles *upper = nullptr);

@@ -851,10 +851,14 @@ F64Op f64tc_prep(const void *src, View2 rv, View2 kv, int64_t R, int64_t K, bool
   return op;
 }
 
+// The largest need of any product of at most M rows and N columns, so that what a caller claims for its first (largest)
+// block or chunk serves the others: a launch takes no more tiles than there are and than SUMS_CAP holds, K splits
+// no more than one unit per SM, and the width of the tiles only grows with N.  (The need of the product itself
+// is not monotone: fewer rows of tiles leave room for more columns of them.)
 size_t f64tc_scratch_bytes(int64_t M, int64_t N) {
   const F64Plan q = plan_of(M, N, SUMS_CAP);
-  // split K: at most one unit per SM
-  return (size_t)std::max<int64_t>((int64_t)q.rows * q.cols, (int64_t)q.nMt * q.nNt <= SPLIT_TILES ? tc_num_sms() : 0) * q.unit;
+  const int64_t fit = std::max<int64_t>(1, (int64_t)SUMS_CAP / q.unit);
+  return (size_t)(std::max<int64_t>(std::min<int64_t>(fit, (int64_t)q.nMt * q.nNt), tc_num_sms()) * q.unit);
 }
 
 void f64tc_gemm(const F64Op &A, int64_t M, const F64Op &B, int64_t N, int64_t K, void *C, View2 rv, View2 cv, zc alpha,

@@ -46,7 +46,8 @@ F64Op f64tc_prep(const void *src, View2 rv, View2 kv, int64_t R, int64_t K, bool
 
 // C(m, n) (+)= alpha sum_k A(m, k) B(k, n), complex128, from prepared operands (A: M rows, B: N embedded
 // columns).  C(m, n) at C + v2off(rv, m) + v2off(cv, n) complex entries; accumulate: added to C, else C is
-// overwritten.  scratch: f64tc_scratch_bytes(M, N) of device memory for the integer sums (at most 256 MB).
+// overwritten.  scratch: f64tc_scratch_bytes of device memory for the integer sums (at most 256 MB), of M and N or of
+// any larger numbers of rows and columns.
 void f64tc_gemm(const F64Op &A, int64_t M, const F64Op &B, int64_t N, int64_t K, void *C, View2 rv, View2 cv, zc alpha,
                 bool accumulate, void *scratch, cudaStream_t st, class UpperTiles *upper = nullptr);
 size_t f64tc_scratch_bytes(int64_t M, int64_t N);
