@@ -819,13 +819,15 @@ struct F64Plan {
   int BN, nMt, nNt, rows, cols;  // tiles in all; tile rows and tile columns per launch
   int64_t unit;                  // bytes of one tile's sums
 };
+// tiles whose sums take cap bytes: as many columns of accumulators at every width
+int64_t tiles_that_fit(int BN, size_t cap) { return (int64_t)cap / (BM * 128 * 12) * (128 / BN); }
 F64Plan plan_of(int64_t M, int64_t N, size_t cap) {
   F64Plan q;
   q.BN = 2 * N <= 32 ? 32 : 2 * N <= 64 ? 64 : 128;
   q.nMt = (int)((M + BM - 1) / BM);
   q.nNt = (int)((2 * N + q.BN - 1) / q.BN);
   q.unit = (int64_t)BM * q.BN * 12;
-  const int64_t fit = std::max<int64_t>(1, (int64_t)cap / q.unit);
+  const int64_t fit = tiles_that_fit(q.BN, cap);
   q.rows = (int)std::min<int64_t>(q.nMt, fit);
   q.cols = (int)std::max<int64_t>(1, std::min<int64_t>(q.nNt, fit / q.rows));
   return q;
@@ -857,7 +859,7 @@ F64Op f64tc_prep(const void *src, View2 rv, View2 kv, int64_t R, int64_t K, bool
 // is not monotone: fewer rows of tiles leave room for more columns of them.)
 size_t f64tc_scratch_bytes(int64_t M, int64_t N) {
   const F64Plan q = plan_of(M, N, SUMS_CAP);
-  const int64_t fit = std::max<int64_t>(1, (int64_t)SUMS_CAP / q.unit);
+  const int64_t fit = tiles_that_fit(q.BN, SUMS_CAP);
   return (size_t)(std::max<int64_t>(std::min<int64_t>(fit, (int64_t)q.nMt * q.nNt), tc_num_sms()) * q.unit);
 }
 

@@ -26,7 +26,7 @@ def test_ladder_groups_fit_the_first_groups_room(v):
 
 
 def test_grows_with_rows_and_columns():
-    sizes = [1, 15, 16, 17, 32, 33, 64, 65, 127, 128, 129, 500, 1000, 4864, 9728, 9729, 50000, 300000]
+    sizes = [1, 15, 16, 17, 32, 33, 64, 65, 127, 128, 129, 500, 1000, 4864, 9728, 9729, 50000, 300000, 1000000]
     need = {(m, n): binding.cc_lr_selftest_f64_scratch(m, n) for m in sizes for n in sizes}
     for i, m in enumerate(sizes):
         for j, n in enumerate(sizes):
