@@ -69,10 +69,12 @@ int cc_lr_selftest_gemm_noalloc(int M, int N, int K, int mode, unsigned seed, do
 /* The FP64 tensor-core GEMM (exact 8-bit slices) on seeded data: C = C0 + alpha A B, complex128, alpha = -0.5
  * (layout bit 8: a general complex alpha), entries normal, rows of A and columns of B scaled by
  * 2^[-spread, spread].  layout bits: 1 A stored [M][K] (else [K][M]), 2 B stored [N][K] (else [K][N]), 4 C
- * stored [N][M] (else [M][N]), 16 a NaN in row 0 of A.  Against sums in extended precision on the host over
+ * stored [N][M] (else [M][N]), 16 a NaN in row 0 of A, 32 graded operands (no row scales; the rows of A fall and the
+ * columns of B rise by 2^spread along k, and the imaginary parts of A lie 2^(spread/2) lower).  Against sums in extended precision on the host over
  * (at most 4000) entries: out[0] = the largest error over its bound, the FP64 rounding of the result plus
  * the dropped slice orders, 8 u (|alpha ref| + |C0|) + |alpha| a b (K 2^-59 + K^2 2^-67), u = 2^-53, a and b the
- * largest entries of the row and the column; out[1] = the number of entries that are NaN where they
+ * largest entries of the row and the column; with graded operands the bound is that of FP64 sums, for the real and the
+ * imaginary part by itself: (2 K + 8) u sum of the terms' magnitudes + 4 u |C0|; out[1] = the number of entries that are NaN where they
  * should not be, or not NaN where they should.  Returns 0 on success, else a cclr_status code. */
 int cc_lr_selftest_f64gemm(int M, int N, int K, int layout, double spread, unsigned seed, double *out);
 

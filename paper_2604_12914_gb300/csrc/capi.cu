@@ -1876,34 +1876,38 @@ int cc_lr_selftest_precond(int n, double omega, double omega_im, unsigned seed, 
 }
 
 int cc_lr_selftest_f64gemm(int M, int N, int K, int layout, double spread, unsigned seed, double *out) {
-  if (M < 1 || N < 1 || K < 1 || layout < 0 || layout > 31 || !(spread >= 0 && spread < 400) || !out)
+  if (M < 1 || N < 1 || K < 1 || layout < 0 || layout > 63 || !(spread >= 0 && spread < 400) || !out)
     return fail(CCLR_EINVAL, "bad selftest_f64gemm arguments");
   return guarded([&] {
     std::mt19937_64 g(seed);
     std::normal_distribution<double> nd(0.0, 1.0);
     std::uniform_real_distribution<double> ud(-spread, spread);
-    const bool ak = layout & 1, bk = layout & 2, cm = layout & 4;
+    const bool ak = layout & 1, bk = layout & 2, cm = layout & 4, graded = layout & 32;
     const zd alpha = layout & 8 ? zd(0.7, -1.3) : zd(-0.5);
     std::vector<zd> a((size_t)M * K), b((size_t)K * N), c0((size_t)M * N), c((size_t)M * N);
     std::vector<double> am(M, 0.0), bm(N, 0.0);
     auto A = [&](int m, int k) -> zd & { return a[ak ? (size_t)m * K + k : (size_t)k * M + m]; };
     auto B = [&](int k, int n) -> zd & { return b[bk ? (size_t)n * K + k : (size_t)k * N + n]; };
     auto at = [&](int m, int n) { return cm ? (size_t)n * M + m : (size_t)m * N + n; };
+    // graded: rows of A fall and columns of B rise by 2^spread along k, the imaginary parts of A lie 2^(spread / 2) lower
+    auto fall = [&](double f) { return graded ? std::exp2(-std::floor(spread * f)) : 1.0; };
     for (int m = 0; m < M; ++m) {
-      const double s = std::exp2(std::floor(ud(g)));
+      const double s = graded ? 1.0 : std::exp2(std::floor(ud(g)));
       for (int k = 0; k < K; ++k) {
-        A(m, k) = zd(s * nd(g), s * nd(g));
+        const double q = s * fall((double)k / K);
+        A(m, k) = zd(q * nd(g), q * fall(0.5) * nd(g));
         am[m] = std::max({am[m], std::abs(A(m, k).real()), std::abs(A(m, k).imag())});
       }
     }
     for (int n = 0; n < N; ++n) {
-      const double s = std::exp2(std::floor(ud(g)));
+      const double s = graded ? 1.0 : std::exp2(std::floor(ud(g)));
       for (int k = 0; k < K; ++k) {
-        B(k, n) = zd(s * nd(g), s * nd(g));
+        const double q = s * fall((double)(K - 1 - k) / K);
+        B(k, n) = zd(q * nd(g), q * nd(g));
         bm[n] = std::max({bm[n], std::abs(B(k, n).real()), std::abs(B(k, n).imag())});
       }
     }
-    for (auto &z : c0) z = zd(nd(g), nd(g));
+    for (auto &z : c0) z = fall(1.5) * zd(nd(g), nd(g));
     if (layout & 16) A(0, K / 2) = zd(std::numeric_limits<double>::quiet_NaN(), 0.0);
     cudaStream_t st;
     CCLR_CUDA(cudaStreamCreate(&st));
@@ -1914,7 +1918,8 @@ int cc_lr_selftest_f64gemm(int M, int N, int K, int layout, double spread, unsig
     CCLR_CUDA(cudaMemcpyAsync(Cd.p, c0.data(), Cd.bytes, cudaMemcpyHostToDevice, st));
     const F64Op oa = f64tc_prep(Ad.p, view1(ak ? K : 1), view1(ak ? 1 : M), M, K, false, As.p, At.as<uint32_t>(), st);
     const F64Op ob = f64tc_prep(Bd.p, view1(bk ? K : 1), view1(bk ? 1 : N), N, K, true, Bs.p, Bt.as<uint32_t>(), st);
-    f64tc_gemm(oa, M, ob, N, K, Cd.p, view1(cm ? 1 : N), view1(cm ? M : 1), zc(alpha.real(), alpha.imag()), true, Sc.p, st);
+    F64Side side;
+    f64tc_gemm(oa, M, ob, N, K, Cd.p, view1(cm ? 1 : N), view1(cm ? M : 1), zc(alpha.real(), alpha.imag()), true, Sc.p, side, st);
     CCLR_CUDA(cudaMemcpyAsync(c.data(), Cd.p, Cd.bytes, cudaMemcpyDeviceToHost, st));
     if (tc_error(st)) throw Error(CCLR_ETIMEOUT, "tensor-core kernel gave up on a bounded wait");
     CCLR_CUDA(cudaStreamDestroy(st));
@@ -1928,15 +1933,25 @@ int cc_lr_selftest_f64gemm(int M, int N, int K, int layout, double spread, unsig
       if (nan != std::isnan(got.real()) || nan != std::isnan(got.imag())) out[1] += 1.0;
       if (nan) continue;
       long double re = 0.0L, im = 0.0L;
+      double sr = 0.0, si = 0.0;  // sums of the terms' magnitudes
       for (int k = 0; k < K; ++k) {
         const zd x = A(m, k), y = B(k, n);
         re += (long double)x.real() * y.real() - (long double)x.imag() * y.imag();
         im += (long double)x.real() * y.imag() + (long double)x.imag() * y.real();
+        sr += std::abs(x.real() * y.real()) + std::abs(x.imag() * y.imag());
+        si += std::abs(x.real() * y.imag()) + std::abs(x.imag() * y.real());
       }
       const long double wr = old.real() + (alpha.real() * re - alpha.imag() * im);
       const long double wi = old.imag() + (alpha.real() * im + alpha.imag() * re);
       const double mag = std::abs(alpha) * std::hypot((double)re, (double)im) + std::abs(old);
-      const double lim = 8 * u * mag + std::abs(alpha) * am[m] * bm[n] * ext;
+      double lim = 8 * u * mag + std::abs(alpha) * am[m] * bm[n] * ext;
+      if (graded) {  // part by part, as FP64 sums in any order: a product and 2K - 1 additions of u each, alpha's, C's
+        const double ar = std::abs(alpha.real()), ai = std::abs(alpha.imag());
+        lim = (2.0 * K + 8) * u * (ar * sr + ai * si) + 4 * u * std::abs(old.real());
+        const double li = (2.0 * K + 8) * u * (ar * si + ai * sr) + 4 * u * std::abs(old.imag());
+        out[0] = std::max({out[0], (double)std::abs(got.real() - wr) / lim, (double)std::abs(got.imag() - wi) / li});
+        continue;
+      }
       out[0] = std::max({out[0], (double)std::abs(got.real() - wr) / lim, (double)std::abs(got.imag() - wi) / lim});
     }
   });

@@ -452,33 +452,39 @@ bool Engine::f64_reclaim() {
   return true;
 }
 
+Engine::PrepEntry *Engine::f64_keep(const std::string &key, size_t bytes) {
+  for (auto &x : f64_kept_)
+    if (x->key == key) return x->buf.bytes == bytes ? x.get() : nullptr;
+  if (f64_kept_bytes_ + bytes > f64_cache_cap) return nullptr;
+  auto n = std::make_unique<PrepEntry>();
+  n->key = key;
+  try {
+    n->buf.alloc(bytes);
+  } catch (const Error &x) {
+    if (x.status != 2) throw;
+    return nullptr;
+  }
+  f64_kept_bytes_ += bytes;
+  f64_kept_.push_back(std::move(n));
+  return f64_kept_.back().get();
+}
+
 F64Op Engine::f64_operand(int slot, const void *src, View2 rv, View2 kv, int64_t R, int64_t K, bool embed,
                           const std::string &key) {
   const size_t sl = ((size_t)f64tc_bytes(R, K, embed) + 255) / 256 * 256, need = sl + (size_t)R * 4;
   if (!key.empty()) {
-    PrepEntry *e = nullptr;
-    for (auto &x : f64_kept_)
-      if (x->key == key) e = x.get();
-    if (e && e->filled && e->buf.bytes == need) {
+    PrepEntry *e = f64_keep(key, need);
+    if (e && e->filled) {
       F64Op op;
       op.p = e->buf.p;
       op.tops = (const uint32_t *)((const char *)e->buf.p + sl);
       op.stride = R;
+      op.src = src;
+      op.rv = rv;
+      op.kv = kv;
       return op;
     }
-    if (!e && f64_kept_bytes_ + need <= f64_cache_cap) {
-      auto n = std::make_unique<PrepEntry>();
-      n->key = key;
-      try {
-        n->buf.alloc(need);
-        f64_kept_bytes_ += need;
-        f64_kept_.push_back(std::move(n));
-        e = f64_kept_.back().get();
-      } catch (const Error &x) {  // no room to keep it: the workspace slot serves
-        if (x.status != 2) throw;
-      }
-    }
-    if (e && e->buf.bytes == need) {
+    if (e) {
       const F64Op op = f64tc_prep(src, rv, kv, R, K, embed, e->buf.p, (uint32_t *)((char *)e->buf.p + sl), st);
       e->filled = true;
       return op;
@@ -500,7 +506,7 @@ void Engine::f64_gemm(const F64Op &A, int64_t M, const F64Op &B, int64_t N, int6
                       bool accumulate, UpperTiles *upper) {
   CCLR_REQUIRE(f64_scr_.bytes >= f64tc_scratch_bytes(M, N), "f64_gemm: no room claimed for the sums");
   tc_pending = true;
-  f64tc_gemm(A, M, B, N, K, C, rv, cv, alpha, accumulate, f64_scr_.p, st, upper);
+  f64tc_gemm(A, M, B, N, K, C, rv, cv, alpha, accumulate, f64_scr_.p, f64_side_, st, upper);
 }
 
 void Engine::check_tc() {
@@ -554,7 +560,7 @@ bool Engine::contract_f64(zc alpha, const Tens &A, const std::string &ma, const 
     return n > cap && u < n ? std::max(u, cap / u * u) : n;
   };
   const int64_t Mc = chunk(M, f64tc_bytes(1, K, false), unit_of(am, cm)), Nc = chunk(N, f64tc_bytes(1, K, true), unit_of(bn, cn));
-  if ((double)F64_SLICES * std::max(Mc, 2 * Nc) >= 2147483648.0) return false;
+  if ((double)F64_PLANES * 2 * std::max(Mc, Nc) >= 2147483648.0) return false;
   const void *Ap = A.p, *Bp = B.p;
   Tens T;
   std::string akey, bkey;
@@ -567,7 +573,7 @@ bool Engine::contract_f64(zc alpha, const Tens &A, const std::string &ma, const 
   auto at = [](const std::string &key, int64_t b, int64_t r) {
     return key.empty() ? key : key + std::to_string(b) + "," + std::to_string(r);
   };
-  // a kept operand whose slices are all there needs no contiguous copy
+  // kept slices need no workspace
   auto have = [&](const std::string &key, int64_t n, int64_t step) {
     if (key.empty()) return false;
     for (int64_t b = 0; b < nb; ++b)
@@ -578,10 +584,17 @@ bool Engine::contract_f64(zc alpha, const Tens &A, const std::string &ma, const 
       }
     return true;
   };
+  // the contiguous copy of an operand, which the direct sums of small entries read (f64_tc.cuh): kept beside the
+  // slices of a constant
+  PrepEntry *a_copy = nullptr, *b_copy = nullptr;
+  auto copy = [&](const std::string &key, int slot, size_t bytes, PrepEntry *&e) -> const void * {
+    e = key.empty() ? nullptr : f64_keep(key + "copy", bytes);
+    return e ? e->buf.p : ws(slot, bytes);
+  };
   F64Hold hold(*this);
   try {
-    if (!a_ok && !have(akey, M, Mc)) Ap = ws(0, nb * M * K * es);
-    if (!b_ok && !have(bkey, N, Nc)) Bp = ws(1, nb * K * N * es);
+    if (!a_ok) Ap = copy(akey, 0, nb * M * K * es, a_copy);
+    if (!b_ok) Bp = copy(bkey, 1, nb * K * N * es, b_copy);
     if (!direct) T = contiguous_like(ws(2, nb * M * N * es), C128, C, mc, bat + Mm + Nm);
     // the workspace for the slices is claimed before anything is computed
     f64_scratch(Mc, Nc);
@@ -591,13 +604,15 @@ bool Engine::contract_f64(zc alpha, const Tens &A, const std::string &ma, const 
     if (e.status != 2) throw;
     return false;
   }
-  if (!a_ok && Ap != A.p) {
+  if (!a_ok && !(a_copy && a_copy->filled)) {
     Tens P = contiguous_like((void *)Ap, C128, A, ma, bat + Mm + Km);
     permute(zc(1.0), A, ma, P, bat + Mm + Km, false);
+    if (a_copy) a_copy->filled = true;
   }
-  if (!b_ok && Bp != B.p) {
+  if (!b_ok && !(b_copy && b_copy->filled)) {
     Tens P = contiguous_like((void *)Bp, C128, B, mb, bat + Km + Nm);
     permute(zc(1.0), B, mb, P, bat + Km + Nm, false);
+    if (b_copy) b_copy->filled = true;
   }
   if (trace_on())
     std::fprintf(stderr, "cclr contract f64 %s,%s->%s nb=%lld M=%lld N=%lld K=%lld A[%s|%s]%s B[%s|%s]%s C[%s|%s]%s\n", ma.c_str(),

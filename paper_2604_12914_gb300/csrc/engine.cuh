@@ -176,10 +176,13 @@ class Engine {
   PrepEntry *prep_find(const std::string &key);
   // the entry to (re)fill, created if needed; nullptr when it would exceed the cap
   PrepEntry *prep_get(const std::string &key, size_t bytes);
-  std::vector<DevBuf> f64_slots_;  // two per slot: slices, tops
+  // the kept entry of that key and size, created if needed; nullptr where there is no room to keep it
+  PrepEntry *f64_keep(const std::string &key, size_t bytes);
+  std::vector<DevBuf> f64_slots_;  // slices, then tops in the same buffer
   std::vector<std::unique_ptr<PrepEntry>> f64_kept_;  // slices, then tops in the same buffer
   size_t f64_kept_bytes_ = 0;
   DevBuf f64_scr_;
+  F64Side f64_side_;
   int f64_holds_ = 0;
 };
 

@@ -57,6 +57,16 @@ struct F64Out {
   View2 rv, cv;
   double ar, ai;        // alpha (used unless pow2)
   int pow2, neg, sh;    // alpha = (-1)^neg 2^sh
+  // entries that are summed directly: the words of tc_magnitude_sums, or its sums (then words is nullptr), for the rows from
+  // m0 on and the ldw columns from n0 on; the operands, and the complex k of this launch
+  const uint4 *words;
+  const float2 *sums;
+  int64_t ldw;
+  float tau;
+  const double2 *A, *B;
+  int64_t ra, rb;  // their first row and column
+  View2 arv, akv, brv, bkv;
+  int64_t k0, k1;
 };
 
 __device__ __forceinline__ void unit_coords(const F64Params &p, int u, int &mt, int &nt, int &sp) {
@@ -492,13 +502,166 @@ __global__ void __launch_bounds__(384, 1)
   }
 }
 
+// Whether a part lies too far below the product of its row's and column's maxima for the slices: bit l of the word for row
+// 32 g + l, or the sums of one entry.
+__device__ __forceinline__ uint32_t small_bits(uint4 w) { return (w.z & ~w.x) | (w.w & ~w.y); }
+__device__ __forceinline__ bool small_sum(float2 s, float tau) { return (s.x < tau && s.x != 0.f) || (s.y < tau && s.y != 0.f); }
+// The FP64 sums alpha sum_k A(row, k) B(k, n) of the entries in 32 rows from r0 on and the columns c0 + lane whose words
+// (lane by lane, the same in every warp) are not zero, which nobody else has written, by the block's 256 threads.  Many
+// short sums: a thread per entry, in the order of k.  Else up to K = 1024 a warp per entry, and beyond it the block for up
+// to four rows of a column, each thread every 32nd or 256th k and the threads' sums added up pairwise.  In the long sums
+// 32 terms that are all zero are passed over: the usual ones are those of a row or column that the difference of two equal
+// products has left, a few roundings among zeros, and the FP64 pipe bounds the loop.  (256 x 256 entries of K = 12100 with
+// 14 such rows: 0.73 ms without, 0.19 with.)  A call: inlined, it costs the conversion its registers.
+__device__ __noinline__ void write_small(const F64Out &p, uint32_t word, int r0, int c0) {
+  __shared__ double part[8][8];
+  const int lane = threadIdx.x, y = threadIdx.y, thread = 32 * y + lane;
+  auto write = [&](int row, int n, double re, double im) {
+    double2 *dst = (double2 *)p.C + v2off(p.rv, row) + v2off(p.cv, n);
+    double2 v = make_double2(p.ar * re - p.ai * im, p.ar * im + p.ai * re);
+    if (p.accumulate) { const double2 o = *dst; v.x += o.x; v.y += o.y; }
+    *dst = v;
+  };
+  auto nonzero = [](double2 z) {  // (in integers: comparisons are the FP64 pipe's too)
+    return ((__double_as_longlong(z.x) | __double_as_longlong(z.y)) << 1) != 0;
+  };
+  const int total = __reduce_add_sync(0xffffffffu, __popc(word));
+  if (p.k1 - p.k0 <= 256 && total >= 64) {
+    for (int t0 = 0; t0 < total; t0 += 256) {
+      int left = t0 + thread, l = -1, n = 0;
+#pragma unroll 1
+      for (int j = 0; j < 16; ++j) {
+        const uint32_t w = __shfl_sync(0xffffffffu, word, j);
+        const int c = __popc(w);
+        if (left >= 0 && left < c) {
+          l = (int)__fns(w, 0, left + 1);
+          n = c0 + j;
+        }
+        left -= c;
+      }
+      if (l < 0) continue;
+      const double2 *a = p.A + v2off(p.arv, p.ra + r0 + l), *b = p.B + v2off(p.brv, p.rb + n);
+      double re = 0.0, im = 0.0;
+#pragma unroll 2
+      for (int64_t k = p.k0; k < p.k1; ++k) {
+        const double2 x = a[v2off(p.akv, k)], z = b[v2off(p.bkv, k)];
+        re = fma(x.x, z.x, re);
+        re = fma(-x.y, z.y, re);
+        im = fma(x.x, z.y, im);
+        im = fma(x.y, z.x, im);
+      }
+      write(r0 + l, n, re, im);
+    }
+    return;
+  }
+  auto add_lanes = [](double &x) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+  };
+  if (p.k1 - p.k0 <= 1024) {
+    int turn = 0;
+    for (uint32_t c = __ballot_sync(0xffffffffu, word != 0); c; c &= c - 1) {
+      const int j = __ffs(c) - 1, n = c0 + j;
+      for (uint32_t w = __shfl_sync(0xffffffffu, word, j); w; w &= w - 1, ++turn) {
+        if ((turn & 7) != y) continue;
+        const int row = r0 + __ffs(w) - 1;
+        const double2 *a = p.A + v2off(p.arv, p.ra + row), *b = p.B + v2off(p.brv, p.rb + n);
+        double re = 0.0, im = 0.0;
+        for (int64_t k = p.k0 + lane; k < p.k1; k += 128) {
+          double2 x[4], z[4];
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            const bool in = k + 32 * q < p.k1;
+            x[q] = in ? a[v2off(p.akv, k + 32 * q)] : make_double2(0.0, 0.0);
+            z[q] = in ? b[v2off(p.bkv, k + 32 * q)] : make_double2(0.0, 0.0);
+          }
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            re = fma(x[q].x, z[q].x, re);
+            re = fma(-x[q].y, z[q].y, re);
+            im = fma(x[q].x, z[q].y, im);
+            im = fma(x[q].y, z[q].x, im);
+          }
+        }
+        add_lanes(re);
+        add_lanes(im);
+        if (lane == 0) write(row, n, re, im);
+      }
+    }
+    return;
+  }
+  for (uint32_t c = __ballot_sync(0xffffffffu, word != 0); c; c &= c - 1) {
+    const int j = __ffs(c) - 1, n = c0 + j;
+    const double2 *b = p.B + v2off(p.brv, p.rb + n);
+    uint32_t w = __shfl_sync(0xffffffffu, word, j);
+    while (w) {
+      const int rows = min(4, __popc(w));
+      int row[4];
+      const double2 *a[4];
+      double re[4] = {0.0, 0.0, 0.0, 0.0}, im[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        row[q] = w ? r0 + __ffs(w) - 1 : r0;
+        a[q] = p.A + v2off(p.arv, p.ra + row[q]);
+        w &= w - 1;
+      }
+      // (a block of the column is loaded under the sums of the one before, and one of zeros needs none of the rows)
+      double2 zn = p.k0 + thread < p.k1 ? b[v2off(p.bkv, p.k0 + thread)] : make_double2(0.0, 0.0);
+#pragma unroll 1
+      for (int64_t k0 = p.k0; k0 < p.k1; k0 += 256) {
+        const int64_t k = k0 + thread;
+        const double2 z = zn;
+        zn = k + 256 < p.k1 ? b[v2off(p.bkv, k + 256)] : make_double2(0.0, 0.0);
+        if (!__any_sync(0xffffffffu, nonzero(z))) continue;
+        const bool in = k < p.k1;
+        const int64_t ko = in ? v2off(p.akv, k) : 0;
+        double2 x[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) x[q] = in && q < rows ? a[q][ko] : make_double2(0.0, 0.0);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          int some = __any_sync(0xffffffffu, nonzero(x[q]) && nonzero(z));
+          asm volatile("" : "+r"(some));
+#pragma unroll 1
+          for (; some > 0; --some) {  // (a loop of at most one pass: as a condition it predicates the FMAs, which take the pipe)
+            re[q] = fma(x[q].x, z.x, re[q]);
+            re[q] = fma(-x[q].y, z.y, re[q]);
+            im[q] = fma(x[q].x, z.y, im[q]);
+            im[q] = fma(x[q].y, z.x, im[q]);
+          }
+        }
+      }
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        if (q >= rows) break;
+        add_lanes(re[q]);
+        add_lanes(im[q]);
+        if (lane == 0) {
+          part[y][2 * q] = re[q];
+          part[y][2 * q + 1] = im[q];
+        }
+      }
+      __syncthreads();
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        if (thread == q && q < rows) {
+          auto sum = [&](int i) {
+            return ((part[0][i] + part[1][i]) + (part[2][i] + part[3][i])) + ((part[4][i] + part[5][i]) + (part[6][i] + part[7][i]));
+          };
+          write(row[q], n, sum(2 * q), sum(2 * q + 1));
+        }
+      __syncthreads();
+    }
+  }
+}
+
 // The integer sums to FP64: a block takes 32 rows by 16 complex columns of a tile, reads the sums of every K
 // split along the rows (as the GEMM wrote them), adds them exactly, and writes C along its contiguous direction
 // (through shared memory when that is the columns).  This is a kernel of its own because the conversion is some
 // hundred dependent integer instructions per value: at the GEMM's eight warps per SM, with the accumulators
 // holding all registers, it took 50 us per tile, as long as the MMAs of K = 250.
 template <int BN>
-__global__ void __launch_bounds__(256) f64_out_kernel(F64Out p) {
+__global__ void __launch_bounds__(256, 4) f64_out_kernel(const __grid_constant__ F64Out p) {
   __shared__ double2 T[32][17];
   const int lane = threadIdx.x, y = threadIdx.y;
   int b = blockIdx.x;
@@ -516,14 +679,15 @@ __global__ void __launch_bounds__(256) f64_out_kernel(F64Out p) {
   if (r0 >= p.M || c0 >= p.N) return;
   const int row = r0 + lane;
   const int er = row < p.M ? scale_of(p.ea[row]) : 0;
+  const uint32_t finite = __ballot_sync(0xffffffffu, er < F64_NONFINITE / 2);
   const int64_t plane = (int64_t)p.nMt * p.nNt * BN * BM;
+  double2 v[2];
 #pragma unroll
   for (int q = 0; q < 2; ++q) {
     const int j = y + 8 * q, n = c0 + j;
     if (n < p.N) {
       const int64_t at = ((int64_t)tile * BN + cg * 32 + 2 * j) * BM + rg * 32 + lane;
       long long hr = 0, hm = 0;
-      double2 v;
       if (p.splits == 1) {
         hr = p.hi[at];
         hm = p.hi[at + BM];
@@ -542,38 +706,59 @@ __global__ void __launch_bounds__(256) f64_out_kernel(F64Out p) {
         lm = (float)im * 0x1p-16f;
       }
       const int e = er + scale_of(p.eb[n]);
-      v.x = combine(hr, lr, e + p.sh, p.neg);
-      v.y = combine(hm, lm, e + p.sh, p.neg);
-      if (!p.pow2) v = make_double2(p.ar * v.x - p.ai * v.y, p.ar * v.y + p.ai * v.x);
-      if (e >= F64_NONFINITE / 2) v.x = v.y = __longlong_as_double(0x7ff8000000000000ll);
-      if (p.cols_fast) {
-        T[lane][j] = v;
-      } else if (row < p.M) {
-        double2 *dst = (double2 *)p.C + v2off(p.rv, row) + v2off(p.cv, n);
-        if (p.accumulate) { const double2 o = *dst; v.x += o.x; v.y += o.y; }
-        *dst = v;
-      }
+      v[q].x = combine(hr, lr, e + p.sh, p.neg);
+      v[q].y = combine(hm, lm, e + p.sh, p.neg);
+      if (!p.pow2) v[q] = make_double2(p.ar * v[q].x - p.ai * v[q].y, p.ar * v[q].y + p.ai * v[q].x);
+      if (e >= F64_NONFINITE / 2) v[q].x = v[q].y = __longlong_as_double(0x7ff8000000000000ll);
+      if (p.cols_fast) T[lane][j] = v[q];
     }
   }
-  if (!p.cols_fast) return;
-  __syncthreads();
-  const int t = y * 32 + lane, j = t & 15, n = c0 + j;
-  if (n >= p.N) return;
-  const int64_t co = v2off(p.cv, n);
-#pragma unroll
-  for (int q = 0; q < 2; ++q) {
-    const int rl = (t >> 4) + 16 * q;
-    if (r0 + rl >= p.M) break;
-    double2 *dst = (double2 *)p.C + v2off(p.rv, r0 + rl) + co, v = T[rl][j];
-    if (p.accumulate) { const double2 o = *dst; v.x += o.x; v.y += o.y; }
-    *dst = v;
+  // the entries to be summed directly, written at the end (the words, of column c0 + lane, are used no earlier: the sums'
+  // loads should not wait for theirs)
+  uint32_t word = 0;
+  if (p.words) {
+    if (lane < 16 && c0 + lane < p.N) word = small_bits(__ldg(p.words + (int64_t)(mt * 4 + rg) * p.ldw + c0 + lane - p.n0));
+  } else {
+    const float2 *mine = p.sums + (int64_t)(row - p.m0) * p.ldw + c0 - p.n0;
+#pragma unroll 8
+    for (int j = 0; j < 16; ++j) {
+      const float2 s = c0 + j < p.N && row < p.M ? __ldg(mine + j) : make_float2(0.f, 0.f);
+      const uint32_t w = __ballot_sync(0xffffffffu, small_sum(s, p.tau));
+      if (lane == j) word = w;
+    }
   }
+  if (word) word = scale_of(p.eb[c0 + lane]) < F64_NONFINITE / 2 ? word & finite : 0u;
+  if (!p.cols_fast) {
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      const int n = c0 + y + 8 * q;
+      const uint32_t small = __shfl_sync(0xffffffffu, word, y + 8 * q);
+      if (n >= p.N || row >= p.M || (small >> lane & 1)) continue;
+      double2 *dst = (double2 *)p.C + v2off(p.rv, row) + v2off(p.cv, n);
+      if (p.accumulate) { const double2 o = *dst; v[q].x += o.x; v[q].y += o.y; }
+      *dst = v[q];
+    }
+  } else {
+    __syncthreads();
+    const int t = y * 32 + lane, j = t & 15, n = c0 + j;
+    const uint32_t small = __shfl_sync(0xffffffffu, word, j);
+    const int64_t co = n < p.N ? v2off(p.cv, n) : 0;
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      const int rl = (t >> 4) + 16 * q;
+      if (n >= p.N || r0 + rl >= p.M || (small >> rl & 1)) continue;
+      double2 *dst = (double2 *)p.C + v2off(p.rv, r0 + rl) + co, z = T[rl][j];
+      if (p.accumulate) { const double2 o = *dst; z.x += o.x; z.y += o.y; }
+      *dst = z;
+    }
+  }
+  if (__any_sync(0xffffffffu, word != 0)) write_small(p, word, r0, c0);
 }
 
 // The same for many K splits of a small C: a block takes 32 rows of one complex column, its eight warps share the
 // splits.
 template <int BN>
-__global__ void __launch_bounds__(256) f64_out_split_kernel(F64Out p) {
+__global__ void __launch_bounds__(256, 4) f64_out_split_kernel(const __grid_constant__ F64Out p) {
   __shared__ long long T[4][8][33];
   const int lane = threadIdx.x, y = threadIdx.y;
   int b = blockIdx.x;
@@ -582,6 +767,7 @@ __global__ void __launch_bounds__(256) f64_out_split_kernel(F64Out p) {
   const int rg = b % 4, tile = b / 4, mt = tile % p.nMt, nt = tile / p.nMt;
   const int row = p.m0 + mt * BM + rg * 32 + lane, n = p.n0 + nt * (BN / 2) + j;
   if (n >= p.N || p.m0 + mt * BM + rg * 32 >= p.M) return;
+  const int er = row < p.M ? scale_of(p.ea[row]) : 0;
   const int64_t plane = (int64_t)p.nMt * p.nNt * BN * BM, at = ((int64_t)tile * BN + 2 * j) * BM + rg * 32 + lane;
   long long t[4] = {0, 0, 0, 0};  // hi and lo 2^16, real and imaginary
 #pragma unroll 4
@@ -594,19 +780,30 @@ __global__ void __launch_bounds__(256) f64_out_split_kernel(F64Out p) {
 #pragma unroll
   for (int k = 0; k < 4; ++k) T[k][y][lane] = t[k];
   __syncthreads();
-  if (y != 0 || row >= p.M) return;
+  uint32_t small;
+  if (p.words) {
+    small = small_bits(__ldg(p.words + (int64_t)(mt * 4 + rg) * p.ldw + n - p.n0));
+  } else {
+    const float2 s = row < p.M ? __ldg(p.sums + (int64_t)(row - p.m0) * p.ldw + n - p.n0) : make_float2(0.f, 0.f);
+    small = __ballot_sync(0xffffffffu, small_sum(s, p.tau));
+  }
+  small &= __ballot_sync(0xffffffffu, er + scale_of(p.eb[n]) < F64_NONFINITE / 2);
+  if (y == 0 && row < p.M && !(small >> lane & 1)) {
 #pragma unroll
-  for (int k = 0; k < 4; ++k)
-    for (int q = 1; q < 8; ++q) t[k] += T[k][q][lane];
-  const int e = scale_of(p.ea[row]) + scale_of(p.eb[n]);
-  double2 v;
-  v.x = combine(t[0], (float)t[2] * 0x1p-16f, e + p.sh, p.neg);
-  v.y = combine(t[1], (float)t[3] * 0x1p-16f, e + p.sh, p.neg);
-  if (!p.pow2) v = make_double2(p.ar * v.x - p.ai * v.y, p.ar * v.y + p.ai * v.x);
-  if (e >= F64_NONFINITE / 2) v.x = v.y = __longlong_as_double(0x7ff8000000000000ll);
-  double2 *dst = (double2 *)p.C + v2off(p.rv, row) + v2off(p.cv, n);
-  if (p.accumulate) { const double2 o = *dst; v.x += o.x; v.y += o.y; }
-  *dst = v;
+    for (int k = 0; k < 4; ++k)
+      for (int q = 1; q < 8; ++q) t[k] += T[k][q][lane];
+    const int e = er + scale_of(p.eb[n]);
+    double2 v;
+    v.x = combine(t[0], (float)t[2] * 0x1p-16f, e + p.sh, p.neg);
+    v.y = combine(t[1], (float)t[3] * 0x1p-16f, e + p.sh, p.neg);
+    if (!p.pow2) v = make_double2(p.ar * v.x - p.ai * v.y, p.ar * v.y + p.ai * v.x);
+    if (e >= F64_NONFINITE / 2) v.x = v.y = __longlong_as_double(0x7ff8000000000000ll);
+    double2 *dst = (double2 *)p.C + v2off(p.rv, row) + v2off(p.cv, n);
+    if (p.accumulate) { const double2 o = *dst; v.x += o.x; v.y += o.y; }
+    *dst = v;
+  }
+  __syncwarp();
+  if (small) write_small(p, lane == 0 ? small : 0u, row - lane, n);
 }
 
 // ---------------- slices ----------------
@@ -635,9 +832,24 @@ __device__ __forceinline__ uint32_t digit(long long &X, int s) {
   return digit_bits(d, s);
 }
 
-// eight slices of one complex entry at real columns 2k, 2k+1 of slice row r (R rows per slice)
+// |x| 2^-e cut off to BF16 (bits); what is not zero counts as 2^-60 at least, so that its products stay above zero
+__device__ __forceinline__ uint32_t magnitude_bits(double x, int e) {
+  const uint32_t h = mag(x);
+  const int ex = (int)(h >> 20), b = ex - 1023 - e + 127;
+  return ex > 0 && b > 67 ? (uint32_t)b << 7 | ((h >> 13) & 0x7fu) : (h | (uint32_t)__double2loint(x)) ? 67u << 7 : 0u;
+}
+
+// eight slices and the magnitudes of one complex entry at real columns 2k, 2k+1 of slice row r (R rows per slice)
 template <bool EMBED>
 __device__ __forceinline__ void put_slices(uint32_t *dst, int64_t R, int64_t ld2, int64_t r, int64_t k, double2 z, int e) {
+  const uint32_t ax = magnitude_bits(z.x, e), ay = magnitude_bits(z.y, e);
+  if (EMBED) {
+    uint32_t *row = dst + ((int64_t)S * 2 * R + 2 * r) * ld2 + k;
+    row[0] = ax | (ay << 16);
+    row[ld2] = ay | (ax << 16);
+  } else {
+    dst[((int64_t)S * R + r) * ld2 + k] = ax | (ay << 16);
+  }
   long long X = fixed63(z.x, e), Y = fixed63(z.y, e);
   if (e == F64_NONFINITE) X = Y = 0;
 #pragma unroll
@@ -773,7 +985,7 @@ template <int BN, bool PAIR> constexpr size_t smem_bytes() {
 
 // one launch of the GEMM over the units of p (rows of A from p.rA, columns of B from p.rB), and its output
 template <int BN, bool PAIR>
-void launch(const F64Op &A, const F64Op &B, const F64Params &p, F64Out &o, int64_t K, cudaStream_t st) {
+void launch(const F64Op &A, const F64Op &B, const F64Params &p, F64Out &o, int64_t K, F64Side &side, cudaStream_t st) {
   static std::atomic<unsigned long long> attr_set{0};  // one bit per device
   constexpr int smem = (int)smem_bytes<BN, PAIR>();
   int dev = 0;
@@ -808,6 +1020,7 @@ void launch(const F64Op &A, const F64Op &B, const F64Params &p, F64Out &o, int64
   o.nMt = p.nMt;
   o.nNt = p.nNt;
   o.splits = p.splits;
+  side.join(st);
   if (p.splits > 8) f64_out_split_kernel<BN><<<(unsigned)(o.ntiles * 4 * (BN / 2)), dim3(32, 8), 0, st>>>(o);
   else f64_out_kernel<BN><<<(unsigned)(o.ntiles * 4 * (BN / 32)), dim3(32, 8), 0, st>>>(o);
   CCLR_CUDA(cudaGetLastError());
@@ -836,13 +1049,31 @@ F64Plan plan_of(int64_t M, int64_t N, size_t cap) {
 int64_t splits_of(int64_t all_tiles, int64_t units, int slots, int n) {
   return all_tiles > SPLIT_TILES ? 1 : std::max<int64_t>(1, std::min<int64_t>(slots / units, n / 2));
 }
-constexpr size_t SUMS_CAP = 256u << 20;  // the most that the sums of one launch take
+constexpr size_t SUMS_CAP = 240u << 20;  // the most that the integer sums of one launch take
 
 }  // namespace
 
+F64Side::~F64Side() {
+  if (s_) cudaStreamDestroy(s_);
+  if (fork_) cudaEventDestroy(fork_);
+  if (join_) cudaEventDestroy(join_);
+}
+cudaStream_t F64Side::fork(cudaStream_t st) {
+  if (!s_) CCLR_CUDA(cudaStreamCreateWithFlags(&s_, cudaStreamNonBlocking));
+  if (!fork_) CCLR_CUDA(cudaEventCreateWithFlags(&fork_, cudaEventDisableTiming));
+  if (!join_) CCLR_CUDA(cudaEventCreateWithFlags(&join_, cudaEventDisableTiming));
+  CCLR_CUDA(cudaEventRecord(fork_, st));
+  CCLR_CUDA(cudaStreamWaitEvent(s_, fork_, 0));
+  return s_;
+}
+void F64Side::join(cudaStream_t st) {
+  CCLR_CUDA(cudaEventRecord(join_, s_));
+  CCLR_CUDA(cudaStreamWaitEvent(st, join_, 0));
+}
+
 F64Op f64tc_prep(const void *src, View2 rv, View2 kv, int64_t R, int64_t K, bool embed, void *dst, uint32_t *tops,
                  cudaStream_t st) {
-  CCLR_REQUIRE(R > 0 && K > 0 && (int64_t)S * 2 * R < (1ll << 31) && 2 * K < (1ll << 31), "f64tc_prep: bad dimensions");
+  CCLR_REQUIRE(R > 0 && K > 0 && (int64_t)F64_PLANES * 2 * R < (1ll << 31) && 2 * K < (1ll << 31), "f64tc_prep: bad dimensions");
   if (embed) prep_launch<true>((const double2 *)src, rv, kv, R, K, (uint32_t *)dst, tops, st);
   else prep_launch<false>((const double2 *)src, rv, kv, R, K, (uint32_t *)dst, tops, st);
   CCLR_CUDA(cudaGetLastError());
@@ -850,6 +1081,9 @@ F64Op f64tc_prep(const void *src, View2 rv, View2 kv, int64_t R, int64_t K, bool
   op.p = dst;
   op.tops = tops;
   op.stride = R;
+  op.src = src;
+  op.rv = rv;
+  op.kv = kv;
   return op;
 }
 
@@ -857,14 +1091,18 @@ F64Op f64tc_prep(const void *src, View2 rv, View2 kv, int64_t R, int64_t K, bool
 // block or chunk serves the others: a launch takes no more tiles than there are and than SUMS_CAP holds, K splits
 // no more than one unit per SM, and the width of the tiles only grows with N.  (The need of the product itself
 // is not monotone: fewer rows of tiles leave room for more columns of them.)
+static size_t sums_bytes(const F64Plan &q) {
+  return (size_t)(std::max<int64_t>(std::min<int64_t>(tiles_that_fit(q.BN, SUMS_CAP), (int64_t)q.nMt * q.nNt), tc_num_sms()) * q.unit);
+}
+// (and behind them the words of a launch's tiles, or the sums that they stand for)
 size_t f64tc_scratch_bytes(int64_t M, int64_t N) {
   const F64Plan q = plan_of(M, N, SUMS_CAP);
-  const int64_t fit = tiles_that_fit(q.BN, SUMS_CAP);
-  return (size_t)(std::max<int64_t>(std::min<int64_t>(fit, (int64_t)q.nMt * q.nNt), tc_num_sms()) * q.unit);
+  const int64_t tiles = std::min<int64_t>(tiles_that_fit(q.BN, SUMS_CAP), (int64_t)q.nMt * q.nNt);
+  return sums_bytes(q) + (size_t)std::max<int64_t>(tiles * (BM / 32) * (q.BN / 2) * 16, std::min<int64_t>(M * 2 * N * 4, tc_magnitude_sums_cap()));
 }
 
 void f64tc_gemm(const F64Op &A, int64_t M, const F64Op &B, int64_t N, int64_t K, void *C, View2 rv, View2 cv, zc alpha,
-                bool accumulate, void *scratch, cudaStream_t st, UpperTiles *upper) {
+                bool accumulate, void *scratch, F64Side &side, cudaStream_t st, UpperTiles *upper) {
   if (M <= 0 || N <= 0 || K <= 0) return;
   CCLR_REQUIRE(A.r0 + M <= A.stride && B.r0 + N <= B.stride, "f64tc_gemm: rows outside the prepared operand");
   CCLR_REQUIRE((uintptr_t)A.p % 16 == 0 && (uintptr_t)B.p % 16 == 0, "f64tc_gemm: operands must be 16-byte aligned");
@@ -888,6 +1126,17 @@ void f64tc_gemm(const F64Op &A, int64_t M, const F64Op &B, int64_t N, int64_t K,
   o.pow2 = alpha.im == 0.0 && std::abs(std::frexp(alpha.re, &ex)) == 0.5;
   o.sh = o.pow2 ? ex - 1 : 0;
   o.neg = o.pow2 && alpha.re < 0.0;
+  o.A = (const double2 *)A.src;
+  o.B = (const double2 *)B.src;
+  o.ra = A.r0;
+  o.rb = B.r0;
+  o.arv = A.rv;
+  o.akv = A.kv;
+  o.brv = B.rv;
+  o.bkv = B.kv;
+  o.tau = (float)std::sqrt(2.0 * (double)K) * 0x1p-8f;
+  const int64_t ld = f64tc_ld(K);
+  void *small = (char *)scratch + sums_bytes(pl);
   const int nk = (int)((2 * K + KC - 1) / KC);
   p.K = (int)(2 * K);
   for (int t0 = 0; t0 < pl.nNt; t0 += pl.cols)
@@ -918,6 +1167,15 @@ void f64tc_gemm(const F64Op &A, int64_t M, const F64Op &B, int64_t N, int64_t K,
           o.ntiles = (int)tiles;
         }
       }
+      {
+        const int64_t mm = std::min<int64_t>(M - o.m0, (int64_t)p.nMt * BM);
+        o.ldw = std::min<int64_t>(N - o.n0, (int64_t)p.nNt * (pl.BN / 2));
+        const bool words = tc_magnitude_sums((const char *)A.p + ((int64_t)S * p.sA + p.rA) * ld * 2, ld,
+                                             (const char *)B.p + ((int64_t)S * p.sB + p.rB) * ld * 2, ld, mm, 2 * o.ldw, 2 * K, o.tau,
+                                             small, side.fork(st));
+        o.words = words ? (const uint4 *)small : nullptr;
+        o.sums = (const float2 *)small;
+      }
       // segments of K that the integer sums can hold, one launch each
       for (p.chunk0 = 0; p.chunk0 < nk; p.chunk0 += MAX_CHUNKS) {
         p.chunk1 = std::min(nk, p.chunk0 + MAX_CHUNKS);
@@ -928,9 +1186,11 @@ void f64tc_gemm(const F64Op &A, int64_t M, const F64Op &B, int64_t N, int64_t K,
         p.hi = (long long *)scratch;
         p.lo = (float *)(p.hi + tiles * p.splits * BM * pl.BN);
         o.accumulate = accumulate || p.chunk0 > 0;
-        if (pl.BN == 32) launch<32, false>(A, B, p, o, K, st);
-        else if (pl.BN == 64) launch<64, false>(A, B, p, o, K, st);
-        else launch<128, true>(A, B, p, o, K, st);
+        o.k0 = (int64_t)p.chunk0 * (KC / 2);
+        o.k1 = std::min<int64_t>(K, (int64_t)p.chunk1 * (KC / 2));
+        if (pl.BN == 32) launch<32, false>(A, B, p, o, K, side, st);
+        else if (pl.BN == 64) launch<64, false>(A, B, p, o, K, side, st);
+        else launch<128, true>(A, B, p, o, K, side, st);
       }
     }
 }

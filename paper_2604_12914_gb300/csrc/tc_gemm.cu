@@ -16,6 +16,7 @@
 #include <map>
 #include <mutex>
 #include <tuple>
+#include <type_traits>
 #include <vector>
 
 #include "engine.cuh"
@@ -43,6 +44,8 @@ struct TcParams {
   int accumulate;       // add to C (always true when split)
   int atomic;           // split-K: combine partial tiles with atomicAdd
   int *err;
+  float tau;            // the kernels that compare their sums instead of storing them (tc_magnitude_sums)
+  uint32_t *words;
 };
 
 // work unit -> (m tile, n tile, split); banded rasterisation: consecutive units share one B
@@ -185,7 +188,28 @@ __device__ __forceinline__ void store16(const TcParams &p, const uint32_t (&r)[1
     if (dst[k]) *reinterpret_cast<float2 *>(dst[k]) = val[k];
 }
 
-template <int KIND>
+// The same chunk compared with p.tau instead (tc_magnitude_sums): a column of 32 sums makes one word per ballot, and lane
+// 4 c + k stores word k of complex column c.
+__device__ __forceinline__ void check16(const TcParams &p, const uint32_t (&r)[16], int row0, int lane, int n1) {
+  uint32_t w = 0;
+#pragma unroll
+  for (int k = 0; k < 16; ++k) {
+    const float s = __uint_as_float(r[k]);
+    const uint32_t reach = __ballot_sync(0xffffffffu, s >= p.tau), some = __ballot_sync(0xffffffffu, s != 0.f);
+    if (lane == 4 * (k >> 1) + (k & 1)) w = reach;
+    if (lane == 4 * (k >> 1) + 2 + (k & 1)) w = some;
+  }
+  const int col = (n1 >> 1) + (lane >> 2);
+  if (row0 >= p.M || 2 * col >= p.N) return;
+  p.words[4 * ((int64_t)(row0 >> 5) * (p.N >> 1) + col) + (lane & 3)] = w;
+}
+struct NoRows {
+  __device__ __forceinline__ NoRows(const TcParams &, int, int) {}
+};
+template <bool CHECK> using Rows = std::conditional_t<CHECK, NoRows, RowPtrs>;
+
+// CHECK: the sums are compared (check16), not stored
+template <int KIND, bool CHECK>
 __global__ void __launch_bounds__(320, 1)
     tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                    TcParams p) {
@@ -308,7 +332,7 @@ __global__ void __launch_bounds__(320, 1)
       int mt, nt, sp;
       unit_coords(p, u, mt, nt, sp);
       const int buf = it & 1;
-      const RowPtrs rows(p, mt * BM + q * 32, lane);
+      const Rows<CHECK> rows(p, mt * BM + q * 32, lane);
       bool ok = mbar_wait_ab(su32(tfull + buf), (uint32_t)(it >> 1) & 1u, p.err, abort_flag);
       ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
       if (!ok) break;
@@ -330,7 +354,8 @@ __global__ void __launch_bounds__(320, 1)
           __syncwarp();
           if (lane == 0) mbar_arrive(su32(tempty + buf));
         }
-        store16(p, r, stg, rows, lane, n0 + c0);
+        if constexpr (CHECK) check16(p, r, mt * BM + q * 32, lane, n0 + c0);
+        else store16(p, r, stg, rows, lane, n0 + c0);
       }
     }
   }
@@ -353,7 +378,7 @@ __global__ void __launch_bounds__(320, 1)
 // 25600 x 2560 x 800 849 and 1063.
 constexpr int PAIR_STAGES = 6;
 
-template <int KIND>
+template <int KIND, bool CHECK>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(320, 1)
     tc_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, TcParams p) {
   extern __shared__ uint8_t smem_raw[];
@@ -476,7 +501,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(320, 1)
       int mt, nt, sp;
       unit_coords(p, u, mt, nt, sp);
       const int buf = it & 1;
-      const RowPtrs rows(p, (2 * mt + (int)rank) * BM + q * 32, lane);
+      const Rows<CHECK> rows(p, (2 * mt + (int)rank) * BM + q * 32, lane);
       bool ok = mbar_wait_ab(su32(tfull + buf), (uint32_t)(it >> 1) & 1u, p.err, abort_flag);
       ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
       if (!ok) break;
@@ -492,7 +517,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(320, 1)
           __syncwarp();
           if (lane == 0) mbar_arrive_cluster(pair_addr(su32(tempty + buf), 0));
         }
-        store16(p, r, stg, rows, lane, n0 + c0);
+        if constexpr (CHECK) check16(p, r, (2 * mt + (int)rank) * BM + q * 32, lane, n0 + c0);
+        else store16(p, r, stg, rows, lane, n0 + c0);
       }
     }
   }
@@ -783,10 +809,12 @@ int current_device() {
 
 // raises the dynamic shared-memory limit of every kernel instantiation on the current device
 void set_smem_limits() {
-  CCLR_CUDA(cudaFuncSetAttribute(tc_gemm_kernel<TC_TF32>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
-  CCLR_CUDA(cudaFuncSetAttribute(tc_gemm_kernel<TC_BF16>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
-  CCLR_CUDA(cudaFuncSetAttribute(tc_pair_kernel<TC_TF32>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
-  CCLR_CUDA(cudaFuncSetAttribute(tc_pair_kernel<TC_BF16>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
+  CCLR_CUDA(cudaFuncSetAttribute(tc_gemm_kernel<TC_TF32, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
+  CCLR_CUDA(cudaFuncSetAttribute(tc_gemm_kernel<TC_BF16, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
+  CCLR_CUDA(cudaFuncSetAttribute(tc_pair_kernel<TC_TF32, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
+  CCLR_CUDA(cudaFuncSetAttribute(tc_pair_kernel<TC_BF16, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
+  CCLR_CUDA(cudaFuncSetAttribute(tc_gemm_kernel<TC_BF16, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
+  CCLR_CUDA(cudaFuncSetAttribute(tc_pair_kernel<TC_BF16, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
   CCLR_CUDA(cudaFuncSetAttribute(tc_split_kernel<TC_TF32>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
   CCLR_CUDA(cudaFuncSetAttribute(tc_split_kernel<TC_BF16>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
 }
@@ -1052,10 +1080,10 @@ static void tc_launch(const void *A, int64_t lda, const void *B, int64_t ldb, in
     const size_t smem = 1024 + (cfg.pair ? (size_t)PAIR_STAGES * (BM + BN / 2) : (size_t)STAGES * (BM + BN)) * BKB + epi;
     if (cfg.pair) {
       const unsigned pairs = (unsigned)std::min<int64_t>(units, std::max(nsm / 2, 1));
-      if (kind == TC_BF16) tc_pair_kernel<TC_BF16><<<2 * pairs, 320, smem, st>>>(ma, mb, p);
-      else tc_pair_kernel<TC_TF32><<<2 * pairs, 320, smem, st>>>(ma, mb, p);
-    } else if (kind == TC_BF16) tc_gemm_kernel<TC_BF16><<<grid, 320, smem, st>>>(ma, mb, p);
-    else tc_gemm_kernel<TC_TF32><<<grid, 320, smem, st>>>(ma, mb, p);
+      if (kind == TC_BF16) tc_pair_kernel<TC_BF16, false><<<2 * pairs, 320, smem, st>>>(ma, mb, p);
+      else tc_pair_kernel<TC_TF32, false><<<2 * pairs, 320, smem, st>>>(ma, mb, p);
+    } else if (kind == TC_BF16) tc_gemm_kernel<TC_BF16, false><<<grid, 320, smem, st>>>(ma, mb, p);
+    else tc_gemm_kernel<TC_TF32, false><<<grid, 320, smem, st>>>(ma, mb, p);
   }
   count_launch();
   CCLR_CUDA(cudaGetLastError());
@@ -1066,6 +1094,52 @@ static void tc_launch(const void *A, int64_t lda, const void *B, int64_t ldb, in
     used->pair = cfg.pair;
   }
 }
+
+// Tiles as wide as 256 columns, by pairs of CTAs from 129 rows and 128 columns on; K in parts of at least four blocks where
+// the tiles leave half the SMs idle.
+bool tc_magnitude_sums(const void *A, int64_t lda, const void *B, int64_t ldb, int64_t M, int64_t Nreal, int64_t Kreal, float tau,
+                       void *out, cudaStream_t st) {
+  CCLR_REQUIRE(Nreal % 2 == 0 && lda % 8 == 0 && ldb % 8 == 0 && (uintptr_t)A % 16 == 0 && (uintptr_t)B % 16 == 0,
+               "tc_magnitude_sums: operands must be whole 16-byte units");
+  const int nsm = num_sms(), nk = (int)((Kreal + BKB / 2 - 1) / (BKB / 2));
+  TcCfg cfg;
+  cfg.pair = M > BM && Nreal >= 128;
+  const int step = cfg.pair ? 32 : 16, rows = cfg.pair ? 2 * BM : BM, slots = cfg.pair ? std::max(nsm / 2, 1) : nsm;
+  cfg.BN = (int)std::min<int64_t>(256, (Nreal + step - 1) / step * step);
+  const int64_t tiles = ((M + rows - 1) / rows) * ((Nreal + cfg.BN - 1) / cfg.BN);
+  cfg.splits = 2 * tiles <= slots ? std::max(1, std::min((int)(slots / tiles), nk / 4)) : 1;
+  if (cfg.splits > 1) {
+    tc_launch(A, lda, B, ldb, M, Nreal, Kreal, TC_BF16, false, (float *)out, view1(Nreal / 2), view1(1), zc(1.0), false,
+              device_err(), st, -1, cfg, nullptr, nullptr);
+    return false;
+  }
+  TcParams p = {};
+  p.M = (int)M;
+  p.N = (int)Nreal;
+  p.K = (int)Kreal;
+  p.BN = cfg.BN;
+  p.nMt = (int)((M + rows - 1) / rows);
+  p.nNt = (int)((Nreal + cfg.BN - 1) / cfg.BN);
+  p.band = std::min(p.nMt, 20 * BM / rows);
+  p.ntiles = (int)tiles;
+  p.splits = 1;
+  p.kb_per_split = nk;
+  p.err = device_err();
+  p.tau = tau;
+  p.words = (uint32_t *)out;
+  const CUtensorMap ma = make_map(A, M, Kreal, lda, BM, BKB, TC_BF16);
+  const CUtensorMap mb = make_map(B, Nreal, Kreal, ldb, cfg.pair ? cfg.BN / 2 : cfg.BN, BKB, TC_BF16);
+  const size_t smem = 1024 + (cfg.pair ? (size_t)PAIR_STAGES * (BM + cfg.BN / 2) : (size_t)STAGES * (BM + cfg.BN)) * BKB +
+                      (size_t)8 * 32 * EPI_PITCH * 4 + (2 * PAIR_STAGES + 5) * 8 + 16;
+  const unsigned grid = (unsigned)std::min<int64_t>(tiles, slots);
+  if (cfg.pair) tc_pair_kernel<TC_BF16, true><<<2 * grid, 320, smem, st>>>(ma, mb, p);
+  else tc_gemm_kernel<TC_BF16, true><<<grid, 320, smem, st>>>(ma, mb, p);
+  count_launch();
+  CCLR_CUDA(cudaGetLastError());
+  return true;
+}
+// (2 tiles <= slots, tiles of 128 x 256 floats per SM)
+int64_t tc_magnitude_sums_cap() { return (int64_t)num_sms() / 2 * BM * 256 * 4; }
 
 // Candidate configurations around the rule's choice: other tile widths for wide outputs (each with its own best
 // number of splits), more or fewer K splits, and the two extreme raster bands.

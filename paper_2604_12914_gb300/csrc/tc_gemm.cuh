@@ -188,6 +188,15 @@ void tc_gemm_seg_v(const void *A, int64_t lda, const void *B, int64_t ldb, int64
                    int seg, int kind, float *C, View2 rv, View2 cv, zc alpha, bool accumulate, cudaStream_t st,
                    UpperTiles *upper = nullptr);
 
+// The sums s(m, n) of A B^T over nonnegative BF16 rows (Nreal rows of B: the real and the imaginary part of Nreal / 2
+// complex columns), compared with tau: true, and out holds four words for every 32 rows and complex column, at
+// 4 ((m / 32) (Nreal / 2) + n / 2), bit m % 32 of which says whether the real part reaches tau, whether the imaginary part
+// does, whether the real part is other than zero, whether the imaginary part is.  Where the tiles leave half the SMs idle
+// K is split and out holds the sums themselves, [M][Nreal] floats of at most tc_magnitude_sums_cap() bytes: false.
+bool tc_magnitude_sums(const void *A, int64_t lda, const void *B, int64_t ldb, int64_t M, int64_t Nreal, int64_t Kreal, float tau,
+                       void *out, cudaStream_t st);
+int64_t tc_magnitude_sums_cap();
+
 // Tile autotuner: while on (per host thread), the first use of a GEMM shape (operand kind, M,
 // real N, real K, epilogue layout) on a device times a handful of launch configurations (tile
 // width, K splits, raster band) around the rules' choice and caches the fastest for that shape
