@@ -78,6 +78,11 @@ int cc_lr_selftest_gemm_noalloc(int M, int N, int K, int mode, unsigned seed, do
  * should not be, or not NaN where they should.  Returns 0 on success, else a cclr_status code. */
 int cc_lr_selftest_f64gemm(int M, int N, int K, int layout, double spread, unsigned seed, double *out);
 
+/* One constant complex128 operand, its slices kept, in two contractions whose results are laid out differently, so that
+ * they cut it into other chunks; the second one under a memory budget that leaves no room for more slices.  err[0], err[1]:
+ * the largest error of each against host sums, over the largest entry. */
+int cc_lr_selftest_f64_kept(unsigned seed, double *err);
+
 /* Device bytes that the FP64 tensor-core GEMM's callers claim for its sums before M x N products (no device call). */
 int cc_lr_selftest_f64_scratch(long long M, long long N, unsigned long long *bytes);
 

@@ -94,6 +94,7 @@ def load(path: str = LIB_PATH):
         "cc_lr_bench_hbm": [I, I, I, P, I],
         "cc_lr_selftest_timeout": [I, ctypes.POINTER(ctypes.c_int)],
         "cc_lr_selftest_f64gemm": [I, I, I, I, D, ctypes.c_uint, P],
+        "cc_lr_selftest_f64_kept": [ctypes.c_uint, P],
         "cc_lr_selftest_f64_scratch": [ctypes.c_longlong, ctypes.c_longlong, ctypes.POINTER(ctypes.c_ulonglong)],
         "cc_lr_selftest_precond": [I, D, D, ctypes.c_uint, ctypes.POINTER(ctypes.c_double)],
     }
@@ -425,6 +426,13 @@ def cc_lr_selftest_f64gemm(M, N, K, layout=0, spread=0.0, seed=1):
     """(largest error over its bound, misplaced NaNs) of the FP64 tensor-core GEMM (include/cclr_testing.h)."""
     out = np.zeros(2, dtype=np.float64)
     _check(load().cc_lr_selftest_f64gemm(M, N, K, layout, float(spread), seed, _ptr(out)))
+    return float(out[0]), float(out[1])
+
+
+def cc_lr_selftest_f64_kept(seed=1):
+    """Errors of two contractions of one kept constant in different chunks (include/cclr_testing.h)."""
+    out = np.zeros(2, dtype=np.float64)
+    _check(load().cc_lr_selftest_f64_kept(seed, _ptr(out)))
     return float(out[0]), float(out[1])
 
 

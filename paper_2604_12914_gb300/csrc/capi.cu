@@ -1957,6 +1957,58 @@ int cc_lr_selftest_f64gemm(int M, int N, int K, int layout, double spread, unsig
   });
 }
 
+int cc_lr_selftest_f64_kept(unsigned seed, double *err) {
+  if (!err) return fail(CCLR_EINVAL, "bad selftest_f64_kept arguments");
+  return guarded([&] {
+    // A[w][p][x][q][y] constant, contracted over (p, q) with B[p][q][n] into C[w][x][y][n], then into C[w][n][x][y]: slices in
+    // chunks of 60 rows (w, x, y) the first time, and of whole (x, y) blocks of 120 the second
+    const int64_t W = 2, P = 10, X = 10, Q = 12, Y = 12, N = 70, nA = W * P * X * Q * Y, nB = P * Q * N, nC = W * X * Y * N;
+    std::mt19937_64 g(seed);
+    std::normal_distribution<double> nd(0.0, 1.0);
+    std::vector<zd> a(nA), b(nB), ref(nC), c(nC);
+    for (auto &z : a) z = zd(nd(g), nd(g));
+    for (auto &z : b) z = zd(nd(g), nd(g));
+    for (int64_t w = 0; w < W; ++w)
+      for (int64_t x = 0; x < X; ++x)
+        for (int64_t y = 0; y < Y; ++y)
+          for (int64_t p = 0; p < P; ++p)
+            for (int64_t q = 0; q < Q; ++q)
+              for (int64_t n = 0; n < N; ++n)
+                ref[((w * X + x) * Y + y) * N + n] += a[(((w * P + p) * X + x) * Q + q) * Y + y] * b[(p * Q + q) * N + n];
+    MemAcct acct;
+    AcctScope scope(&acct);
+    Engine E;
+    CCLR_CUDA(cudaStreamCreate(&E.st));
+    DevBuf Ad(nA * 16), Bd(nB * 16), Cd(nC * 16);
+    CCLR_CUDA(cudaMemcpyAsync(Ad.p, a.data(), Ad.bytes, cudaMemcpyHostToDevice, E.st));
+    CCLR_CUDA(cudaMemcpyAsync(Bd.p, b.data(), Bd.bytes, cudaMemcpyHostToDevice, E.st));
+    const Tens At = make_tens(Ad.p, C128, {W, P, X, Q, Y}), Bt = make_tens(Bd.p, C128, {P, Q, N});
+    const Tens C1 = make_tens(Cd.p, C128, {W, X, Y, N}), C2 = make_tens(Cd.p, C128, {W, N, X, Y});
+    for (int s = 0; s < 3; ++s) E.ws(s, (size_t)std::max(nA, nC) * 16);  // what the CUDA cores would need
+    E.f64_scratch(W * X * Y, N);
+    E.f64_cache_cap = (size_t)1 << 30;
+    E.f64_operand_cap = 60 * f64tc_bytes(1, P * Q, false);
+    E.cst_hint = Ad.p;
+    double mx = 0.0;
+    for (const auto &z : ref) mx = std::max(mx, std::abs(z));
+    for (int k = 0; k < 2; ++k) {
+      E.zero(C1);
+      E.contract(zc(1), At, "wpxqy", Bt, "pqn", k == 0 ? C1 : C2, k == 0 ? "wxyn" : "wnxy");
+      CCLR_CUDA(cudaMemcpyAsync(c.data(), Cd.p, Cd.bytes, cudaMemcpyDeviceToHost, E.st));
+      CCLR_CUDA(cudaStreamSynchronize(E.st));
+      E.check_tc();
+      err[k] = 0.0;
+      for (int64_t w = 0; w < W; ++w)
+        for (int64_t xy = 0; xy < X * Y; ++xy)
+          for (int64_t n = 0; n < N; ++n)
+            err[k] = std::max(err[k], std::abs(c[k == 0 ? (w * X * Y + xy) * N + n : (w * N + n) * X * Y + xy] -
+                                               ref[(w * X * Y + xy) * N + n]) / mx);
+      acct.budget = acct.used;  // the second one finds no room for more slices
+    }
+    CCLR_CUDA(cudaStreamDestroy(E.st));
+  });
+}
+
 int cc_lr_selftest_f64_scratch(long long M, long long N, unsigned long long *bytes) {
   if (M < 1 || N < 1 || !bytes) return fail(CCLR_EINVAL, "bad selftest_f64_scratch arguments");
   *bytes = f64tc_scratch_bytes(M, N);

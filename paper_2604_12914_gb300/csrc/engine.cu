@@ -555,8 +555,8 @@ bool Engine::contract_f64(zc alpha, const Tens &A, const std::string &ma, const 
     if (y.din != TC_ONE_LEVEL) u = std::lcm(u, y.din);
     return u;
   };
-  auto chunk = [](int64_t n, int64_t per, int64_t u) {
-    const int64_t cap = (2ll << 30) / per;
+  auto chunk = [&](int64_t n, int64_t per, int64_t u) {
+    const int64_t cap = f64_operand_cap / per;
     return n > cap && u < n ? std::max(u, cap / u * u) : n;
   };
   const int64_t Mc = chunk(M, f64tc_bytes(1, K, false), unit_of(am, cm)), Nc = chunk(N, f64tc_bytes(1, K, true), unit_of(bn, cn));
@@ -570,8 +570,9 @@ bool Engine::contract_f64(zc alpha, const Tens &A, const std::string &ma, const 
     if (cst_hint == A.p) akey = std::string("A") + hint + ma + "|" + bat + "|" + Mm + "|" + Km + "|";
     else bkey = std::string("B") + hint + mb + "|" + bat + "|" + Km + "|" + Nm + "|";
   }
-  auto at = [](const std::string &key, int64_t b, int64_t r) {
-    return key.empty() ? key : key + std::to_string(b) + "," + std::to_string(r);
+  // a chunk by its batch, first row and length (which follow C's layout too, not the operand's alone)
+  auto at = [](const std::string &key, int64_t b, int64_t r, int64_t len) {
+    return key.empty() ? key : key + std::to_string(b) + "," + std::to_string(r) + "+" + std::to_string(len);
   };
   // kept slices need no workspace
   auto have = [&](const std::string &key, int64_t n, int64_t step) {
@@ -579,7 +580,7 @@ bool Engine::contract_f64(zc alpha, const Tens &A, const std::string &ma, const 
     for (int64_t b = 0; b < nb; ++b)
       for (int64_t r = 0; r < n; r += step) {
         bool f = false;
-        for (auto &x : f64_kept_) f = f || (x->key == at(key, b, r) && x->filled);
+        for (auto &x : f64_kept_) f = f || (x->key == at(key, b, r, std::min(step, n - r)) && x->filled);
         if (!f) return false;
       }
     return true;
@@ -624,10 +625,10 @@ bool Engine::contract_f64(zc alpha, const Tens &A, const std::string &ma, const 
     char *Cb = (char *)(direct ? C.p : T.p) + b * c0 * es;
     for (int64_t n0 = 0; n0 < N; n0 += Nc) {
       const int64_t nn = std::min(Nc, N - n0);
-      const F64Op ob = f64_operand(1, (const char *)Bp + (b * b0 + v2off(bn, n0)) * es, bn, bk, nn, K, true, at(bkey, b, n0));
+      const F64Op ob = f64_operand(1, (const char *)Bp + (b * b0 + v2off(bn, n0)) * es, bn, bk, nn, K, true, at(bkey, b, n0, nn));
       for (int64_t m0 = 0; m0 < M; m0 += Mc) {
         const int64_t mm = std::min(Mc, M - m0);
-        const F64Op oa = f64_operand(0, (const char *)Ap + (b * a0 + v2off(am, m0)) * es, am, ak, mm, K, false, at(akey, b, m0));
+        const F64Op oa = f64_operand(0, (const char *)Ap + (b * a0 + v2off(am, m0)) * es, am, ak, mm, K, false, at(akey, b, m0, mm));
         f64_gemm(oa, mm, ob, nn, K, Cb + (v2off(cm, m0) + v2off(cn, n0)) * es, cm, cn, alpha, true);
       }
     }

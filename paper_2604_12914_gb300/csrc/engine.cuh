@@ -132,6 +132,7 @@ class Engine {
   // claims workspace slot `slot` for R rows of K entries.  Throws status 2.
   void f64_reserve(int slot, int64_t R, int64_t K, bool embed);
   size_t f64_cache_cap = 0;
+  int64_t f64_operand_cap = 2ll << 30;  // bytes of one operand's slices in contract_f64: in chunks above that
   // Holds off f64_reclaim() while prepared slices are in use on the host side.
   struct F64Hold {
     Engine &e;
