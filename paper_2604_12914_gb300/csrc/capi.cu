@@ -816,13 +816,25 @@ struct cclr_ctx {
   // ---- ground-state CCSD: the amplitude equations Omega(T) = 0 and the energy (Sec. 2.2) ----
   CstSet gs;  // intermediates at s T, s a quadrature node of the residual (scratch)
   // amplitudes, residual and product of a residual call, and the energy's effective doubles: kept for the next call up to
-  // 64 MB each, outside budgeted contexts
+  // 64 MB each, outside budgeted contexts (GsScope)
   AVec gv[3];
   DevBuf gtau;
   void release_gs_vectors() {
     for (auto &b : gv) b.b.release();
     gtau.release();
   }
+  // Ends a ground-state call, one that throws too: a budgeted context keeps nothing of it, others no vector above 64 MB.
+  struct GsScope {
+    cclr_ctx &c;
+    ~GsScope() {
+      if (c.M->lean) {
+        c.M->release_set(c.gs);
+        c.release_scratch();
+      } else if ((size_t)c.ntot() * 16 > (64u << 20)) {
+        c.release_gs_vectors();
+      }
+    }
+  };
 
   // the arithmetic of a ground-state product: a cclr_prec, or -1 for the context's own
   int gs_prec(int p) const {
@@ -1658,6 +1670,7 @@ cclr_status cc_lr_ccsd_residual(cclr_ctx *c, int prec, const double *t1, const d
   if (!c || !t1 || !t2 || !r1 || !r2) return (cclr_status)fail(CCLR_EINVAL, "bad ccsd_residual arguments");
   return (cclr_status)guarded_ctx(c, [&] {
     const int p = c->gs_prec(prec);
+    cclr_ctx::GsScope scope{*c};
     c->alloc_full(c->fullB);
     AVec &tv = c->gv[0], &rv = c->gv[1];
     c->alloc_vec(tv);
@@ -1676,8 +1689,6 @@ cclr_status cc_lr_ccsd_residual(cclr_ctx *c, int prec, const double *t1, const d
     from_dev(c, c->fullA.p2(c->n1), r2, (size_t)c->n2 * 16);
     CCLR_CUDA(cudaStreamSynchronize(c->st));
     c->M->retire_set(c->gs);
-    if (c->M->lean) c->release_scratch();
-    else if ((size_t)c->ntot() * 16 > (64u << 20)) c->release_gs_vectors();
   });
 }
 
@@ -1687,6 +1698,7 @@ cclr_status cc_lr_ccsd(cclr_ctx *c, int prec, double tol, int max_iterations, in
   bool conv = false;
   int st = guarded_ctx(c, [&] {
     const int p = c->gs_prec(prec);
+    cclr_ctx::GsScope scope{*c};
     AVec tv;
     int its = 0;
     const double rn = c->ccsd_solve(p, tol, max_iterations, diis_depth, tv, &its);
@@ -1699,7 +1711,6 @@ cclr_status cc_lr_ccsd(cclr_ctx *c, int prec, double tol, int max_iterations, in
     }
     if (res_norm) *res_norm = rn;
     if (iterations) *iterations = its;
-    if (c->M->lean) c->release_scratch();
   });
   if (st == CCLR_OK && !conv) return (cclr_status)fail(CCLR_ENOCONV, "ground-state CCSD did not reach the tolerance");
   return (cclr_status)st;
