@@ -78,6 +78,11 @@ int cc_lr_selftest_gemm_noalloc(int M, int N, int K, int mode, unsigned seed, do
  * should not be, or not NaN where they should.  Returns 0 on success, else a cclr_status code. */
 int cc_lr_selftest_f64gemm(int M, int N, int K, int layout, double spread, unsigned seed, double *out);
 
+/* The 16 x 16 tiles of (e, f), e < f < v, that the tensor-core ladder reads to pack the pairs q0 .. q0 + nq - 1 (numbered row
+ * by row): out[0] those read, out[1] those that hold one of the pairs, out[2] those that hold one and are not read (no
+ * device call). */
+int cc_lr_selftest_pack_tiles(int v, long long q0, long long nq, long long *out);
+
 /* One constant complex128 operand, its slices kept, in two contractions whose results are laid out differently, so that
  * they cut it into other chunks; the second one under a memory budget that leaves no room for more slices.  err[0], err[1]:
  * the largest error of each against host sums, over the largest entry. */

@@ -94,6 +94,7 @@ def load(path: str = LIB_PATH):
         "cc_lr_bench_hbm": [I, I, I, P, I],
         "cc_lr_selftest_timeout": [I, ctypes.POINTER(ctypes.c_int)],
         "cc_lr_selftest_f64gemm": [I, I, I, I, D, ctypes.c_uint, P],
+        "cc_lr_selftest_pack_tiles": [I, ctypes.c_longlong, ctypes.c_longlong, P],
         "cc_lr_selftest_f64_kept": [ctypes.c_uint, P],
         "cc_lr_selftest_f64_scratch": [ctypes.c_longlong, ctypes.c_longlong, ctypes.POINTER(ctypes.c_ulonglong)],
         "cc_lr_selftest_precond": [I, D, D, ctypes.c_uint, ctypes.POINTER(ctypes.c_double)],
@@ -427,6 +428,13 @@ def cc_lr_selftest_f64gemm(M, N, K, layout=0, spread=0.0, seed=1):
     out = np.zeros(2, dtype=np.float64)
     _check(load().cc_lr_selftest_f64gemm(M, N, K, layout, float(spread), seed, _ptr(out)))
     return float(out[0]), float(out[1])
+
+
+def cc_lr_selftest_pack_tiles(v, q0, nq):
+    """(tiles read, tiles that hold a pair, tiles missed) of the ladder's packing of a chunk of pairs."""
+    out = np.zeros(3, dtype=np.int64)
+    _check(load().cc_lr_selftest_pack_tiles(v, q0, nq, _ptr(out)))
+    return tuple(int(k) for k in out)
 
 
 def cc_lr_selftest_f64_kept(seed=1):

@@ -1968,6 +1968,15 @@ int cc_lr_selftest_f64gemm(int M, int N, int K, int layout, double spread, unsig
   });
 }
 
+int cc_lr_selftest_pack_tiles(int v, long long q0, long long nq, long long *out) {
+  if (v < 2 || q0 < 0 || nq < 1 || q0 + nq > (long long)v * (v - 1) / 2 || !out)
+    return fail(CCLR_EINVAL, "bad selftest_pack_tiles arguments");
+  int64_t t[3];
+  ladder_pack_tiles(v, q0, nq, t);
+  for (int k = 0; k < 3; ++k) out[k] = t[k];
+  return CCLR_OK;
+}
+
 int cc_lr_selftest_f64_kept(unsigned seed, double *err) {
   if (!err) return fail(CCLR_EINVAL, "bad selftest_f64_kept arguments");
   return guarded([&] {

@@ -55,8 +55,19 @@ __global__ void pack_y_a(const float2 *Y, int o, int v, const int2 *op, const in
 // A block takes one a, PW values of b and a PW x PW tile of (e, f), e-tile <= f-tile: both images are read along
 // their rows (whole 128-byte lines, 32 of them in flight per thread), one is turned around through shared memory,
 // and the result is written along q (mode 0) or, turned again, along r (mode 1), in 128-byte runs.  HBM-bound: W is
-// read once and the block written once.
+// read once and the block written once, also where the pairs go in several chunks: a tile without a pair of the chunk is
+// left before its loads (o=56 v=480, two and four chunks: ladder TF32 1139 -> 1115 ms, 3xTF32 3104 -> 3010).
 constexpr int PW = 16;
+__host__ __device__ __forceinline__ int64_t pair_index(int p, int q, int v) {
+  return (int64_t)p * v - (int64_t)p * (p + 1) / 2 + (q - p - 1);
+}
+// Whether the tile at (e0, f0) may hold one of the pairs q0 .. q0 + nq - 1: whether its first pair and its last one lie around
+// or among them (exact for chunks of at least v pairs).
+__host__ __device__ __forceinline__ bool tile_in_chunk(int e0, int f0, int v, int64_t q0, int64_t nq) {
+  const int f1 = f0 + PW < v ? f0 + PW - 1 : v - 1, e1 = e0 + PW - 1 < f1 ? e0 + PW - 1 : f1 - 1;
+  if (e0 >= f1) return false;
+  return pair_index(e1, f1, v) >= q0 && pair_index(e0, f0 > e0 ? f0 : e0 + 1, v) < q0 + nq;
+}
 template <int KIND, int MODE>
 __global__ void __launch_bounds__(PW *PW) pack_w(const float2 *__restrict__ W, int64_t ldw, int v, int a0, int64_t p0,
                                                  int64_t q0, int64_t nq, int64_t Kp, int seg,
@@ -68,7 +79,8 @@ __global__ void __launch_bounds__(PW *PW) pack_w(const float2 *__restrict__ W, i
   const int nt = (v + PW - 1) / PW;
   while (t >= nt - te) { t -= nt - te; ++te; }
   const int e0 = te * PW, f0 = (te + t) * PW, x = threadIdx.x & (PW - 1), y = threadIdx.x / PW;
-  auto pair = [&](int p, int q) { return (int64_t)p * v - (int64_t)p * (p + 1) / 2 + (q - p - 1); };
+  if (!tile_in_chunk(e0, f0, v, q0, nq)) return;
+  auto pair = [&](int p, int q) { return pair_index(p, q, v); };
   const int nb = min(PW, v - b0);
   const float2 *Wa = W + (int64_t)(a - a0) * v;
   float2 w[PW];
@@ -223,6 +235,23 @@ std::vector<int2> pairs(int n) {
 int64_t pair_start(int v, int a) { return (int64_t)a * v - (int64_t)a * (a + 1) / 2; }
 
 }  // namespace
+
+void ladder_pack_tiles(int v, int64_t q0, int64_t nq, int64_t *out) {
+  out[0] = out[1] = out[2] = 0;
+  for (int e0 = 0; e0 < v; e0 += PW)
+    for (int f0 = e0; f0 < v; f0 += PW) {
+      const bool read = tile_in_chunk(e0, f0, v, q0, nq);
+      bool holds = false;
+      for (int e = e0; e < std::min(v, e0 + PW); ++e)
+        for (int f = std::max(f0, e + 1); f < std::min(v, f0 + PW); ++f) {
+          const int64_t q = pair_index(e, f, v);
+          holds = holds || (q >= q0 && q < q0 + nq);
+        }
+      out[0] += read;
+      out[1] += holds;
+      out[2] += holds && !read;
+    }
+}
 
 void ladder_unpack_sig_bench(int o, int v, const void *S, void *out, cudaStream_t st) {
   static thread_local DevBuf opairs, vpairs;

@@ -15,6 +15,9 @@ namespace cclr {
 // Times nothing itself: runs the ladder's result scatter (unpack_sig) once on a packed result S
 // [(a<b)][(i<j)] (complex64) into out [o][o][v][v] (complex64), with its own pair tables (for the
 // HBM kernel benchmark).
+// The tiles of (e, f) that the packing of the pairs q0 .. q0 + nq - 1 reads, those that hold one of them, and those that hold
+// one and are not read.
+void ladder_pack_tiles(int v, int64_t q0, int64_t nq, int64_t *out);
 void ladder_unpack_sig_bench(int o, int v, const void *S, void *out, cudaStream_t st);
 
 class LadderTC {
