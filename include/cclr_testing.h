@@ -83,6 +83,9 @@ int cc_lr_selftest_f64gemm(int M, int N, int K, int layout, double spread, unsig
  * device call). */
 int cc_lr_selftest_pack_tiles(int v, long long q0, long long nq, long long *out);
 
+/* Sets the context's limit on the FP64 slices of one operand that are not kept (2 GiB by default; more go in chunks). */
+int cc_lr_selftest_f64_operand_cap(cclr_ctx *ctx, long long bytes);
+
 /* One constant complex128 operand, its slices kept, in two contractions whose results are laid out differently, so that
  * they cut it into other chunks; the second one under a memory budget that leaves no room for more slices.  err[0], err[1]:
  * the largest error of each against host sums, over the largest entry. */

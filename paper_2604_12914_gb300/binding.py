@@ -94,6 +94,7 @@ def load(path: str = LIB_PATH):
         "cc_lr_bench_hbm": [I, I, I, P, I],
         "cc_lr_selftest_timeout": [I, ctypes.POINTER(ctypes.c_int)],
         "cc_lr_selftest_f64gemm": [I, I, I, I, D, ctypes.c_uint, P],
+        "cc_lr_selftest_f64_operand_cap": [P, ctypes.c_longlong],
         "cc_lr_selftest_pack_tiles": [I, ctypes.c_longlong, ctypes.c_longlong, P],
         "cc_lr_selftest_f64_kept": [ctypes.c_uint, P],
         "cc_lr_selftest_f64_scratch": [ctypes.c_longlong, ctypes.c_longlong, ctypes.POINTER(ctypes.c_ulonglong)],
@@ -428,6 +429,11 @@ def cc_lr_selftest_f64gemm(M, N, K, layout=0, spread=0.0, seed=1):
     out = np.zeros(2, dtype=np.float64)
     _check(load().cc_lr_selftest_f64gemm(M, N, K, layout, float(spread), seed, _ptr(out)))
     return float(out[0]), float(out[1])
+
+
+def cc_lr_selftest_f64_operand_cap(ctx, size):
+    """Limits the FP64 slices of one operand of the context that are not kept to size bytes."""
+    _check(load().cc_lr_selftest_f64_operand_cap(ctx._h, int(size)))
 
 
 def cc_lr_selftest_pack_tiles(v, q0, nq):

@@ -1968,6 +1968,12 @@ int cc_lr_selftest_f64gemm(int M, int N, int K, int layout, double spread, unsig
   });
 }
 
+int cc_lr_selftest_f64_operand_cap(cclr_ctx *c, long long bytes) {
+  if (!c || bytes < 1) return fail(CCLR_EINVAL, "bad selftest_f64_operand_cap arguments");
+  c->M->E.f64_operand_cap = bytes;
+  return CCLR_OK;
+}
+
 int cc_lr_selftest_pack_tiles(int v, long long q0, long long nq, long long *out) {
   if (v < 2 || q0 < 0 || nq < 1 || q0 + nq > (long long)v * (v - 1) / 2 || !out)
     return fail(CCLR_EINVAL, "bad selftest_pack_tiles arguments");

@@ -469,27 +469,34 @@ Engine::PrepEntry *Engine::f64_keep(const std::string &key, size_t bytes) {
   return f64_kept_.back().get();
 }
 
-F64Op Engine::f64_operand(int slot, const void *src, View2 rv, View2 kv, int64_t R, int64_t K, bool embed,
-                          const std::string &key) {
+bool Engine::f64_kept(const void *src, View2 rv, View2 kv, int64_t R, int64_t K, bool embed, const std::string &key, F64Op &op) {
   const size_t sl = ((size_t)f64tc_bytes(R, K, embed) + 255) / 256 * 256, need = sl + (size_t)R * 4;
   if (!key.empty()) {
     PrepEntry *e = f64_keep(key, need);
     if (e && e->filled) {
-      F64Op op;
       op.p = e->buf.p;
       op.tops = (const uint32_t *)((const char *)e->buf.p + sl);
       op.stride = R;
+      op.r0 = 0;
       op.src = src;
       op.rv = rv;
       op.kv = kv;
-      return op;
+      return true;
     }
     if (e) {
-      const F64Op op = f64tc_prep(src, rv, kv, R, K, embed, e->buf.p, (uint32_t *)((char *)e->buf.p + sl), st);
+      op = f64tc_prep(src, rv, kv, R, K, embed, e->buf.p, (uint32_t *)((char *)e->buf.p + sl), st);
       e->filled = true;
-      return op;
+      return true;
     }
   }
+  return false;
+}
+
+F64Op Engine::f64_operand(int slot, const void *src, View2 rv, View2 kv, int64_t R, int64_t K, bool embed,
+                          const std::string &key) {
+  F64Op op;
+  if (f64_kept(src, rv, kv, R, K, embed, key, op)) return op;
+  const size_t sl = ((size_t)f64tc_bytes(R, K, embed) + 255) / 256 * 256;
   f64_reserve(slot, R, K, embed);
   char *b = (char *)f64_slots_[slot].p;
   return f64tc_prep(src, rv, kv, R, K, embed, b, (uint32_t *)(b + sl), st);
@@ -503,10 +510,10 @@ void Engine::f64_scratch(int64_t M, int64_t N) {
 }
 
 void Engine::f64_gemm(const F64Op &A, int64_t M, const F64Op &B, int64_t N, int64_t K, void *C, View2 rv, View2 cv, zc alpha,
-                      bool accumulate, UpperTiles *upper) {
+                      bool accumulate, UpperTiles *upper, int64_t upper_row, int64_t upper_col) {
   CCLR_REQUIRE(f64_scr_.bytes >= f64tc_scratch_bytes(M, N), "f64_gemm: no room claimed for the sums");
   tc_pending = true;
-  f64tc_gemm(A, M, B, N, K, C, rv, cv, alpha, accumulate, f64_scr_.p, f64_side_, st, upper);
+  f64tc_gemm(A, M, B, N, K, C, rv, cv, alpha, accumulate, f64_scr_.p, f64_side_, st, upper, upper_row, upper_col);
 }
 
 void Engine::check_tc() {

@@ -120,11 +120,13 @@ class Engine {
   // clear_prep_cache() like the other constant operands (at most f64_cache_cap bytes).  Throws status 2.
   F64Op f64_operand(int slot, const void *src, View2 rv, View2 kv, int64_t R, int64_t K, bool embed,
                     const std::string &key);
+  // the kept slices of an operand (made here if there is room to keep them); false, and nothing done, where there is none
+  bool f64_kept(const void *src, View2 rv, View2 kv, int64_t R, int64_t K, bool embed, const std::string &key, F64Op &op);
   // room for the sums of f64tc_gemms of up to M x N (throws status 2), and a product itself on this engine's stream; the
   // room has to be claimed before: nothing is allocated, and so nothing can fail, between the products of a call
   void f64_scratch(int64_t M, int64_t N);
   void f64_gemm(const F64Op &A, int64_t M, const F64Op &B, int64_t N, int64_t K, void *C, View2 rv, View2 cv, zc alpha,
-                bool accumulate, UpperTiles *upper = nullptr);
+                bool accumulate, UpperTiles *upper = nullptr, int64_t upper_row = 0, int64_t upper_col = 0);
   // Throws status 5 if a tensor-core kernel launched since the last check gave up on a bounded wait
   // (synchronises the stream; nothing is done when none was launched).
   void check_tc();
@@ -132,7 +134,7 @@ class Engine {
   // claims workspace slot `slot` for R rows of K entries.  Throws status 2.
   void f64_reserve(int slot, int64_t R, int64_t K, bool embed);
   size_t f64_cache_cap = 0;
-  int64_t f64_operand_cap = 2ll << 30;  // bytes of one operand's slices in contract_f64: in chunks above that
+  int64_t f64_operand_cap = 2ll << 30;  // bytes of an operand's slices that are not kept: in chunks above that
   // Holds off f64_reclaim() while prepared slices are in use on the host side.
   struct F64Hold {
     Engine &e;

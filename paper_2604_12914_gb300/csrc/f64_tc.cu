@@ -1102,7 +1102,8 @@ size_t f64tc_scratch_bytes(int64_t M, int64_t N) {
 }
 
 void f64tc_gemm(const F64Op &A, int64_t M, const F64Op &B, int64_t N, int64_t K, void *C, View2 rv, View2 cv, zc alpha,
-                bool accumulate, void *scratch, F64Side &side, cudaStream_t st, UpperTiles *upper) {
+                bool accumulate, void *scratch, F64Side &side, cudaStream_t st, UpperTiles *upper,
+                int64_t upper_row, int64_t upper_col) {
   if (M <= 0 || N <= 0 || K <= 0) return;
   CCLR_REQUIRE(A.r0 + M <= A.stride && B.r0 + N <= B.stride, "f64tc_gemm: rows outside the prepared operand");
   CCLR_REQUIRE((uintptr_t)A.p % 16 == 0 && (uintptr_t)B.p % 16 == 0, "f64tc_gemm: operands must be 16-byte aligned");
@@ -1158,8 +1159,9 @@ void f64tc_gemm(const F64Op &A, int64_t M, const F64Op &B, int64_t N, int64_t K,
       o.ntiles = (int)tiles;
       p.list = o.list = nullptr;
       if (upper && all > SPLIT_TILES) {  // (a product with few tiles splits K instead)
-        o.list = upper->get(p.nMt, p.nNt, 12, BM, pl.BN / 2, o.m0, o.n0, M, st, &o.ntiles);
-        p.list = pair ? upper->get(p.uMt, p.nNt, p.band, 2 * BM, pl.BN / 2, o.m0, o.n0, M, st, &p.ntiles) : o.list;
+        const int64_t um = upper_row + o.m0, un = upper_col + o.n0;
+        o.list = upper->get(p.nMt, p.nNt, 12, BM, pl.BN / 2, um, un, upper_row + M, st, &o.ntiles);
+        p.list = pair ? upper->get(p.uMt, p.nNt, p.band, 2 * BM, pl.BN / 2, um, un, upper_row + M, st, &p.ntiles) : o.list;
         if (!pair && o.list) p.ntiles = o.ntiles;
         if (!p.list || !o.list) {
           p.list = o.list = nullptr;

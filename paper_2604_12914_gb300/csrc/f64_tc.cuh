@@ -74,9 +74,11 @@ class F64Side {
 // C(m, n) (+)= alpha sum_k A(m, k) B(k, n), complex128, from prepared operands (A: M rows, B: N embedded
 // columns).  C(m, n) at C + v2off(rv, m) + v2off(cv, n) complex entries; accumulate: added to C, else C is
 // overwritten.  scratch: f64tc_scratch_bytes of device memory for the integer sums (at most 256 MB), of M and N or of
-// any larger numbers of rows and columns.
+// any larger numbers of rows and columns.  upper: only tiles with an entry b > a are needed, counting the rows (b, f) from
+// upper_row and the columns (a, e) from upper_col.
 void f64tc_gemm(const F64Op &A, int64_t M, const F64Op &B, int64_t N, int64_t K, void *C, View2 rv, View2 cv, zc alpha,
-                bool accumulate, void *scratch, F64Side &side, cudaStream_t st, class UpperTiles *upper = nullptr);
+                bool accumulate, void *scratch, F64Side &side, cudaStream_t st, class UpperTiles *upper = nullptr,
+                int64_t upper_row = 0, int64_t upper_col = 0);
 size_t f64tc_scratch_bytes(int64_t M, int64_t N);
 
 }  // namespace cclr

@@ -139,18 +139,33 @@ void LadderCC::apply(Engine &E, int dt, const Tens &Lvv, int o, int v, int naux,
   Engine::F64Hold hold(E);
   bool tc = f64 && (double)naux * Pv * vv >= 2.0e7 && Pv < (1ll << 26) && NR * Po < (1ll << 26) && vv < (1ll << 26);
   F64Op La, Lb, Xo;
+  // L~ rows (b,f) and embedded columns (a,e), K = naux: whole and kept while L~_vv stands, where they fit among the kept
+  // operands of an unbudgeted context; else made again for every group, in chunks of lrows rows and lcols columns
+  bool keep_a = false, keep_b = false;
+  int64_t lrows = vv, lcols = (int64_t)ga * v;
+  // the packed block's slices, in chunks of its rows (a,b) or, in the transpose, of its columns (e,f); the packed vectors' are
+  // whole (4.5 times the vectors)
+  int64_t wpart = dir > 0 ? maxpairs : Pv;
   if (tc) {
     try {
       char hint[64];
       std::snprintf(hint, sizeof hint, "ladder|%p|%d|%d|", Lvv.p, v, naux);
-      // L~ rows (b,f) and embedded columns (a,e), K = naux; kept while L~_vv stands, in unbudgeted contexts
-      La = E.f64_operand(2, Lvv.p, view1(1), view1(vv), vv, naux, false, std::string(hint) + "A");
-      Lb = E.f64_operand(3, Lvv.p, view1(1), view1(vv), vv, naux, true, std::string(hint) + "B");
+      keep_a = E.f64_kept(Lvv.p, view1(1), view1(vv), vv, naux, false, std::string(hint) + "A", La);
+      keep_b = E.f64_kept(Lvv.p, view1(1), view1(vv), vv, naux, true, std::string(hint) + "B", Lb);
+      if (!keep_a) {
+        lrows = std::min(lrows, std::max<int64_t>(1, E.f64_operand_cap / f64tc_bytes(1, naux, false)));
+        E.f64_reserve(2, lrows, naux, false);
+      }
+      if (!keep_b) {
+        lcols = std::min(lcols, std::max<int64_t>(1, E.f64_operand_cap / f64tc_bytes(1, naux, true)));
+        E.f64_reserve(3, lcols, naux, true);
+      }
       E.f64_scratch((int64_t)v * v, (int64_t)ga * v);
       if (dir > 0) E.f64_scratch(maxpairs, NR * Po);
       else E.f64_scratch(NR * Po, Pv);
-      // the packed block's and the packed vectors' slices for the largest group
-      E.f64_reserve(4, dir > 0 ? maxpairs : Pv, dir > 0 ? Pv : maxpairs, dir < 0);
+      const int64_t wk = dir > 0 ? Pv : maxpairs;
+      wpart = std::min(wpart, std::max<int64_t>(1, E.f64_operand_cap / f64tc_bytes(1, wk, dir < 0)));
+      E.f64_reserve(4, wpart, wk, dir < 0);
       E.f64_reserve(5, NR * Po, dir > 0 ? Pv : maxpairs, dir > 0);
     } catch (const Error &e) {
       if (e.status != 2) throw;
@@ -179,8 +194,20 @@ void LadderCC::apply(Engine &E, int dt, const Tens &Lvv, int o, int v, int naux,
     // formation: W[(b - a0, f)][(a - a0, e)] = sum_P L[P,b,f] L[P,a,e], b >= a0
     const int64_t rows = (int64_t)(v - a0) * v, cols = (int64_t)(a1 - a0) * v;
     if (tc) {
-      E.f64_gemm(La.rows((int64_t)a0 * v), rows, Lb.rows((int64_t)a0 * v), cols, naux, W.p, view1(cols), view1(1), zc(1.0),
-                 false, &upper_);
+      const int64_t first = (int64_t)a0 * v;
+      auto chunk = [&](bool b, int64_t at, int64_t n) {  // L~ rows or columns first + at ..
+        return E.f64_operand(b ? 3 : 2, (const char *)Lvv.p + (first + at) * es, view1(1), view1(vv), n, naux, b, "");
+      };
+      for (int64_t c0 = 0; c0 < cols; c0 += lcols) {
+        const int64_t nc = std::min(lcols, cols - c0);
+        const F64Op lb = keep_b ? Lb.rows(first + c0) : chunk(true, c0, nc);
+        for (int64_t m0 = 0; m0 < rows; m0 += lrows) {
+          const int64_t nr = std::min(lrows, rows - m0);
+          const F64Op la = keep_a ? La.rows(first + m0) : chunk(false, m0, nr);
+          E.f64_gemm(la, nr, lb, nc, naux, (char *)W.p + (m0 * cols + c0) * es, view1(cols), view1(1), zc(1.0), false, &upper_, m0,
+                     c0);
+        }
+      }
     } else {
       GemmArgs g;
       g.A = (const char *)Lvv.p + (size_t)a0 * v * es;
@@ -201,8 +228,11 @@ void LadderCC::apply(Engine &E, int dt, const Tens &Lvv, int o, int v, int naux,
     if (dir > 0) {
       // sig[(ab)][(r, ij)] = sum_{e<f} <ab||ef>~ X_r[i,j,e,f] for the group's pairs
       if (tc) {
-        const F64Op wo = E.f64_operand(4, Wp.p, view1(Pv), view1(1), np, Pv, false, "");
-        E.f64_gemm(wo, np, Xo, NR * Po, Pv, (char *)sig.p + (size_t)p0 * NR * Po * es, view1(NR * Po), view1(1), zc(1.0), false);
+        for (int64_t m0 = 0; m0 < np; m0 += wpart) {
+          const int64_t nr = std::min(wpart, np - m0);
+          const F64Op wo = E.f64_operand(4, (char *)Wp.p + m0 * Pv * es, view1(Pv), view1(1), nr, Pv, false, "");
+          E.f64_gemm(wo, nr, Xo, NR * Po, Pv, (char *)sig.p + (p0 + m0) * NR * Po * es, view1(NR * Po), view1(1), zc(1.0), false);
+        }
         continue;
       }
       GemmArgs c;
@@ -226,8 +256,11 @@ void LadderCC::apply(Engine &E, int dt, const Tens &Lvv, int o, int v, int naux,
       // Z[(r, ij)][(ef)] += sum_{(ab) in group} Y'_r[(ij)][(ab)] <ab||ef>~
       if (tc) {
         const F64Op yo = E.f64_operand(5, Xp.p, view1(np), view1(1), NR * Po, np, false, "");
-        const F64Op wo = E.f64_operand(4, Wp.p, view1(1), view1(Pv), Pv, np, true, "");
-        E.f64_gemm(yo, NR * Po, wo, Pv, np, sig.p, view1(Pv), view1(1), zc(1.0), true);
+        for (int64_t q0 = 0; q0 < Pv; q0 += wpart) {
+          const int64_t nq = std::min(wpart, Pv - q0);
+          const F64Op wo = E.f64_operand(4, (char *)Wp.p + q0 * es, view1(1), view1(Pv), nq, np, true, "");
+          E.f64_gemm(yo, NR * Po, wo, nq, np, (char *)sig.p + q0 * es, view1(Pv), view1(1), zc(1.0), true);
+        }
         continue;
       }
       GemmArgs c;
