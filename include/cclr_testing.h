@@ -52,7 +52,7 @@ int cc_lr_bench_hbm(int o, int v, int reps, double *out, int n);
  *   tensor-core operands and the bounded-wait flag) lives in one file-scope device array of
  *   CCLR_SELFTEST_NOALLOC_SCRATCH_BYTES; sizes that do not fit return CCLR_EINVAL (1) and a
  *   message naming the bytes needed (cc_lr_last_error).  About 24(MK + KN) + 32MN +
- *   8(M + 2N)(K + 1)s bytes are needed, s = 1 for TF32 and 2 for 3xTF32; M = N = K = 384
+ *   8(M + 2N)(K + 1)s bytes are needed (rows take whole 128-byte blocks where there is room, K + 7 on average), s = 1 for TF32 and 2 for 3xTF32; M = N = K = 384
  *   fits with 3xTF32.  Nothing is allocated: no cudaMalloc, no cudaFree, no allocating
  *   library routine; host staging uses fixed stack buffers.
  *   Set-up: the first call on each device (with that device current) looks the array up with

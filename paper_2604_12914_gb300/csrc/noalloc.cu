@@ -70,9 +70,11 @@ struct Layout {
   int64_t ld;
 };
 
-Layout plan(int64_t M, int64_t N, int64_t K, int seg) {
+// Operand rows as the library prepares them (whole 128-byte K blocks from K = 64 on); of whole 16-byte units where those
+// would not fit.
+Layout plan(int64_t M, int64_t N, int64_t K, int seg, bool blocks = true) {
   Layout l;
-  l.ld = 2 * tc_kpad(K) * seg;
+  l.ld = 2 * (blocks ? tc_kpad(K, TC_TF32) : tc_kpad(K)) * seg;
   size_t off = 0;
   auto take = [&](size_t bytes) {
     const size_t at = off;
@@ -90,6 +92,7 @@ Layout plan(int64_t M, int64_t N, int64_t K, int seg) {
   l.ao = take((size_t)M * l.ld * 4);
   l.bo = take((size_t)2 * N * l.ld * 4);
   l.total = off;
+  if (blocks && off > (size_t)CCLR_SELFTEST_NOALLOC_SCRATCH_BYTES) return plan(M, N, K, seg, false);
   return l;
 }
 
@@ -167,7 +170,7 @@ extern "C" int cc_lr_selftest_gemm_noalloc(int M, int N, int K, int mode, unsign
     tc_prep_a(at(l.a64), K, 1, M, K, seg, TC_TF32, at(l.ao), l.ld, s);
     tc_prep_b(at(l.b64), N, 1, K, N, seg, TC_TF32, at(l.bo), l.ld, s);
     tc_gemm_seg_flagged((const float *)at(l.ao), l.ld, (const float *)at(l.bo), l.ld, M, 2 * (int64_t)N,
-                        2 * tc_kpad(K), seg, (float *)at(l.ct), 2 * (int64_t)N, zc(1.0), true, (int *)at(l.flag), s);
+                        l.ld / seg, seg, (float *)at(l.ct), 2 * (int64_t)N, zc(1.0), true, (int *)at(l.flag), s);
     gemm_plain(C64, at(l.a64), at(l.b64), at(l.cs), M, N, K, s);  // FP32 CUDA cores
     int flag = 0;
     CCLR_CUDA(cudaMemcpyAsync(&flag, at(l.flag), sizeof(int), cudaMemcpyDeviceToHost, s));
