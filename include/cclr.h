@@ -263,7 +263,7 @@ cclr_status cc_lr_set_solver(cclr_ctx *ctx, int method, int subspace, int max_it
 
 /* Tensor-core GEMM tile autotuner (on by default): the first eager use of each GEMM shape
  * (operand type, M, N, K, output layout) on a device times a handful of launch configurations
- * -- tile width, K splits, raster band -- around the rules' choice on the real operands (an
+ * -- tile width, K splits, raster band, single CTAs or pairs -- around the rules' choice on the real operands (an
  * accumulated output is tuned into a scratch block) and keeps the fastest for that shape and
  * device; later products, and other contexts on the device, launch it.  on = 0: untuned shapes
  * keep the rules. */
@@ -271,8 +271,11 @@ cclr_status cc_lr_set_autotune(cclr_ctx *ctx, int on);
 
 /* The tuned GEMM shapes of the current device: writes *n (the number of shapes) and the first
  * min(*n, cap) rows of 10 doubles (operand type 0 TF32 / 1 BF16, M, N, K (real elements), tile
- * width, K splits, raster band, best milliseconds, the rules' milliseconds, candidates timed). */
+ * width, K splits, raster band, best milliseconds, the rules' milliseconds, candidates timed).
+ * cc_lr_gemm_tuning_pairs writes one int per shape, in the same order: 1 where the shape runs by pairs of CTAs
+ * on tiles of 256 rows, 0 where by single CTAs on tiles of 128 rows; the raster band counts rows of those tiles. */
 cclr_status cc_lr_gemm_tuning(cclr_ctx *ctx, int cap, int *n, double *rec);
+cclr_status cc_lr_gemm_tuning_pairs(cclr_ctx *ctx, int cap, int *n, int *pair);
 
 /* Device memory held by the context now (*in_use), the most it has held (*peak), and its
  * budget (*budget, 0 = none), in bytes.  Host-side bookkeeping only (no device call). */

@@ -26,7 +26,7 @@ EXPORTS = ["cc_lr_init", "cc_lr_sigma", "cc_lr_sigma_T", "cc_lr_sigma_packed", "
            "cc_lr_lambda", "cc_lr_get_t", "cc_lr_ccsd_residual", "cc_lr_ccsd", "cc_lr_set_precision", "cc_lr_set_refinement", "cc_lr_set_graphs",
            "cc_lr_graph_stats", "cc_lr_ladder_tuning", "cc_lr_set_ladder_storage", "cc_lr_set_solver",
            "cc_lr_last_timings", "cc_lr_memory", "cc_lr_set_autotune", "cc_lr_gemm_tuning",
-           "cc_lr_free", "cc_lr_strerror", "cc_lr_last_error", "cc_lr_launch_count"]
+           "cc_lr_gemm_tuning_pairs", "cc_lr_free", "cc_lr_strerror", "cc_lr_last_error", "cc_lr_launch_count"]
 
 
 class CclrError(RuntimeError):
@@ -84,6 +84,7 @@ def load(path: str = LIB_PATH):
         "cc_lr_memory": [P, ctypes.POINTER(S), ctypes.POINTER(S), ctypes.POINTER(S)],
         "cc_lr_set_autotune": [P, I],
         "cc_lr_gemm_tuning": [P, I, ctypes.POINTER(ctypes.c_int), P],
+        "cc_lr_gemm_tuning_pairs": [P, I, ctypes.POINTER(ctypes.c_int), P],
         "cc_lr_free": [P],
         "cc_lr_strerror": [I],
         "cc_lr_last_error": [],
@@ -363,6 +364,15 @@ class Context:
         _check(load().cc_lr_gemm_tuning(self._h, cap, ctypes.byref(n), _ptr(rec)))
         keys = ["kind", "M", "N", "K", "BN", "splits", "band", "ms_best", "ms_rule", "tried"]
         return [dict(zip(keys, map(float, rec[k]))) for k in range(min(n.value, cap))]
+
+    def cc_lr_gemm_tuning_pairs(self):
+        """For every row of cc_lr_gemm_tuning(): whether the shape runs by pairs of CTAs on 256-row tiles."""
+        n = ctypes.c_int(0)
+        _check(load().cc_lr_gemm_tuning_pairs(self._h, 0, ctypes.byref(n), None))
+        cap = max(1, n.value)
+        pair = np.zeros(cap, dtype=np.int32)
+        _check(load().cc_lr_gemm_tuning_pairs(self._h, cap, ctypes.byref(n), _ptr(pair)))
+        return [bool(k) for k in pair[:min(n.value, cap)]]
 
     def cc_lr_memory(self):
         """(bytes held, peak bytes held, budget) of this context's device memory."""

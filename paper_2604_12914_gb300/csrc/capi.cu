@@ -1813,7 +1813,12 @@ cclr_status cc_lr_set_autotune(cclr_ctx *c, int on) {
 
 cclr_status cc_lr_gemm_tuning(cclr_ctx *c, int cap, int *n, double *rec) {
   if (!c || !n || cap < 0 || (cap > 0 && !rec)) return (cclr_status)fail(CCLR_EINVAL, "bad gemm_tuning arguments");
-  return (cclr_status)guarded_ctx(c, [&] { *n = tc_tuning_table(cap, rec); });
+  return (cclr_status)guarded_ctx(c, [&] { *n = tc_tuning_table(cap, rec, nullptr); });
+}
+
+cclr_status cc_lr_gemm_tuning_pairs(cclr_ctx *c, int cap, int *n, int *pair) {
+  if (!c || !n || cap < 0 || (cap > 0 && !pair)) return (cclr_status)fail(CCLR_EINVAL, "bad gemm_tuning_pairs arguments");
+  return (cclr_status)guarded_ctx(c, [&] { *n = tc_tuning_table(cap, nullptr, pair); });
 }
 
 cclr_status cc_lr_memory(cclr_ctx *c, size_t *in_use, size_t *peak, size_t *budget) {

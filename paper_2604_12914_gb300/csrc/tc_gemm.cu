@@ -1358,12 +1358,13 @@ CUtensorMap tc_make_map(const void *base, int64_t rows, int64_t cols, int64_t ld
 
 void tc_set_autotune(bool on) { g_tune_on = on; }
 
-int tc_tuning_table(int cap, double *rec) {
+int tc_tuning_table(int cap, double *rec, int *pair) {
   const int dev = current_device();
   std::lock_guard<std::mutex> lock(g_tune_mu);
   int n = 0;
   for (const auto &kv : g_tune) {
     if (kv.first.dev != dev) continue;
+    if (n < cap && pair) pair[n] = kv.second.cfg.pair ? 1 : 0;
     if (n < cap && rec) {
       double *r = rec + 10 * n;
       const TuneKey &k = kv.first;

@@ -203,8 +203,9 @@ int64_t tc_magnitude_sums_cap();
 // and device; later uses launch the cached configuration.  Never tunes inside a stream capture.
 void tc_set_autotune(bool on);
 // Rows of 10 doubles per tuned shape of the current device (kind, M, N, K, BN, splits, band,
-// best ms, the rule's ms, candidates timed), up to cap rows; returns the number of shapes.
-int tc_tuning_table(int cap, double *rec);
+// best ms, the rule's ms, candidates timed), up to cap rows, and whether pairs of CTAs run it (either may be nullptr);
+// returns the number of shapes.
+int tc_tuning_table(int cap, double *rec, int *pair);
 
 // For kernels of other translation units: the current device's bounded-wait flag (the first use on a device
 // sets it up and fetches the tensor-map encoder), its SM count, and the 2-D tensor map of a row-major operand
