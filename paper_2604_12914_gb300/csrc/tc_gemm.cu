@@ -1004,10 +1004,11 @@ thread_local bool g_tune_on = false;
 
 // a_cols: operand elements A actually holds per row (<= Kreal; the rest reads as zero).
 // lda, ldb, Kreal in elements of the operand type; split: rows of two segments (hi, lo) of Kreal elements.  cfg
-// overrides the rules; *used receives the configuration launched.
+// overrides the rules; *used receives the configuration launched.  prepare: makes the list of tiles of that configuration if
+// there is none yet, and launches nothing (the list is allocated and copied, which a timed launch should not contain).
 static void tc_launch(const void *A, int64_t lda, const void *B, int64_t ldb, int64_t M, int64_t Nreal, int64_t Kreal,
                       int kind, bool split, float *C, View2 rv, View2 cv, zc alpha, bool accumulate, int *err,
-                      cudaStream_t st, int64_t a_cols, TcCfg cfg, TcCfg *used, UpperTiles *upper) {
+                      cudaStream_t st, int64_t a_cols, TcCfg cfg, TcCfg *used, UpperTiles *upper, bool prepare = false) {
   const int64_t es = tc_esize(kind), BK = BKB / es;
   const int nk = (int)((Kreal + BK - 1) / BK), nsm = num_sms();
   // K splits need an accumulating or plain output (split partial tiles are added atomically)
@@ -1051,13 +1052,14 @@ static void tc_launch(const void *A, int64_t lda, const void *B, int64_t ldb, in
   p.atomic = splits > 1 ? 1 : 0;
   p.accumulate = (accumulate || splits > 1) ? 1 : 0;
   p.err = err;
+  p.ntiles = (int)tiles;
+  p.list = upper ? upper->get(p.nMt, p.nNt, p.band, rows, BN / 2, 0, 0, M, st, &p.ntiles) : nullptr;
+  if (prepare) return;
   if (splits > 1 && !accumulate) {
     CCLR_REQUIRE(rv.din == TC_ONE_LEVEL && cv.din == TC_ONE_LEVEL && cv.sin == 1,
                  "tc_gemm: split K without accumulation needs a plain C layout");
     CCLR_CUDA(cudaMemset2DAsync(C, (size_t)rv.sin * 8, 0, (size_t)Nreal * 4, (size_t)M, st));
   }
-  p.ntiles = (int)tiles;
-  p.list = upper ? upper->get(p.nMt, p.nNt, p.band, rows, BN / 2, 0, 0, M, st, &p.ntiles) : nullptr;
   const int64_t units = (int64_t)p.ntiles * splits;
   CCLR_REQUIRE(units < (1ll << 31), "tc_gemm: too many work units");
   static const bool trace = std::getenv("CCLR_TRACE") && std::getenv("CCLR_TRACE")[0] == '1';
@@ -1236,6 +1238,8 @@ static void tc_gemm_core(const void *A, int64_t lda, const void *B, int64_t ldb,
       const bool plain = trv.din == TC_ONE_LEVEL && tcv.din == TC_ONE_LEVEL && tcv.sin == 1;
       for (const TcCfg &cand : candidates(rule, M, Nreal, Kreal, kind, accumulate || plain, split)) {
         TcCfg used;
+        tc_launch(A, lda, B, ldb, M, Nreal, Kreal, kind, split, Ct, trv, tcv, alpha, false, err, st, a_cols, cand, nullptr,
+                  upper, true);
         CCLR_CUDA(cudaEventRecord(e0, st));
         tc_launch(A, lda, B, ldb, M, Nreal, Kreal, kind, split, Ct, trv, tcv, alpha, false, err, st, a_cols,
                   cand, &used, upper);
