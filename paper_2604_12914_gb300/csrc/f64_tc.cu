@@ -1049,7 +1049,7 @@ F64Plan plan_of(int64_t M, int64_t N, size_t cap) {
 int64_t splits_of(int64_t all_tiles, int64_t units, int slots, int n) {
   return all_tiles > SPLIT_TILES ? 1 : std::max<int64_t>(1, std::min<int64_t>(slots / units, n / 2));
 }
-constexpr size_t SUMS_CAP = 240u << 20;  // the most that the integer sums of one launch take
+constexpr size_t SUMS_CAP = 250u << 20;  // the most that the integer sums of one launch take
 
 }  // namespace
 
@@ -1091,14 +1091,13 @@ F64Op f64tc_prep(const void *src, View2 rv, View2 kv, int64_t R, int64_t K, bool
 // block or chunk serves the others: a launch takes no more tiles than there are and than SUMS_CAP holds, K splits
 // no more than one unit per SM, and the width of the tiles only grows with N.  (The need of the product itself
 // is not monotone: fewer rows of tiles leave room for more columns of them.)
-static size_t sums_bytes(const F64Plan &q) {
-  return (size_t)(std::max<int64_t>(std::min<int64_t>(tiles_that_fit(q.BN, SUMS_CAP), (int64_t)q.nMt * q.nNt), tc_num_sms()) * q.unit);
-}
-// (and behind them the words of a launch's tiles, or the sums that they stand for)
+// Behind the integer sums lie the words of the launch's tiles, or the magnitudes' sums that they stand for: those are there
+// only where the tiles leave half the SMs idle, and then the integer sums take one unit per SM at most.
 size_t f64tc_scratch_bytes(int64_t M, int64_t N) {
   const F64Plan q = plan_of(M, N, SUMS_CAP);
   const int64_t tiles = std::min<int64_t>(tiles_that_fit(q.BN, SUMS_CAP), (int64_t)q.nMt * q.nNt);
-  return sums_bytes(q) + (size_t)std::max<int64_t>(tiles * (BM / 32) * (q.BN / 2) * 16, std::min<int64_t>(M * 2 * N * 4, tc_magnitude_sums_cap()));
+  const int64_t small = std::min<int64_t>(std::max<int64_t>(M, 2) * 2 * N * 4, tc_magnitude_sums_cap());
+  return (size_t)std::max<int64_t>(tiles * (q.unit + (BM / 32) * (q.BN / 2) * 16), tc_num_sms() * q.unit + small);
 }
 
 void f64tc_gemm(const F64Op &A, int64_t M, const F64Op &B, int64_t N, int64_t K, void *C, View2 rv, View2 cv, zc alpha,
@@ -1137,7 +1136,6 @@ void f64tc_gemm(const F64Op &A, int64_t M, const F64Op &B, int64_t N, int64_t K,
   o.bkv = B.kv;
   o.tau = (float)std::sqrt(2.0 * (double)K) * 0x1p-8f;
   const int64_t ld = f64tc_ld(K);
-  void *small = (char *)scratch + sums_bytes(pl);
   const int nk = (int)((2 * K + KC - 1) / KC);
   p.K = (int)(2 * K);
   for (int t0 = 0; t0 < pl.nNt; t0 += pl.cols)
@@ -1170,6 +1168,8 @@ void f64tc_gemm(const F64Op &A, int64_t M, const F64Op &B, int64_t N, int64_t K,
         }
       }
       {
+        // behind the integer sums of as many K splits as any segment of K below takes
+        void *small = (char *)scratch + tiles * splits_of(all, (int64_t)p.uMt * p.nNt, slots, std::min(nk, MAX_CHUNKS)) * pl.unit;
         const int64_t mm = std::min<int64_t>(M - o.m0, (int64_t)p.nMt * BM);
         o.ldw = std::min<int64_t>(N - o.n0, (int64_t)p.nNt * (pl.BN / 2));
         const bool words = tc_magnitude_sums((const char *)A.p + ((int64_t)S * p.sA + p.rA) * ld * 2, ld,
