@@ -3,7 +3,8 @@
 // This GPU's FP64 pipe does two FMAs per clock and SM, so a complex GEMM on it stops near 1 TFLOP/s.  The
 // 36 BF16 slice products (orders q <= 7) cost 36 times a BF16 GEMM and still leave some 25 times more.
 // Measured (GEMM and output kernel, operands sliced): M = N = K = 1760 complex 1.24 ms (35 TFLOP/s, 1270 TFLOP/s of
-// BF16 MMAs) against 42 ms on the FP64 pipe; 12100 x 1760 x 500 2.6 ms against 90; 400^3 44 us against 617.
+// BF16 MMAs) against 42 ms on the FP64 pipe; 12100 x 1760 x 500 2.67 ms against 90; 400^3 49 us against 617 (44 without the
+// comparison of the magnitudes, which runs beside the slice products).
 // What bounds it: MMAs alone (never waiting for the epilogue) 0.89 ms at 1760^3; handing each sum to the epilogue and
 // its accumulator back, 0.99 ms; with the epilogue's integer work, 1.24 ms.  With chunks of 32 real K (eight sums per
 // chunk, each of its own order) and 128-row tiles by single CTAs it was 1.09, 1.5 and 1.81 ms: twice as many sums to
@@ -508,8 +509,10 @@ __device__ __forceinline__ uint32_t small_bits(uint4 w) { return (w.z & ~w.x) | 
 __device__ __forceinline__ bool small_sum(float2 s, float tau) { return (s.x < tau && s.x != 0.f) || (s.y < tau && s.y != 0.f); }
 // The FP64 sums alpha sum_k A(row, k) B(k, n) of the entries in 32 rows from r0 on and the columns c0 + lane whose words
 // (lane by lane, the same in every warp) are not zero, which nobody else has written, by the block's 256 threads.  Many
-// short sums: a thread per entry, in the order of k.  Else up to K = 1024 a warp per entry, and beyond it the block for up
-// to four rows of a column, each thread every 32nd or 256th k and the threads' sums added up pairwise.  In the long sums
+// entries (64 of short sums, 256 of any): a thread per entry, in the order of k.  Else up to K = 1024 a warp per entry, and
+// beyond it the block for up to four rows of a column, each thread every 32nd or 256th k and the threads' sums added up
+// pairwise: few entries are bound by latency, many by the FP64 pipe, which the pairwise sums take too (all entries,
+// 1760^3: 57 ms by four rows, 37 by threads; 12100 x 1760 x 500: 96 by warps, 72; the CUDA-core kernel 42 and 90).  In the long sums
 // 32 terms that are all zero are passed over: the usual ones are those of a row or column that the difference of two equal
 // products has left, a few roundings among zeros, and the FP64 pipe bounds the loop.  (256 x 256 entries of K = 12100 with
 // 14 such rows: 0.73 ms without, 0.19 with.)  A call: inlined, it costs the conversion its registers.
@@ -526,7 +529,7 @@ __device__ __noinline__ void write_small(const F64Out &p, uint32_t word, int r0,
     return ((__double_as_longlong(z.x) | __double_as_longlong(z.y)) << 1) != 0;
   };
   const int total = __reduce_add_sync(0xffffffffu, __popc(word));
-  if (p.k1 - p.k0 <= 256 && total >= 64) {
+  if (total >= (p.k1 - p.k0 <= 256 ? 64 : 256)) {
     for (int t0 = 0; t0 < total; t0 += 256) {
       int left = t0 + thread, l = -1, n = 0;
 #pragma unroll 1
