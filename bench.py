@@ -86,7 +86,7 @@ def algorithmic(o, v, naux):
 
 # DRAM bytes (read + write) per executed FLOP of the formation GEMM: one ncu capture of one
 # formation launch of the workload (M = 28800 rows (b,f), N = 7680 complex columns (a,e),
-# K = 1200: 1.793388 GB read + 1.740861 GB written for 8 M N K = 2.1234e12 FLOP).  With K =
+# K = 1200: 2.618338 GB read + 1.743082 GB written for 8 M N K = 2.1234e12 FLOP).  With K =
 # naux fixed, both the output writes and the per-band operand reads scale with M N, so the
 # ratio carries over to every group of the same workload.
 FORMATION_BYTES_PER_FLOP = (2.618338e9 + 1.743082e9) / (8 * 28800 * 7680 * 1200)
@@ -115,7 +115,9 @@ def ladder_peak(prec):
     """Peak (TFLOP/s) of the unit the ladder runs on, and how it was obtained."""
     d, how = peaks()
     if prec in ("tf32", "3xtf32"):
-        # tf32 dense is half the bf16 dense rate (1.1 vs 2.25 PFLOP/s nominal)
+        # tf32 dense is half the bf16 dense rate (1.1 vs 2.25 PFLOP/s nominal), here of a measured
+        # cuBLAS GEMM: the tensor pipe's own rate is about a quarter higher (1210 in tf32), so a
+        # fraction near 1 of this peak is near 0.8 of the pipe
         return "tensor", d["bf16_tflops"] * (1.1 / 2.25), f"{how} bf16 x nominal tf32/bf16 ratio"
     if prec == "bf16x3":
         return "tensor", d["bf16_tflops"], f"{how} bf16"
@@ -480,8 +482,8 @@ def ground_state(cfg, scale, prec, tol, fp64_check=False):
     steps with DIIS, each residual from two intermediate builds and two sigma products (exact
     two-point Gauss-Legendre rule); wall time, residuals formed, energy, and (fp64_check) the FP64
     residual norm of the final amplitudes, an independent check that the mixed-precision solve met
-    its tolerance (at o=32 v=240 that one FP64 residual takes over a minute on this GPU's FP64
-    rate).  The Cholesky scale keeps the synthetic system weakly correlated enough for the
+    its tolerance (two FP64 sigma products of 0.90 s at o=32 v=240, and two builds of FP64
+    intermediates).  The Cholesky scale keeps the synthetic system weakly correlated enough for the
     first-order start: |Omega(T1st)| is about 500 at o=32 v=240 with s = 0.05."""
     import numpy as np
     from paper_2604_12914_gb300 import binding

@@ -45,3 +45,17 @@ def test_captured_products_with_slices():
     captures, launches = ctx.cc_lr_graph_stats()
     assert captures == 2 and launches >= 6
     ctx.close()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("M,N", [(129, 16), (129, 32), (20, 70)])
+@pytest.mark.parametrize("K", [31, 32, 33, 32768, 33001])
+def test_f64_gemm_at_chunks_and_segments_of_k(M, N, K):
+    """K around a chunk (32 complex) in tiles of 32, 64 and 128 columns, and beyond what the integer sums of one launch hold
+    (32768 complex), with ordinary entries and with graded ones; the library divides by the bound of each."""
+    if K > 30000:
+        M = min(M, 9)  # (the reference sums on the host take K per entry)
+    for layout, spread in ((0, 20.0), (35, 40.0)):
+        err, nans = binding.cc_lr_selftest_f64gemm(M, N, K, layout, spread=spread, seed=M + N + K)
+        assert err <= 1.0, (layout, err)
+        assert nans == 0
